@@ -39,12 +39,14 @@ cudaError_t film_adjoint_launch(int precision, const Desc& d, const double* v, d
                                 double* sbar, int iters, const double* g, double* gbar,
                                 double* jcbar, const double* wbar_out, double* wbar_in,
                                 cudaStream_t s);
-cudaError_t adj_warm_io(int precision, long long n, int load, const uint8_t* mask, void* hd,
+cudaError_t adj_warm_io(int precision, int nx, int ny, int load, const uint8_t* mask, void* hd,
                         double A, double* dst, const double* src, cudaStream_t s);
 cudaError_t adj_lincomb(long long n, double* out, int nt, const double* const* x, const double* c,
                         double b, cudaStream_t s);
 cudaError_t adj_sums(long long n, const double* x, double* out, cudaStream_t s);
 cudaError_t adj_to_float(long long n, const double* x, float* y, cudaStream_t s);
+cudaError_t film_to_units(int precision, int nx, int ny, const double* x, void* y, cudaStream_t s);
+cudaError_t film_relayout(int precision, int nx, int ny, bool to_rows, const void* src, void* dst, cudaStream_t s);
 }  // namespace mf
 
 namespace {
@@ -116,9 +118,9 @@ Layout layout(const mf_params* p) {
   L.q2 = take(p->dim == 2 ? L.ncell * ts : 0);
   L.jc = take(p->jc_map ? L.ncell * ts : 0);
   L.mask = take(L.ncell);
-  L.twx = take(2 * p->nx * 2 * ts);             // stage-ordered tables A and B (< 2 L entries)
-  L.twy = take(2 * p->ny * 2 * ts);
-  L.twz = take(2 * nz * 2 * ts);
+  L.twx = take(TWIDDLE_VALUES * p->nx * ts);
+  L.twy = take(TWIDDLE_VALUES * p->ny * ts);
+  L.twz = take(TWIDDLE_VALUES * nz * ts);
   const int nk = p->nx / 2 + 1 + p->ny + nz;
   L.ktab = take(nk * ts);
   L.gtab = take(nk * ts);
@@ -135,15 +137,16 @@ Layout layout(const mf_params* p) {
 }
 
 template <typename T>
-void fill_tables(const mf_params* p, double sigma, std::vector<char>& tw, std::vector<char>& kt,
+void fill_tables(const mf_params* p, const Desc& d, std::vector<char>& tw, std::vector<char>& kt,
                  std::vector<char>& gt) {
   const int nz = p->dim == 2 ? 1 : p->nz;
   const int ns[3] = {p->nx, p->ny, nz};
-  // per axis: stage-ordered twiddle tables, each block padded to 2 L complex entries
+  // per axis: twiddle tables, each block padded to TWIDDLE_VALUES L values
   std::vector<T> t;
   for (int a = 0; a < 3; ++a) {
-    std::vector<T> blk(4 * (size_t)ns[a], (T)0);
-    stage_twiddles<T>(ns[a], blk.data());
+    std::vector<T> blk(TWIDDLE_VALUES * (size_t)ns[a], (T)0);
+    if (p->dim == 3) stage_twiddles<T>(ns[a], blk.data());
+    else if (a < 2) core_twiddles<T>(ns[a], a == 0 ? d.ex : d.ey, blk.data());
     t.insert(t.end(), blk.begin(), blk.end());
   }
   tw.assign((const char*)t.data(), (const char*)(t.data() + t.size()));
@@ -157,7 +160,7 @@ void fill_tables(const mf_params* p, double sigma, std::vector<char>& tw, std::v
       if (a == 0 && i == n / 2) m = -n / 2;
       const double kv = M_PI * (double)m / Ls[a];
       k.push_back((T)kv);
-      g.push_back((T)std::exp(-kv * kv * sigma * sigma / 2.0));
+      g.push_back((T)std::exp(-kv * kv * d.sigma * d.sigma / 2.0));
     }
   }
   kt.assign((const char*)k.data(), (const char*)(k.data() + k.size()));
@@ -303,6 +306,7 @@ mf_status mf_create(const mf_params* p, void* d_workspace, size_t bytes, void* s
   d.dev = (const Desc*)(w + L.desc);
 
   // launch configuration: all CTAs co-resident, no more than the widest pass can use
+  if (p->dim == 2) { d.ex = elems_per_thread(d, d.nx); d.ey = elems_per_thread(d, d.ny); }
   const size_t smem = kernel_smem_bytes(d);
   int per_sm = p->dim == 2 ? film_max_blocks(p->precision, smem) : bulk_max_blocks(p->precision, smem);
   int nsm = 0;
@@ -315,15 +319,7 @@ mf_status mf_create(const mf_params* p, void* d_workspace, size_t bytes, void* s
   }
   const int coresident = per_sm * nsm;
   if (p->dim == 2) {
-    int rb1 = std::min(p->ny, 2 * BATCH / p->nx);
-    int rb2 = std::min(p->ny, BATCH / p->nx);
-    const int want = std::max(p->nx / 2 + 1, 1);
-    const int grid = std::min(coresident, want);
-    while (rb1 > 2 && p->ny / rb1 < grid) rb1 /= 2;
-    while (rb2 > 2 && p->ny / rb2 < grid) rb2 /= 2;
-    d.rows_per_item = rb1;
-    d.zs_per_item = rb2;
-    d.grid = std::max(1, std::min(coresident, std::max(want, p->ny / rb1)));
+    film_shape(d, coresident);
   } else {
     // x pass: rb rows of 3 fields; y pass: zs z-lines of 3 fields
     int rb = std::min(p->ny, 2 * BATCH / (3 * p->nx));
@@ -349,16 +345,21 @@ mf_status mf_create(const mf_params* p, void* d_workspace, size_t bytes, void* s
 
   // tables and inputs
   std::vector<char> tw, kt, gt;
-  if (p->precision) fill_tables<float>(p, d.sigma, tw, kt, gt);
-  else fill_tables<double>(p, d.sigma, tw, kt, gt);
+  if (p->precision) fill_tables<float>(p, d, tw, kt, gt);
+  else fill_tables<double>(p, d, tw, kt, gt);
   const size_t ts = p->precision ? 4 : 8;
   std::vector<char> jcbuf;
+  const int ru = p->dim == 2 ? row_unit(p->precision) : 1;    // films: kept by row units
   if (p->jc_map) {
     jcbuf.resize(L.ncell * ts);
-    for (long long i = 0; i < L.ncell; ++i) {
-      if (p->precision) ((float*)jcbuf.data())[i] = (float)p->jc_map[i];
-      else ((double*)jcbuf.data())[i] = p->jc_map[i];
-    }
+    const long long units = L.ncell / ((long long)ru * p->nx);
+    if (p->precision) field_by_units(p->jc_map, p->nx, ru, units, (float*)jcbuf.data());
+    else field_by_units(p->jc_map, p->nx, ru, units, (double*)jcbuf.data());
+  }
+  std::vector<unsigned char> units;
+  if (p->dim == 2) {
+    units.resize(L.ncell / ru);
+    pack_mask(p->mask, p->nx, ru, p->ny / ru, units.data());
   }
   std::vector<double> knots(2 * (p->he_knots > 0 ? p->he_knots : 1), 0.0);
   for (int i = 0; i < p->he_knots; ++i) { knots[i] = p->he_t[i]; knots[p->he_knots + i] = p->he_v[i]; }
@@ -372,9 +373,10 @@ mf_status mf_create(const mf_params* p, void* d_workspace, size_t bytes, void* s
   auto cp = [&](void* dst, const void* src, size_t n) {
     if (e == cudaSuccess && n) e = cudaMemcpyAsync(dst, src, n, cudaMemcpyHostToDevice, st);
   };
-  cp(w + L.mask, p->mask, L.ncell);
+  if (p->dim == 2) cp(w + L.mask, units.data(), units.size());
+  else cp(w + L.mask, p->mask, L.ncell);
   if (p->jc_map) cp(w + L.jc, jcbuf.data(), jcbuf.size());
-  const size_t twx = 2 * p->nx * 2 * ts, twy = 2 * p->ny * 2 * ts, twz = 2 * nz * 2 * ts;
+  const size_t twx = TWIDDLE_VALUES * p->nx * ts, twy = TWIDDLE_VALUES * p->ny * ts, twz = TWIDDLE_VALUES * nz * ts;
   cp(w + L.twx, tw.data(), twx);
   cp(w + L.twy, tw.data() + twx, twy);
   cp(w + L.twz, tw.data() + twx + twy, twz);
@@ -528,7 +530,9 @@ static void advance_films_together(mf_problem* const* pbs, const std::vector<int
     return;
   }
   const int prec = p0->d.precision;
-  const int per_sm = film_batch_max_blocks(prec, kernel_smem_bytes(p0->d));
+  size_t smem = 0;                       // of the widest film
+  for (int i : idx) smem = std::max(smem, kernel_smem_bytes(pbs[i]->d));
+  const int per_sm = film_batch_max_blocks(prec, smem);
   int nsm = 0;
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, p0->device);
   e = cudaGetLastError();
@@ -590,7 +594,7 @@ static void advance_films_together(mf_problem* const* pbs, const std::vector<int
       b += ctas[k];
       members.push_back(live[k]);
     }
-    if (e == cudaSuccess) e = film_batch_launch(prec, tab, b, s);
+    if (e == cudaSuccess) e = film_batch_launch(prec, tab, b, smem, s);
     for (int i : members) {
       if (e == cudaSuccess) shared.push_back(i);
       else st[i] = cuda_fail(pbs[i], e, "shared persistent launch");
@@ -785,9 +789,7 @@ static std::vector<std::array<int, 3>> tuning_candidates(const mf_problem* pb, i
       if (g >= 1 && g <= coresident) c.push_back({rb, zs, g});
   };
   if (d.dim == 2) {
-    // row passes: rb one-field rows (and min(rb, BATCH / nx) two-field rows) per item
-    const int rb_max = std::min(d.ny, 2 * BATCH / d.nx);
-    for (int rb = 2; rb <= rb_max; rb *= 2) add(rb, std::max(2, std::min(rb, BATCH / d.nx)));
+    add(d.rows_per_item, d.zs_per_item);     // row units are fixed by the precision: launch widths only
   } else {
     // x pass: rb rows of 3 fields; y pass: zs z-lines of 3 fields
     for (int rb = 2; rb <= d.ny && 3 * d.nx * (rb / 2) <= BATCH; rb *= 2)
@@ -903,6 +905,12 @@ std::vector<std::pair<void*, size_t>> ckpt_regions(const mf_problem* pb) {
   r.push_back({(void*)d.log, (size_t)d.log_cap * sizeof(StepLog)});
   return r;
 }
+// a film's h_dot buffers, kept by row units, are row-major in the blob: a spectrum buffer (free
+// between calls) to convert them through, null for every other region
+void* ckpt_rows(const mf_problem* pb, const void* region) {
+  if (pb->d.dim != 2) return nullptr;
+  return region == pb->d.hd ? pb->d.Sa : region == pb->d.hd2 ? pb->d.Sb : nullptr;
+}
 size_t ckpt_bytes(const mf_problem* pb) {
   size_t b = sizeof(CkptHeader);
   for (const auto& x : ckpt_regions(pb)) b += x.second;
@@ -922,6 +930,13 @@ mf_status mf_checkpoint_save(mf_problem* pb, void* dst) {
   MF_CUDA(pb, cudaMemcpyAsync(o, &h, sizeof(h), cudaMemcpyDefault, pb->stream));
   o += sizeof(h);
   for (const auto& x : ckpt_regions(pb)) {
+    if (void* rows = ckpt_rows(pb, x.first)) {
+      cudaError_t e = film_relayout(pb->d.precision, pb->d.nx, pb->d.ny, true, x.first, rows, pb->stream);
+      if (e != cudaSuccess) return cuda_fail(pb, e, "checkpoint layout");
+      MF_CUDA(pb, cudaMemcpyAsync(o, rows, x.second, cudaMemcpyDefault, pb->stream));
+      o += x.second;
+      continue;
+    }
     MF_CUDA(pb, cudaMemcpyAsync(o, x.first, x.second, cudaMemcpyDefault, pb->stream));
     o += x.second;
   }
@@ -943,12 +958,22 @@ mf_status mf_checkpoint_restore(mf_problem* pb, const void* src) {
   }
   const char* i = (const char*)src + sizeof(h);
   for (const auto& x : ckpt_regions(pb)) {
+    if (void* rows = ckpt_rows(pb, x.first)) {
+      MF_CUDA(pb, cudaMemcpyAsync(rows, i, x.second, cudaMemcpyDefault, pb->stream));
+      cudaError_t e = film_relayout(pb->d.precision, pb->d.nx, pb->d.ny, false, rows, x.first, pb->stream);
+      if (e != cudaSuccess) return cuda_fail(pb, e, "checkpoint layout");
+      i += x.second;
+      continue;
+    }
     MF_CUDA(pb, cudaMemcpyAsync(x.first, i, x.second, cudaMemcpyDefault, pb->stream));
     i += x.second;
   }
-  // the work-item shape (it sets the order of the sums) and launch width it was saved with
-  pb->d.rows_per_item = h.rows_per_item;
-  pb->d.zs_per_item = h.zs_per_item;
+  // the work-item shape (it sets the order of the sums; a film's is fixed) and launch width it was
+  // saved with
+  if (pb->d.dim == 3) {
+    pb->d.rows_per_item = h.rows_per_item;
+    pb->d.zs_per_item = h.zs_per_item;
+  }
   pb->d.grid = h.grid;
   MF_CUDA(pb, cudaMemcpyAsync((void*)pb->d.dev, &pb->d, sizeof(Desc), cudaMemcpyHostToDevice, pb->stream));
   MF_CUDA(pb, cudaStreamSynchronize(pb->stream));
@@ -1005,7 +1030,7 @@ static mf_status warm_save(mf_problem* pb, double* dst) {
   SolverState s;
   MF_TRY_STATUS(read_state(pb, &s));
   void* hd = s.hd_sel ? pb->d.hd2 : pb->d.hd;
-  cudaError_t e = adj_warm_io(pb->d.precision, pb->d.ncell, 0, pb->d.mask, hd, s.A_prev, dst, nullptr,
+  cudaError_t e = adj_warm_io(pb->d.precision, pb->d.nx, pb->d.ny, 0, pb->d.mask, hd, s.A_prev, dst, nullptr,
                               pb->stream);
   return e == cudaSuccess ? MF_OK : cuda_fail(pb, e, "warm start save");
 }
@@ -1013,7 +1038,7 @@ static mf_status warm_load(mf_problem* pb, const double* src) {
   SolverState s;
   MF_TRY_STATUS(read_state(pb, &s));
   s.hd_sel = 0; s.warm_valid = 1; s.A_prev = 0.0; s.com_valid = 0; s.A_com = 0.0;
-  cudaError_t e = adj_warm_io(pb->d.precision, pb->d.ncell, 1, pb->d.mask, pb->d.hd, 0.0, nullptr, src,
+  cudaError_t e = adj_warm_io(pb->d.precision, pb->d.nx, pb->d.ny, 1, pb->d.mask, pb->d.hd, 0.0, nullptr, src,
                               pb->stream);
   if (e != cudaSuccess) return cuda_fail(pb, e, "warm start load");
   return write_state(pb, &s);
@@ -1225,7 +1250,10 @@ mf_status mf_set_jc_map(mf_problem* pb, const double* d_jc) {
   }
   MF_CUDA(pb, cudaSetDevice(pb->device));
   const long long n = pb->d.ncell;
-  if (pb->d.precision) {
+  if (pb->d.dim == 2) {
+    cudaError_t e = film_to_units(pb->d.precision, pb->d.nx, pb->d.ny, d_jc, (void*)pb->d.jcmap, pb->stream);
+    if (e != cudaSuccess) return cuda_fail(pb, e, "jc map conversion");
+  } else if (pb->d.precision) {
     cudaError_t e = adj_to_float(n, d_jc, (float*)pb->d.jcmap, pb->stream);
     if (e != cudaSuccess) return cuda_fail(pb, e, "jc map conversion");
   } else {

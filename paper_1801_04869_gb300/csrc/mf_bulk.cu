@@ -744,7 +744,7 @@ __global__ void __launch_bounds__(NT, 2) bulk_kernel(const Desc* __restrict__ dg
     if (!ok) status = ST_BARRIER;
   } else if (a.mode == MODE_ADVANCE) {
     BulkRhs<T> R{B};
-    status = bs23_advance(R, d, st, a, leader);
+    status = bs23_advance(R, d, st, a, leader, sh.ctl);
   }
   if (leader) {
     st->warm_valid = sh.warm_valid;

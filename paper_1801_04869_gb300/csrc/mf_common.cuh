@@ -171,6 +171,7 @@ struct Desc {
   int rows_per_item;             // 2D row pass / 3D x pass rows per work item (even)
   int zs_per_item;               // 3D y pass z-lines per work item
   int grid;                      // CTAs of the persistent launch
+  int ex, ey;                    // elements per thread of the transform core along x, y
   unsigned long long barrier_ns; // time limit of one grid-barrier wait (ns)
   const struct Desc* dev;        // device copy of this descriptor (what the kernels read)
 };
@@ -213,10 +214,11 @@ __device__ __forceinline__ bool grid_sync(GridBarrier* gb, unsigned int nblocks,
     unsigned long long v = ld_acquire_u64(&gb->count);
     if ((v & ~BARRIER_ABORT) < target && !(v & BARRIER_ABORT)) {
       const unsigned long long t0 = globaltimer_ns();
-      unsigned int nap = 32;
+      // a sleep of at least 32 ns between polls would be a large share of the shortest phases: the
+      // polls follow one another (an L2 round trip each) and sleep only in long waits
+      int polls = 0;
       do {
-        __nanosleep(nap);
-        if (nap < 128) nap <<= 1;
+        if (++polls > 64) __nanosleep(64);
         if (globaltimer_ns() - t0 > lim) {
           atomicOr(&gb->count, BARRIER_ABORT);
           atomicExch(&gb->where, where);
@@ -303,43 +305,30 @@ __device__ __forceinline__ double block_max(double v, double* red) {
 }
 
 // Sum (or max) of partials[slot * max_items + i] over i < n, in a fixed order, computed
-// identically by every CTA.
-// The first warp does it alone (loads through L2 only: the partials were written by other CTAs
-// in this launch), so the CTA synchronises once instead of four times.
+// identically by every CTA (loads through L2 only: the partials were written by other CTAs in this
+// launch).  Every thread loads, the warps reduce, thread 0 combines: one load latency and a short
+// chain of FP64 additions (64 cycles each per warp) instead of one warp's walk over all items.
 __device__ __forceinline__ double reduce_partials(const double* partials, int max_items, int slot,
                                                   int n, bool is_max, double* red) {
   const double* p = partials + (size_t)slot * max_items;
-  if (threadIdx.x < 32) {
-    double v = 0.0;
-    for (int i = threadIdx.x; i < n; i += 32) {
-      const double x = __ldcg(p + i);
-      v = is_max ? fmax(v, x) : v + x;
-    }
-    v = is_max ? warp_max(v) : warp_sum(v);
-    if (threadIdx.x == 0) red[0] = v;
+  double v = 0.0;
+  for (int i = threadIdx.x; i < n; i += NT) {
+    const double x = __ldcg(p + i);
+    v = is_max ? fmax(v, x) : v + x;
+  }
+  v = is_max ? warp_max(v) : warp_sum(v);
+  __syncthreads();
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double s = red[0];
+    for (int k = 1; k < NT / 32; ++k) s = is_max ? fmax(s, red[k]) : s + red[k];
+    red[0] = s;
   }
   __syncthreads();
   const double s = red[0];
   __syncthreads();
   return s;
-}
-
-// Sums of two slots over i < n (fixed order, as reduce_partials), read in one pass by the first
-// warp; red[0], red[1] receive them.  The caller combines them in thread 0 and broadcasts.
-__device__ __forceinline__ void reduce_partials2(const double* partials, int max_items, int slot_a,
-                                                 int slot_b, int n, double* red) {
-  if (threadIdx.x < 32) {
-    const double* pa = partials + (size_t)slot_a * max_items;
-    const double* pb = partials + (size_t)slot_b * max_items;
-    double a = 0.0, b = 0.0;
-    for (int i = threadIdx.x; i < n; i += 32) {
-      a += __ldcg(pa + i);
-      b += __ldcg(pb + i);
-    }
-    a = warp_sum(a);
-    b = warp_sum(b);
-    if (threadIdx.x == 0) { red[0] = a; red[1] = b; }
-  }
 }
 
 // ------------------------------------------------------------------------------------------
@@ -376,11 +365,30 @@ struct BatchTable {
 
 // launch helpers implemented next to each kernel
 cudaError_t film_launch(int precision, const Desc& d, const KernelArgs& a, cudaStream_t s);
-cudaError_t film_batch_launch(int precision, const BatchTable& tab, int grid, cudaStream_t s);
+cudaError_t film_batch_launch(int precision, const BatchTable& tab, int grid, size_t smem, cudaStream_t s);
 int film_batch_max_blocks(int precision, size_t smem);
 cudaError_t bulk_launch(int precision, const Desc& d, const KernelArgs& a, cudaStream_t s);
 int film_max_blocks(int precision, size_t smem);
 int bulk_max_blocks(int precision, size_t smem);
 size_t kernel_smem_bytes(const Desc& d);
+
+// Entries (16 bytes each) of the core's twiddle table of length 2^lg for E elements per thread
+__host__ __device__ constexpr int core_table_len(int lg, int E) {
+  const int e = E == 2 ? 1 : E == 4 ? 2 : E == 8 ? 3 : 4;
+  int n = 0, lgp = e;
+  for (int rem = lg - e; rem > 0; rem -= e, lgp += e) n += rem >= e ? e << lgp : rem << (lg - e);
+  return n;
+}
+// a film's shared memory: the exchange buffer's elements, then the tables (one if the axes agree)
+__host__ __device__ constexpr int slots_of(int E) { return NT * E + (NT * E >> (E == 16 ? 4 : 3)); }
+__host__ __device__ inline int film_slots(const Desc& d) { return slots_of(d.ex > d.ey ? d.ex : d.ey); }
+__host__ __device__ inline bool film_one_table(const Desc& d) { return d.lgx == d.lgy && d.ex == d.ey; }
+// the most that any film needs (what the kernels' attribute is set to, whatever is launched first)
+constexpr size_t FILM_SMEM_MAX = 16 * ((size_t)slots_of(8) + 2 * core_table_len(11, 8));
+inline size_t film_smem_bytes(const Desc& d) {
+  return 16 * ((size_t)film_slots(d) + core_table_len(d.lgx, d.ex) + (film_one_table(d) ? 0 : core_table_len(d.lgy, d.ey)));
+}
+// Rows of the real fields that a film's row passes keep together (mf_film.cuh)
+constexpr int row_unit(int precision) { return precision ? 4 : 2; }
 
 }  // namespace mf

@@ -6,22 +6,24 @@ namespace mf {
 
 // one film on the whole grid
 template <typename T>
-__global__ void __launch_bounds__(NT, 2) film_kernel(const Desc* __restrict__ dg, KernelArgs a) {
+__global__ void __launch_bounds__(NT, FILM_CTAS) film_kernel(const Desc* __restrict__ dg, KernelArgs a) {
   film_main<T>(*dg, a, (int)blockIdx.x, gridDim.x);
 }
 
-// film passes: two FFT buffers; bulk passes: a third one for the next item's gather
+// film passes: the core's exchange buffer and twiddle tables; bulk passes: two FFT buffers and a third one for the next
+// item's gather
 size_t kernel_smem_bytes(const Desc& d) {
-  return film_smem_bytes(d.precision) / 2 * (d.dim == 3 ? 3 : 2);
+  if (d.dim == 2) return film_smem_bytes(d);
+  return 3 * (size_t)BATCH_PAD * (d.precision ? sizeof(C2<float>) : sizeof(C2<double>));
 }
 
 int film_max_blocks(int precision, size_t smem) {
   int nb = 0;
   if (precision) {
-    cudaFuncSetAttribute(film_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaFuncSetAttribute(film_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FILM_SMEM_MAX);
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, film_kernel<float>, NT, smem);
   } else {
-    cudaFuncSetAttribute(film_kernel<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaFuncSetAttribute(film_kernel<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FILM_SMEM_MAX);
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, film_kernel<double>, NT, smem);
   }
   return nb;

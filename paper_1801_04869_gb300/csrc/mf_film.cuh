@@ -18,12 +18,133 @@
 // The centring constant C (Eq. 11), the mean over free space of raw - A q1, is known before
 // the x pass that forms g_dot: K1 is real and even, so sum_out F^-1[K1 F h] = <q1, h>, and
 // C = (<q1, h> - A sum_out q1) / n_out with <q1, h> summed where h is written (P5, P10).
+//
+// Both passes run on the transform core (mf_core.cuh).  The real fields of the workspace (h_dot,
+// g_dot, q1, q2, the jc map) and the mask are kept by row units: the RU rows that one element of a
+// row pass holds (4 in FP32, 2 in FP64) lie together for each x, 16 bytes, and their mask classes
+// in one byte, so that an epilogue moves one 16-byte vector per element.
+//
+// What bounds a pass, and what it measured (one right-hand side, 5 outside iterations = 24 passes with
+// their grid barriers; the design before transformed through two shared buffers at 16 values per
+// thread): small grids are bound by one thread's chain of instructions, the barrier and the load
+// latencies (128^2: FP32 250 -> 190 us, FP64 514 -> 251 us); FP64 grids from 512^2 by the FP64 unit,
+// 2 lanes per cycle and SM (1024^2 2.85 -> 2.10 ms, 2048^2 11.2 -> 8.6 ms); 2048^2 FP32 by exchanges
+// through shared memory and their latencies (979 -> 786 us), 512^2 and 1024^2 by both (350 -> 216 us,
+// 513 -> 304 us).
 #pragma once
+#include "mf_core.cuh"
 #include "mf_rhs_common.cuh"
 
 namespace mf {
 
 enum Op2 { OP_GRAD = 0, OP_CURLNEG = 1, OP_K1 = 2, OP_K2 = 3, OP_KH = 4, OP_ID = 5 };
+
+// ------------------------------------------------------------------------------------------
+// row units
+// ------------------------------------------------------------------------------------------
+// the RU rows of one element at one x: 16 bytes
+template <typename T> struct Q { T v[Lane<T>::RU]; };
+__device__ __forceinline__ Q<float> ld_q(const float* p) {
+  Q<float> r;
+  asm volatile("ld.global.L1::no_allocate.v4.f32 {%0, %1, %2, %3}, [%4];"
+               : "=f"(r.v[0]), "=f"(r.v[1]), "=f"(r.v[2]), "=f"(r.v[3]) : "l"(p) : "memory");
+  return r;
+}
+__device__ __forceinline__ Q<double> ld_q(const double* p) {
+  Q<double> r;
+  asm volatile("ld.global.L1::no_allocate.v2.f64 {%0, %1}, [%2];" : "=d"(r.v[0]), "=d"(r.v[1]) : "l"(p) : "memory");
+  return r;
+}
+// read-only for the whole launch (non-coherent path)
+__device__ __forceinline__ Q<float> ldg_q(const float* p) {
+  Q<float> r;
+  asm("ld.global.nc.L1::no_allocate.v4.f32 {%0, %1, %2, %3}, [%4];"
+      : "=f"(r.v[0]), "=f"(r.v[1]), "=f"(r.v[2]), "=f"(r.v[3]) : "l"(p));
+  return r;
+}
+__device__ __forceinline__ Q<double> ldg_q(const double* p) {
+  Q<double> r;
+  asm("ld.global.nc.L1::no_allocate.v2.f64 {%0, %1}, [%2];" : "=d"(r.v[0]), "=d"(r.v[1]) : "l"(p));
+  return r;
+}
+__device__ __forceinline__ void st_q(float* p, const Q<float>& q) { *(float4*)p = make_float4(q.v[0], q.v[1], q.v[2], q.v[3]); }
+__device__ __forceinline__ void st_q(double* p, const Q<double>& q) { *(double2*)p = make_double2(q.v[0], q.v[1]); }
+// element <-> rows: lines pack rows (0, 2) and (1, 3) in FP32, (0, 1) in FP64, as a + i b
+__device__ __forceinline__ Q<float> to_q(const CV<F2>& e) {
+  Q<float> q;
+  upk(e.x, q.v[0], q.v[1]);
+  upk(e.y, q.v[2], q.v[3]);
+  return q;
+}
+__device__ __forceinline__ Q<double> to_q(const CV<double>& e) { return Q<double>{{e.x, e.y}}; }
+__device__ __forceinline__ CV<F2> to_e(const Q<float>& q) { return {pk(q.v[0], q.v[1]), pk(q.v[2], q.v[3])}; }
+__device__ __forceinline__ CV<double> to_e(const Q<double>& q) { return {q.v[0], q.v[1]}; }
+// mask classes of a unit's rows, 2 bits each
+__device__ __forceinline__ int ld_mask(const uint8_t* p) {
+  unsigned m;
+  asm("ld.global.nc.L1::no_allocate.u8 %0, [%1];" : "=r"(m) : "l"(p));
+  return (int)m;
+}
+__device__ __forceinline__ int cls(int m, int r) { return (m >> (2 * r)) & 3; }
+
+// 32 bytes of one half-spectrum column: the complex values of a unit's rows at one x-wavenumber
+struct B32f { float a[8]; };
+struct B32d { double a[4]; };
+__device__ __forceinline__ B32f ld_b32(const C2<float>* p) {
+  B32f r;
+  asm volatile("ld.global.L1::no_allocate.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+               : "=f"(r.a[0]), "=f"(r.a[1]), "=f"(r.a[2]), "=f"(r.a[3]), "=f"(r.a[4]), "=f"(r.a[5]),
+                 "=f"(r.a[6]), "=f"(r.a[7]) : "l"(p) : "memory");
+  return r;
+}
+__device__ __forceinline__ B32d ld_b32(const C2<double>* p) {
+  B32d r;
+  asm volatile("ld.global.L1::no_allocate.v4.f64 {%0, %1, %2, %3}, [%4];"
+               : "=d"(r.a[0]), "=d"(r.a[1]), "=d"(r.a[2]), "=d"(r.a[3]) : "l"(p) : "memory");
+  return r;
+}
+// position k of the packed lines (a + i b per pair of rows) from the rows' half spectra A, B at k:
+// A + i B; at nx - k: conj(A) + i conj(B); at k = 0 and nx/2 the imaginary parts are dropped
+__device__ __forceinline__ CV<F2> pack_lo(const B32f& s) { return {pk(s.a[0] - s.a[5], s.a[2] - s.a[7]), pk(s.a[1] + s.a[4], s.a[3] + s.a[6])}; }
+__device__ __forceinline__ CV<F2> pack_hi(const B32f& s) { return {pk(s.a[0] + s.a[5], s.a[2] + s.a[7]), pk(s.a[4] - s.a[1], s.a[6] - s.a[3])}; }
+__device__ __forceinline__ CV<F2> pack_re(const B32f& s) { return {pk(s.a[0], s.a[2]), pk(s.a[4], s.a[6])}; }
+__device__ __forceinline__ CV<double> pack_lo(const B32d& s) { return {s.a[0] - s.a[3], s.a[1] + s.a[2]}; }
+__device__ __forceinline__ CV<double> pack_hi(const B32d& s) { return {s.a[0] + s.a[3], s.a[2] - s.a[1]}; }
+__device__ __forceinline__ CV<double> pack_re(const B32d& s) { return {s.a[0], s.a[2]}; }
+// twice the rows' half spectra at k from the packed lines' transforms at k and nx - k (the factor
+// 1/2 is in the column passes' scale)
+__device__ __forceinline__ void st_b32(C2<float>* p, const CV<F2>& zk, const CV<F2>& zm) {
+  float r[8];
+  upk(vadd(zk.x, zm.x), r[0], r[2]);
+  upk(vsub(zk.y, zm.y), r[1], r[3]);
+  upk(vadd(zk.y, zm.y), r[4], r[6]);
+  upk(vsub(zm.x, zk.x), r[5], r[7]);
+  asm volatile("st.global.v8.f32 [%8], {%0, %1, %2, %3, %4, %5, %6, %7};"
+               :: "f"(r[0]), "f"(r[1]), "f"(r[2]), "f"(r[3]), "f"(r[4]), "f"(r[5]), "f"(r[6]), "f"(r[7]), "l"(p) : "memory");
+}
+__device__ __forceinline__ void st_b32(C2<double>* p, const CV<double>& zk, const CV<double>& zm) {
+  asm volatile("st.global.v4.f64 [%4], {%0, %1, %2, %3};"
+               :: "d"(zk.x + zm.x), "d"(zk.y - zm.y), "d"(zk.y + zm.y), "d"(zm.x - zk.x), "l"(p) : "memory");
+}
+// one column element: the values of line kx (and, in FP32, of line kx + 1 at `stride`)
+__device__ __forceinline__ CV<F2> ld_col(const C2<float>* p, long long stride, bool two) {
+  const C2<float> a = lds_c2(p);
+  C2<float> b = {0.f, 0.f};
+  if (two) b = lds_c2(p + stride);
+  return {pk(a.x, b.x), pk(a.y, b.y)};
+}
+__device__ __forceinline__ CV<double> ld_col(const C2<double>* p, long long, bool) {
+  const C2<double> a = lds_c2(p);
+  return {a.x, a.y};
+}
+__device__ __forceinline__ void st_col(C2<float>* p, long long stride, bool two, const CV<F2>& e) {
+  C2<float> a, b;
+  upk(e.x, a.x, b.x);
+  upk(e.y, a.y, b.y);
+  p[0] = a;
+  if (two) p[stride] = b;
+}
+__device__ __forceinline__ void st_col(C2<double>* p, long long, bool, const CV<double>& e) { p[0] = C2<double>{e.x, e.y}; }
 
 // raw pointers and sizes the x-pass epilogues need, held by value (registers)
 template <typename T>
@@ -39,9 +160,10 @@ struct FilmPtrs {
 
 template <typename T>
 struct Film {
+  using V = typename Lane<T>::V;
+  static constexpr int RU = Lane<T>::RU, NL = Lane<T>::NL;
   const Desc& d;
-  C2<T>* sm;         // shared buffer A (BATCH values)
-  C2<T>* sm2;        // shared buffer B
+  CV<V>* sm;         // the CTA's exchange buffer
   Shared& sh;
   int nx, ny, lgx, lgy, half, nkx;
   long long nspec, ncell;
@@ -53,349 +175,502 @@ struct Film {
   const T* q2;
   const uint8_t* mask;
   const T* jcmap;
-  const C2<T>* twx;
-  const C2<T>* twy;
+  const CV<V>* twx;  // twiddle tables, behind the exchange buffer in shared memory
+  const CV<V>* twy;
   const T* ktab;     // kx values (half entries), then ky values (ny entries)
   const T* gtab;     // Gaussian factors, same layout
-  int rb1, rb2;      // rows per item for one- and two-field row passes
+  T lam, scale, ig2;  // lambda; 1/(2 cells); 1/gamma^2
+  int ex, ey;        // elements per thread of the x and y passes
+  int max_items;     // members of the descriptor that every phase reads, at hand in shared memory (a
+  double* partials;  // grid barrier's acquire empties L1)
+  GridBarrier* gb;
+  unsigned long long barrier_ns;
+  double iter_tol;
   int vb;            // this CTA's index among the CTAs that run this film
   unsigned nblocks;  // how many CTAs run this film
 
-  __device__ Film(const Desc& dd, C2<T>* s, Shared& shr, int vblock, unsigned nblk)
-      : d(dd), sm(s), sm2(s + BATCH_PAD), sh(shr) {
+  __device__ Film(const Desc& dd, unsigned char* smem, Shared& shr, int vblock, unsigned nblk)
+      : d(dd), sm((CV<V>*)smem), sh(shr) {
     nx = d.nx; ny = d.ny; lgx = d.lgx; lgy = d.lgy; half = nx / 2; nkx = half + 1;
     nspec = (long long)nkx * ny;
     ncell = (long long)nx * ny;
     Sa = (C2<T>*)d.Sa; Sb = (C2<T>*)d.Sb;
     hd = (T*)d.hd; u = (T*)d.u; q1 = (const T*)d.q1; q2 = (const T*)d.q2;
     mask = d.mask; jcmap = (const T*)d.jcmap;
-    twx = (const C2<T>*)d.tw_x;                 // stage-ordered twiddle tables (read-only)
-    twy = (const C2<T>*)d.tw_y;
+    ex = d.ex; ey = d.ey;
+    const int slots = film_slots(d);
+    twx = sm + slots;
+    twy = film_one_table(d) ? twx : twx + core_table_len(lgx, ex);
+    max_items = d.max_items;
+    partials = d.partials;
+    gb = d.gb;
+    barrier_ns = d.barrier_ns;
+    iter_tol = d.iter_tol;
     ktab = (const T*)d.ktab;
     gtab = (const T*)d.gtab;
-    rb1 = d.rows_per_item;
-    rb2 = d.zs_per_item;
+    lam = (T)d.lam;
+    scale = (T)0.5 / (T)ncell;         // a power of two
+    ig2 = (T)(1.0 / (d.gamma * d.gamma));
     vb = vblock;
     nblocks = nblk;
+    sh.N = (double)ncell;
+    sh.inv_nout = d.nout > 0 ? 1.0 / (double)d.nout : 0.0;
   }
 
-  __device__ bool sync(int where) { return grid_sync(d.gb, nblocks, where, &sh.bar_passed, d.barrier_ns); }
+  __device__ bool sync(int where) { return grid_sync(gb, nblocks, where, &sh.bar_passed, barrier_ns); }
 
   __device__ FilmPtrs<T> ptrs() const { return FilmPtrs<T>{mask, jcmap, hd, u, q1, q2, nx}; }
 
-  // ---- y pass: forward, multiplier, inverse on nl consecutive x-wavenumber lines ----
-  // shared line f * nl + l holds field f of line kx0 + l
-  __device__ __noinline__ void col_item(int kx0, int nl, const C2<T>* Sin, int nin, C2<T>* Sout, int nout, int op) {
-    if (fft_plan<T>(lgy).m >= 2) {
-      // fused round trip: global -> first stage, multiplier between the forward last and the
-      // inverse first stage, last stage -> global.  Everything the lambdas use is a copy held
-      // in registers.
-      const long long nspec = this->nspec;
-      const int ny = this->ny, nkx = this->nkx, half = this->half;
-      const T* const ktab = this->ktab;
-      const T* const gtab = this->gtab;
-      const T lam = (T)d.lam;
-      auto src = [=](int f, int l) { return Sin + f * nspec + (long long)(kx0 + l) * ny; };
-      auto dst = [=](int g, int l) { return Sout + g * nspec + (long long)(kx0 + l) * ny; };
-      const T s = (T)1 / (T)ncell;
-      // single precision: k_y = pi m / L_y (m in FFT order) and its Gaussian factor are
-      // computed from the index (a few ulp from the tables); double precision reads the tables
-      const T ky_scale = (T)(PI_D / d.Ly), g_half = (T)(0.5 * d.sigma * d.sigma);
-      auto coef = [=](int l, int ky, T& kxo, T& kyo, T& k2, T& G) {
-        const int kx = kx0 + l;
-        const T kxv = ldg_tab(&ktab[kx]);
-        T kyv, gy;
-        if constexpr (sizeof(T) == 4) {
-          kyv = (T)(ky < ny / 2 ? ky : ky - ny) * ky_scale;
-          gy = __expf(-kyv * kyv * g_half);
-        } else {
-          kyv = ldg_tab(&ktab[nkx + ky]);
-          gy = ldg_tab(&gtab[nkx + ky]);
-        }
-        kxo = (kx == half) ? (T)0 : kxv;
-        kyo = (ky == ny / 2) ? (T)0 : kyv;
-        k2 = kxv * kxv + kyv * kyv;
-        G = ldg_tab(&gtab[kx]) * gy;
-      };
-      if (op == OP_GRAD) {
-        fft_round_trip<T, 1, 2>(sm, sm2, lgy, nl, twy, src, dst,
-            [=](int l, int ky, const C2<T>* x, C2<T>* y) {
-              T kxo, kyo, k2, G; coef(l, ky, kxo, kyo, k2, G);
-              y[0] = cmul_si(cscale(x[0], kxo * G * s), 1);
-              y[1] = cmul_si(cscale(x[0], kyo * G * s), 1);
-            }, [] {});
-      } else if (op == OP_CURLNEG) {
-        fft_round_trip<T, 2, 1>(sm, sm2, lgy, nl, twy, src, dst,
-            [=](int l, int ky, const C2<T>* x, C2<T>* y) {
-              T kxo, kyo, k2, G; coef(l, ky, kxo, kyo, k2, G);
-              // -(i kx G e_y - i ky G e_x) = i G (ky e_x - kx e_y)
-              const C2<T> c = {kyo * x[0].x - kxo * x[1].x, kyo * x[0].y - kxo * x[1].y};
-              y[0] = cmul_si(cscale(c, G * s), 1);
-            }, [] {});
-      } else {
-        fft_round_trip<T, 1, 1>(sm, sm2, lgy, nl, twy, src, dst,
-            [=](int l, int ky, const C2<T>* x, C2<T>* y) {
-              T kxo, kyo, k2, G; coef(l, ky, kxo, kyo, k2, G);
-              // |k| and 1/|k| from one reciprocal square root in single precision (a few ulp,
-              // far below the FP32 transform error); correctly rounded sqrt and divide in double
-              T kabs, kinv;
-              if constexpr (sizeof(T) == 4) {
-                kinv = k2 > (T)0 ? rsqrtf(k2) : (T)0;
-                kabs = k2 * kinv;
-              } else {
-                kabs = sqrt(k2);
-                kinv = k2 > (T)0 ? (T)1 / kabs : (T)0;
-              }
-              T m;
-              if (op == OP_K1) m = (T)2 * kinv;
-              else if (op == OP_K2) m = lam * kabs * (T)0.5 * G;
-              else if (op == OP_KH) m = kabs * (T)0.5;
-              else m = (T)1;
-              y[0] = cscale(x[0], m * s);
-            }, [] {});
-      }
-      return;
+  // ---- y pass: forward, multiplier, inverse on the lines of NL consecutive x-wavenumbers ----
+  struct Coef { V kxo, kx2, gx; };     // per line: k_x (0 at its Nyquist index), k_x^2, G_x
+  __device__ __forceinline__ Coef coef_x(int kx) const {
+    if constexpr (sizeof(T) == 4) {
+      const int k1 = kx + 1 < nkx ? kx + 1 : kx;
+      const float a = ldg_tab(&ktab[kx]), b = ldg_tab(&ktab[k1]);
+      return {pk(kx == half ? 0.f : a, k1 == half ? 0.f : b), pk(a * a, b * b),
+              pk(ldg_tab(&gtab[kx]), ldg_tab(&gtab[k1]))};
+    } else {
+      const double a = ldg_tab(&ktab[kx]);
+      return {kx == half ? 0.0 : a, a * a, ldg_tab(&gtab[kx])};
     }
-    gather_batched<T, 4>(sm, Sin, (nin * nl) << lgy,
-        [=](int e) {
-          const int j = e >> lgy, f = j / nl, l = j - f * nl;
-          return f * nspec + (long long)(kx0 + l) * ny + (e & (ny - 1));
-        },
-        [](int e) { return e; });
-    C2<T>* X = fft_lines<T, -1>(sm, sm2, lgy, nin * nl, twy);
-    C2<T>* Y = X == sm ? sm2 : sm;
-    const T s = (T)1 / (T)ncell;
-    for (int e = threadIdx.x; e < (nl << lgy); e += NT) {
-      const int l = e >> lgy, ky = e & (ny - 1);
-      const int kx = kx0 + l;
-      const T kxv = ldg_tab(&ktab[kx]), gx = ldg_tab(&gtab[kx]);
-      const T kxo = (kx == half) ? (T)0 : kxv;
-      const T kyv = ldg_tab(&ktab[nkx + ky]), G = gx * ldg_tab(&gtab[nkx + ky]);
-      const T kyo = (ky == ny / 2) ? (T)0 : kyv;
-      const T k2 = kxv * kxv + kyv * kyv;
-      const int i0 = (0 * nl + l) * ny + ky, i1 = (1 * nl + l) * ny + ky;
-      C2<T> a = X[sp(i0)];
-      if (op == OP_GRAD) {
-        const T fx = kxo * G * s, fy = kyo * G * s;
-        X[sp(i0)] = cmul_si(cscale(a, fx), 1);
-        X[sp(i1)] = cmul_si(cscale(a, fy), 1);
-      } else if (op == OP_CURLNEG) {
-        const C2<T> b = X[sp(i1)];
-        // -(i kx G e_y - i ky G e_x) = i G (ky e_x - kx e_y)
-        C2<T> c = {kyo * a.x - kxo * b.x, kyo * a.y - kxo * b.y};
-        X[sp(i0)] = cmul_si(cscale(c, G * s), 1);
-      } else {
-        T m;
-        const T kabs = sqrt(k2);
-        if (op == OP_K1) m = (k2 > (T)0) ? (T)2 / kabs : (T)0;
-        else if (op == OP_K2) m = (T)d.lam * kabs * (T)0.5 * G;
-        else if (op == OP_KH) m = kabs * (T)0.5;
-        else m = (T)1;
-        X[sp(i0)] = cscale(a, m * s);
-      }
-    }
-    __syncthreads();
-    const C2<T>* Z = fft_lines<T, +1>(X, Y, lgy, nout * nl, twy);
-    for (int e = threadIdx.x; e < ((nout * nl) << lgy); e += NT) {
-      const int j = e >> lgy, f = j / nl, l = j - f * nl;
-      Sout[f * nspec + (long long)(kx0 + l) * ny + (e & (ny - 1))] = Z[sp(e)];
-    }
-    __syncthreads();
   }
-
-  // ---- y pass of one line kx with a one-field multiplier, by half of the CTA (group g, its
-  // own line region of both shared buffers and its own named barrier) ----
-  __device__ __noinline__ void col_line_half(int kx, const C2<T>* Sin, C2<T>* Sout, int op, int g) {
-    const int ny = this->ny, half = this->half;
-    const T* const ktab = this->ktab;
-    const T* const gtab = this->gtab;
-    const T lam = (T)d.lam;
-    const C2<T>* const src0 = Sin + (long long)kx * ny;
-    C2<T>* const dst0 = Sout + (long long)kx * ny;
-    auto src = [=](int, int) { return src0; };
-    auto dst = [=](int, int) { return dst0; };
-    const T s = (T)1 / (T)ncell;
-    const T ky_scale = (T)(PI_D / d.Ly), g_half = (T)(0.5 * d.sigma * d.sigma);
-    const T kxv = ldg_tab(&ktab[kx]), gx = ldg_tab(&gtab[kx]);
-    const int nkx = this->nkx;
-    (void)half;
-    fft_round_trip<T, 1, 1>(sm + sp(g << lgy), sm2 + sp(g << lgy), lgy, 1, twy, src, dst,
-        [=](int, int ky, const C2<T>* x, C2<T>* y) {
-          T kyv, gy;
-          if constexpr (sizeof(T) == 4) {
-            kyv = (T)(ky < ny / 2 ? ky : ky - ny) * ky_scale;
-            gy = __expf(-kyv * kyv * g_half);
-          } else {
-            kyv = ldg_tab(&ktab[nkx + ky]);
-            gy = ldg_tab(&gtab[nkx + ky]);
-          }
-          const T k2 = kxv * kxv + kyv * kyv;
-          T kabs, kinv;
-          if constexpr (sizeof(T) == 4) {
-            kinv = k2 > (T)0 ? rsqrtf(k2) : (T)0;
-            kabs = k2 * kinv;
-          } else {
-            kabs = sqrt(k2);
-            kinv = k2 > (T)0 ? (T)1 / kabs : (T)0;
-          }
-          T m;
-          if (op == OP_K1) m = (T)2 * kinv;
-          else if (op == OP_K2) m = lam * kabs * (T)0.5 * (gx * gy);
-          else if (op == OP_KH) m = kabs * (T)0.5;
-          else m = (T)1;
-          y[0] = cscale(x[0], m * s);
-        }, [] {}, HalfCta{g});
+  // k_y (m in FFT order) and its Gaussian factor
+  __device__ __forceinline__ void coef_y(int ky, T& k, T& g) const {
+    k = ldg_tab(&ktab[nkx + ky]);
+    g = ldg_tab(&gtab[nkx + ky]);
   }
-
-  // lines per column item: fill the shared batch (two lines for single-field operators)
-  __device__ int col_lines(int nf) const {
-    int nl = BATCH / (nf * ny);
-    return nl < 1 ? 1 : (nl > 2 ? 2 : nl);
+  // multiplier of a one-field operator at |k|^2 = k2.  |k| and 1/|k| come from one reciprocal
+  // square root (1 ulp in double; a few ulp in single, far below the transform's error)
+  __device__ __forceinline__ static T inv_abs(T k2) {
+    if constexpr (sizeof(T) == 4) return k2 > 0.f ? rsqrtf(k2) : 0.f;
+    else return k2 > 0.0 ? rsqrt(k2) : 0.0;
   }
-
-  __device__ void cols(const C2<T>* Sin, int nin, C2<T>* Sout, int nout, int op) {
-    const int nl = col_lines(nin > nout ? nin : nout);
-    const int nitems = (nkx + nl - 1) / nl;
-    if (nin == 1 && nout == 1 && nl == 2 && fft_plan<T>(lgy).m >= 2) {
-      // one line per half of the CTA: the halves run their transforms independently
-      const int g = (int)threadIdx.x / (NT / 2);
-      for (int it = vb; it < nitems; it += (int)nblocks) {
-        const int kx = it * 2 + g;
-        if (kx < nkx) col_line_half(kx, Sin, Sout, op, g);
-      }
-      return;
+  // c1 / |k| (OP_K1: c1 = 2) or c2 |k| g (OP_K2: c2 = lambda/2, g the Gaussian; OP_KH: 1/2 and 1)
+  __device__ __forceinline__ static V mult_k1(const V& kx2, T ky, T c1) {
+    if constexpr (sizeof(T) == 4) {
+      float a, b;
+      upk(vfma(pk(ky, ky), pk(ky, ky), kx2), a, b);
+      return vmul(pk(inv_abs(a), inv_abs(b)), pk(c1, c1));
+    } else {
+      return inv_abs(fma(ky, ky, kx2)) * c1;
     }
-    for (int it = vb; it < nitems; it += (int)nblocks) {
-      const int kx0 = it * nl;
-      col_item(kx0, kx0 + nl <= nkx ? nl : nkx - kx0, Sin, nin, Sout, nout, op);
+  }
+  __device__ __forceinline__ static V mult_k(const V& kx2, T ky, const V& g) {
+    if constexpr (sizeof(T) == 4) {
+      float a, b;
+      const F2 k2 = vfma(pk(ky, ky), pk(ky, ky), kx2);
+      upk(k2, a, b);
+      return vmul(vmul(k2, pk(inv_abs(a), inv_abs(b))), g);
+    } else {
+      const double k2 = fma(ky, ky, kx2);
+      return k2 * inv_abs(k2) * g;
     }
   }
 
-  // ---- x pass over rows [y0, y0 + rb): inverse of NIN fields, epilogue, forward of NOUT ----
-  // epi(row, x, in[], out[]) is called for every cell of the item.
-  template <int NIN, int NOUT, class Epi>
-  __device__ __forceinline__ void row_item(int y0, int rb, const C2<T>* Sin, C2<T>* Sout, Epi& epi_io) {
-    // inlined into the pass loop (a call per item cost a save and restore of the caller's live
-    // registers); works on register copies of the epilogue and of the members used in the loops
-    Epi epi = epi_io;
-    C2<T>* const smA = sm;
-    C2<T>* const smB = sm2;
-    const int nx = this->nx, lgx = this->lgx, ny = this->ny;
+  template <int E, int NIN, int NOUT>
+  __device__ __noinline__ void cols_e(const C2<T>* Sin, C2<T>* Sout, int op) {
+    const int ny = this->ny;
     const long long nspec = this->nspec;
-    const C2<T>* const twx = this->twx;
-    const int npair = rb / 2;
-    C2<T>* X = smA;
-    const int lgpair = __ffs(npair) - 1;
-    if constexpr (NIN > 0) X = rows_gather_inverse<T, NIN>(smA, smB, Sin + y0, nspec, ny, npair, lgpair, lgx, twx);
-    C2<T>* Y = X == smA ? smB : smA;
-    C2<T>* const S = dsm<T>();
-    const int ix = dsm_off(X);
-    // four consecutive cells of both rows of a pair per step; the epilogue issues its global
-    // loads for the four cells together (x0 is a multiple of 4: one padding group)
-    const int lgq = lgx - 2;
-#pragma unroll 4
-    for (int e = threadIdx.x; e < (npair << lgq); e += NT) {
-      const int pr = e >> lgq, x0 = (e & ((1 << lgq) - 1)) << 2;
-      V4<T> ina[NIN > 0 ? NIN : 1], inb[NIN > 0 ? NIN : 1], oa[NOUT > 0 ? NOUT : 1], ob[NOUT > 0 ? NOUT : 1];
+    Team<T, E> t(sm, twy, lgy);
+    const int units = (nkx + NL - 1) / NL;
+    const int per = NT / t.threads();
+    // lines that a CTA runs at a time: as few as spread the pass over all CTAs
+    const int want = (units + (int)nblocks - 1) / (int)nblocks;
+    const int nuc = want < per ? want : per;
+    const int q = t.step();
+    for (int u0 = vb * nuc; u0 < units; u0 += (int)nblocks * nuc) {
+      const int first = ((int)threadIdx.x & ~31) >> (lgy - Team<T, E>::LGE);   // slot of the warp's first lane
+      if (first >= nuc || u0 + first >= units) continue;
+      const bool mine = t.slot < nuc && u0 + t.slot < units;
+      const int kx = mine ? (u0 + t.slot) * NL : 0;
+      const bool two = NL == 2 && kx + 1 < nkx;
+      const C2<T>* const src = Sin + (long long)kx * ny + t.i;
+      C2<T>* const dst = Sout + (long long)kx * ny + t.i;
+      const Coef c = coef_x(kx);
+      CV<V> v[E];
 #pragma unroll
-      for (int f = 0; f < NIN; ++f) {
+      for (int j = 0; j < E; ++j) v[j] = ld_col(src + j * q, ny, two);
+      core_fft<-1>(v, t);
+      if constexpr (NIN == 1 && NOUT == 1) {
+        if (op == OP_K1) {
+          const T c1 = (T)2 * scale;
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          const C2<T> z = S[ix + sp(((f * npair + pr) << lgx) + x0) + j];
-          ina[f].v[j] = z.x; inb[f].v[j] = z.y;
+          for (int j = 0; j < E; ++j)
+            v[j] = escale(v[j], mult_k1(c.kx2, ldg_tab(&ktab[nkx + t.i + j * q]), c1));
+        } else if (op == OP_ID) {
+#pragma unroll
+          for (int j = 0; j < E; ++j) v[j] = escale(v[j], vset(scale, (V*)nullptr));
+        } else {
+          const bool smooth = op == OP_K2;
+          const T c2 = (smooth ? lam : (T)1) * (T)0.5 * scale;
+          const V gx = smooth ? vmul(c.gx, vset(c2, (V*)nullptr)) : vset(c2, (V*)nullptr);
+#pragma unroll
+          for (int j = 0; j < E; ++j) {
+            T ky, gy;
+            coef_y(t.i + j * q, ky, gy);
+            v[j] = escale(v[j], mult_k(c.kx2, ky, smooth ? vmul(gx, vset(gy, (V*)nullptr)) : gx));
+          }
+        }
+      } else if constexpr (NOUT == 2) {
+        // smoothed gradient i k G (odd factors are 0 at the Nyquist index of their axis); the
+        // transformed line waits in the second output's place (the same thread's positions)
+#pragma unroll
+        for (int j = 0; j < E; ++j) {
+          T ky, gy;
+          coef_y(t.i + j * q, ky, gy);
+          const V g = vmul(vmul(c.gx, vset(gy * scale, (V*)nullptr)), c.kxo);
+          if (mine) st_col(dst + nspec + j * q, ny, two, v[j]);
+          v[j] = CV<V>{vneg(vmul(v[j].y, g)), vmul(v[j].x, g)};
+        }
+        core_fft<+1>(v, t);
+#pragma unroll
+        for (int j = 0; j < E; ++j) {
+          if (mine) st_col(dst + j * q, ny, two, v[j]);
+          v[j] = ld_col(dst + nspec + j * q, ny, two);
+        }
+#pragma unroll
+        for (int j = 0; j < E; ++j) {
+          const int ky = t.i + j * q;
+          T k, gy;
+          coef_y(ky, k, gy);
+          if (ky == (ny >> 1)) k = (T)0;
+          const V g = vmul(c.gx, vset(gy * scale * k, (V*)nullptr));
+          v[j] = CV<V>{vneg(vmul(v[j].y, g)), vmul(v[j].x, g)};
+        }
+      } else {
+        // -(i kx G e_y - i ky G e_x) = i G (ky e_x - kx e_y); the first field's part waits in the
+        // output's place
+#pragma unroll
+        for (int j = 0; j < E; ++j) {
+          if (mine) st_col(dst + j * q, ny, two, v[j]);
+          v[j] = ld_col(src + nspec + j * q, ny, two);
+        }
+        core_fft<-1>(v, t);
+#pragma unroll
+        for (int j = 0; j < E; ++j) {
+          const int ky = t.i + j * q;
+          T k, gy;
+          coef_y(ky, k, gy);
+          if (ky == (ny >> 1)) k = (T)0;
+          const CV<V> a = ld_col(dst + j * q, ny, two);
+          const V kv = vset(k, (V*)nullptr), kn = vneg(c.kxo);
+          const V g = vmul(c.gx, vset(gy * scale, (V*)nullptr));
+          const CV<V> b = {vfma(kv, a.x, vmul(kn, v[j].x)), vfma(kv, a.y, vmul(kn, v[j].y))};
+          v[j] = CV<V>{vneg(vmul(b.y, g)), vmul(b.x, g)};
         }
       }
-      const long long i0 = (long long)(y0 + 2 * pr) * nx + x0;
-      if constexpr (Epi::kPair) {
-        epi.pair(i0, i0 + nx, ina, inb, oa, ob);
-      } else {
-        epi(i0, ina, oa);
-        epi(i0 + nx, inb, ob);
-      }
+      core_fft<+1>(v, t);
+      C2<T>* const out = NOUT == 2 ? dst + nspec : dst;
+      if (mine) {
 #pragma unroll
-      for (int f = 0; f < NOUT; ++f) {
-#pragma unroll
-        for (int j = 0; j < 4; ++j) S[ix + sp(((f * npair + pr) << lgx) + x0) + j] = C2<T>{oa[f].v[j], ob[f].v[j]};
+        for (int j = 0; j < E; ++j) st_col(out + j * q, ny, two, v[j]);
       }
     }
-    __syncthreads();
-    if constexpr (NOUT > 0) rows_forward_scatter<T, NOUT>(X, Y, Sout + y0, nspec, ny, npair, lgpair, lgx, twx);
-    epi_io.acc = epi.acc;
-    epi_io.accmax = epi.accmax;
-    epi_io.acc2 = epi.acc2;
+  }
+  template <int NIN, int NOUT>
+  __device__ __forceinline__ void cols_n(const C2<T>* Sin, C2<T>* Sout, int op) {
+    if (ey == 2) cols_e<2, NIN, NOUT>(Sin, Sout, op);
+    else if (sizeof(T) == 4 && ey == 4) cols_e<(sizeof(T) == 4 ? 4 : 2), NIN, NOUT>(Sin, Sout, op);
+    else cols_e<8, NIN, NOUT>(Sin, Sout, op);
+  }
+  __device__ __forceinline__ void cols(const C2<T>* Sin, int nin, C2<T>* Sout, int nout, int op) {
+    if (nin == 2) cols_n<2, 1>(Sin, Sout, op);
+    else if (nout == 2) cols_n<1, 2>(Sin, Sout, op);
+    else cols_n<1, 1>(Sin, Sout, op);
   }
 
-  // rows pass with optional per-item reductions into partials slots `slot` (acc or accmax)
-  // and `slot2` (acc2)
-  template <int NIN, int NOUT, class Epi>
-  __device__ void rows(int rb, const C2<T>* Sin, C2<T>* Sout, Epi& epi, int slot, int slot2 = -1) {
-    const int nitems = ny / rb;
-    for (int it = vb; it < nitems; it += (int)nblocks) {
-      epi.acc = 0.0;
-      epi.accmax = 0.0;
-      epi.acc2 = 0.0;
-      row_item<NIN, NOUT>(it * rb, rb, Sin, Sout, epi);
-      if (slot >= 0) {
-        const double v = epi.is_max ? block_max(epi.accmax, sh.red) : block_sum(epi.acc, sh.red);
-        if (threadIdx.x == 0) d.partials[(size_t)slot * d.max_items + it] = v;
-      }
-      if (slot2 >= 0) {
-        const double v = block_sum(epi.acc2, sh.red);
-        if (threadIdx.x == 0) d.partials[(size_t)slot2 * d.max_items + it] = v;
+  // ---- x pass over units of RU rows: inverse of NIN fields, epilogue, forward of NOUT ----
+  // The packed lines' upper half (positions nx - k) passes through the shared buffer: a thread
+  // loads the half spectrum at its k < nx/2 once, keeps Z[k] and hands Z[nx - k] over.
+  template <int E>
+  __device__ __forceinline__ void gather(CV<V> (&v)[E], const Team<T, E>& t, const C2<T>* src) {
+    const int nx = this->nx, q = t.step();
+    const long long ny = this->ny;
+    t.sync();
+#pragma unroll
+    for (int j = 0; j < E / 2; ++j) {
+      const int k = t.i + j * q;
+      const auto s = ld_b32(src + k * ny);
+      if (k == 0) {
+        v[j] = pack_re(s);
+      } else {
+        v[j] = pack_lo(s);
+        t.at(nx - k) = pack_hi(s);
       }
     }
+    if (t.i == 0) t.at(nx >> 1) = pack_re(ld_b32(src + (nx >> 1) * ny));
+    t.sync();
+#pragma unroll
+    for (int j = E / 2; j < E; ++j) v[j] = t.at(t.i + j * q);
   }
-  __device__ double total(int slot, int rb, bool is_max = false) {
-    return reduce_partials(d.partials, d.max_items, slot, ny / rb, is_max, sh.red);
+  template <int E>
+  __device__ __forceinline__ void scatter(CV<V> (&v)[E], const Team<T, E>& t, C2<T>* dst, bool mine) {
+    const int nx = this->nx, q = t.step();
+    const long long ny = this->ny;
+    t.sync();
+#pragma unroll
+    for (int j = E / 2; j < E; ++j) t.at(t.i + j * q) = v[j];
+    t.sync();
+#pragma unroll
+    for (int j = 0; j < E / 2; ++j) {
+      const int k = t.i + j * q;
+      const CV<V> zm = k == 0 ? v[j] : t.at(nx - k);
+      if (mine) st_b32(dst + k * ny, v[j], zm);
+    }
+    if (t.i == 0 && mine) st_b32(dst + (nx >> 1) * ny, v[E / 2], v[E / 2]);
+  }
+
+  // Row pass over the units of RU rows with optional per-unit sums into partials slots `slot` (acc,
+  // or the maximum of accmax) and `slot2` (acc2).  epi(i, r, in, out) is called for every element: i
+  // is the index of the unit's 16-byte vector (and mask byte), r the row-major index of its first
+  // row's cell.  With two inputs or two outputs one of the fields waits in `tmp` (a real field by row
+  // units) while the other one is transformed, so that a thread never holds two fields' elements.
+  // The sums are per unit whatever the number of CTAs, so a film gives the same bits on any launch.
+  template <int E, int NIN, int NOUT, class Epi>
+  __device__ __noinline__ void rows_e(const C2<T>* Sin, C2<T>* Sout, const Epi& epi_in, int slot, int slot2, T* tmp) {
+    Epi epi = epi_in;                   // register copy of the epilogue
+    const int nx = this->nx;
+    const long long nspec = this->nspec;
+    Team<T, E> t(sm, twx, lgx);
+    const int q = t.step(), tt = t.threads();
+    const int units = ny / RU;
+    const int want = (units + (int)nblocks - 1) / (int)nblocks, per = NT / tt;
+    const int nuc = want < per ? want : per;       // units that a CTA runs at a time
+    const int first = ((int)threadIdx.x & ~31) >> (lgx - Team<T, E>::LGE);   // slot of the warp's first lane
+    for (int u0 = vb * nuc; u0 < units; u0 += (int)nblocks * nuc) {
+      if (first >= nuc || u0 + first >= units) continue;
+      const bool mine = t.slot < nuc && u0 + t.slot < units;
+      const int unit = mine ? u0 + t.slot : u0;
+      const int y0 = unit * RU;
+      const long long iu = (long long)unit * nx + t.i;
+      const long long ir = (long long)y0 * nx + t.i;
+      epi.acc = 0;
+      epi.accmax = 0;
+      epi.acc2 = 0;
+      CV<V> v[E];
+      // the epilogue's fields, B elements at a time: the first batch is on its way during the
+      // inverse transform, each further one while the batch before is worked on
+      constexpr int B = Epi::kBatch < E ? Epi::kBatch : E;
+      typename Epi::Ld ld[2][B];
+      if constexpr (NIN > 0) gather<E>(v, t, Sin + y0);
+      if constexpr (NIN == 2) {
+        core_fft<+1>(v, t);
+        if (mine) {
+#pragma unroll
+          for (int j = 0; j < E; ++j) st_q(tmp + (iu + j * q) * RU, to_q(v[j]));
+        }
+        gather<E>(v, t, Sin + nspec + y0);
+      }
+#pragma unroll
+      for (int b = 0; b < B; ++b) ld[0][b] = epi.load(iu + b * q, ir + b * q);
+      if constexpr (NIN > 0) core_fft<+1>(v, t);
+#pragma unroll
+      for (int j0 = 0; j0 < E; j0 += B) {
+        if (j0 + B < E) {
+#pragma unroll
+          for (int b = 0; b < B; ++b) ld[(j0 / B + 1) & 1][b] = epi.load(iu + (j0 + B + b) * q, ir + (j0 + B + b) * q);
+        }
+        Q<T> in0[B];
+        if constexpr (NIN == 2) {
+#pragma unroll
+          for (int b = 0; b < B; ++b) in0[b] = ld_q(tmp + (iu + (j0 + b) * q) * RU);
+        }
+        if (mine) {
+#pragma unroll
+          for (int b = 0; b < B; ++b) {
+            const int j = j0 + b;
+            Q<T> in[NIN > 0 ? NIN : 1], out[NOUT > 0 ? NOUT : 1];
+            const long long i = iu + j * q;
+            if constexpr (NIN == 2) { in[0] = in0[b]; in[1] = to_q(v[j]); }
+            if constexpr (NIN == 1) in[0] = to_q(v[j]);
+            epi.apply(ld[(j0 / B) & 1][b], i, ir + j * q, in, out);
+            if constexpr (NOUT > 0) v[j] = to_e(out[0]);
+            if constexpr (NOUT == 2) st_q(tmp + i * RU, out[1]);
+          }
+        }
+      }
+      if constexpr (NOUT > 0) {
+        core_fft<-1>(v, t);
+        scatter<E>(v, t, Sout + y0, mine);
+      }
+      if constexpr (NOUT == 2) {
+#pragma unroll
+        for (int j = 0; j < E; ++j) v[j] = to_e(ld_q(tmp + (iu + j * q) * RU));
+        core_fft<-1>(v, t);
+        scatter<E>(v, t, Sout + nspec + y0, mine);
+      }
+      if (slot >= 0) unit_sums(epi, t, unit, mine, slot, slot2);
+    }
+  }
+  // a unit's sums: over the lanes of its team, then (teams of several warps) over the team's warps in
+  // FP64 by one thread per sum (threads of two sub-partitions: an FP64 addition takes 64 cycles)
+  template <int E, class Epi>
+  __device__ __forceinline__ void unit_sums(const Epi& epi, const Team<T, E>& t, int unit, bool mine, int slot, int slot2) {
+    const int tt = t.threads(), w = threadIdx.x >> 5, l = threadIdx.x & 31;
+    const int width = tt < 32 ? tt : 32;
+    auto a = epi.is_max ? epi.accmax : epi.acc;
+    auto b = epi.acc2;
+    for (int o = width >> 1; o > 0; o >>= 1) {
+      const auto x = __shfl_xor_sync(0xffffffffu, a, o);
+      a = epi.is_max ? (x > a ? x : a) : a + x;
+      if (slot2 >= 0) b += __shfl_xor_sync(0xffffffffu, b, o);
+    }
+    double* const pa = partials + (size_t)slot * max_items + unit;
+    double* const pb = partials + (size_t)slot2 * max_items + unit;
+    if (tt <= 32) {
+      if (t.i == 0 && mine) {
+        *pa = (double)a;
+        if (slot2 >= 0) *pb = (double)b;
+      }
+      return;
+    }
+    t.sync();                           // the unit before has been summed
+    if (l == 0) {
+      sh.red[w] = (double)a;
+      if (slot2 >= 0) sh.red2[w] = (double)b;
+    }
+    t.sync();
+    // by lanes 0 .. warps - 1 of the team's first warp (acc) and second warp (acc2)
+    const int nw = tt / 32;
+    if ((t.i >> 5) == 0) {
+      double s = sh.red[w + (l & (nw - 1))];
+      for (int o = nw >> 1; o > 0; o >>= 1) {
+        const double x = __shfl_xor_sync(0xffffffffu, s, o);
+        s = epi.is_max ? (x > s ? x : s) : s + x;
+      }
+      if (l == 0) *pa = s;
+    } else if ((t.i >> 5) == 1 && slot2 >= 0) {
+      double s = sh.red2[w - 1 + (l & (nw - 1))];
+      for (int o = nw >> 1; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+      if (l == 0) *pb = s;
+    }
+  }
+  template <int NIN, int NOUT, class Epi>
+  __device__ __forceinline__ void rows(const C2<T>* Sin, C2<T>* Sout, const Epi& epi, int slot, int slot2 = -1, T* tmp = nullptr) {
+    if (ex == 2) rows_e<2, NIN, NOUT>(Sin, Sout, epi, slot, slot2, tmp);
+    else if (sizeof(T) == 4 && ex == 4) rows_e<(sizeof(T) == 4 ? 4 : 2), NIN, NOUT>(Sin, Sout, epi, slot, slot2, tmp);
+    else rows_e<8, NIN, NOUT>(Sin, Sout, epi, slot, slot2, tmp);
+  }
+  // Sums over the units of slots a and (b >= 0) b, in a fixed order: the last warps first, which have
+  // no line to run while the pass before is narrow, so that the sums of a small film are formed
+  // beside its column pass.  The result is valid in thread SUMS, which the caller lets go on.
+  static constexpr int SUMS = NT - 32;
+  __device__ double2 partial_sums(int a, int b) {
+    const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
+    const int n = ny / RU;
+    const bool few = n <= 128;             // two warps per slot, else four
+    const int per = few ? 2 : 4;
+    const int sl = few ? (w < 4 ? -1 : w < 6 ? a : b) : (w < 4 ? b : a);
+    if (sl >= 0) {
+      const double* p = partials + (size_t)sl * max_items;
+      double v = 0.0;
+      for (int i = (w & (per - 1)) * 32 + l; i < n; i += per * 32) v += __ldcg(p + i);
+      v = warp_sum(v);
+      if (l == 0) sh.red[w] = v;
+    }
+    __syncthreads();
+    double2 r = make_double2(0.0, 0.0);
+    if (threadIdx.x == SUMS) {
+      const double* q = sh.red;
+      if (few) {
+        r.x = q[4] + q[5];
+        if (b >= 0) r.y = q[6] + q[7];
+      } else {
+        r.x = (q[4] + q[5]) + (q[6] + q[7]);
+        if (b >= 0) r.y = (q[0] + q[1]) + (q[2] + q[3]);
+      }
+    }
+    return r;
+  }
+  // sum (max) over the units of a slot, the same in every thread of every CTA
+  __device__ double total(int slot, bool is_max = false) {
+    return reduce_partials(partials, max_items, slot, ny / RU, is_max, sh.red);
   }
   // Eq. 10 and Eq. 11 constants from the sums of h (slot 0) and q1 h (slot 5) of the pass that
-  // wrote h: A = (sum h - N h_e_dot) / n_out, C = (<q1, h> - A sum_out q1) / n_out; computed once
-  // by thread 0 and broadcast (the double-precision division runs at a low rate on this part)
-  __device__ void shifts(int rb, double N, double hed, double nout, double& A, double& C) {
-    reduce_partials2(d.partials, d.max_items, 0, 5, ny / rb, sh.red);
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      const double a = (sh.red[0] - N * hed) / nout;
-      sh.red[2] = a;
-      sh.red[3] = (sh.red[1] - a * sh.q11) / nout;
+  // wrote h: A = (sum h - N h_e_dot) / n_out, C = (<q1, h> - A sum_out q1) / n_out
+  __device__ void shifts() {
+    const double2 t = partial_sums(0, 5);
+    if (threadIdx.x == SUMS) {
+      const double A = (t.x - sh.N * sh.hed) * sh.inv_nout;
+      const double C = (t.y - A * sh.q11) * sh.inv_nout;
+      sh.A = A;
+      sh.C = C;
+      sh.Af = (float)A;
+      sh.Cf = (float)C;
     }
     __syncthreads();
-    A = sh.red[2];
-    C = sh.red[3];
-    __syncthreads();
   }
-  // mean over free space of the residual sum in slot 2 (broadcast like shifts)
-  __device__ double mean_out(int slot, int rb, double nout) {
-    const double s = reduce_partials(d.partials, d.max_items, slot, ny / rb, false, sh.red);
-    if (threadIdx.x == 0) sh.red[2] = s / nout;
+  // the sum of a slot / n_out (sh.A), in the transform precision
+  __device__ T mean_of(int slot) {
+    const double2 t = partial_sums(slot, -1);
+    if (threadIdx.x == SUMS) {
+      sh.A = t.x * sh.inv_nout;
+      sh.Af = (float)sh.A;
+    }
     __syncthreads();
-    const double r = sh.red[2];
+    return At();
+  }
+  // the outside iteration's scalars in the transform precision
+  __device__ __forceinline__ T At() const { if constexpr (sizeof(T) == 4) return sh.Af; else return sh.A; }
+  __device__ __forceinline__ T Ct() const { if constexpr (sizeof(T) == 4) return sh.Cf; else return sh.C; }
+  // Section 2.3: r = mean over free space of |g_dot| (slot 2) and the decision to stop
+  __device__ void stop_test(bool by_count, bool last) {
+    const double2 t = partial_sums(2, -1);
+    if (threadIdx.x == SUMS) {
+      const double r = t.x * sh.inv_nout;
+      sh.r = r;
+      sh.stop = by_count ? last : (r < iter_tol || last);
+    }
     __syncthreads();
-    return r;
   }
 };
 
 // ------------------------------------------------------------------------------------------
 // epilogues
 // ------------------------------------------------------------------------------------------
-// Epilogues of the x pass: called with the index i of the first of four consecutive cells of
-// one row, the inverse-transformed inputs in[f].v[0..3] and outputs out[f].v[0..3].
+// Epilogues of the x pass: load(i, r) reads the fields of the RU rows of one element, with the index
+// i of their 16-byte vector and the row-major index r of the first row's cell (the others nx
+// apart); apply(ld, i, r, in, out) works on them with the inverse-transformed inputs
+// in[f].v[0 .. RU) and sets the outputs out[f].v[0 .. RU).  kBatch elements are loaded together
+// (a store could alias a later load as far as the compiler knows, so a load placed behind a store
+// waits for the whole latency of the loads before it).
+struct NoLd {};
+
+// FP64 state fields are row-major (the caller's layout)
+__device__ __forceinline__ double ld_s(const double* p) {
+  double v;
+  asm volatile("ld.global.L1::no_allocate.f64 %0, [%1];" : "=d"(v) : "l"(p) : "memory");
+  return v;
+}
 
 // P1 / readouts: field from the FP64 stage input
 template <typename T>
 struct EpiStage : EpiBase<T> {
+  static constexpr int RU = Lane<T>::RU;
   FilmPtrs<T> P;
   StageIn in;
-  __device__ void operator()(long long i, const V4<T>*, V4<T>* out) {
-    V4<double> v = ld4(in.y + i);
+  static constexpr int kBatch = 2;
+  struct Ld { double v[RU]; };
+  __device__ __forceinline__ Ld load(long long, long long r) const {
+    Ld l;
+#pragma unroll
+    for (int q = 0; q < RU; ++q) l.v[q] = ld_s(in.y + r + (long long)q * P.nx);
     for (int j = 0; j < in.nk; ++j) {
-      const V4<double> k = ld4(in.k[j] + i);
+      double k[RU];
 #pragma unroll
-      for (int q = 0; q < 4; ++q) v.v[q] += in.c[j] * k.v[q];
+      for (int q = 0; q < RU; ++q) k[q] = ld_s(in.k[j] + r + (long long)q * P.nx);
+#pragma unroll
+      for (int q = 0; q < RU; ++q) l.v[q] += in.c[j] * k[q];
     }
-    if (in.ynew) st4(in.ynew + i, v);
+    return l;
+  }
+  __device__ __forceinline__ void apply(const Ld& l, long long, long long r, const Q<T>*, Q<T>* out) {
+    if (in.ynew) {
 #pragma unroll
-    for (int q = 0; q < 4; ++q) out[0].v[q] = (T)v.v[q];
+      for (int q = 0; q < RU; ++q) in.ynew[r + (long long)q * P.nx] = l.v[q];
+    }
+#pragma unroll
+    for (int q = 0; q < RU; ++q) out[0].v[q] = (T)l.v[q];
   }
 };
 
@@ -403,10 +678,12 @@ struct EpiStage : EpiBase<T> {
 template <typename T>
 struct EpiOut : EpiBase<T> {
   FilmPtrs<T> P;
-  __device__ void operator()(long long i, const V4<T>*, V4<T>* out) {
-    const uchar4 m = ldmask4(P.mask + i);
+  static constexpr int kBatch = 4;
+  struct Ld { int m; };
+  __device__ __forceinline__ Ld load(long long i, long long) const { return Ld{ld_mask(P.mask + i)}; }
+  __device__ __forceinline__ void apply(const Ld& l, long long, long long, const Q<T>*, Q<T>* out) {
 #pragma unroll
-    for (int q = 0; q < 4; ++q) out[0].v[q] = mask_at(m, q) == 0 ? (T)1 : (T)0;
+    for (int q = 0; q < Lane<T>::RU; ++q) out[0].v[q] = cls(l.m, q) == 0 ? (T)1 : (T)0;
   }
 };
 
@@ -415,12 +692,14 @@ template <typename T>
 struct EpiStoreT : EpiBase<T> {
   FilmPtrs<T> P;
   T* dst;
-  __device__ void operator()(long long i, const V4<T>* in, V4<T>*) {
-    st4(dst + i, in[0]);
-    const uchar4 m = ldmask4(P.mask + i);
+  static constexpr int kBatch = 4;
+  struct Ld { int m; };
+  __device__ __forceinline__ Ld load(long long i, long long) const { return Ld{ld_mask(P.mask + i)}; }
+  __device__ __forceinline__ void apply(const Ld& l, long long i, long long, const Q<T>* in, Q<T>*) {
+    st_q(dst + i * Lane<T>::RU, in[0]);
 #pragma unroll
-    for (int q = 0; q < 4; ++q)
-      if (mask_at(m, q) == 0) this->acc += (double)in[0].v[q];
+    for (int q = 0; q < Lane<T>::RU; ++q)
+      if (cls(l.m, q) == 0) this->acc += (double)in[0].v[q];
   }
 };
 // h_z readout (FP64)
@@ -429,11 +708,12 @@ struct EpiStoreHz : EpiBase<T> {
   FilmPtrs<T> P;
   double* dst;
   double he;
-  __device__ void operator()(long long i, const V4<T>* in, V4<T>*) {
-    V4<double> o;
+  static constexpr int kBatch = 4;
+  using Ld = NoLd;
+  __device__ __forceinline__ Ld load(long long, long long) const { return Ld{}; }
+  __device__ __forceinline__ void apply(const Ld&, long long, long long r, const Q<T>* in, Q<T>*) {
 #pragma unroll
-    for (int q = 0; q < 4; ++q) o.v[q] = he + (double)in[0].v[q];
-    st4(dst + i, o);
+    for (int q = 0; q < Lane<T>::RU; ++q) dst[r + (long long)q * P.nx] = he + (double)in[0].v[q];
   }
 };
 
@@ -444,18 +724,27 @@ template <typename T>
 struct EpiPower : EpiBase<T> {
   FilmPtrs<T> P;
   T n, e0, jc, rho_out, ig2;
-  __device__ void operator()(long long i, const V4<T>* in, V4<T>* out) {
-    const uchar4 m = ldmask4(P.mask + i);
-    V4<T> jcl;
-    if (P.jcmap) jcl = ldg4(P.jcmap + i);
-    else jcl = V4<T>{{jc, jc, jc, jc}};
+  static constexpr int kBatch = 4;
+  struct Ld { int m; Q<T> jc; };
+  __device__ __forceinline__ Ld load(long long i, long long) const {
+    Ld l;
+    l.m = ld_mask(P.mask + i);
+    if (P.jcmap) {
+      l.jc = ldg_q(P.jcmap + i * Lane<T>::RU);
+    } else {
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
+      for (int q = 0; q < Lane<T>::RU; ++q) l.jc.v[q] = jc;
+    }
+    return l;
+  }
+  __device__ __forceinline__ void apply(const Ld& l, long long, long long, const Q<T>* in, Q<T>* out) {
+#pragma unroll
+    for (int q = 0; q < Lane<T>::RU; ++q) {
       const T gx = in[0].v[q], gy = in[1].v[q];
       const T jx = gy, jy = -gx;                              // Eq. 2
-      const int mq = mask_at(m, q);
+      const int mq = cls(l.m, q);
       const T a = mq == 1 ? ig2 : (T)1;
-      const T rho = resistivity<T>(jx * jx + jy * jy * a, jcl.v[q], mq, n, e0, rho_out);
+      const T rho = resistivity<T>(jx * jx + jy * jy * a, l.jc.v[q], mq, n, e0, rho_out);
       out[0].v[q] = rho * jx;                                 // Eq. 3
       out[1].v[q] = rho * jy * a;
     }
@@ -469,59 +758,51 @@ struct EpiInit : EpiBase<T, T> {
   bool warm;
   const T* wsrc;          // warm start (the previous time step's or the most recent iterate)
   T A_prev, hed;
-  struct Ld { uchar4 m; V4<T> w, q1; };
-  __device__ __forceinline__ Ld load(long long i) const {
+  static constexpr int kBatch = 4;
+  struct Ld { int m; Q<T> w, q1; };
+  __device__ __forceinline__ Ld load(long long i, long long) const {
     Ld l;
-    l.m = ldmask4(P.mask + i);
-    if (warm) l.w = ld4(wsrc + i);
-    l.q1 = ldg4(P.q1 + i);
+    l.m = ld_mask(P.mask + i);
+    if (warm) l.w = ld_q(wsrc + i * Lane<T>::RU);
+    l.q1 = ldg_q(P.q1 + i * Lane<T>::RU);
     return l;
   }
-  __device__ __forceinline__ V4<T> apply(const Ld& l, const V4<T>* in) {
-    V4<T> h;
+  __device__ __forceinline__ void apply(const Ld& l, long long i, long long, const Q<T>* in, Q<T>* out) {
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      if (mask_at(l.m, q) != 0) h.v[q] = in[0].v[q];           // h_dot_in on the conductor
-      else h.v[q] = warm ? l.w.v[q] - A_prev : hed;           // warm start (Section 2.2)
-      this->acc += h.v[q];
-      this->acc2 += l.q1.v[q] * h.v[q];                       // <q1, h> for C
+    for (int q = 0; q < Lane<T>::RU; ++q) {
+      T h;
+      if (cls(l.m, q) != 0) h = in[0].v[q];                   // h_dot_in on the conductor
+      else h = warm ? l.w.v[q] - A_prev : hed;                // warm start (Section 2.2)
+      this->acc += h;
+      this->acc2 += l.q1.v[q] * h;                              // <q1, h> for C
+      out[0].v[q] = h;
     }
-    return h;
-  }
-  __device__ void operator()(long long i, const V4<T>* in, V4<T>* out) {
-    const V4<T> h = apply(load(i), in);
-    st4(P.hd + i, h);
-    out[0] = h;
-  }
-  static constexpr bool kPair = true;
-  __device__ __forceinline__ void pair(long long ia, long long ib, const V4<T>* ina, const V4<T>* inb,
-                                       V4<T>* oa, V4<T>* ob) {
-    const Ld la = load(ia), lb = load(ib);
-    oa[0] = apply(la, ina);
-    ob[0] = apply(lb, inb);
-    st4(P.hd + ia, oa[0]);
-    st4(P.hd + ib, ob[0]);
+    st_q(P.hd + i * Lane<T>::RU, out[0]);
   }
 };
 
-// P7: g_dot = raw - A q1 - C (Eq. 11), stored; residual sum over free space of |g_dot|
-// (Section 2.3); forward of mask_out g_dot (the input of Eq. 12)
+// P7: g_dot = raw - A q1 - C (Eq. 11), stored where the unit touches the conductor (all that the
+// final pass reads); residual sum over free space of |g_dot| (Section 2.3); forward of
+// mask_out g_dot (the input of Eq. 12)
 template <typename T>
 struct EpiU : EpiBase<T, T> {
   FilmPtrs<T> P;
   T A, C;
-  __device__ void operator()(long long i, const V4<T>* in, V4<T>* out) {
-    const uchar4 m = ldmask4(P.mask + i);
-    const V4<T> q1 = ldg4(P.q1 + i);
-    V4<T> v;
+  static constexpr int kBatch = 4;
+  struct Ld { int m; Q<T> q1; };
+  __device__ __forceinline__ Ld load(long long i, long long) const {
+    return Ld{ld_mask(P.mask + i), ldg_q(P.q1 + i * Lane<T>::RU)};
+  }
+  __device__ __forceinline__ void apply(const Ld& l, long long i, long long, const Q<T>* in, Q<T>* out) {
+    Q<T> v;
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      v.v[q] = (in[0].v[q] - A * q1.v[q]) - C;
-      const bool o = mask_at(m, q) == 0;
+    for (int q = 0; q < Lane<T>::RU; ++q) {
+      v.v[q] = (in[0].v[q] - A * l.q1.v[q]) - C;
+      const bool o = cls(l.m, q) == 0;
       if (o) this->acc += fabs(v.v[q]);
       out[0].v[q] = o ? v.v[q] : (T)0;
     }
-    st4(P.u + i, v);
+    if (l.m != 0) st_q(P.u + i * Lane<T>::RU, v);
   }
 };
 
@@ -531,73 +812,68 @@ template <typename T>
 struct EpiUpdate : EpiBase<T, T> {
   FilmPtrs<T> P;
   T A;
-  struct Ld { uchar4 m; V4<T> h, q1; };
-  __device__ __forceinline__ Ld load(long long i) const {
-    return Ld{ldmask4(P.mask + i), ld4(P.hd + i), ldg4(P.q1 + i)};
+  static constexpr int kBatch = 4;
+  struct Ld { int m; Q<T> h, q1; };
+  __device__ __forceinline__ Ld load(long long i, long long) const {
+    return Ld{ld_mask(P.mask + i), ld_q(P.hd + i * Lane<T>::RU), ldg_q(P.q1 + i * Lane<T>::RU)};
   }
-  __device__ __forceinline__ V4<T> apply(Ld l, const V4<T>* in) {
+  __device__ __forceinline__ void apply(const Ld& l, long long i, long long, const Q<T>* in, Q<T>* out) {
+    Q<T> h = l.h;
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      if (mask_at(l.m, q) == 0) l.h.v[q] = (l.h.v[q] - A) - in[0].v[q];
-      this->acc += l.h.v[q];
-      this->acc2 += l.q1.v[q] * l.h.v[q];
+    for (int q = 0; q < Lane<T>::RU; ++q) {
+      if (cls(l.m, q) == 0) h.v[q] = (h.v[q] - A) - in[0].v[q];
+      this->acc += h.v[q];
+      this->acc2 += l.q1.v[q] * h.v[q];
     }
-    return l.h;
-  }
-  __device__ void operator()(long long i, const V4<T>* in, V4<T>* out) {
-    const V4<T> h = apply(load(i), in);
-    st4(P.hd + i, h);
+    st_q(P.hd + i * Lane<T>::RU, h);
     out[0] = h;
-  }
-  static constexpr bool kPair = true;
-  __device__ __forceinline__ void pair(long long ia, long long ib, const V4<T>* ina, const V4<T>* inb,
-                                       V4<T>* oa, V4<T>* ob) {
-    const Ld la = load(ia), lb = load(ib);
-    oa[0] = apply(la, ina);
-    ob[0] = apply(lb, inb);
-    st4(P.hd + ia, oa[0]);
-    st4(P.hd + ib, ob[0]);
   }
 };
 
 // finalize: g_dot (stored by P7) on the conductor; optional BS23 error contribution
-template <typename T>
-struct EpiFinal : EpiBase<T> {
+template <typename T, bool err>
+struct EpiFinal : EpiBase<T, T> {
   FilmPtrs<T> P;
   double* kout;
-  // error estimate (stage 4 of a step): E = h (e1 k1 + e2 k2 + e3 k3 + e4 k4)
-  bool err;
+  // err: error estimate (stage 4 of a step): E = h (e1 k1 + e2 k2 + e3 k3 + e4 k4)
   double h, rtol, atol;
   const double* k1; const double* k2; const double* k3; const double* y; const double* ynew;
-  __device__ void operator()(long long i, const V4<T>*, V4<T>*) {
-    const uchar4 m = ldmask4(P.mask + i);
-    const V4<T> u = ld4(P.u + i);
-    V4<double> g;
+  static constexpr int RU = Lane<T>::RU, NE = err ? RU : 1, kBatch = err ? 1 : 4;
+  struct Ld { int m; Q<T> u; double a1[NE], a2[NE], a3[NE], y[NE], yn[NE]; };
+  __device__ __forceinline__ Ld load(long long i, long long r) const {
+    Ld l;
+    l.m = ld_mask(P.mask + i);
+    l.u = ld_q(P.u + i * RU);                              // defined on the conductor's units only
+    if constexpr (err) {
 #pragma unroll
-    for (int q = 0; q < 4; ++q) g.v[q] = mask_at(m, q) != 0 ? (double)u.v[q] : 0.0;
-    if (err) {
-      // the loads before the store (a store could alias a later load as far as the compiler
-      // knows, which would put the loads behind it)
-      const V4<double> a1 = ld4(k1 + i), a2 = ld4(k2 + i), a3 = ld4(k3 + i), yy = ld4(y + i), yn = ld4(ynew + i);
-      st4(kout + i, g);
+      for (int q = 0; q < RU; ++q) {
+        const long long c = r + (long long)q * P.nx;
+        l.a1[q] = ld_s(k1 + c); l.a2[q] = ld_s(k2 + c); l.a3[q] = ld_s(k3 + c);
+        l.y[q] = ld_s(y + c); l.yn[q] = ld_s(ynew + c);
+      }
+    }
+    return l;
+  }
+  __device__ __forceinline__ void apply(const Ld& l, long long, long long r, const Q<T>*, Q<T>*) {
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const double E = h * (-5.0 / 72.0 * a1.v[q] + 1.0 / 12.0 * a2.v[q] + 1.0 / 9.0 * a3.v[q] - 0.125 * g.v[q]);
-        const double sc = atol + rtol * fmax(fabs(yy.v[q]), fabs(yn.v[q]));
+    for (int q = 0; q < RU; ++q) {
+      const bool in = cls(l.m, q) != 0;
+      const double g = in ? (double)l.u.v[q] : 0.0;
+      kout[r + (long long)q * P.nx] = g;
+      if constexpr (err) {
+        const double E = h * (-5.0 / 72.0 * l.a1[q] + 1.0 / 12.0 * l.a2[q] + 1.0 / 9.0 * l.a3[q] - 0.125 * g);
+        const double sc = atol + rtol * fmax(fabs(l.y[q]), fabs(l.yn[q]));
         // E and its scale in FP64; their ratio, which only feeds the accept test and the step
         // size factor, in the transform precision (FP64 division runs at a small fraction of the
         // FP32 rate on this part)
-        double r;
-        if constexpr (sizeof(T) == 4) r = (double)__fdiv_rn((float)fabs(E), (float)sc);
-        else r = fabs(E) / sc;
-        if (!(r == r) || isinf(r)) r = 1e300;                // non-finite -> rejected step
-        this->accmax = fmax(this->accmax, r);
+        T e;
+        if constexpr (sizeof(T) == 4) e = __fdiv_rn((float)fabs(E), (float)sc);
+        else e = fabs(E) / sc;
+        if (!(e == e)) e = (T)INFINITY;                      // non-finite -> rejected step
+        this->accmax = this->accmax > e ? this->accmax : e;
+      } else if (in && !isfinite(l.u.v[q])) {
+        this->accmax = (T)1;
       }
-    } else {
-      st4(kout + i, g);
-#pragma unroll
-      for (int q = 0; q < 4; ++q)
-        if (!isfinite(g.v[q])) this->accmax = 1.0;
     }
   }
 };
@@ -610,23 +886,22 @@ struct EpiStoreE : EpiBase<T> {
   T n, e0, jc, rho_out, ig2;
   double* dst;
   long long ncell;
-  __device__ void operator()(long long i, const V4<T>* in, V4<T>*) {
-    const uchar4 m = ldmask4(P.mask + i);
-    V4<T> jcl;
-    if (P.jcmap) jcl = ldg4(P.jcmap + i);
-    else jcl = V4<T>{{jc, jc, jc, jc}};
-    V4<double> ex, ey;
+  static constexpr int kBatch = 4;
+  using Ld = typename EpiPower<T>::Ld;
+  __device__ __forceinline__ EpiPower<T> law() const {       // the law of P3
+    EpiPower<T> p;
+    p.P = P; p.n = n; p.e0 = e0; p.jc = jc; p.rho_out = rho_out; p.ig2 = ig2;
+    return p;
+  }
+  __device__ __forceinline__ Ld load(long long i, long long r) const { return law().load(i, r); }
+  __device__ __forceinline__ void apply(const Ld& l, long long i, long long r, const Q<T>* in, Q<T>*) {
+    Q<T> e[2];
+    law().apply(l, i, r, in, e);
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const T jx = in[1].v[q], jy = -in[0].v[q];
-      const int mq = mask_at(m, q);
-      const T a = mq == 1 ? ig2 : (T)1;                       // elliptic law, as in EpiPower
-      const T rho = resistivity<T>(jx * jx + jy * jy * a, jcl.v[q], mq, n, e0, rho_out);
-      ex.v[q] = (double)(rho * jx);
-      ey.v[q] = (double)(rho * jy * a);
+    for (int q = 0; q < Lane<T>::RU; ++q) {
+      dst[r + (long long)q * P.nx] = (double)e[0].v[q];
+      dst[ncell + r + (long long)q * P.nx] = (double)e[1].v[q];
     }
-    st4(dst + i, ex);
-    st4(dst + ncell + i, ey);
   }
 };
 
@@ -635,9 +910,17 @@ template <typename T>
 struct EpiMoment : EpiBase<T> {
   FilmPtrs<T> P;
   const double* g;
-  __device__ void operator()(long long i, const V4<T>*, V4<T>*) {
-    const V4<double> v = ld4(g + i);
-    this->acc += (v.v[0] + v.v[1]) + (v.v[2] + v.v[3]);
+  static constexpr int kBatch = 4;
+  struct Ld { double v[Lane<T>::RU]; };
+  __device__ __forceinline__ Ld load(long long, long long r) const {
+    Ld l;
+#pragma unroll
+    for (int q = 0; q < Lane<T>::RU; ++q) l.v[q] = ld_s(g + r + (long long)q * P.nx);
+    return l;
+  }
+  __device__ __forceinline__ void apply(const Ld& l, long long, long long, const Q<T>*, Q<T>*) {
+#pragma unroll
+    for (int q = 0; q < Lane<T>::RU; ++q) this->acc += l.v[q];
   }
 };
 
@@ -651,18 +934,23 @@ __device__ __noinline__ RhsOut film_rhs(Film<T>& F, double t, int seg, const Sta
                            const double* e_ynew) {
   const Desc& d = F.d;
   RhsOut res{ST_OK, 0, 0.0, 0.0, 0};
-  const double hed = he_dot(d, t, seg);
-  const double N = (double)F.ncell;
-  const double nout = (double)d.nout;
   const bool first = F.sh.attempt_first != 0;   // read by every thread before it is cleared
   // h_dot buffers: this call writes hdw; hdc holds the committed (accepted-step) h_dot
   T* const hdw = (T*)(F.sh.hd_sel ? d.hd2 : d.hd);
   const T* const hdc = (const T*)(F.sh.hd_sel ? d.hd : d.hd2);
+  if (threadIdx.x == 0) {               // scalar FP64 work: one thread (see Control)
+    const double hed = he_dot(d, t, seg);
+    const double Ap = first && F.sh.com_valid != 0 ? F.sh.A_com : F.sh.A_prev;
+    F.sh.hed = hed;
+    F.sh.rq = (float)hed;
+    F.sh.A = Ap;
+    F.sh.Af = (float)Ap;
+  }
 
   // P1
   {
     EpiStage<T> e; e.P = F.ptrs(); e.in = sin;
-    F.rows<0, 1>(F.rb1, nullptr, F.Sa, e, -1);
+    F.rows<0, 1>(nullptr, F.Sa, e, -1);
   }
   if (!F.sync(1)) { res.status = ST_BARRIER; return res; }
   F.cols(F.Sa, 1, F.Sa, 2, OP_GRAD);                                    // P2
@@ -670,8 +958,8 @@ __device__ __noinline__ RhsOut film_rhs(Film<T>& F, double t, int seg, const Sta
   {
     EpiPower<T> e; e.P = F.ptrs();
     e.n = (T)d.n; e.e0 = (T)d.e0; e.jc = (T)d.jc; e.rho_out = (T)d.rho_out;
-    e.ig2 = (T)(1.0 / (d.gamma * d.gamma));
-    F.rows<2, 2>(F.rb2, F.Sa, F.Sb, e, -1);                             // P3
+    e.ig2 = F.ig2;
+    F.rows<2, 2>(F.Sa, F.Sb, e, -1, -1, F.u);                           // P3
   }
   if (!F.sync(3)) { res.status = ST_BARRIER; return res; }
   F.cols(F.Sb, 2, F.Sb, 1, OP_CURLNEG);                                 // P4
@@ -686,62 +974,72 @@ __device__ __noinline__ RhsOut film_rhs(Film<T>& F, double t, int seg, const Sta
     const bool com = first && F.sh.com_valid != 0;
     e.warm = com || F.sh.warm_valid != 0;
     e.wsrc = com ? hdc : hdw;
-    e.A_prev = (T)(com ? F.sh.A_com : F.sh.A_prev); e.hed = (T)hed;
-    F.rows<1, 1>(F.rb1, F.Sb, F.Sa, e, 0, 5);                           // P5
+    e.A_prev = F.At();                   // the warm start's shift (set above)
+    if constexpr (sizeof(T) == 4) e.hed = F.sh.rq;
+    else e.hed = F.sh.hed;
+    F.rows<1, 1>(F.Sb, F.Sa, e, 0, 5);                                  // P5
   }
   if (!F.sync(5)) { res.status = ST_BARRIER; return res; }
-  // Eq. 10: A; Eq. 11: C = (<q1, h> - A sum_out q1) / n_out (K1 is real and even)
-  double A = 0.0, C = 0.0;
-  if (have_out) F.shifts(F.rb1, N, hed, nout, A, C);
-  double r = 0.0;
+  if (!have_out) {
+    if (threadIdx.x == 0) { F.sh.A = 0.0; F.sh.C = 0.0; F.sh.Af = 0.f; F.sh.Cf = 0.f; F.sh.r = 0.0; }
+    __syncthreads();
+  }
   const bool forced = force_iters > 0;
-  const bool fixed = d.iter_tol <= 0.0;
+  const bool by_count = forced || d.iter_tol <= 0.0;
   int itmax = forced ? force_iters : d.iter_max;
   if (!have_out) itmax = 1;
   int i = 0;
   for (; i < itmax; ++i) {
     F.cols(F.Sa, 1, F.Sa, 1, OP_K1);                                    // P6
+    // Eq. 10: A; Eq. 11: C = (<q1, h> - A sum_out q1) / n_out (K1 is real and even).  P6 does not
+    // need them, so the sums of P5 / P10 are combined beside it.
+    if (have_out) F.shifts();
     if (!F.sync(6)) { res.status = ST_BARRIER; return res; }
     {
-      EpiU<T> e; e.P = F.ptrs(); e.A = (T)A; e.C = (T)C;
-      F.rows<1, 1>(F.rb1, F.Sa, F.Sb, e, 2);                            // P7
+      EpiU<T> e; e.P = F.ptrs(); e.A = F.At(); e.C = F.Ct();
+      F.rows<1, 1>(F.Sa, F.Sb, e, 2);                                   // P7
     }
     if (!F.sync(7)) { res.status = ST_BARRIER; return res; }
-    if (!have_out) { r = 0.0; break; }
-    r = F.mean_out(2, F.rb1, nout);                                     // Section 2.3
-    const bool last = (i == itmax - 1);
-    const bool stop = (forced || fixed) ? last : (r < d.iter_tol || last);
-    if (stop) break;
+    if (!have_out) break;
+    if (!by_count || i == itmax - 1) {
+      F.stop_test(by_count, i == itmax - 1);                            // Section 2.3
+      if (F.sh.stop) break;
+    }
     F.cols(F.Sb, 1, F.Sb, 1, OP_K2);                                    // P9 (Eq. 12)
     if (!F.sync(8)) { res.status = ST_BARRIER; return res; }
     {
-      EpiUpdate<T> e; e.P = F.ptrs(); e.P.hd = hdw; e.A = (T)A;
-      F.rows<1, 1>(F.rb1, F.Sb, F.Sa, e, 0, 5);                         // P10
+      EpiUpdate<T> e; e.P = F.ptrs(); e.P.hd = hdw; e.A = F.At();
+      F.rows<1, 1>(F.Sb, F.Sa, e, 0, 5);                                // P10
     }
     if (!F.sync(10)) { res.status = ST_BARRIER; return res; }
-    F.shifts(F.rb1, N, hed, nout, A, C);                                // Eq. 10, Eq. 11
   }
   res.iters = i + 1;
-  res.r = r;
-  res.status = (!have_out || fixed || r < d.iter_tol) ? ST_OK : ST_NOCONV;
-  // warm start for the next call: h_dot stored, A still to subtract on free space.  A call that
-  // failed with a residual above 1e3 tol (or not finite) diverged: the next call starts cold.
-  const bool diverged = res.status == ST_NOCONV && !(r < 1e3 * d.iter_tol);
-  F.sh.warm_valid = diverged ? 0 : 1;
-  F.sh.A_prev = A;
-  F.sh.attempt_first = 0;
+  if (threadIdx.x == 0) {
+    const double r = F.sh.r;
+    F.sh.ok = !have_out || d.iter_tol <= 0.0 || r < d.iter_tol;
+    // warm start for the next call: h_dot stored, A still to subtract on free space.  A call that
+    // failed with a residual above 1e3 tol (or not finite) diverged: the next call starts cold.
+    F.sh.warm_valid = !F.sh.ok && !(r < 1e3 * d.iter_tol) ? 0 : 1;
+    F.sh.A_prev = F.sh.A;
+    F.sh.attempt_first = 0;
+  }
 
   // finalize
   {
-    EpiFinal<T> e; e.P = F.ptrs(); e.kout = kout; e.is_max = true;
-    e.err = want_err; e.h = h_err; e.rtol = d.rtol; e.atol = d.atol;
-    e.k1 = e_k1; e.k2 = e_k2; e.k3 = e_k3; e.y = e_y; e.ynew = e_ynew;
-    F.rows<0, 0>(F.rb1, nullptr, nullptr, e, 3);
+    auto fill = [&](auto& e) {
+      e.P = F.ptrs(); e.kout = kout; e.is_max = true;
+      e.h = h_err; e.rtol = d.rtol; e.atol = d.atol;
+      e.k1 = e_k1; e.k2 = e_k2; e.k3 = e_k3; e.y = e_y; e.ynew = e_ynew;
+    };
+    if (want_err) { EpiFinal<T, true> e; fill(e); F.rows<0, 0>(nullptr, nullptr, e, 3); }
+    else { EpiFinal<T, false> e; fill(e); F.rows<0, 0>(nullptr, nullptr, e, 3); }
   }
   if (!F.sync(11)) { res.status = ST_BARRIER; return res; }
-  const double q = F.total(3, F.rb1, true);
-  if (want_err) res.err = q;
-  else res.nonfinite = q > 0.0;
+  res.status = F.sh.ok ? ST_OK : ST_NOCONV;
+  res.r = F.sh.r;
+  const double q = F.total(3, true);
+  if (want_err) res.err = isinf(q) ? 1e300 : q;
+  else res.nonfinite = __double_as_longlong(q) > 0;
   return res;
 }
 
@@ -757,7 +1055,6 @@ struct FilmRhs {
   // the integrator accepted a step: the last call's h_dot (written to hd_sel) becomes the
   // committed initial approximation, and later calls write the other buffer
   __device__ void on_attempt() {
-    __syncthreads();
     if (threadIdx.x == 0) F.sh.attempt_first = 1;
     __syncthreads();
   }
@@ -774,10 +1071,20 @@ struct FilmRhs {
 // ------------------------------------------------------------------------------------------
 // the persistent kernel
 // ------------------------------------------------------------------------------------------
+// The twiddle tables into shared memory, behind the exchange buffer (a grid barrier's acquire empties
+// L1, so tables in global memory would come from L2 again in every phase).
+template <typename T>
+__device__ __forceinline__ void film_tables(const Desc& d) {
+  uint4* const to = (uint4*)mf_dsmem + film_slots(d);
+  const uint4* const x = (const uint4*)d.tw_x;
+  const uint4* const y = (const uint4*)d.tw_y;
+  const int nx = core_table_len(d.lgx, d.ex), ny = film_one_table(d) ? 0 : core_table_len(d.lgy, d.ey);
+  for (int k = threadIdx.x; k < nx; k += NT) to[k] = x[k];
+  for (int k = threadIdx.x; k < ny; k += NT) to[nx + k] = y[k];
+}
 // The body of a launch for one film, run by CTAs vb = 0 .. vn - 1 of that film.
 template <typename T>
 __device__ __forceinline__ void film_main(const Desc& d, const KernelArgs& a, int vb, unsigned vn) {
-  C2<T>* sm = dsm<T>();
   __shared__ Shared sh;
   // one copy of the pass object per CTA, in shared memory: its members are read as broadcasts
   // instead of per-thread local-memory copies
@@ -793,7 +1100,8 @@ __device__ __forceinline__ void film_main(const Desc& d, const KernelArgs& a, in
     sh.attempt_first = 0;
     sh.q11 = st->q11;
   }
-  if (threadIdx.x == 0) new (objraw) Film<T>(d, sm, sh, vb, vn);
+  if (threadIdx.x == 0) new (objraw) Film<T>(d, mf_dsmem, sh, vb, vn);
+  film_tables<T>(d);
   __syncthreads();
   Film<T>& F = *reinterpret_cast<Film<T>*>(objraw);
   const bool leader = vb == 0 && threadIdx.x == 0;
@@ -803,45 +1111,46 @@ __device__ __forceinline__ void film_main(const Desc& d, const KernelArgs& a, in
     // q1 = F^-1[K1 F(out)], q2 = F^-1[K2 F(out)]
     for (int pass = 0; pass < 2; ++pass) {
       EpiOut<T> eo; eo.P = F.ptrs();
-      F.rows<0, 1>(F.rb1, nullptr, F.Sa, eo, -1);
+      F.rows<0, 1>(nullptr, F.Sa, eo, -1);
       if (!F.sync(20)) { status = ST_BARRIER; break; }
       F.cols(F.Sa, 1, F.Sa, 1, pass == 0 ? OP_K1 : OP_K2);
       if (!F.sync(21)) { status = ST_BARRIER; break; }
       EpiStoreT<T> es; es.P = F.ptrs(); es.dst = (T*)(pass == 0 ? d.q1 : d.q2);
-      F.rows<1, 0>(F.rb1, F.Sa, nullptr, es, 4);
+      F.rows<1, 0>(F.Sa, nullptr, es, 4);
       if (!F.sync(22)) { status = ST_BARRIER; break; }
       if (pass == 0) {
-        const double q11 = F.total(4, F.rb1);          // sum over free space of q1
+        const double q11 = F.total(4);          // sum over free space of q1
         if (leader) st->q11 = q11;
       }
     }
   } else if (a.mode == MODE_HZ) {
     EpiStage<T> e; e.P = F.ptrs(); e.in = StageIn{a.y_in, 0, {0, 0, 0}, {nullptr, nullptr, nullptr}, nullptr};
-    F.rows<0, 1>(F.rb1, nullptr, F.Sa, e, -1);
+    if (threadIdx.x == 0) sh.hed = he_value(d, a.t);
+    F.rows<0, 1>(nullptr, F.Sa, e, -1);
     if (F.sync(30)) {
       F.cols(F.Sa, 1, F.Sa, 1, OP_KH);
       if (F.sync(31)) {
-        EpiStoreHz<T> es; es.P = F.ptrs(); es.dst = a.out; es.he = he_value(d, a.t);
-        F.rows<1, 0>(F.rb1, F.Sa, nullptr, es, -1);
+        EpiStoreHz<T> es; es.P = F.ptrs(); es.dst = a.out; es.he = sh.hed;
+        F.rows<1, 0>(F.Sa, nullptr, es, -1);
       } else status = ST_BARRIER;
     } else status = ST_BARRIER;
   } else if (a.mode == MODE_E) {
     EpiStage<T> e; e.P = F.ptrs(); e.in = StageIn{a.y_in, 0, {0, 0, 0}, {nullptr, nullptr, nullptr}, nullptr};
-    F.rows<0, 1>(F.rb1, nullptr, F.Sa, e, -1);
+    F.rows<0, 1>(nullptr, F.Sa, e, -1);
     if (F.sync(50)) {
       F.cols(F.Sa, 1, F.Sa, 2, OP_GRAD);
       if (F.sync(51)) {
         EpiStoreE<T> es; es.P = F.ptrs(); es.dst = a.out; es.ncell = F.ncell;
         es.n = (T)d.n; es.e0 = (T)d.e0; es.jc = (T)d.jc; es.rho_out = (T)d.rho_out;
-        es.ig2 = (T)(1.0 / (d.gamma * d.gamma));
-        F.rows<2, 0>(F.rb2, F.Sa, nullptr, es, -1);
+        es.ig2 = F.ig2;
+        F.rows<2, 0>(F.Sa, nullptr, es, -1, -1, F.u);
       } else status = ST_BARRIER;
     } else status = ST_BARRIER;
   } else if (a.mode == MODE_MOMENT) {
     EpiMoment<T> e; e.P = F.ptrs(); e.g = a.y_in;
-    F.rows<0, 0>(F.rb1, nullptr, nullptr, e, 4);
+    F.rows<0, 0>(nullptr, nullptr, e, 4);
     if (F.sync(40)) {
-      const double s = F.total(4, F.rb1);
+      const double s = F.total(4);
       if (leader) a.out[0] = s * d.dx * d.dy;
     } else status = ST_BARRIER;
   } else if (a.mode == MODE_RHS) {
@@ -852,7 +1161,7 @@ __device__ __forceinline__ void film_main(const Desc& d, const KernelArgs& a, in
     if (leader) { st->last_iters = r.iters; st->last_r = r.r; st->n_rhs += 1; st->n_iters += r.iters; }
   } else if (a.mode == MODE_ADVANCE) {
     FilmRhs<T> R{F};
-    status = bs23_advance(R, d, st, a, leader);
+    status = bs23_advance(R, d, st, a, leader, sh.ctl);
   }
   if (leader) {
     st->warm_valid = sh.warm_valid;
@@ -864,9 +1173,9 @@ __device__ __forceinline__ void film_main(const Desc& d, const KernelArgs& a, in
   }
 }
 
-// the two FFT buffers (twiddles stay in global memory, read through L1)
-inline size_t film_smem_bytes(int precision) {
-  return 2 * (size_t)BATCH_PAD * (precision ? sizeof(C2<float>) : sizeof(C2<double>));
-}
+// CTAs per SM of the film kernels: 2 leave 128 registers per thread.  4 (64 registers) spill in every
+// pass (2048^2 FP32, 5 iterations: 922 us against 852 us on otherwise the same source); 3 leave the 513
+// line pairs of a 2048^2 pass 456 places (1193 us).
+constexpr int FILM_CTAS = 2;
 
 }  // namespace mf

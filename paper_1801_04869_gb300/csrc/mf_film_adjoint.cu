@@ -48,22 +48,35 @@ struct AdjArgs {
   double* wbar_in;      // cotangent of the warm start (FP64, ncell, 0 on the conductor) or null
 };
 
+// FP64 cotangent fields are row-major (the caller's layout): the RU rows of one element
+template <typename T>
+__device__ __forceinline__ void ld_rows(double (&v)[Lane<T>::RU], const double* p, int nx) {
+#pragma unroll
+  for (int q = 0; q < Lane<T>::RU; ++q) v[q] = ld_s(p + (long long)q * nx);
+}
+
 // full product, V1: gbar_{I-1} = conductor * v (with its sum) and g, forward of both
 template <typename T>
 struct EpiPT0g : EpiBase<T, T> {
   FilmPtrs<T> P;
   const double* v;
   const double* g;
-  __device__ void operator()(long long i, const V4<T>*, V4<T>* out) {
-    const uchar4 m = ldmask4(P.mask + i);
-    const V4<double> x = ld4(v + i);
-    const V4<double> y = ld4(g + i);
+  static constexpr int kBatch = 2;
+  struct Ld { int m; double x[Lane<T>::RU], y[Lane<T>::RU]; };
+  __device__ __forceinline__ Ld load(long long i, long long r) const {
+    Ld l;
+    l.m = ld_mask(P.mask + i);
+    ld_rows<T>(l.x, v + r, P.nx);
+    ld_rows<T>(l.y, g + r, P.nx);
+    return l;
+  }
+  __device__ __forceinline__ void apply(const Ld& l, long long, long long, const Q<T>*, Q<T>* out) {
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const T gb = mask_at(m, q) != 0 ? (T)x.v[q] : (T)0;
+    for (int q = 0; q < Lane<T>::RU; ++q) {
+      const T gb = cls(l.m, q) != 0 ? (T)l.x[q] : (T)0;
       this->acc += gb;
       out[0].v[q] = gb;
-      out[1].v[q] = (T)y.v[q];
+      out[1].v[q] = (T)l.y[q];
     }
   }
 };
@@ -74,12 +87,15 @@ struct EpiStoreJ : EpiBase<T, T> {
   FilmPtrs<T> P;
   T* jx;
   T* jy;
-  __device__ void operator()(long long i, const V4<T>* in, V4<T>*) {
-    V4<T> a, b;
+  static constexpr int kBatch = 4;
+  using Ld = NoLd;
+  __device__ __forceinline__ Ld load(long long, long long) const { return Ld{}; }
+  __device__ __forceinline__ void apply(const Ld&, long long i, long long, const Q<T>* in, Q<T>*) {
+    Q<T> b;
 #pragma unroll
-    for (int q = 0; q < 4; ++q) { a.v[q] = in[1].v[q]; b.v[q] = -in[0].v[q]; }
-    st4(jx + i, a);
-    st4(jy + i, b);
+    for (int q = 0; q < Lane<T>::RU; ++q) b.v[q] = -in[0].v[q];
+    st_q(jx + i * Lane<T>::RU, in[1]);
+    st_q(jy + i * Lane<T>::RU, b);
   }
 };
 
@@ -89,16 +105,17 @@ struct EpiRbar : EpiBase<T, T> {
   FilmPtrs<T> P;
   T t_q;
   double* wdst;         // cotangent of the warm start (free space) or null
-  __device__ void operator()(long long i, const V4<T>*, V4<T>* out) {
-    const uchar4 m = ldmask4(P.mask + i);
-    const V4<T> h = ld4(P.hd + i);
-    V4<double> w;
+  static constexpr int kBatch = 4;
+  struct Ld { int m; Q<T> h; };
+  __device__ __forceinline__ Ld load(long long i, long long) const {
+    return Ld{ld_mask(P.mask + i), ld_q(P.hd + i * Lane<T>::RU)};
+  }
+  __device__ __forceinline__ void apply(const Ld& l, long long, long long r, const Q<T>*, Q<T>* out) {
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      out[0].v[q] = mask_at(m, q) != 0 ? -(h.v[q] - t_q) : (T)0;
-      w.v[q] = mask_at(m, q) == 0 ? (double)(h.v[q] - t_q) : 0.0;
+    for (int q = 0; q < Lane<T>::RU; ++q) {
+      out[0].v[q] = cls(l.m, q) != 0 ? -(l.h.v[q] - t_q) : (T)0;
+      if (wdst) wdst[r + (long long)q * P.nx] = cls(l.m, q) == 0 ? (double)(l.h.v[q] - t_q) : 0.0;
     }
-    if (wdst) st4(wdst + i, w);
   }
 };
 
@@ -113,22 +130,31 @@ struct EpiPowVJP : EpiBase<T, T> {
   const T* jy;
   double* jcbar;
   T n, e0, jc, rho_out, ig2;
-  __device__ void operator()(long long i, const V4<T>* in, V4<T>* out) {
-    const uchar4 m = ldmask4(P.mask + i);
-    V4<T> jcl;
-    if (P.jcmap) jcl = ldg4(P.jcmap + i);
-    else jcl = V4<T>{{jc, jc, jc, jc}};
-    const V4<T> ax = ld4(jx + i), ay = ld4(jy + i);
-    V4<double> cb;
+  static constexpr int kBatch = 2;
+  struct Ld { int m; Q<T> ax, ay, jc; };
+  __device__ __forceinline__ Ld load(long long i, long long) const {
+    Ld l;
+    l.m = ld_mask(P.mask + i);
+    l.ax = ld_q(jx + i * Lane<T>::RU);
+    l.ay = ld_q(jy + i * Lane<T>::RU);
+    if (P.jcmap) {
+      l.jc = ldg_q(P.jcmap + i * Lane<T>::RU);
+    } else {
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
+      for (int q = 0; q < Lane<T>::RU; ++q) l.jc.v[q] = jc;
+    }
+    return l;
+  }
+  __device__ __forceinline__ void apply(const Ld& l, long long, long long r, const Q<T>* in, Q<T>* out) {
+#pragma unroll
+    for (int q = 0; q < Lane<T>::RU; ++q) {
       const T ex = in[1].v[q], ey = -in[0].v[q];                 // transposed -curl
-      const T x = ax.v[q], y = ay.v[q];
-      const int mq = mask_at(m, q);
+      const T x = l.ax.v[q], y = l.ay.v[q];
+      const int mq = cls(l.m, q);
       const T a = mq == 1 ? ig2 : (T)1;
       const T Ay = y * a;                                          // (A j)_y
       const T j2 = x * x + y * Ay;
-      const T rho = resistivity<T>(j2, jcl.v[q], mq, n, e0, rho_out);
+      const T rho = resistivity<T>(j2, l.jc.v[q], mq, n, e0, rho_out);
       T bx = rho * ex, by = rho * ey * a;
       double c = 0.0;
       if (mq == 1) {
@@ -139,13 +165,12 @@ struct EpiPowVJP : EpiBase<T, T> {
           bx += pr * ux;
           by += pr * uy;
         }
-        c = -(double)(n / jcl.v[q]) * (double)(rho * (ex * x + ey * Ay));
+        c = -(double)(n / l.jc.v[q]) * (double)(rho * (ex * x + ey * Ay));
       }
       out[0].v[q] = bx;
       out[1].v[q] = by;
-      cb.v[q] = c;
+      jcbar[r + (long long)q * P.nx] = c;
     }
-    st4(jcbar + i, cb);
   }
 };
 
@@ -154,11 +179,12 @@ template <typename T>
 struct EpiGbar : EpiBase<T, T> {
   FilmPtrs<T> P;
   double* dst;
-  __device__ void operator()(long long i, const V4<T>* in, V4<T>*) {
-    V4<double> r;
+  static constexpr int kBatch = 4;
+  using Ld = NoLd;
+  __device__ __forceinline__ Ld load(long long, long long) const { return Ld{}; }
+  __device__ __forceinline__ void apply(const Ld&, long long, long long r, const Q<T>* in, Q<T>*) {
 #pragma unroll
-    for (int q = 0; q < 4; ++q) r.v[q] = -(double)in[0].v[q];
-    st4(dst + i, r);
+    for (int q = 0; q < Lane<T>::RU; ++q) dst[r + (long long)q * P.nx] = -(double)in[0].v[q];
   }
 };
 
@@ -167,12 +193,18 @@ template <typename T>
 struct EpiPT0 : EpiBase<T, T> {
   FilmPtrs<T> P;
   const double* v;
-  __device__ void operator()(long long i, const V4<T>*, V4<T>* out) {
-    const uchar4 m = ldmask4(P.mask + i);
-    const V4<double> x = ld4(v + i);
+  static constexpr int kBatch = 4;
+  struct Ld { int m; double x[Lane<T>::RU]; };
+  __device__ __forceinline__ Ld load(long long i, long long r) const {
+    Ld l;
+    l.m = ld_mask(P.mask + i);
+    ld_rows<T>(l.x, v + r, P.nx);
+    return l;
+  }
+  __device__ __forceinline__ void apply(const Ld& l, long long, long long, const Q<T>*, Q<T>* out) {
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const T g = mask_at(m, q) != 0 ? (T)x.v[q] : (T)0;
+    for (int q = 0; q < Lane<T>::RU; ++q) {
+      const T g = cls(l.m, q) != 0 ? (T)l.x[q] : (T)0;
       this->acc += g;
       out[0].v[q] = g;
     }
@@ -186,25 +218,34 @@ struct EpiPTh : EpiBase<T, T> {
   const T* zbar;        // null on the first backward iteration
   const double* om;     // first backward iteration: cotangent of the last iterate, or null
   T s_q1;               // S / n_out
-  __device__ void operator()(long long i, const V4<T>* in, V4<T>* out) {
-    const uchar4 m = ldmask4(P.mask + i);
-    const V4<T> q1 = ldg4(P.q1 + i);
-    V4<T> z;
-    if (zbar) z = ld4(zbar + i);
-    else if (om) {
-      const V4<double> w = ld4(om + i);
+  static constexpr int kBatch = 4;
+  struct Ld { int m; Q<T> q1, z; };
+  __device__ __forceinline__ Ld load(long long i, long long r) const {
+    Ld l;
+    l.m = ld_mask(P.mask + i);
+    l.q1 = ldg_q(P.q1 + i * Lane<T>::RU);
 #pragma unroll
-      for (int q = 0; q < 4; ++q) z.v[q] = mask_at(m, q) == 0 ? (T)w.v[q] : (T)0;
+    for (int q = 0; q < Lane<T>::RU; ++q) l.z.v[q] = (T)0;
+    if (zbar) {
+      l.z = ld_q(zbar + i * Lane<T>::RU);
+    } else if (om) {
+      double w[Lane<T>::RU];
+      ld_rows<T>(w, om + r, P.nx);
+#pragma unroll
+      for (int q = 0; q < Lane<T>::RU; ++q) l.z.v[q] = cls(l.m, q) == 0 ? (T)w[q] : (T)0;
     }
-    V4<T> h;
+    return l;
+  }
+  __device__ __forceinline__ void apply(const Ld& l, long long i, long long, const Q<T>* in, Q<T>* out) {
+    Q<T> h;
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      h.v[q] = ((zbar || om) ? z.v[q] : (T)0) + in[0].v[q] - s_q1 * q1.v[q];
-      const bool o = mask_at(m, q) == 0;
+    for (int q = 0; q < Lane<T>::RU; ++q) {
+      h.v[q] = l.z.v[q] + in[0].v[q] - s_q1 * l.q1.v[q];
+      const bool o = cls(l.m, q) == 0;
       if (o) this->acc += h.v[q];
       out[0].v[q] = o ? -h.v[q] : (T)0;
     }
-    st4(P.hd + i, h);
+    st_q(P.hd + i * Lane<T>::RU, h);
   }
 };
 
@@ -214,19 +255,21 @@ struct EpiPTg : EpiBase<T, T> {
   FilmPtrs<T> P;
   T* zbuf;
   T t_q;                // tot / n_out
-  __device__ void operator()(long long i, const V4<T>* in, V4<T>* out) {
-    const uchar4 m = ldmask4(P.mask + i);
-    const V4<T> q2 = ldg4(P.q2 + i);
-    const V4<T> h = ld4(P.hd + i);
-    V4<T> z;
+  static constexpr int kBatch = 4;
+  struct Ld { int m; Q<T> q2, h; };
+  __device__ __forceinline__ Ld load(long long i, long long) const {
+    return Ld{ld_mask(P.mask + i), ldg_q(P.q2 + i * Lane<T>::RU), ld_q(P.hd + i * Lane<T>::RU)};
+  }
+  __device__ __forceinline__ void apply(const Ld& l, long long i, long long, const Q<T>* in, Q<T>* out) {
+    Q<T> h = l.h;
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const T g = mask_at(m, q) == 0 ? in[0].v[q] + t_q * q2.v[q] : (T)0;
+    for (int q = 0; q < Lane<T>::RU; ++q) {
+      const T g = cls(l.m, q) == 0 ? in[0].v[q] + t_q * l.q2.v[q] : (T)0;
       this->acc += g;
       out[0].v[q] = g;
-      z.v[q] = h.v[q] - t_q;
+      h.v[q] -= t_q;
     }
-    st4(zbuf + i, z);
+    st_q(zbuf + i * Lane<T>::RU, h);
   }
 };
 
@@ -237,82 +280,82 @@ struct EpiPTout : EpiBase<T, T> {
   double* dst;
   double* wdst;         // cotangent of the warm start (free space) or null
   T t_q;
-  __device__ void operator()(long long i, const V4<T>*, V4<T>*) {
-    const uchar4 m = ldmask4(P.mask + i);
-    const V4<T> h = ld4(P.hd + i);
-    V4<double> r, w;
+  static constexpr int kBatch = 4;
+  struct Ld { int m; Q<T> h; };
+  __device__ __forceinline__ Ld load(long long i, long long) const {
+    return Ld{ld_mask(P.mask + i), ld_q(P.hd + i * Lane<T>::RU)};
+  }
+  __device__ __forceinline__ void apply(const Ld& l, long long, long long r, const Q<T>*, Q<T>*) {
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      r.v[q] = mask_at(m, q) != 0 ? (double)(h.v[q] - t_q) : 0.0;
-      w.v[q] = mask_at(m, q) == 0 ? (double)(h.v[q] - t_q) : 0.0;
+    for (int q = 0; q < Lane<T>::RU; ++q) {
+      const double x = (double)(l.h.v[q] - t_q);
+      dst[r + (long long)q * P.nx] = cls(l.m, q) != 0 ? x : 0.0;
+      if (wdst) wdst[r + (long long)q * P.nx] = cls(l.m, q) == 0 ? x : 0.0;
     }
-    st4(dst + i, r);
-    if (wdst) st4(wdst + i, w);
   }
 };
 
 template <typename T>
-__global__ void __launch_bounds__(NT, 2) film_adjoint_kernel(const Desc* __restrict__ dg, AdjArgs a) {
-  C2<T>* sm = dsm<T>();
+__global__ void __launch_bounds__(NT, FILM_CTAS) film_adjoint_kernel(const Desc* __restrict__ dg, AdjArgs a) {
   __shared__ Shared sh;
   __shared__ __align__(16) unsigned char objraw[sizeof(Film<T>)];
   const Desc& d = *dg;
   SolverState* st = d.st;
   if (threadIdx.x == 0) {
     sh.bar_passed = 0;
-    new (objraw) Film<T>(d, sm, sh, (int)blockIdx.x, gridDim.x);
+    new (objraw) Film<T>(d, mf_dsmem, sh, (int)blockIdx.x, gridDim.x);
   }
+  film_tables<T>(d);
   __syncthreads();
   Film<T>& F = *reinterpret_cast<Film<T>*>(objraw);
   const bool leader = blockIdx.x == 0 && threadIdx.x == 0;
-  const double nout = (double)d.nout, N = (double)F.ncell;
   T* const zbuf = (T*)d.hd2;
   int status = ST_OK;
-  double sbar = 0.0;
+  double sbar = 0.0;                             // thread 0
   const bool full = a.g != nullptr;
   T* const jx = (T*)d.u;                         // j for the full product: the raw g_dot buffer
   T* const jy = (T*)(F.Sb + 2 * F.nspec);        // and the third field of Sb, as real storage
   do {
-    double S;
+    T S, tot;                                    // the sums over free space, / n_out
     if (full) {
       EpiPT0g<T> e; e.P = F.ptrs(); e.v = a.v; e.g = a.g;
-      F.rows<0, 2>(F.rb2, nullptr, F.Sa, e, 0);                         // V1 (+ g)
+      F.rows<0, 2>(nullptr, F.Sa, e, 0, -1, F.hd);                         // V1 (+ g)
       if (!F.sync(60)) { status = ST_BARRIER; break; }
-      S = F.total(0, F.rb2);
+      S = F.mean_of(0);
     } else {
       EpiPT0<T> e; e.P = F.ptrs(); e.v = a.v;
-      F.rows<0, 1>(F.rb1, nullptr, F.Sa, e, 0);                         // V1
+      F.rows<0, 1>(nullptr, F.Sa, e, 0);                         // V1
       if (!F.sync(50)) { status = ST_BARRIER; break; }
-      S = F.total(0, F.rb1);
+      S = F.mean_of(0);
     }
     F.cols(F.Sa, 1, F.Sa, 1, OP_K1);                                    // V2
     if (full) F.cols(F.Sa + F.nspec, 1, F.Sa + F.nspec, 2, OP_GRAD);    // grad g -> Sa 1, 2
     if (!F.sync(51)) { status = ST_BARRIER; break; }
     if (full) {
       EpiStoreJ<T> e; e.P = F.ptrs(); e.jx = jx; e.jy = jy;
-      F.rows<2, 0>(F.rb2, F.Sa + F.nspec, nullptr, e, -1);              // j (Eq. 2)
+      F.rows<2, 0>(F.Sa + F.nspec, nullptr, e, -1, -1, F.hd);              // j (Eq. 2)
       if (!F.sync(61)) { status = ST_BARRIER; break; }
     }
     for (int i = a.iters - 1; i >= 0; --i) {
       const bool first = i == a.iters - 1;
       {
-        EpiPTh<T> e; e.P = F.ptrs(); e.zbar = first ? nullptr : zbuf; e.s_q1 = (T)(S / nout);
+        EpiPTh<T> e; e.P = F.ptrs(); e.zbar = first ? nullptr : zbuf; e.s_q1 = S;
         e.om = first ? a.wbar_out : nullptr;
-        if (i > 0) F.rows<1, 1>(F.rb1, F.Sa, F.Sb, e, 1);               // V3
-        else F.rows<1, 0>(F.rb1, F.Sa, nullptr, e, 1);
+        if (i > 0) F.rows<1, 1>(F.Sa, F.Sb, e, 1);               // V3
+        else F.rows<1, 0>(F.Sa, nullptr, e, 1);
       }
       if (!F.sync(52)) { status = ST_BARRIER; break; }
-      const double tot = F.total(1, F.rb1);
-      sbar += N / nout * tot;
+      tot = F.mean_of(1);
+      if (threadIdx.x == 0) sbar += sh.N * sh.A;     // sh.A: the mean, tot / n_out
       if (i == 0) {
         if (!full) {
-          EpiPTout<T> e; e.P = F.ptrs(); e.dst = a.hin_bar; e.wdst = a.wbar_in; e.t_q = (T)(tot / nout);
-          F.rows<0, 0>(F.rb1, nullptr, nullptr, e, -1);
+          EpiPTout<T> e; e.P = F.ptrs(); e.dst = a.hin_bar; e.wdst = a.wbar_in; e.t_q = tot;
+          F.rows<0, 0>(nullptr, nullptr, e, -1);
           break;
         }
         {
-          EpiRbar<T> e; e.P = F.ptrs(); e.t_q = (T)(tot / nout); e.wdst = a.wbar_in;
-          F.rows<0, 1>(F.rb1, nullptr, F.Sb, e, -1);                    // r
+          EpiRbar<T> e; e.P = F.ptrs(); e.t_q = tot; e.wdst = a.wbar_in;
+          F.rows<0, 1>(nullptr, F.Sb, e, -1);                    // r
         }
         if (!F.sync(62)) { status = ST_BARRIER; break; }
         F.cols(F.Sb, 1, F.Sb, 2, OP_GRAD);                              // grad r -> Sb 0, 1
@@ -320,26 +363,26 @@ __global__ void __launch_bounds__(NT, 2) film_adjoint_kernel(const Desc* __restr
         {
           EpiPowVJP<T> e; e.P = F.ptrs(); e.jx = jx; e.jy = jy; e.jcbar = a.jcbar;
           e.n = (T)d.n; e.e0 = (T)d.e0; e.jc = (T)d.jc; e.rho_out = (T)d.rho_out;
-          e.ig2 = (T)(1.0 / (d.gamma * d.gamma));
-          F.rows<2, 2>(F.rb2, F.Sb, F.Sa, e, -1);                       // jbar, jcbar (Eq. 3)
+          e.ig2 = F.ig2;
+          F.rows<2, 2>(F.Sb, F.Sa, e, -1, -1, F.hd);                       // jbar, jcbar (Eq. 3)
         }
         if (!F.sync(64)) { status = ST_BARRIER; break; }
         F.cols(F.Sa, 2, F.Sa, 1, OP_CURLNEG);                           // -curl jbar
         if (!F.sync(65)) { status = ST_BARRIER; break; }
         {
           EpiGbar<T> e; e.P = F.ptrs(); e.dst = a.gbar;
-          F.rows<1, 0>(F.rb1, F.Sa, nullptr, e, -1);                    // gbar
+          F.rows<1, 0>(F.Sa, nullptr, e, -1);                    // gbar
         }
         break;
       }
       F.cols(F.Sb, 1, F.Sb, 1, OP_K2);                                  // V4
       if (!F.sync(53)) { status = ST_BARRIER; break; }
       {
-        EpiPTg<T> e; e.P = F.ptrs(); e.zbuf = zbuf; e.t_q = (T)(tot / nout);
-        F.rows<1, 1>(F.rb1, F.Sb, F.Sa, e, 0);                          // V5
+        EpiPTg<T> e; e.P = F.ptrs(); e.zbuf = zbuf; e.t_q = tot;
+        F.rows<1, 1>(F.Sb, F.Sa, e, 0);                          // V5
       }
       if (!F.sync(54)) { status = ST_BARRIER; break; }
-      S = F.total(0, F.rb1);
+      S = F.mean_of(0);
       F.cols(F.Sa, 1, F.Sa, 1, OP_K1);                                  // V6
       if (!F.sync(55)) { status = ST_BARRIER; break; }
     }
@@ -416,23 +459,71 @@ cudaError_t adj_sums(long long n, const double* x, double* out, cudaStream_t s) 
   return cudaGetLastError();
 }
 
+// Fields by row units (mf_film.cuh): element of (unit, x, row) for the row-major cell (y, x)
+__device__ __forceinline__ long long unit_index(long long cell, int nx, int ru) {
+  const long long y = cell / nx, x = cell - y * nx, u = y / ru;
+  return (u * nx + x) * ru + (y - u * ru);
+}
 // the warm start of a film right-hand side: dst = h_dot - A on free space, 0 elsewhere (FP64) for
 // save; h_dot = src on free space for load (the caller sets A = 0)
 template <typename T>
-__global__ void warm_io_kernel(long long n, int load, const uint8_t* mask, T* hd, double A,
+__global__ void warm_io_kernel(int nx, long long n, int load, const uint8_t* mask, T* hd, double A,
                                double* dst, const double* src) {
+  constexpr int ru = Lane<T>::RU;
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
        i += (long long)gridDim.x * blockDim.x) {
-    const bool o = mask[i] == 0;
-    if (load) hd[i] = o ? (T)src[i] : (T)0;
-    else dst[i] = o ? (double)hd[i] - A : 0.0;
+    const long long o = unit_index(i, nx, ru);
+    const bool out = cls(mask[o / ru], (int)(o % ru)) == 0;
+    if (load) hd[o] = out ? (T)src[i] : (T)0;
+    else dst[i] = out ? (double)hd[o] - A : 0.0;
   }
 }
 
-cudaError_t adj_warm_io(int precision, long long n, int load, const uint8_t* mask, void* hd,
+cudaError_t adj_warm_io(int precision, int nx, int ny, int load, const uint8_t* mask, void* hd,
                         double A, double* dst, const double* src, cudaStream_t s) {
-  if (precision) warm_io_kernel<float><<<304, 256, 0, s>>>(n, load, mask, (float*)hd, A, dst, src);
-  else warm_io_kernel<double><<<304, 256, 0, s>>>(n, load, mask, (double*)hd, A, dst, src);
+  const long long n = (long long)nx * ny;
+  if (precision) warm_io_kernel<float><<<608, 256, 0, s>>>(nx, n, load, mask, (float*)hd, A, dst, src);
+  else warm_io_kernel<double><<<608, 256, 0, s>>>(nx, n, load, mask, (double*)hd, A, dst, src);
+  return cudaGetLastError();
+}
+
+// row-major FP64 field -> transform precision by row units (a jc map set after creation)
+template <typename T>
+__global__ void to_units_kernel(int nx, long long n, const double* x, T* y) {
+  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
+       i += (long long)gridDim.x * blockDim.x)
+    y[unit_index(i, nx, Lane<T>::RU)] = (T)x[i];
+}
+cudaError_t film_to_units(int precision, int nx, int ny, const double* x, void* y, cudaStream_t s) {
+  const long long n = (long long)nx * ny;
+  if (precision) to_units_kernel<float><<<608, 256, 0, s>>>(nx, n, x, (float*)y);
+  else to_units_kernel<double><<<608, 256, 0, s>>>(nx, n, x, (double*)y);
+  return cudaGetLastError();
+}
+
+// a field by row units <-> row-major (checkpoints): one thread per 16-byte vector
+template <typename T>
+__global__ void relayout_kernel(int nx, long long nvec, bool to_rows, const T* src, T* dst) {
+  constexpr int ru = Lane<T>::RU;
+  for (long long v = (long long)blockIdx.x * blockDim.x + threadIdx.x; v < nvec;
+       v += (long long)gridDim.x * blockDim.x) {
+    const long long u = v / nx, x = v - u * nx, r0 = u * ru * nx + x;
+    Q<T> q;
+    if (to_rows) {
+      q = ldg_q(src + v * ru);
+#pragma unroll
+      for (int r = 0; r < ru; ++r) dst[r0 + (long long)r * nx] = q.v[r];
+    } else {
+#pragma unroll
+      for (int r = 0; r < ru; ++r) q.v[r] = src[r0 + (long long)r * nx];
+      st_q(dst + v * ru, q);
+    }
+  }
+}
+cudaError_t film_relayout(int precision, int nx, int ny, bool to_rows, const void* src, void* dst, cudaStream_t s) {
+  const long long nvec = (long long)nx * ny / row_unit(precision);
+  if (precision) relayout_kernel<float><<<608, 256, 0, s>>>(nx, nvec, to_rows, (const float*)src, (float*)dst);
+  else relayout_kernel<double><<<608, 256, 0, s>>>(nx, nvec, to_rows, (const double*)src, (double*)dst);
   return cudaGetLastError();
 }
 
@@ -443,11 +534,11 @@ cudaError_t film_adjoint_launch(int precision, const Desc& d, const double* v, d
   const Desc* dg = d.dev;
   AdjArgs a{v, hin_bar, sbar, iters, g, gbar, jcbar, wbar_out, wbar_in};
   void* args[] = {&dg, &a};
-  const size_t smem = film_smem_bytes(precision);
+  const size_t smem = film_smem_bytes(d);
   const void* fn = precision ? (const void*)film_adjoint_kernel<float> : (const void*)film_adjoint_kernel<double>;
   cudaError_t e = precision
-      ? cudaFuncSetAttribute(film_adjoint_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)
-      : cudaFuncSetAttribute(film_adjoint_kernel<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      ? cudaFuncSetAttribute(film_adjoint_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FILM_SMEM_MAX)
+      : cudaFuncSetAttribute(film_adjoint_kernel<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FILM_SMEM_MAX);
   if (e != cudaSuccess) return e;
   return cudaLaunchCooperativeKernel(fn, dim3(d.grid), dim3(NT), args, smem, s);
 }

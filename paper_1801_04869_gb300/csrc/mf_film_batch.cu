@@ -8,7 +8,7 @@ namespace mf {
 
 // several films in one launch, each advanced (MODE_ADVANCE) by its own range of CTAs
 template <typename T>
-__global__ void __launch_bounds__(NT, 2) film_batch_kernel(const __grid_constant__ BatchTable tab) {
+__global__ void __launch_bounds__(NT, FILM_CTAS) film_batch_kernel(const __grid_constant__ BatchTable tab) {
   __shared__ int s_job;
   if (threadIdx.x == 0) {
     // the job whose range [b0, b0 + nb) holds this CTA (ranges ascend and tile the grid)
@@ -33,19 +33,18 @@ __global__ void __launch_bounds__(NT, 2) film_batch_kernel(const __grid_constant
 int film_batch_max_blocks(int precision, size_t smem) {
   int nb = 0;
   if (precision) {
-    cudaFuncSetAttribute(film_batch_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaFuncSetAttribute(film_batch_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FILM_SMEM_MAX);
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, film_batch_kernel<float>, NT, smem);
   } else {
-    cudaFuncSetAttribute(film_batch_kernel<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaFuncSetAttribute(film_batch_kernel<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FILM_SMEM_MAX);
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, film_batch_kernel<double>, NT, smem);
   }
   return nb;
 }
 
-cudaError_t film_batch_launch(int precision, const BatchTable& tab, int grid, cudaStream_t s) {
+cudaError_t film_batch_launch(int precision, const BatchTable& tab, int grid, size_t smem, cudaStream_t s) {
   BatchTable t = tab;
   void* args[] = {&t};
-  const size_t smem = film_smem_bytes(precision);
   const void* fn = precision ? (const void*)film_batch_kernel<float> : (const void*)film_batch_kernel<double>;
   return cudaLaunchCooperativeKernel(fn, dim3(grid), dim3(NT), args, smem, s);
 }

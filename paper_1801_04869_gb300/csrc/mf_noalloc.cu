@@ -96,7 +96,7 @@ extern "C" mf_status mf_film_rhs_noalloc(const mf_params* p, double t, const dou
   const size_t oSa = take(2 * nspec * 2 * ts), oSb = take(2 * nspec * 2 * ts);
   const size_t ohd = take(ncell * ts), ou = take(ncell * ts), oq1 = take(ncell * ts), oq2 = take(ncell * ts);
   const size_t ojc = take(p->jc_map ? ncell * ts : 0), omask = take(ncell);
-  const size_t otwx = take(2 * nx * 2 * ts), otwy = take(2 * ny * 2 * ts), otwz = take(2 * ts);
+  const size_t otwx = take(TWIDDLE_VALUES * nx * ts), otwy = take(TWIDDLE_VALUES * ny * ts), otwz = take(TWIDDLE_VALUES * ts);
   const size_t okt = take(nk * ts), ogt = take(nk * ts);
   const size_t opart = take((size_t)8 * ny * 8), ost = take(sizeof(SolverState)), ogb = take(sizeof(GridBarrier));
   const size_t oknots = take(2 * (size_t)(p->he_knots > 0 ? p->he_knots : 1) * 8);
@@ -140,22 +140,14 @@ extern "C" mf_status mf_film_rhs_noalloc(const mf_params* p, double t, const dou
   d.dev = (const Desc*)(w + odesc);
 
   d.nz = 1;
+  d.ex = elems_per_thread(d, nx);
+  d.ey = elems_per_thread(d, ny);
   const size_t smem = kernel_smem_bytes(d);
   const int per_sm = film_max_blocks(precision, smem);
   int nsm = 0;
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
   if (per_sm < 1 || nsm < 1) { set_err(err, err_len, "kernel does not fit on this device"); return MF_ERR_CUDA; }
-  {
-    const int coresident = per_sm * nsm;
-    int rb1 = std::min(ny, 2 * BATCH / nx), rb2 = std::min(ny, BATCH / nx);
-    const int want = nx / 2 + 1;
-    const int grid = std::min(coresident, want);
-    while (rb1 > 2 && ny / rb1 < grid) rb1 /= 2;
-    while (rb2 > 2 && ny / rb2 < grid) rb2 /= 2;
-    d.rows_per_item = rb1;
-    d.zs_per_item = rb2;
-    d.grid = std::max(1, std::min(coresident, std::max(want, ny / rb1)));
-  }
+  film_shape(d, per_sm * nsm);
 
   // inputs and tables, staged through fixed-size stack buffers (synchronous copies)
   cudaError_t e = cudaSuccess;
@@ -163,23 +155,26 @@ extern "C" mf_status mf_film_rhs_noalloc(const mf_params* p, double t, const dou
     if (e == cudaSuccess && n) e = cudaMemcpyAsync(dst, src, n, cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   };
-  copy_sync(w + omask, p->mask, (size_t)ncell);
+  const int ru = row_unit(precision);
   {
-    double tw[4 * NOALLOC_MAX_N], kt[NOALLOC_MAX_N / 2 + 1 + NOALLOC_MAX_N + 1],
+    unsigned char chunk[NOALLOC_MAX_N];   // mask classes of one row unit
+    for (int u = 0; u < ny / ru && e == cudaSuccess; ++u) {
+      pack_mask(p->mask + (size_t)u * ru * nx, nx, ru, 1, chunk);
+      copy_sync(w + omask + (size_t)u * nx, chunk, (size_t)nx);
+    }
+  }
+  {
+    double tw[TWIDDLE_VALUES * NOALLOC_MAX_N], kt[NOALLOC_MAX_N / 2 + 1 + NOALLOC_MAX_N + 1],
         gt[NOALLOC_MAX_N / 2 + 1 + NOALLOC_MAX_N + 1];
-    float twf[4 * NOALLOC_MAX_N], ktf[NOALLOC_MAX_N / 2 + 1 + NOALLOC_MAX_N + 1],
+    float twf[TWIDDLE_VALUES * NOALLOC_MAX_N], ktf[NOALLOC_MAX_N / 2 + 1 + NOALLOC_MAX_N + 1],
         gtf[NOALLOC_MAX_N / 2 + 1 + NOALLOC_MAX_N + 1];
     const int ns[2] = {nx, ny};
     const size_t to[2] = {otwx, otwy};
     for (int a = 0; a < 2; ++a) {
-      // stage-ordered twiddle tables (A then B), as mf_create writes them
-      if (precision) {
-        const int n = stage_twiddles<float>(ns[a], twf);
-        copy_sync(w + to[a], twf, (size_t)n * 2 * 4);
-      } else {
-        const int n = stage_twiddles<double>(ns[a], tw);
-        copy_sync(w + to[a], tw, (size_t)n * 2 * 8);
-      }
+      // the core's twiddle tables, as mf_create writes them
+      const int E = a == 0 ? d.ex : d.ey;
+      if (precision) copy_sync(w + to[a], twf, core_twiddles<float>(ns[a], E, twf) * 4);
+      else copy_sync(w + to[a], tw, core_twiddles<double>(ns[a], E, tw) * 8);
     }
     int c = 0;
     const double Ls[2] = {p->Lx, p->Ly};
@@ -206,16 +201,14 @@ extern "C" mf_status mf_film_rhs_noalloc(const mf_params* p, double t, const dou
       copy_sync(w + oknots + (size_t)K * 8, p->he_v, (size_t)K * 8);
     }
   }
-  if (p->jc_map) {
-    if (!precision) {
-      copy_sync(w + ojc, p->jc_map, (size_t)ncell * 8);
-    } else {
-      float chunk[1024];
-      for (long long i0 = 0; i0 < ncell && e == cudaSuccess; i0 += 1024) {
-        const long long n = std::min<long long>(1024, ncell - i0);
-        for (long long i = 0; i < n; ++i) chunk[i] = (float)p->jc_map[i0 + i];
-        copy_sync(w + ojc + i0 * 4, chunk, (size_t)n * 4);
-      }
+  if (p->jc_map) {                        // by row units
+    float chunk_f[4 * NOALLOC_MAX_N];
+    double chunk_d[2 * NOALLOC_MAX_N];
+    for (int u = 0; u < ny / ru && e == cudaSuccess; ++u) {
+      const double* f = p->jc_map + (size_t)u * ru * nx;
+      if (precision) field_by_units(f, nx, ru, 1, chunk_f);
+      else field_by_units(f, nx, ru, 1, chunk_d);
+      copy_sync(w + ojc + (size_t)u * ru * nx * ts, precision ? (const void*)chunk_f : (const void*)chunk_d, (size_t)ru * nx * ts);
     }
   }
   // state that must start at zero: solver state (cold start), barrier

@@ -18,19 +18,33 @@ struct StageIn {
   double* ynew;
 };
 
+// Scalars of the integrator's current step attempt.  Thread 0 computes them and the others read
+// them: an FP64 instruction occupies an SM sub-partition for 64 cycles, so the same scalar
+// arithmetic done by every warp of an SM would take tens of thousands of cycles per step.
+struct Control {
+  double t, h, h_prop, t_lim, t_new;
+  double ts[4];                  // stage times
+  double c[4][3];                // stage coefficients of the derivatives
+  int go, clipped, seg, outcome, status;
+};
+
 // per-CTA copy of the scalars every CTA agrees on
 struct Shared {
-  double red[NT / 32];
-  double A, C, r, hed;
+  double red[NT / 32], red2[NT / 32];
+  double A, C, r, hed, N;
+  float Af, Cf, rq;              // (2D) A, C and h_e_dot in the transform precision's FP32 form
+  int stop, ok, diverged;        // decisions of the outside iteration
   int warm_valid;
   double A_prev;
   int com_valid, hd_sel;         // (2D) accepted-step initial approximation, see SolverState
   double A_com;
   double q11;                    // (2D) sum over free space of q1 (from the solver state)
+  double inv_nout;               // 1 / free-space cells
   int attempt_first;             // (2D) the next right-hand side is the first of a step attempt
   unsigned long long bar_passed;  // grid barriers passed in this launch (thread 0)
   unsigned long long tma_bar;     // (3D) mbarrier of the bulk copies into the staging buffer
   unsigned tma_parity;            // (3D) phase parity the next wait on tma_bar expects
+  Control ctl;
 };
 
 // ------------------------------------------------------------------------------------------
@@ -91,116 +105,142 @@ struct RhsOut {
 
 // ------------------------------------------------------------------------------------------
 // BS23 integrator loop shared by the film and bulk kernels: adaptive steps until t_target or
-// max_attempts, first same as last, every decision taken identically by every CTA.
+// max_attempts, first same as last, every decision taken identically by every CTA (by its
+// thread 0, from the same sums).
 // R(t, seg, stage_in, k_out, force_iters, want_err, h, k1, k2, k3, y, ynew) evaluates one
 // right-hand side.  Returns the launch status.
 // ------------------------------------------------------------------------------------------
 template <class Rhs>
-__device__ int bs23_advance(Rhs& R, const Desc& d, SolverState* st, const KernelArgs& a, bool leader) {
+__device__ int bs23_advance(Rhs& R, const Desc& d, SolverState* st, const KernelArgs& a, bool leader,
+                            Control& ctl) {
+  const bool t0 = threadIdx.x == 0;
+  if (t0) { ctl.t = st->t; ctl.h = st->h; ctl.status = ST_OK; }
+  int failed = st->failed, k1_valid = st->k1_valid;
+  int iy = st->ybuf, iyn = st->ynewbuf, ik1 = st->k1buf, ik4 = st->k4buf;
+  // k2, k3 live in the two remaining buffers
+  int others[2], no = 0;
+  for (int b = 0; b < 6 && no < 2; ++b)
+    if (b != iy && b != iyn && b != ik1 && b != ik4) others[no++] = b;
+  const int ik2 = others[0], ik3 = others[1];
+  long long att = 0, n_rhs = 0, n_it = 0, n_acc = 0, n_rej = 0, n_nc = 0;
+  double last_r = 0.0, last_err = 0.0;             // thread 0
   int status = ST_OK;
-    // BS23 with first-same-as-last, all decisions on the device
-    double t = st->t, h = st->h;
-    int failed = st->failed, k1_valid = st->k1_valid;
-    int iy = st->ybuf, iyn = st->ynewbuf, ik1 = st->k1buf, ik4 = st->k4buf;
-    // k2, k3 live in the two remaining buffers
-    int others[2], no = 0;
-    for (int b = 0; b < 6 && no < 2; ++b)
-      if (b != iy && b != iyn && b != ik1 && b != ik4) others[no++] = b;
-    const int ik2 = others[0], ik3 = others[1];
-    long long att = 0, n_rhs = 0, n_it = 0, n_acc = 0, n_rej = 0, n_nc = 0;
-    double last_r = 0.0, last_err = 0.0;
-    while (t < a.t_target && att < a.max_attempts) {
-      const double t_lim = fmin(a.t_target, he_next_knot(d, t));
-      const double h_prop = h;         // the controller's proposal before clipping
-      const bool clipped = t + 1.1 * h >= t_lim;
-      if (clipped) h = t_lim - t;
-      R.on_attempt();                  // the attempt's first evaluation starts from the accepted step
-      const int seg = he_segment(d, t);
-      int it[4] = {-1, -1, -1, -1};
-      double* y = d.fbuf[iy];
-      double* yn = d.fbuf[iyn];
-      double* k1 = d.fbuf[ik1];
-      double* k2 = d.fbuf[ik2];
-      double* k3 = d.fbuf[ik3];
-      double* k4 = d.fbuf[ik4];
-      RhsOut r;
-      r.status = ST_OK;
-      r.r = 0.0;
-      if (!k1_valid) {
-        // a k1 whose outside iteration did not converge rejects the attempt like any other
-        // stage; the warm start keeps the progress, so the next attempt continues from it
-        StageIn in{y, 0, {0, 0, 0}, {nullptr, nullptr, nullptr}, nullptr};
-        r = R(t, seg, in, k1, 0, false, 0, nullptr, nullptr, nullptr, nullptr, nullptr);
-        ++n_rhs; n_it += r.iters; it[0] = r.iters;
-        if (r.status == ST_BARRIER) { status = ST_BARRIER; break; }
-        if (r.status == ST_OK && r.nonfinite) { status = ST_NONFINITE; break; }
-        if (r.status == ST_OK) k1_valid = 1;
+  for (;;) {
+    __syncthreads();
+    if (t0) {
+      ctl.go = ctl.t < a.t_target && att < a.max_attempts;
+      if (ctl.go) {
+        ctl.t_lim = fmin(a.t_target, he_next_knot(d, ctl.t));
+        ctl.h_prop = ctl.h;            // the controller's proposal before clipping
+        ctl.clipped = ctl.t + 1.1 * ctl.h >= ctl.t_lim;
+        if (ctl.clipped) ctl.h = ctl.t_lim - ctl.t;
+        ctl.seg = he_segment(d, ctl.t);
+        const double t = ctl.t, h = ctl.h;
+        ctl.t_new = ctl.clipped ? ctl.t_lim : t + h;
+        ctl.ts[0] = t; ctl.ts[1] = t + 0.5 * h; ctl.ts[2] = t + 0.75 * h; ctl.ts[3] = ctl.t_new;
+        ctl.c[1][0] = 0.5 * h; ctl.c[2][0] = 0.75 * h;
+        ctl.c[3][0] = h * (2.0 / 9.0); ctl.c[3][1] = h * (1.0 / 3.0); ctl.c[3][2] = h * (4.0 / 9.0);
       }
-      int outcome = 1;
-      double err = INFINITY;
-      if (r.status == ST_OK) {
-        StageIn s2{y, 1, {0.5 * h, 0, 0}, {k1, nullptr, nullptr}, nullptr};
-        r = R(t + 0.5 * h, seg, s2, k2, 0, false, 0, nullptr, nullptr, nullptr, nullptr, nullptr);
-        ++n_rhs; n_it += r.iters; it[1] = r.iters;
-        if (r.status == ST_BARRIER) { status = ST_BARRIER; break; }
-      }
-      if (r.status == ST_OK) {
-        StageIn s3{y, 1, {0.75 * h, 0, 0}, {k2, nullptr, nullptr}, nullptr};
-        r = R(t + 0.75 * h, seg, s3, k3, 0, false, 0, nullptr, nullptr, nullptr, nullptr, nullptr);
-        ++n_rhs; n_it += r.iters; it[2] = r.iters;
-        if (r.status == ST_BARRIER) { status = ST_BARRIER; break; }
-      }
-      const double t_new = clipped ? t_lim : t + h;
-      if (r.status == ST_OK) {
-        StageIn s4{y, 3, {h * (2.0 / 9.0), h * (1.0 / 3.0), h * (4.0 / 9.0)}, {k1, k2, k3}, yn};
-        r = R(t_new, seg, s4, k4, 0, true, h, k1, k2, k3, y, yn);
-        ++n_rhs; n_it += r.iters; it[3] = r.iters;
-        if (r.status == ST_BARRIER) { status = ST_BARRIER; break; }
-        if (r.status == ST_OK) err = r.err;
-      }
+    }
+    __syncthreads();
+    if (!ctl.go) break;
+    R.on_attempt();                    // the attempt's first evaluation starts from the accepted step
+    const int seg = ctl.seg;
+    const double h = ctl.h;
+    int it[4] = {-1, -1, -1, -1};
+    double* y = d.fbuf[iy];
+    double* yn = d.fbuf[iyn];
+    double* k1 = d.fbuf[ik1];
+    double* k2 = d.fbuf[ik2];
+    double* k3 = d.fbuf[ik3];
+    double* k4 = d.fbuf[ik4];
+    RhsOut r;
+    r.status = ST_OK;
+    r.r = 0.0;
+    if (!k1_valid) {
+      // a k1 whose outside iteration did not converge rejects the attempt like any other
+      // stage; the warm start keeps the progress, so the next attempt continues from it
+      StageIn in{y, 0, {0, 0, 0}, {nullptr, nullptr, nullptr}, nullptr};
+      r = R(ctl.ts[0], seg, in, k1, 0, false, 0, nullptr, nullptr, nullptr, nullptr, nullptr);
+      ++n_rhs; n_it += r.iters; it[0] = r.iters;
+      if (r.status == ST_BARRIER) { status = ST_BARRIER; break; }
+      if (r.status == ST_OK && r.nonfinite) { status = ST_NONFINITE; break; }
+      if (r.status == ST_OK) k1_valid = 1;
+    }
+    if (r.status == ST_OK) {
+      StageIn s2{y, 1, {ctl.c[1][0], 0, 0}, {k1, nullptr, nullptr}, nullptr};
+      r = R(ctl.ts[1], seg, s2, k2, 0, false, 0, nullptr, nullptr, nullptr, nullptr, nullptr);
+      ++n_rhs; n_it += r.iters; it[1] = r.iters;
+      if (r.status == ST_BARRIER) { status = ST_BARRIER; break; }
+    }
+    if (r.status == ST_OK) {
+      StageIn s3{y, 1, {ctl.c[2][0], 0, 0}, {k2, nullptr, nullptr}, nullptr};
+      r = R(ctl.ts[2], seg, s3, k3, 0, false, 0, nullptr, nullptr, nullptr, nullptr, nullptr);
+      ++n_rhs; n_it += r.iters; it[2] = r.iters;
+      if (r.status == ST_BARRIER) { status = ST_BARRIER; break; }
+    }
+    if (r.status == ST_OK) {
+      StageIn s4{y, 3, {ctl.c[3][0], ctl.c[3][1], ctl.c[3][2]}, {k1, k2, k3}, yn};
+      r = R(ctl.ts[3], seg, s4, k4, 0, true, h, k1, k2, k3, y, yn);
+      ++n_rhs; n_it += r.iters; it[3] = r.iters;
+      if (r.status == ST_BARRIER) { status = ST_BARRIER; break; }
+    }
+    const bool reached = r.status == ST_OK;
+    if (t0) {
+      const double err = reached ? r.err : (double)INFINITY;
+      ctl.outcome = !reached ? 2 : (err <= 1.0 ? 1 : 0);
       last_r = r.r;
-      if (r.status != ST_OK) { outcome = 2; ++n_nc; }
-      else outcome = err <= 1.0 ? 1 : 0;
-      if (leader && st->log_count < d.log_cap) {
-        StepLog L; L.t = t; L.h = h; L.t_new = outcome == 1 ? t_new : t; L.err = err;
-        L.outcome = outcome; for (int q = 0; q < 4; ++q) L.iters[q] = it[q]; L.pad = 0;
-        d.log[st->log_count] = L;
+      const bool clipped = ctl.clipped != 0;
+      if (leader) {
+        if (st->log_count < d.log_cap) {
+          StepLog L; L.t = ctl.t; L.h = h; L.t_new = ctl.outcome == 1 ? ctl.t_new : ctl.t; L.err = err;
+          L.outcome = ctl.outcome; for (int q = 0; q < 4; ++q) L.iters[q] = it[q]; L.pad = 0;
+          d.log[st->log_count] = L;
+        }
+        st->log_count += 1;
       }
-      if (leader) st->log_count += 1;
-      ++att;
-      if (outcome == 1) {
-        R.on_accept();                 // the last evaluation's iterate starts later calls
-        const bool knot_hit = clipped && t_lim == he_next_knot(d, t);
-        t = t_new;
-        int tmp = iy; iy = iyn; iyn = tmp;
-        tmp = ik1; ik1 = ik4; ik4 = tmp;
-        k1_valid = knot_hit ? 0 : 1;
+      if (ctl.outcome == 1) {
+        const bool knot_hit = clipped && ctl.t_lim == he_next_knot(d, ctl.t);
+        ctl.t = ctl.t_new;
+        ctl.go = knot_hit ? 0 : 1;     // k4 serves as the next k1
         double fac = err == 0.0 ? 5.0 : fmin(5.0, fmax(0.2, 0.9 * pow(err, -1.0 / 3.0)));
         if (failed) fac = fmin(fac, 1.0);
         // a step shortened to end on a knot or output time says nothing about longer steps:
         // the next one starts from the proposal it replaced (never above it)
-        h = (clipped && h < h_prop) ? h_prop * fmin(fac, 1.0) : h * fac;
-        failed = 0;
-        ++n_acc;
+        ctl.h = (clipped && h < ctl.h_prop) ? ctl.h_prop * fmin(fac, 1.0) : h * fac;
         last_err = err;
-      } else if (outcome == 0) {
-        h = h * fmax(0.2, 0.9 * pow(err, -1.0 / 3.0));
-        failed = 1;
-        ++n_rej;
+      } else if (ctl.outcome == 0) {
+        ctl.h = h * fmax(0.2, 0.9 * pow(err, -1.0 / 3.0));
       } else {
-        h = 0.5 * h;
-        failed = 1;
-        ++n_rej;
+        ctl.h = 0.5 * h;
       }
-      if (h < d.h_min) { status = ST_UNDERFLOW; break; }
+      if (ctl.h < d.h_min) ctl.status = ST_UNDERFLOW;
     }
-    if (leader) {
-      st->t = t; st->h = h; st->failed = failed; st->k1_valid = k1_valid;
-      st->ybuf = iy; st->ynewbuf = iyn; st->k1buf = ik1; st->k4buf = ik4;
-      st->n_attempts += att; st->n_rhs += n_rhs; st->n_iters += n_it; st->n_accepted += n_acc;
-      st->n_rejected += n_rej; st->n_noconv += n_nc; st->last_r = last_r; st->last_err = last_err;
+    __syncthreads();
+    ++att;
+    const int outcome = ctl.outcome;
+    if (outcome == 1) {
+      R.on_accept();                   // the last evaluation's iterate starts later calls
+      int tmp = iy; iy = iyn; iyn = tmp;
+      tmp = ik1; ik1 = ik4; ik4 = tmp;
+      k1_valid = ctl.go;
+      failed = 0;
+      ++n_acc;
+    } else {
+      if (outcome == 2) ++n_nc;
+      failed = 1;
+      ++n_rej;
     }
-    return status;
+    status = ctl.status;
+    if (status != ST_OK) break;
+  }
+  if (leader) {
+    st->t = ctl.t; st->h = ctl.h; st->failed = failed; st->k1_valid = k1_valid;
+    st->ybuf = iy; st->ynewbuf = iyn; st->k1buf = ik1; st->k4buf = ik4;
+    st->n_attempts += att; st->n_rhs += n_rhs; st->n_iters += n_it; st->n_accepted += n_acc;
+    st->n_rejected += n_rej; st->n_noconv += n_nc; st->last_r = last_r; st->last_err = last_err;
+  }
+  return status;
 }
 
 }  // namespace mf

@@ -54,4 +54,83 @@ inline int stage_twiddles(int L, T* out) {
   return n;
 }
 
+// Values of type T set aside per point of an axis for its twiddle tables: the bulk's tables A and B
+// hold fewer than 2 L complex entries; the core's hold fewer than L entries of 4 (single) or 2
+// (double) values
+constexpr size_t TWIDDLE_VALUES = 4;
+
+// Table of the transform core (mf_core.cuh) for length L and E = 2^e elements per thread, stage after
+// stage: p = E, E^2, ...: w^(2^m), m < e, with w = exp(-2 pi i k / (E p)) for k < p; a last stage of
+// radix 2^r < E holds m < r with w = exp(-2 pi i k / L) for k < L / E.  A single-precision entry is
+// stored twice over, (re, re, im, im), for the packed instructions.  Returns the number of values of
+// type T written.
+template <typename T>
+inline size_t core_twiddles(int L, int E, T* out) {
+  int lg = 0, e = 0;
+  while ((1 << lg) < L) ++lg;
+  while ((1 << e) < E) ++e;
+  size_t n = 0;
+  int lgp = e;
+  for (int rem = lg - e; rem > 0; rem -= e, lgp += e) {
+    const int nk = rem >= e ? 1 << lgp : L >> e;
+    const int den = rem >= e ? E << lgp : L;
+    for (int m = 0; m < (rem >= e ? e : rem); ++m)
+      for (int k = 0; k < nk; ++k) {
+        const double ang = -2.0 * M_PI * (double)(k << m) / (double)den;
+        const T c = (T)std::cos(ang), s = (T)std::sin(ang);
+        if (sizeof(T) == 4) { out[n++] = c; out[n++] = c; out[n++] = s; out[n++] = s; }
+        else { out[n++] = c; out[n++] = s; }
+      }
+  }
+  return n;
+}
+
+// Launch shape of a film: a CTA per unit of the wider pass (its lines run on as few CTAs' threads
+// as the pass leaves idle), no more than fit the GPU at once.
+inline void film_shape(Desc& d, int coresident) {
+  const int ru = row_unit(d.precision);
+  const int rows = d.ny / ru, cols = (d.nx / 2 + 1 + ru / 2 - 1) / (ru / 2);
+  const int want = rows > cols ? rows : cols;
+  d.rows_per_item = ru;
+  d.zs_per_item = ru;
+  d.grid = want < coresident ? want : coresident;
+}
+// Elements per thread E of a film's passes along an axis of n points (mf_core.cuh).  A radix-E stage
+// costs one exchange through shared memory, so the large films take E = 8 (2048 points: 3 exchanges
+// per transform).  Where a pass does not fill the chip, its time is one thread's chain of
+// instructions, and fewer elements per thread make it shorter.
+//   FP64: an FP64 instruction occupies an SM sub-partition for 64 cycles whatever the number of
+//     active lanes, so while E = 2 gives at most one warp per sub-partition (256^2 cells: 512 warps
+//     on 608) the pass takes a quarter of the instructions of E = 8.  One right-hand side with 4 / 5 /
+//     5 iterations at 64^2 / 128^2 / 256^2: 202 / 251 / 288 us against 389 / 514 / 550 us.
+//   FP32: E = 4 up to 2^20 cells (1024^2: 256 lines of 256 threads): 64^2 / 512^2 / 1024^2 with 5
+//     iterations 171 / 216 / 304 us against 230 / 240 / 339 us with E = 8; lines of 2048 points would
+//     need 512 threads.
+inline int elems_per_thread(const Desc& d, int n) {
+  const long long cells = (long long)d.nx * d.ny;
+  if (d.precision == 0) return cells <= 65536 && n <= 2 * NT ? 2 : 8;
+  return cells <= 1048576 && n <= 4 * NT ? 4 : 8;
+}
+
+// mask classes of `units` row units from the row-major mask of their rows, 2 bits per row
+inline void pack_mask(const unsigned char* mask, int nx, int ru, long long units, unsigned char* out) {
+  for (long long u = 0; u < units; ++u, mask += (long long)ru * nx, out += nx) {
+    const unsigned char *a = mask, *b = mask + nx, *c = a, *d = b;
+    if (ru == 4) {
+      c = mask + 2 * (long long)nx;
+      d = mask + 3 * (long long)nx;
+      for (int x = 0; x < nx; ++x) out[x] = (unsigned char)(a[x] | b[x] << 2 | c[x] << 4 | d[x] << 6);
+    } else {
+      for (int x = 0; x < nx; ++x) out[x] = (unsigned char)(a[x] | b[x] << 2);
+    }
+  }
+}
+// a row-major field by row units, in the transform precision
+template <typename T>
+inline void field_by_units(const double* f, int nx, int ru, long long units, T* out) {
+  for (long long u = 0; u < units; ++u, f += (long long)ru * nx)
+    for (int x = 0; x < nx; ++x)
+      for (int r = 0; r < ru; ++r) *out++ = (T)f[(long long)r * nx + x];
+}
+
 }  // namespace mf
