@@ -48,7 +48,7 @@ def hbm_peak():
 
 
 # the sources the persistent kernels are compiled from (host-only API code excluded)
-KERNEL_SOURCES = ("mf_common.cuh", "mf_fft.cuh", "mf_passes.cuh", "mf_rhs_common.cuh",
+KERNEL_SOURCES = ("mf_common.cuh", "mf_core.cuh", "mf_units.cuh", "mf_rhs_common.cuh",
                   "mf_tables.h", "mf_film.cuh", "mf_film.cu", "mf_film_batch.cu", "mf_bulk.cu")
 
 

@@ -44,9 +44,8 @@ cudaError_t adj_warm_io(int precision, int nx, int ny, int load, const uint8_t* 
 cudaError_t adj_lincomb(long long n, double* out, int nt, const double* const* x, const double* c,
                         double b, cudaStream_t s);
 cudaError_t adj_sums(long long n, const double* x, double* out, cudaStream_t s);
-cudaError_t adj_to_float(long long n, const double* x, float* y, cudaStream_t s);
-cudaError_t film_to_units(int precision, int nx, int ny, const double* x, void* y, cudaStream_t s);
-cudaError_t film_relayout(int precision, int nx, int ny, bool to_rows, const void* src, void* dst, cudaStream_t s);
+cudaError_t field_to_units(int precision, int nx, long long rows, const double* x, void* y, cudaStream_t s);
+cudaError_t field_relayout(int precision, int nx, long long rows, bool to_rows, const void* src, void* dst, cudaStream_t s);
 }  // namespace mf
 
 namespace {
@@ -145,8 +144,7 @@ void fill_tables(const mf_params* p, const Desc& d, std::vector<char>& tw, std::
   std::vector<T> t;
   for (int a = 0; a < 3; ++a) {
     std::vector<T> blk(TWIDDLE_VALUES * (size_t)ns[a], (T)0);
-    if (p->dim == 3) stage_twiddles<T>(ns[a], blk.data());
-    else if (a < 2) core_twiddles<T>(ns[a], a == 0 ? d.ex : d.ey, blk.data());
+    if (p->dim == 3 || a < 2) core_twiddles<T>(ns[a], a == 0 ? d.ex : a == 1 ? d.ey : d.ez, blk.data());
     t.insert(t.end(), blk.begin(), blk.end());
   }
   tw.assign((const char*)t.data(), (const char*)(t.data() + t.size()));
@@ -306,7 +304,8 @@ mf_status mf_create(const mf_params* p, void* d_workspace, size_t bytes, void* s
   d.dev = (const Desc*)(w + L.desc);
 
   // launch configuration: all CTAs co-resident, no more than the widest pass can use
-  if (p->dim == 2) { d.ex = elems_per_thread(d, d.nx); d.ey = elems_per_thread(d, d.ny); }
+  if (p->dim == 2) { d.ex = elems_per_thread(d, d.nx); d.ey = elems_per_thread(d, d.ny); d.ez = 2; }
+  else bulk_shape(d, 1);
   const size_t smem = kernel_smem_bytes(d);
   int per_sm = p->dim == 2 ? film_max_blocks(p->precision, smem) : bulk_max_blocks(p->precision, smem);
   int nsm = 0;
@@ -321,26 +320,7 @@ mf_status mf_create(const mf_params* p, void* d_workspace, size_t bytes, void* s
   if (p->dim == 2) {
     film_shape(d, coresident);
   } else {
-    // x pass: rb rows of 3 fields; y pass: zs z-lines of 3 fields
-    int rb = std::min(p->ny, 2 * BATCH / (3 * p->nx));
-    rb = std::max(2, rb & ~1);
-    while (rb & (rb - 1)) rb &= rb - 1;
-    int zs = std::min(nz, BATCH / (3 * p->ny));
-    zs = std::max(1, zs);
-    while (zs & (zs - 1)) zs &= zs - 1;
-    const long long xitems = (long long)p->ny * nz / rb;
-    const long long zlines = (long long)(p->nx / 2 + 1) * p->ny;
-    const int grid = (int)std::min<long long>(coresident, std::max(xitems, zlines));
-    while (rb > 2 && (long long)p->ny * nz / rb < grid) rb /= 2;
-    while (zs > 1 && (long long)(p->nx / 2 + 1) * nz / zs < grid) zs /= 2;
-    d.rows_per_item = rb;
-    d.zs_per_item = zs;
-    d.grid = std::max(1, grid);
-    if (3 * p->nx * (rb / 2) > BATCH || 3 * p->ny * zs > BATCH || 3 * nz > BATCH) {
-      pb->err = "grid too large for the shared-memory batch";
-      delete pb;
-      return MF_ERR_ARG;
-    }
+    bulk_shape(d, coresident);
   }
 
   // tables and inputs
@@ -349,18 +329,15 @@ mf_status mf_create(const mf_params* p, void* d_workspace, size_t bytes, void* s
   else fill_tables<double>(p, d, tw, kt, gt);
   const size_t ts = p->precision ? 4 : 8;
   std::vector<char> jcbuf;
-  const int ru = p->dim == 2 ? row_unit(p->precision) : 1;    // films: kept by row units
+  const int ru = row_unit(p->precision);           // fields and mask are kept by row units
   if (p->jc_map) {
     jcbuf.resize(L.ncell * ts);
     const long long units = L.ncell / ((long long)ru * p->nx);
     if (p->precision) field_by_units(p->jc_map, p->nx, ru, units, (float*)jcbuf.data());
     else field_by_units(p->jc_map, p->nx, ru, units, (double*)jcbuf.data());
   }
-  std::vector<unsigned char> units;
-  if (p->dim == 2) {
-    units.resize(L.ncell / ru);
-    pack_mask(p->mask, p->nx, ru, p->ny / ru, units.data());
-  }
+  std::vector<unsigned char> units(L.ncell / ru);
+  pack_mask(p->mask, p->nx, ru, (long long)p->ny * nz / ru, units.data());
   std::vector<double> knots(2 * (p->he_knots > 0 ? p->he_knots : 1), 0.0);
   for (int i = 0; i < p->he_knots; ++i) { knots[i] = p->he_t[i]; knots[p->he_knots + i] = p->he_v[i]; }
   SolverState s0;
@@ -373,8 +350,7 @@ mf_status mf_create(const mf_params* p, void* d_workspace, size_t bytes, void* s
   auto cp = [&](void* dst, const void* src, size_t n) {
     if (e == cudaSuccess && n) e = cudaMemcpyAsync(dst, src, n, cudaMemcpyHostToDevice, st);
   };
-  if (p->dim == 2) cp(w + L.mask, units.data(), units.size());
-  else cp(w + L.mask, p->mask, L.ncell);
+  cp(w + L.mask, units.data(), units.size());
   if (p->jc_map) cp(w + L.jc, jcbuf.data(), jcbuf.size());
   const size_t twx = TWIDDLE_VALUES * p->nx * ts, twy = TWIDDLE_VALUES * p->ny * ts, twz = TWIDDLE_VALUES * nz * ts;
   cp(w + L.twx, tw.data(), twx);
@@ -791,9 +767,9 @@ static std::vector<std::array<int, 3>> tuning_candidates(const mf_problem* pb, i
   if (d.dim == 2) {
     add(d.rows_per_item, d.zs_per_item);     // row units are fixed by the precision: launch widths only
   } else {
-    // x pass: rb rows of 3 fields; y pass: zs z-lines of 3 fields
-    for (int rb = 2; rb <= d.ny && 3 * d.nx * (rb / 2) <= BATCH; rb *= 2)
-      for (int zs = 1; zs <= d.nz && 3 * d.ny * zs <= BATCH; zs *= 2) add(rb, zs);
+    // row units per x item that a CTA holds
+    const int ru = row_unit(d.precision);
+    for (int ub = 1; ub <= NT / (d.nx / d.ex) && (long long)d.ny * d.nz / ru % ub == 0; ub *= 2) add(ub * ru, d.zs_per_item);
   }
   return c;
 }
@@ -905,12 +881,14 @@ std::vector<std::pair<void*, size_t>> ckpt_regions(const mf_problem* pb) {
   r.push_back({(void*)d.log, (size_t)d.log_cap * sizeof(StepLog)});
   return r;
 }
-// a film's h_dot buffers, kept by row units, are row-major in the blob: a spectrum buffer (free
-// between calls) to convert them through, null for every other region
+// the h_dot buffers, kept by row units, are row-major in the blob: a spectrum buffer (free between
+// calls) to convert them through, null for every other region
 void* ckpt_rows(const mf_problem* pb, const void* region) {
-  if (pb->d.dim != 2) return nullptr;
-  return region == pb->d.hd ? pb->d.Sa : region == pb->d.hd2 ? pb->d.Sb : nullptr;
+  if (region == pb->d.hd) return pb->d.Sa;
+  return pb->d.dim == 2 && region == pb->d.hd2 ? pb->d.Sb : nullptr;
 }
+// rows of the h_dot buffer (units do not straddle planes or components)
+long long field_rows(const mf_problem* pb) { return (long long)pb->d.ny * pb->d.nz * (pb->d.dim == 2 ? 1 : 3); }
 size_t ckpt_bytes(const mf_problem* pb) {
   size_t b = sizeof(CkptHeader);
   for (const auto& x : ckpt_regions(pb)) b += x.second;
@@ -931,7 +909,7 @@ mf_status mf_checkpoint_save(mf_problem* pb, void* dst) {
   o += sizeof(h);
   for (const auto& x : ckpt_regions(pb)) {
     if (void* rows = ckpt_rows(pb, x.first)) {
-      cudaError_t e = film_relayout(pb->d.precision, pb->d.nx, pb->d.ny, true, x.first, rows, pb->stream);
+      cudaError_t e = field_relayout(pb->d.precision, pb->d.nx, field_rows(pb), true, x.first, rows, pb->stream);
       if (e != cudaSuccess) return cuda_fail(pb, e, "checkpoint layout");
       MF_CUDA(pb, cudaMemcpyAsync(o, rows, x.second, cudaMemcpyDefault, pb->stream));
       o += x.second;
@@ -960,7 +938,7 @@ mf_status mf_checkpoint_restore(mf_problem* pb, const void* src) {
   for (const auto& x : ckpt_regions(pb)) {
     if (void* rows = ckpt_rows(pb, x.first)) {
       MF_CUDA(pb, cudaMemcpyAsync(rows, i, x.second, cudaMemcpyDefault, pb->stream));
-      cudaError_t e = film_relayout(pb->d.precision, pb->d.nx, pb->d.ny, false, rows, x.first, pb->stream);
+      cudaError_t e = field_relayout(pb->d.precision, pb->d.nx, field_rows(pb), false, rows, x.first, pb->stream);
       if (e != cudaSuccess) return cuda_fail(pb, e, "checkpoint layout");
       i += x.second;
       continue;
@@ -971,8 +949,8 @@ mf_status mf_checkpoint_restore(mf_problem* pb, const void* src) {
   // the work-item shape (it sets the order of the sums; a film's is fixed) and launch width it was
   // saved with
   if (pb->d.dim == 3) {
-    pb->d.rows_per_item = h.rows_per_item;
-    pb->d.zs_per_item = h.zs_per_item;
+    const int ru = row_unit(pb->d.precision), most = NT / (pb->d.nx / pb->d.ex) * ru;
+    pb->d.rows_per_item = std::min(std::max(h.rows_per_item, ru), most);
   }
   pb->d.grid = h.grid;
   MF_CUDA(pb, cudaMemcpyAsync((void*)pb->d.dev, &pb->d, sizeof(Desc), cudaMemcpyHostToDevice, pb->stream));
@@ -1249,17 +1227,8 @@ mf_status mf_set_jc_map(mf_problem* pb, const double* d_jc) {
     return MF_ERR_ARG;
   }
   MF_CUDA(pb, cudaSetDevice(pb->device));
-  const long long n = pb->d.ncell;
-  if (pb->d.dim == 2) {
-    cudaError_t e = film_to_units(pb->d.precision, pb->d.nx, pb->d.ny, d_jc, (void*)pb->d.jcmap, pb->stream);
-    if (e != cudaSuccess) return cuda_fail(pb, e, "jc map conversion");
-  } else if (pb->d.precision) {
-    cudaError_t e = adj_to_float(n, d_jc, (float*)pb->d.jcmap, pb->stream);
-    if (e != cudaSuccess) return cuda_fail(pb, e, "jc map conversion");
-  } else {
-    MF_CUDA(pb, cudaMemcpyAsync((void*)pb->d.jcmap, d_jc, n * sizeof(double), cudaMemcpyDeviceToDevice,
-                                pb->stream));
-  }
+  cudaError_t e = field_to_units(pb->d.precision, pb->d.nx, (long long)pb->d.ny * pb->d.nz, d_jc, (void*)pb->d.jcmap, pb->stream);
+  if (e != cudaSuccess) return cuda_fail(pb, e, "jc map conversion");
   MF_CUDA(pb, cudaStreamSynchronize(pb->stream));
   return MF_OK;
 }

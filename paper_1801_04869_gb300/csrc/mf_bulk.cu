@@ -3,29 +3,26 @@
 //
 // Method: Section 3.1 of Prigozhin & Sokolovsky (arXiv:1801.04869).  The state h has three
 // components (component-major).  A vector "round trip" F^-1[M F(v)] runs as five passes
-// separated by grid barriers:
-//   X   x pass: rows of the real field, R2C along x           -> S1[c][z][kx][y]
-//   Yf  y pass: forward along y                                -> S2[c][kx][ky][z]
-//   Z   z pass: forward along z, the 3x3 multiplier M, inverse along z (in place in S2)
-//   Yi  y pass: inverse along y                                -> S1
-//   X   x pass: C2R along x, epilogue on all three components, and the forward x pass of the
-//       next round trip's input
+// separated by grid barriers, all on one spectrum S[c][z][kx][y] in place:
+//   X   x pass: rows of the real field, R2C along x
+//   Yf  y pass: forward along y (contiguous lines)
+//   Z   z pass: forward along z, the 3x3 multiplier M, inverse along z
+//   Yi  y pass: inverse along y
+//   X   x pass: C2R along x, epilogue, and the forward x pass of the next round trip's input
 // Multipliers: the Gaussian-smoothed curl i G k x (Section 3.1, last paragraph) and the
 // Biot-Savart operator Phi = (i/|k|^2) k x (Eq. 17, 1/|k|^2 -> 0 at k = 0).
 // One right-hand side (Eqs. 13-14 and the iteration of Eq. 18):
 //   j = curl h;  e = rho(|j|) j (Eq. 13) or rho_out j;  h_dot_in = -curl e on the conductor
 //   repeat: j_dot = curl h_dot, kept on the conductor;  h_dot_out = h_e_dot + Phi[j_dot] on
 //   free space;  stop when mean_out |h_dot^{i+1} - h_dot^i| < delta_it max(|h_e_dot|, 1).
-#include "mf_rhs_common.cuh"
+//
+// The passes run on the transform core (mf_core.cuh); real fields and the mask lie by row units
+// (mf_units.cuh).
+#include "mf_units.cuh"
 
 namespace mf {
 
 enum Op3 { OP3_CURL = 0, OP3_CURLNEG = 1, OP3_PHI = 2 };
-
-// y and z lines of at least 2^TMA_MIN_LG points are staged by bulk copies (tensor memory
-// accelerator); shorter ones by per-thread cp.async into a rotating third buffer, which issues
-// the next item's gather earlier (measured faster for the 128-point lines of a 128^3 grid)
-constexpr int TMA_MIN_LG = 8;
 
 // raw pointers and sizes the x-pass epilogues need, held by value (registers)
 template <typename T>
@@ -35,566 +32,652 @@ struct BulkPtrs {
   T* hd;
   long long ncell;
   int nx, ny;
-  double Lx, Ly, Lz, dx, dy, dz;
+};
+
+// The threads of a group of G = 2^lgG neighbouring lines of the z pass: a line's element z lies nkx ny
+// values behind element z - 1, so the group's lines are interleaved on the lanes and a warp reads
+// G x 16 contiguous bytes per z.  Line u's buffer is 8/G elements longer than its padded length, which
+// spreads the lines of 8 neighbouring lanes over the banks.
+template <typename T, int E> struct GroupTeam {
+  using V = typename Lane<T>::V;
+  static constexpr int LGE = lg_of(E);
+  CV<V>* s;
+  const CV<V>* tw;
+  int i, lg, slot, u, lgt, fs;     // position; log2 length; group of the CTA; line of the group; log2 threads
+  __device__ __forceinline__ GroupTeam(CV<V>* buf, const CV<V>* table, int lgL, int lgG) : tw(table), lg(lgL) {
+    lgt = lg - LGE + lgG;
+    slot = (int)threadIdx.x >> lgt;
+    u = (int)threadIdx.x & ((1 << lgG) - 1);
+    i = ((int)threadIdx.x >> lgG) & ((1 << (lg - LGE)) - 1);
+    const int stride = spe<E>(1 << lg) + (8 >> lgG);
+    s = buf + ((slot << lgG) + u) * stride;
+    fs = ((NT >> lgt) << lgG) * stride;
+  }
+  __device__ __forceinline__ CV<V>& at(int e) const { return s[spe<E>(e)]; }
+  __device__ __forceinline__ void sync() const {
+    if (lgt <= 5) __syncwarp();
+    else asm volatile("bar.sync %0, %1;" :: "r"(1 + slot), "r"(1 << lgt) : "memory");
+  }
 };
 
 template <typename T>
 struct Bulk {
+  using V = typename Lane<T>::V;
+  static constexpr int RU = Lane<T>::RU, NL = Lane<T>::NL;
   const Desc& d;
-  C2<T>* sm;
-  C2<T>* sm2;
-  C2<T>* sm3;        // third buffer: the next item's gather in the y and z passes
+  CV<V>* sm;         // the CTA's exchange buffer
   Shared& sh;
   int nx, ny, nz, lgx, lgy, lgz, half, nkx;
   long long nspec, ncell;
-  C2<T>* S1;
-  C2<T>* S2;
+  C2<T>* S;          // spectra of the three components, [c][z][kx][y]
+  T* tmp;            // two real fields by row units (joint epilogues)
   T* hd;
   const uint8_t* mask;
   const T* jcmap;
-  const C2<T>* twx; const C2<T>* twy; const C2<T>* twz;
+  const CV<V>* twx; const CV<V>* twy; const CV<V>* twz;   // twiddle tables in shared memory
   const T* ktab; const T* gtab;     // kx (nkx), ky (ny), kz (nz)
-  int rb, zs, P;
-  unsigned nblocks;
+  T scale;           // 1/(2 cells): the x pass leaves twice the half spectra
+  T ig2, ib0;        // 1/gamma^2; 1/b0 of the Kim law, 0: none
+  int ex, ey, ez, lgG, ub, lgu;     // elements per thread; lines per z group; row units per x item; log2 units per z
+  int max_items;
+  double* partials;
+  GridBarrier* gb;
+  unsigned long long barrier_ns;
 
-  __device__ Bulk(const Desc& dd, C2<T>* s, Shared& shr)
-      : d(dd), sm(s), sm2(s + BATCH_PAD), sm3(s + 2 * BATCH_PAD), sh(shr) {
+  __device__ Bulk(const Desc& dd, unsigned char* smem, Shared& shr) : d(dd), sm((CV<V>*)smem), sh(shr) {
     nx = d.nx; ny = d.ny; nz = d.nz; lgx = d.lgx; lgy = d.lgy; lgz = d.lgz;
     half = nx / 2; nkx = half + 1;
     nspec = (long long)nkx * ny * nz;
     ncell = (long long)nx * ny * nz;
-    S1 = (C2<T>*)d.Sa; S2 = (C2<T>*)d.Sb;
+    S = (C2<T>*)d.Sa; tmp = (T*)d.Sb;
     hd = (T*)d.hd;
     mask = d.mask; jcmap = (const T*)d.jcmap;
-    twx = (const C2<T>*)d.tw_x;
-    twy = (const C2<T>*)d.tw_y;
-    twz = (const C2<T>*)d.tw_z;
+    ex = d.ex; ey = d.ey; ez = d.ez;
+    twx = sm + bulk_slots(d);
+    twy = twx + core_table_len(lgx, ex);
+    twz = twy + core_table_len(lgy, ey);
     ktab = (const T*)d.ktab; gtab = (const T*)d.gtab;
-    rb = d.rows_per_item;
-    zs = d.zs_per_item;
-    P = BATCH / (3 * nz);
-    if (P > ny) P = ny;
-    int p2 = 1;
-    while (p2 * 2 <= P) p2 *= 2;
-    P = p2;
-    nblocks = gridDim.x;
+    scale = (T)0.5 / (T)ncell;
+    ig2 = (T)(1.0 / (d.gamma * d.gamma));
+    ib0 = d.b0 > 0.0 ? (T)(1.0 / d.b0) : (T)0;
+    lgG = z_group_lg(lgz, ez);
+    ub = d.rows_per_item / RU;
+    lgu = lgy - (RU == 4 ? 2 : 1);
+    max_items = d.max_items;
+    partials = d.partials;
+    gb = d.gb;
+    barrier_ns = d.barrier_ns;
+    sh.inv_nout = d.nout > 0 ? 1.0 / (double)d.nout : 0.0;
   }
 
-  __device__ bool sync(int where) { return grid_sync(d.gb, nblocks, where, &sh.bar_passed, d.barrier_ns); }
+  __device__ bool sync(int where) { return grid_sync(gb, gridDim.x, where, &sh.bar_passed, barrier_ns); }
 
-  __device__ BulkPtrs<T> ptrs() const {
-    return BulkPtrs<T>{mask, jcmap, hd, ncell, nx, ny, d.Lx, d.Ly, d.Lz, d.dx, d.dy, d.dz};
+  // members of the law's epilogues
+  template <class Epi> __device__ __forceinline__ void law(Epi& e) const {
+    e.n = (T)d.n; e.e0 = (T)d.e0; e.jc = (T)d.jc; e.rho_out = (T)d.rho_out;
+    e.ig2 = ig2; e.ib0 = ib0;
   }
 
-  // ---- x pass over rows (z, y0 .. y0 + rb): inverse of NIN = 0|3 fields, epilogue, forward ----
-  // With inputs, the item's half spectra arrive staged in the third buffer (cp.async); once the
-  // first inverse stage has read them, the next item's (x pass item `next`, -1: none) are
-  // issued into the same buffer and load while this item finishes.
-  __device__ __forceinline__ void xstage(int it, int nin) {
-    const int per_z = ny / rb;
-    const long long off = (long long)(it / per_z) * nkx * ny + (it % per_z) * rb;
-    if (nin == 3) stage_rows_async<T, 3>(sm3, S1 + off, nspec, ny, rb, lgx);
-  }
-  template <int NIN, int NOUT, class Epi>
-  __device__ __forceinline__ void xitem(int z, int y0, int next, Epi& epi_io) {
-    Epi epi = epi_io;                   // register copy of the epilogue
-    const int nx = this->nx, ny = this->ny, lgx = this->lgx, nkx = this->nkx, rb = this->rb;
-    const long long nspec = this->nspec;
-    C2<T>* const sm = this->sm;
-    C2<T>* const sm2 = this->sm2;
-    C2<T>* const S1 = this->S1;
-    const C2<T>* const twx = this->twx;
-    const int npair = rb / 2;
-    const long long off = (long long)z * nkx * ny + y0;
-    C2<T>* X = sm;
-    const int lgpair = __ffs(npair) - 1;
-    (void)off;
-    if constexpr (NIN > 0) {
-      cp_async_wait<0>();
-      __syncthreads();
-      X = rows_inverse_staged<T, NIN>(sm3, sm, sm2, npair, lgpair, lgx, twx, [&] {
-        if (next >= 0) xstage(next, NIN);
-      });
-    }
-    C2<T>* Y = X == sm ? sm2 : sm;
-    // not unrolled: a second cell in flight spilled the epilogues' live values (26% slower
-    // per outside iteration on the 128^3 grid)
-#pragma unroll 1
-    for (int e = threadIdx.x; e < (npair << lgx); e += NT) {
-      const int pr = e >> lgx, x = e & (nx - 1);
-      T ina[3], inb[3], oa[3], ob[3];
-#pragma unroll
-      for (int f = 0; f < NIN; ++f) {
-        const C2<T> v = X[sp(((f * npair + pr) << lgx) + x)];
-        ina[f] = v.x; inb[f] = v.y;
-      }
-      const long long i0 = ((long long)z * ny + y0 + 2 * pr) * nx + x;
-      if constexpr (Epi::kPair) {
-        epi.pair(i0, i0 + nx, ina, inb, oa, ob);
-      } else {
-        epi(i0, ina, oa);
-        epi(i0 + nx, inb, ob);
-      }
-#pragma unroll
-      for (int f = 0; f < NOUT; ++f) X[sp(((f * npair + pr) << lgx) + x)] = C2<T>{oa[f], ob[f]};
-    }
-    __syncthreads();
-    if constexpr (NOUT > 0) rows_forward_scatter<T, NOUT>(X, Y, S1 + off, nspec, ny, npair, lgpair, lgx, twx);
-    epi_io.acc = epi.acc;
-    epi_io.accmax = epi.accmax;
-  }
-  template <int NIN, int NOUT, class Epi>
-  __device__ void xpass(Epi& epi, int slot) {
-    const int per_z = ny / rb;
-    const int nitems = per_z * nz;
-    if (NIN > 0 && (int)blockIdx.x < nitems) xstage((int)blockIdx.x, NIN);
+  __device__ BulkPtrs<T> ptrs() const { return BulkPtrs<T>{mask, jcmap, hd, ncell, nx, ny}; }
+
+  // ---- x pass: items of ub row units; per unit the components one after the other: inverse (NIN),
+  // epilogue, forward (NOUT).  An epilogue that needs the three components of a cell together (kJoint)
+  // lets the first two wait in `tmp` (the same thread's elements) while the third is transformed. ----
+  template <int E, bool NIN, bool NOUT, class Epi>
+  __device__ __noinline__ void xpass_e(const Epi& epi_in, int slot) {
+    Epi epi = epi_in;                   // register copy of the epilogue
+    const int nx = this->nx, ub = this->ub;
+    const long long ny = this->ny, nspec = this->nspec, ncell = this->ncell;
+    Team<T, E> t(sm, twx, lgx);
+    const int q = t.step();
+    const int nitems = (nz << lgu) / ub;
+    const int first = ((int)threadIdx.x & ~31) >> (lgx - lg_of(E));      // slot of the warp's first lane
+    const bool mine = t.slot < ub;
     for (int it = (int)blockIdx.x; it < nitems; it += (int)gridDim.x) {
-      epi.acc = 0.0;
-      epi.accmax = 0.0;
-      const int next = it + (int)gridDim.x < nitems ? it + (int)gridDim.x : -1;
-      xitem<NIN, NOUT>(it / per_z, (it % per_z) * rb, next, epi);
-      if (slot >= 0) {
-        const double v = epi.is_max ? block_max(epi.accmax, sh.red) : block_sum(epi.acc, sh.red);
-        if (threadIdx.x == 0) d.partials[(size_t)slot * d.max_items + it] = v;
+      epi.reset();
+      if (first < ub) {
+        const int unit = it * ub + (mine ? t.slot : 0);
+        const int z = unit >> lgu, y0 = (unit - (z << lgu)) * RU;
+        C2<T>* const Su = S + (long long)z * nkx * ny + y0;
+        const long long iu = (long long)unit * nx + t.i;                 // 16-byte vector of a component
+        const long long ir = (long long)unit * RU * nx + t.i;            // row-major cell of the first row
+        constexpr int B = Epi::kBatch < E ? Epi::kBatch : E;
+        if constexpr (Epi::kJoint) {
+          T* const tmp = this->tmp;
+          CV<V> v[E];
+#pragma unroll 1
+          for (int c = 0; c < 3; ++c) {
+            row_gather(v, t, Su + c * nspec, nx, ny);
+            core_fft<+1>(v, t);
+            if (c < 2 && mine) {
+#pragma unroll
+              for (int j = 0; j < E; ++j) st_q(tmp + c * ncell + (iu + j * q) * RU, to_q(v[j]));
+            }
+          }
+          if (mine) {
+#pragma unroll
+            for (int j0 = 0; j0 < E; j0 += B) {
+              typename Epi::Ld ld[B];
+              Q<T> in[B][3], out[3];
+#pragma unroll
+              for (int b = 0; b < B; ++b) {
+                const long long i = iu + (j0 + b) * q;
+                ld[b] = epi.load(i, ir + (j0 + b) * q);
+                in[b][0] = ld_q(tmp + i * RU);
+                in[b][1] = ld_q(tmp + ncell + i * RU);
+                in[b][2] = to_q(v[j0 + b]);
+              }
+#pragma unroll
+              for (int b = 0; b < B; ++b) {
+                const long long i = iu + (j0 + b) * q;
+                epi.apply(ld[b], t.i + (j0 + b) * q, unit, ir + (j0 + b) * q, in[b], out);
+                if constexpr (NOUT) {
+                  st_q(tmp + i * RU, out[0]);
+                  st_q(tmp + ncell + i * RU, out[1]);
+                  v[j0 + b] = to_e(out[2]);
+                }
+              }
+            }
+          }
+          if constexpr (NOUT) {
+#pragma unroll 1
+            for (int c = 2; c >= 0; --c) {
+              if (c < 2) {
+#pragma unroll
+                for (int j = 0; j < E; ++j) v[j] = to_e(ld_q(tmp + c * ncell + (iu + j * q) * RU));
+              }
+              core_fft<-1>(v, t);
+              row_scatter(v, t, Su + c * nspec, nx, ny, mine);
+            }
+          }
+        } else {
+#pragma unroll 1
+          for (int c = 0; c < 3; ++c) {
+            CV<V> v[E];
+            typename Epi::Ld ld[2][B];
+            if constexpr (NIN) row_gather(v, t, Su + c * nspec, nx, ny);
+#pragma unroll
+            for (int b = 0; b < B; ++b) ld[0][b] = epi.load(c, iu + b * q, ir + b * q);
+            if constexpr (NIN) core_fft<+1>(v, t);
+#pragma unroll
+            for (int j0 = 0; j0 < E; j0 += B) {
+              if (j0 + B < E) {
+#pragma unroll
+                for (int b = 0; b < B; ++b) ld[(j0 / B + 1) & 1][b] = epi.load(c, iu + (j0 + B + b) * q, ir + (j0 + B + b) * q);
+              }
+              if (mine) {
+#pragma unroll
+                for (int b = 0; b < B; ++b) {
+                  const int j = j0 + b;
+                  Q<T> in, out;
+                  if constexpr (NIN) in = to_q(v[j]);
+                  epi.apply(ld[(j0 / B) & 1][b], c, j, iu + j * q, ir + j * q, in, out);
+                  if constexpr (NOUT) v[j] = to_e(out);
+                }
+              }
+            }
+            if constexpr (NOUT) {
+              core_fft<-1>(v, t);
+              row_scatter(v, t, Su + c * nspec, nx, ny, mine);
+            }
+          }
+          if (mine) epi.done(iu, q);
+        }
       }
+      if (slot >= 0) {
+        const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
+        constexpr int NS = Epi::kSums;
+        __syncthreads();                // the item before has been summed
+#pragma unroll
+        for (int k = 0; k < NS; ++k) {
+          if constexpr (Epi::kMax) {
+            const auto m = warp_max((double)epi.acc[k]);
+            if (l == 0) sh.redn[k][w] = m;
+          } else {
+            const auto s = warp_sum(epi.acc[k]);
+            if (l == 0) sh.redn[k][w] = (double)s;
+          }
+        }
+        __syncthreads();
+        if (l == 0 && w < NS) {         // one sum per warp: an FP64 addition takes 64 cycles
+          double s = sh.redn[w][0];
+          for (int k = 1; k < NT / 32; ++k) s = Epi::kMax ? fmax(s, sh.redn[w][k]) : s + sh.redn[w][k];
+          partials[(size_t)(slot + w) * max_items + it] = s;
+        }
+      }
+    }
+  }
+  // fill(epi) sets the epilogue's members
+  template <template <class, int> class EPI, bool NIN, bool NOUT, class Fill>
+  __device__ __forceinline__ void xpass(Fill fill, int slot = -1) {
+    constexpr int SMALL = sizeof(T) == 4 ? 4 : 2;
+    if (ex == SMALL) {
+      EPI<T, SMALL> e;
+      e.P = ptrs();
+      fill(e);
+      xpass_e<SMALL, NIN, NOUT>(e, slot);
+    } else {
+      EPI<T, 8> e;
+      e.P = ptrs();
+      fill(e);
+      xpass_e<8, NIN, NOUT>(e, slot);
     }
   }
   __device__ double total(int slot, bool is_max = false) {
-    return reduce_partials(d.partials, d.max_items, slot, (ny / rb) * nz, is_max, sh.red);
+    return reduce_partials(partials, max_items, slot, (nz << lgu) / ub, is_max, sh.red);
   }
 
-  // ---- the y and z passes: items it = blockIdx.x, + gridDim.x, ... with the gather of the next
-  // item in flight (cp.async into the third shared buffer) while the current one transforms in
-  // the other two.  issue(it, buf) starts item it's gather into buf; work(it, a, b) transforms
-  // the item gathered in a (b is its second buffer), writes its result and ends with a CTA
-  // barrier.  The buffers rotate: the next input is the prefetch buffer, the next prefetch goes
-  // to the buffer the finished item used last. ----
-  template <class Issue, class Work>
-  __device__ __forceinline__ void pipelined(int nitems, Issue issue, Work work) {
-    C2<T>* a = sm;
-    C2<T>* b = sm2;
-    C2<T>* c = sm3;
-    int it = (int)blockIdx.x;
-    if (it < nitems) issue(it, a);
-    for (; it < nitems; it += (int)gridDim.x) {
-      const int nxt = it + (int)gridDim.x;
-      if (nxt < nitems) {
-        issue(nxt, c);
-        cp_async_wait<1>();                 // this item's group; the next one stays in flight
+  // ---- y pass: contiguous lines in place, z neighbours together in FP32; kx slowest ----
+  template <int E, int DIR>
+  __device__ __noinline__ void ypass_e() {
+    const long long ny = this->ny, nspec = this->nspec, nkx = this->nkx;
+    Team<T, E> t(sm, twy, lgy);
+    const int q = t.step();
+    const int nzp = nz / NL, units = 3 * nzp * (int)nkx;
+    const int per = NT / t.threads(), want = (units + (int)gridDim.x - 1) / (int)gridDim.x;
+    const int nuc = want < per ? want : per;
+    const int first = ((int)threadIdx.x & ~31) >> (lgy - lg_of(E));
+    for (int u0 = (int)blockIdx.x * nuc; u0 < units; u0 += (int)gridDim.x * nuc) {
+      if (first >= nuc || u0 + first >= units) continue;
+      const bool mine = t.slot < nuc && u0 + t.slot < units;
+      const int u = mine ? u0 + t.slot : u0;
+      const int kx = u / (3 * nzp), r = u - kx * 3 * nzp, c = r / nzp, z = (r - c * nzp) * NL;
+      C2<T>* const p = S + c * nspec + (z * nkx + kx) * ny + t.i;
+      const long long next = nkx * ny;       // the line of z + 1
+      CV<V> v[E];
+#pragma unroll
+      for (int j = 0; j < E; ++j) v[j] = ld_col(p + j * q, next, true);
+      core_fft<DIR>(v, t);
+      if (mine) {
+#pragma unroll
+        for (int j = 0; j < E; ++j) st_col(p + j * q, next, true, v[j]);
+      }
+    }
+  }
+  template <int DIR> __device__ __forceinline__ void ypass() {
+    constexpr int BIG = sizeof(T) == 4 ? 16 : 8;
+    if (ey == 4) ypass_e<4, DIR>();
+    else ypass_e<BIG, DIR>();
+  }
+
+  // ---- z pass: forward, 3x3 multiplier, inverse on groups of lines (kx, y0 ..) ----
+  static __device__ __forceinline__ CV<F2> ld_z(const C2<float>* p) {
+    float a, b, c, e;
+    asm volatile("ld.global.L1::no_allocate.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(a), "=f"(b), "=f"(c), "=f"(e) : "l"(p) : "memory");
+    return {pk(a, c), pk(b, e)};
+  }
+  static __device__ __forceinline__ CV<double> ld_z(const C2<double>* p) { return ld_col(p, 0, false); }
+  static __device__ __forceinline__ void st_z(C2<float>* p, const CV<F2>& v) {
+    float4 f;
+    upk(v.x, f.x, f.z);
+    upk(v.y, f.y, f.w);
+    *(float4*)p = f;
+  }
+  static __device__ __forceinline__ void st_z(C2<double>* p, const CV<double>& v) { st_col(p, 0, false, v); }
+  // 1/k2 (0 at k = 0)
+  static __device__ __forceinline__ T inv(T k2) {
+    if constexpr (sizeof(T) == 4) return k2 > 0.f ? __frcp_rn(k2) : 0.f;
+    const T r = k2 > (T)0 ? rsqrt(k2) : (T)0;
+    return r * r;
+  }
+  template <int E>
+  __device__ __noinline__ void zpass_e(int op) {
+    const int ny = this->ny, half = this->half;
+    const long long nspec = this->nspec, zs = (long long)nkx * ny;
+    GroupTeam<T, E> t(sm, twz, lgz, lgG);
+    const int q = 1 << (lgz - lg_of(E));
+    const int gl = NL << lgG, ngy = ny / gl;                  // y lines per group, groups per kx
+    const int units = nkx * ngy;
+    const int per = NT >> t.lgt, want = (units + (int)gridDim.x - 1) / (int)gridDim.x;
+    const int nuc = want < per ? want : per;
+    const int first = ((int)threadIdx.x & ~31) >> t.lgt;
+    for (int u0 = (int)blockIdx.x * nuc; u0 < units; u0 += (int)gridDim.x * nuc) {
+      if (first >= nuc || u0 + first >= units) continue;
+      const bool mine = t.slot < nuc && u0 + t.slot < units;
+      // from the last kx to the first: what the y pass before left in L2 last comes first
+      const int g = units - 1 - (mine ? u0 + t.slot : u0);
+      const int kx = g / ngy, y = (g - kx * ngy) * gl + t.u * NL;
+      C2<T>* const p = S + (long long)kx * ny + y + t.i * zs;
+      CV<V> v[3][E];
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+#pragma unroll
+        for (int j = 0; j < E; ++j) v[c][j] = ld_z(p + c * nspec + j * q * zs);
+      }
+      // wavenumbers of the line(s); odd multipliers are 0 at the Nyquist index of their axis
+      const T kx1 = ldg_tab(&ktab[kx]), gx = ldg_tab(&gtab[kx]);
+      const T kxo = kx == half ? (T)0 : kx1;
+      V ky, ky2, gxy;
+      if constexpr (sizeof(T) == 4) {
+        const float a = ldg_tab(&ktab[nkx + y]), b = ldg_tab(&ktab[nkx + y + 1]);
+        ky = pk(y == (ny >> 1) ? 0.f : a, y + 1 == (ny >> 1) ? 0.f : b);
+        ky2 = pk(fmaf(kx1, kx1, a * a), fmaf(kx1, kx1, b * b));
+        gxy = pk(gx * ldg_tab(&gtab[nkx + y]), gx * ldg_tab(&gtab[nkx + y + 1]));
       } else {
-        cp_async_wait<0>();
+        const double a = ldg_tab(&ktab[nkx + y]);
+        ky = y == (ny >> 1) ? 0.0 : a;
+        ky2 = fma(kx1, kx1, a * a);
+        gxy = gx * ldg_tab(&gtab[nkx + y]);
       }
-      __syncthreads();
-      work(it, a, b);
-      C2<T>* const t = a;
-      a = c;
-      c = b;
-      b = t;
-    }
-  }
-
-  // ---- passes whose items are contiguous lines: item it's `nl` lines of length 2^lg (line l
-  // at src(it, l)) are copied by the tensor memory accelerator (cp.async.bulk) into the third
-  // buffer, line l at l (2^lg + 2) (the two spare values per line shift successive lines by
-  // four banks), completion counted on the CTA's mbarrier.  work(it, after_first) runs the item
-  // and calls after_first() once its first transform stage has read the staging buffer; that
-  // issues the next item's copies, which then land while this item finishes. ----
-  template <class Src, class Work>
-  __device__ __forceinline__ void tma_lines(int nitems, int nl, int lg, Src src, Work work) {
-    unsigned long long* const bar = &sh.tma_bar;
-    const int stride = (1 << lg) + 2;
-    const unsigned bytes = (unsigned)sizeof(C2<T>) << lg;
-    C2<T>* const stg = sm3;
-    auto issue = [&](int it) {
-      if (threadIdx.x == 0) {
-        fence_proxy_async();
-        mbar_expect_tx(bar, bytes * (unsigned)nl);
-        for (int l = 0; l < nl; ++l) bulk_g2s(stg + l * stride, src(it, l), bytes, bar);
-      }
-    };
-    unsigned parity = sh.tma_parity;
-    int it = (int)blockIdx.x;
-    if (it < nitems) issue(it);
-    for (; it < nitems; it += (int)gridDim.x) {
-      mbar_wait(bar, parity, d.gb, d.barrier_ns);
-      parity ^= 1u;
-      const int nxt = it + (int)gridDim.x;
-      work(it, [&] { if (nxt < nitems) issue(nxt); });
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) sh.tma_parity = parity;
-    __syncthreads();
-  }
-  // first (inverse or forward) transform stage of nl staged lines into `out`, then after_first()
-  template <int DIR, class AfterFirst>
-  __device__ __forceinline__ void first_from_stage(int lg, int nl, C2<T>* out, AfterFirst after_first) {
-    C2<T>* const S = dsm<T>();
-    const int st = dsm_off(sm3);
-    const int stride = (1 << lg) + 2;
-    const FftPlan P = fft_plan<T>(lg);
-    fft_first_io_any<T, DIR>(P.lgr(0), lg, nl, [=](int line, int pos) { return S[st + line * stride + pos]; }, out);
-    after_first();
-  }
-
-  // ---- y pass, forward: S1[c][z][kx][:] -> S2[c][kx][:][z] for z in [z0, z0 + zs) ----
-  __device__ __noinline__ void yfwd() {
-    const int ny = this->ny, nz = this->nz, lgy = this->lgy, nkx = this->nkx, zs = this->zs;
-    const long long nspec = this->nspec;
-    C2<T>* const S1 = this->S1;
-    C2<T>* const S2 = this->S2;
-    const C2<T>* const twy = this->twy;
-    const int per_kx = nz / zs;
-    const int nl = 3 * zs;
-    // transposed write of the item's transformed lines (X: line c zs + dz, wavenumber ky)
-    auto scatter = [=](const C2<T>* X, int kx, int z0) {
-      for (int e = threadIdx.x; e < (nl << lgy); e += NT) {
-        const int dz = e % zs, rest = e / zs;
-        const int ky = rest & (ny - 1), c = rest >> lgy;
-        S2[c * nspec + ((long long)kx * ny + ky) * nz + z0 + dz] = X[sp(((c * zs + dz) << lgy) + ky)];
-      }
-      __syncthreads();
-    };
-    if (lgy >= TMA_MIN_LG) {
-      tma_lines(nkx * per_kx, nl, lgy,
-          [=](int it, int l) {
-            const int kx = it / per_kx, z0 = (it % per_kx) * zs;
-            const int c = l / zs, dz = l - c * zs;
-            return (const C2<T>*)(S1 + c * nspec + ((long long)(z0 + dz) * nkx + kx) * ny);
-          },
-          [&](int it, auto after_first) {
-            first_from_stage<-1>(lgy, nl, sm, after_first);
-            scatter(fft_lines_from<T, -1>(sm, sm2, lgy, nl, twy, 1), it / per_kx, (it % per_kx) * zs);
-          });
-      return;
-    }
-    pipelined(nkx * per_kx,
-        [=](int it, C2<T>* buf) {
-          const int kx = it / per_kx, z0 = (it % per_kx) * zs;
-          gather_async<T>(buf, S1, nl << lgy,
-              [=](int e) {
-                const int l = e >> lgy, y = e & (ny - 1);
-                const int c = l / zs, dz = l - c * zs;
-                return c * nspec + ((long long)(z0 + dz) * nkx + kx) * ny + y;
-              },
-              [](int e) { return e; });
-        },
-        [=](int it, C2<T>* a, C2<T>* b) {
-          scatter(fft_lines<T, -1>(a, b, lgy, nl, twy), it / per_kx, (it % per_kx) * zs);
-        });
-  }
-  // ---- y pass, inverse: S2 -> S1 ----
-  __device__ __noinline__ void yinv() {
-    const int ny = this->ny, nz = this->nz, lgy = this->lgy, nkx = this->nkx, zs = this->zs;
-    const long long nspec = this->nspec;
-    C2<T>* const S1 = this->S1;
-    C2<T>* const S2 = this->S2;
-    const C2<T>* const twy = this->twy;
-    const int per_kx = nz / zs;
-    const int nl = 3 * zs;
-    pipelined(nkx * per_kx,
-        [=](int it, C2<T>* buf) {
-          const int kx = it / per_kx, z0 = (it % per_kx) * zs;
-          gather_async<T>(buf, S2, nl << lgy,
-              [=](int e) {
-                const int dz = e % zs, rest = e / zs;
-                const int ky = rest & (ny - 1), c = rest >> lgy;
-                return c * nspec + ((long long)kx * ny + ky) * nz + z0 + dz;
-              },
-              [=](int e) {
-                const int dz = e % zs, rest = e / zs;
-                const int ky = rest & (ny - 1), c = rest >> lgy;
-                return ((c * zs + dz) << lgy) + ky;
-              });
-        },
-        [=](int it, C2<T>* a, C2<T>* b) {
-          const int kx = it / per_kx, z0 = (it % per_kx) * zs;
-          const C2<T>* X = fft_lines<T, +1>(a, b, lgy, nl, twy);
-          for (int e = threadIdx.x; e < (nl << lgy); e += NT) {
-            const int l = e >> lgy, y = e & (ny - 1);
-            const int c = l / zs, dz = l - c * zs;
-            S1[c * nspec + ((long long)(z0 + dz) * nkx + kx) * ny + y] = X[sp(e)];
+      core_fft_n<-1, 3>(v, t);
+      const V kxv = vset(kxo, (V*)nullptr), nkxv = vneg(kxv), nky = vneg(ky);
+      const T sc = op == OP3_CURLNEG ? -scale : scale;
+#pragma unroll
+      for (int j = 0; j < E; ++j) {
+        const int kz = t.i + j * q;
+        const T kz1 = ldg_tab(&ktab[nkx + ny + kz]);
+        const V kzv = vset(kz == (nz >> 1) ? (T)0 : kz1, (V*)nullptr), nkz = vneg(kzv);
+        V f;
+        if (op == OP3_PHI) {                                 // Eq. 17
+          const V k2 = vfma(vset(kz1, (V*)nullptr), vset(kz1, (V*)nullptr), ky2);
+          if constexpr (sizeof(T) == 4) {
+            float a, b;
+            upk(k2, a, b);
+            f = pk(inv(a) * sc, inv(b) * sc);
+          } else {
+            f = inv(k2) * sc;
           }
-          __syncthreads();
-        });
-  }
-  // ---- z pass: forward, 3x3 multiplier, inverse on lines (kx, ky0 .. ky0 + P) ----
-  __device__ __noinline__ void zpass(int op) {
-    const int ny = this->ny, nz = this->nz, lgz = this->lgz, nkx = this->nkx, half = this->half, P = this->P;
-    const long long nspec = this->nspec, ncell = this->ncell;
-    C2<T>* const S2 = this->S2;
-    const C2<T>* const twz = this->twz;
-    const T* const ktab = this->ktab;
-    const T* const gtab = this->gtab;
-    const int per_kx = ny / P;
-    const T s = (T)1 / (T)ncell;
-    const int pl = P << lgz;                         // values per component
-    // multiplier, inverse transform and write of an item whose forward transform is in X (Y:
-    // the other buffer)
-    auto finish = [=](C2<T>* X, C2<T>* Y, int kx, int ky0) {
-      const long long base = ((long long)kx * ny + ky0) * nz;
-      const T kxv = ldg_tab(&ktab[kx]), gx = ldg_tab(&gtab[kx]);
-      const T kxo = kx == half ? (T)0 : kxv;
-      for (int e = threadIdx.x; e < pl; e += NT) {
-        const int p = e >> lgz, kz = e & (nz - 1);
-        const int ky = ky0 + p;
-        const T kyv = ldg_tab(&ktab[nkx + ky]), kzv = ldg_tab(&ktab[nkx + ny + kz]);
-        const T kyo = ky == ny / 2 ? (T)0 : kyv;
-        const T kzo = kz == nz / 2 ? (T)0 : kzv;
-        const C2<T> va = X[sp(e)], vb = X[sp(pl + e)], vc = X[sp(2 * pl + e)];
-        // cross product k x v with the odd (Nyquist-free) wavenumbers
-        C2<T> cx = {kyo * vc.x - kzo * vb.x, kyo * vc.y - kzo * vb.y};
-        C2<T> cy = {kzo * va.x - kxo * vc.x, kzo * va.y - kxo * vc.y};
-        C2<T> cz = {kxo * vb.x - kyo * va.x, kxo * vb.y - kyo * va.y};
-        T f;
-        if (op == OP3_PHI) {
-          const T k2 = kxv * kxv + kyv * kyv + kzv * kzv;
-          f = k2 > (T)0 ? s / k2 : (T)0;                   // Eq. 17
-        } else {
-          const T G = gx * ldg_tab(&gtab[nkx + ky]) * ldg_tab(&gtab[nkx + ny + kz]);
-          f = (op == OP3_CURL ? G : -G) * s;               // smoothed curl
+        } else {                                             // smoothed curl
+          f = vmul(gxy, vset(ldg_tab(&gtab[nkx + ny + kz]) * sc, (V*)nullptr));
         }
-        X[sp(e)] = cmul_si(cscale(cx, f), 1);
-        X[sp(pl + e)] = cmul_si(cscale(cy, f), 1);
-        X[sp(2 * pl + e)] = cmul_si(cscale(cz, f), 1);
+        // i f (k x v)
+        const CV<V> a = v[0][j], b = v[1][j], c = v[2][j];
+        const CV<V> x = {vfma(ky, c.x, vmul(nkz, b.x)), vfma(ky, c.y, vmul(nkz, b.y))};
+        const CV<V> yv = {vfma(kzv, a.x, vmul(nkxv, c.x)), vfma(kzv, a.y, vmul(nkxv, c.y))};
+        const CV<V> z = {vfma(kxv, b.x, vmul(nky, a.x)), vfma(kxv, b.y, vmul(nky, a.y))};
+        const V nf = vneg(f);
+        v[0][j] = {vmul(x.y, nf), vmul(x.x, f)};
+        v[1][j] = {vmul(yv.y, nf), vmul(yv.x, f)};
+        v[2][j] = {vmul(z.y, nf), vmul(z.x, f)};
       }
-      __syncthreads();
-      const C2<T>* Z = fft_lines<T, +1>(X, Y, lgz, 3 * P, twz);
-      for (int e = threadIdx.x; e < 3 * pl; e += NT) {
-        const int c = e / pl, r = e - c * pl;
-        S2[c * nspec + base + r] = Z[sp(e)];
+      core_fft_n<+1, 3>(v, t);
+      if (mine) {
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+#pragma unroll
+          for (int j = 0; j < E; ++j) st_z(p + c * nspec + j * q * zs, v[c][j]);
+        }
       }
-      __syncthreads();
-    };
-    if (lgz >= TMA_MIN_LG) {
-      tma_lines(nkx * per_kx, 3 * P, lgz,
-          [=](int it, int l) {
-            const int kx = it / per_kx, ky0 = (it % per_kx) * P;
-            const int c = l / P, p = l - c * P;
-            return (const C2<T>*)(S2 + c * nspec + ((long long)kx * ny + ky0 + p) * nz);
-          },
-          [&](int it, auto after_first) {
-            first_from_stage<-1>(lgz, 3 * P, sm, after_first);
-            C2<T>* X = fft_lines_from<T, -1>(sm, sm2, lgz, 3 * P, twz, 1);
-            finish(X, X == sm ? sm2 : sm, it / per_kx, (it % per_kx) * P);
-          });
-      return;
     }
-    pipelined(nkx * per_kx,
-        [=](int it, C2<T>* buf) {
-          const long long base = ((long long)(it / per_kx) * ny + (it % per_kx) * P) * nz;
-          gather_async<T>(buf, S2, 3 * pl,
-              [=](int e) { const int c = e / pl; return c * nspec + base + (e - c * pl); },
-              [](int e) { return e; });
-        },
-        [=](int it, C2<T>* a, C2<T>* b) {
-          C2<T>* X = fft_lines<T, -1>(a, b, lgz, 3 * P, twz);
-          finish(X, X == a ? b : a, it / per_kx, (it % per_kx) * P);
-        });
+  }
+  __device__ __forceinline__ void zpass(int op) {
+    if constexpr (sizeof(T) == 8) {
+      if (ez == 2) { zpass_e<2>(op); return; }
+    }
+    zpass_e<4>(op);
   }
 
   // Yf, Z(op), Yi with barriers; the x passes before and after are separate
   __device__ bool yzy(int op, int where) {
-    yfwd();
+    ypass<-1>();
     if (!sync(where)) return false;
     zpass(op);
     if (!sync(where + 1)) return false;
-    yinv();
+    ypass<+1>();
     return sync(where + 2);
   }
 };
 
 // ------------------------------------------------------------------------------------------
-// epilogues of the x pass (cell index i, three components in / out)
+// Epilogues of the x pass.  load(c, i, r) reads what the RU rows of one element of component c need (i:
+// the component's 16-byte vector, r: the row-major cell of the first row, the others nx apart);
+// apply(ld, c, j, i, r, in, out) works on the thread's element j; done(i, q) follows the last component
+// (element j's vector is i + j q); reset() starts a unit.  Joint ones take the three components at once.
 // ------------------------------------------------------------------------------------------
-// Stage state y + sum c_j k_j.  With a field-dependent critical current (kim) the stage
-// field's magnitude |h| is kept, in the transform precision, in the first component of the
-// h_dot iterate at superconductor cells: those entries are rewritten by BInit before anything
-// reads them as an iterate, and the warm start lives on free space only.
-template <typename T>
-struct BStage : EpiBase<T> {
+template <typename T, int NS = 1, bool MAX = false>
+struct BEpi {
   BulkPtrs<T> P;
+  static constexpr int RU = Lane<T>::RU, kSums = NS, kBatch = 4;
+  static constexpr bool kJoint = false, kMax = MAX;
+  T acc[NS];
+  __device__ __forceinline__ void reset() {
+#pragma unroll
+    for (int k = 0; k < NS; ++k) acc[k] = 0;
+  }
+  __device__ __forceinline__ void done(long long, int) {}
+  __device__ __forceinline__ int msk(long long i) const { return ld_mask(P.mask + i); }
+};
+
+// Stage state y + sum c_j k_j.  With a field-dependent critical current (KIM) the stage field's
+// magnitude |h| is kept, in the transform precision, in the first component of the h_dot iterate at
+// superconductor cells: those entries are rewritten by BInit before anything reads them as an iterate,
+// and the warm start lives on free space only.
+template <typename T, int E, bool KIM>
+struct BStageT : BEpi<T> {
+  static constexpr int RU = Lane<T>::RU, kBatch = 2;
   StageIn in;
-  bool kim;
-  __device__ void operator()(long long i, const T*, T* out) {
-    // every load of the cell before its first store (a store could alias a later load as far
-    // as the compiler knows, which would put each load behind the previous store)
-    double v[3];
+  double h2[KIM ? E : 1][RU];
+  struct Ld { double v[RU]; };
+  __device__ __forceinline__ Ld load(int c, long long, long long r) const {
+    Ld l;
+    const long long o = c * this->P.ncell + r;
 #pragma unroll
-    for (int c = 0; c < 3; ++c) v[c] = in.y[c * P.ncell + i];
+    for (int q = 0; q < RU; ++q) l.v[q] = ld_s(in.y + o + (long long)q * this->P.nx);
     for (int j = 0; j < in.nk; ++j) {
+      double k[RU];
 #pragma unroll
-      for (int c = 0; c < 3; ++c) v[c] += in.c[j] * in.k[j][c * P.ncell + i];
-    }
-    double h2 = 0.0;
+      for (int q = 0; q < RU; ++q) k[q] = ld_s(in.k[j] + o + (long long)q * this->P.nx);
 #pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      if (in.ynew) in.ynew[c * P.ncell + i] = v[c];
-      out[c] = (T)v[c];
-      h2 += v[c] * v[c];
+      for (int q = 0; q < RU; ++q) l.v[q] += in.c[j] * k[q];
     }
-    if (kim && __ldg(&P.mask[i]) == 1) P.hd[i] = (T)sqrt(h2);
+    return l;
   }
-};
-
-// local law of the superconductor: critical current (Kim-type jc / (1 + |h|/b0) when ib0 > 0,
-// |h| left by BStage) and the elliptic weight a = 1/gamma^2 of j_z
-template <typename T>
-__device__ __forceinline__ T bulk_jc(const BulkPtrs<T>& P, long long i, int m, T jc, T ib0) {
-  T jcl = P.jcmap ? __ldg(&P.jcmap[i]) : jc;
-  if (ib0 > (T)0 && m == 1) jcl = jcl / ((T)1 + P.hd[i] * ib0);
-  return jcl;
-}
-
-template <typename T>
-struct BPower : EpiBase<T> {               // j -> e (Eq. 13 / Ohm law; elliptic and Kim laws)
-  BulkPtrs<T> P;
-  T n, e0, jc, rho_out, ig2, ib0;
-  __device__ void operator()(long long i, const T* in, T* out) {
-    const int m = __ldg(&P.mask[i]);
-    const T jcl = bulk_jc(P, i, m, jc, ib0);
-    const T a = m == 1 ? ig2 : (T)1;
-    const T rho = resistivity<T>(in[0] * in[0] + in[1] * in[1] + in[2] * in[2] * a, jcl, m, n, e0, rho_out);
-    out[0] = rho * in[0]; out[1] = rho * in[1]; out[2] = rho * in[2] * a;
-  }
-};
-
-template <typename T>
-struct BInit : EpiBase<T> {                // h_dot^0: h_dot_in on the conductor, warm or h_e_dot outside
-  BulkPtrs<T> P;
-  bool warm;
-  T hed[3];
-  static constexpr bool kPair = true;
-  __device__ __forceinline__ void pair(long long ia, long long ib, const T* ina, const T* inb, T* oa, T* ob) {
-    const bool ca = __ldg(&P.mask[ia]) != 0, cb = __ldg(&P.mask[ib]) != 0;
-    T wa[3], wb[3];
+  __device__ __forceinline__ void apply(const Ld& l, int c, int j, long long, long long r, const Q<T>&, Q<T>& out) {
 #pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      wa[c] = (!ca && warm) ? P.hd[c * P.ncell + ia] : hed[c];
-      wb[c] = (!cb && warm) ? P.hd[c * P.ncell + ib] : hed[c];
-    }
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      oa[c] = ca ? ina[c] : wa[c];                         // -curl e (Eq. 14) on the conductor
-      ob[c] = cb ? inb[c] : wb[c];
-    }
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      P.hd[c * P.ncell + ia] = oa[c];
-      P.hd[c * P.ncell + ib] = ob[c];
+    for (int q = 0; q < RU; ++q) {
+      if (in.ynew) in.ynew[c * this->P.ncell + r + (long long)q * this->P.nx] = l.v[q];
+      out.v[q] = (T)l.v[q];
+      if constexpr (KIM) h2[j][q] = l.v[q] * l.v[q] + (c == 0 ? 0.0 : h2[j][q]);
     }
   }
-};
-
-template <typename T>
-struct BMaskCond : EpiBase<T> {            // j_dot_in: keep on the conductor only
-  BulkPtrs<T> P;
-  __device__ void operator()(long long i, const T* in, T* out) {
-    const bool cond = __ldg(&P.mask[i]) != 0;
-    out[0] = cond ? in[0] : (T)0; out[1] = cond ? in[1] : (T)0; out[2] = cond ? in[2] : (T)0;
-  }
-};
-
-template <typename T>
-struct BUpdate : EpiBase<T, T> {           // Eq. 18 on free space, residual, forward
-  BulkPtrs<T> P;
-  T hed[3];
-  static constexpr bool kPair = true;
-  __device__ __forceinline__ void pair(long long ia, long long ib, const T* ina, const T* inb, T* oa, T* ob) {
-    const bool fa = __ldg(&P.mask[ia]) == 0, fb = __ldg(&P.mask[ib]) == 0;
-    T ha[3], hb[3];
+  __device__ __forceinline__ void done(long long i, int q) {
+    if constexpr (KIM) {
 #pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      ha[c] = P.hd[c * P.ncell + ia];
-      hb[c] = P.hd[c * P.ncell + ib];
-    }
-    T sa = 0, sb = 0;
+      for (int j = 0; j < E; ++j) {
+        const int m = this->msk(i + (long long)j * q);
 #pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      const T na = hed[c] + ina[c], nb = hed[c] + inb[c];
-      sa += (na - ha[c]) * (na - ha[c]);
-      sb += (nb - hb[c]) * (nb - hb[c]);
-      oa[c] = fa ? na : ha[c];
-      ob[c] = fb ? nb : hb[c];
-    }
-    if (fa) this->acc += sqrt(sa);
-    if (fb) this->acc += sqrt(sb);
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      if (fa) P.hd[c * P.ncell + ia] = oa[c];
-      if (fb) P.hd[c * P.ncell + ib] = ob[c];
-    }
-  }
-};
-
-template <typename T>
-struct BFinal : EpiBase<T> {               // h_dot out (FP64); optional BS23 error contribution
-  BulkPtrs<T> P;
-  double* kout;
-  bool err;
-  double h, rtol, atol;
-  const double* k1; const double* k2; const double* k3; const double* y; const double* ynew;
-  __device__ void operator()(long long i, const T*, T*) {
-    double g[3];                                             // loads before the stores (see BStage)
-#pragma unroll
-    for (int c = 0; c < 3; ++c) g[c] = (double)P.hd[c * P.ncell + i];
-#pragma unroll
-    for (int c = 0; c < 3; ++c) kout[c * P.ncell + i] = g[c];
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      const long long k = c * P.ncell + i;
-      if (err) {
-        const double E = h * (-5.0 / 72.0 * k1[k] + 1.0 / 12.0 * k2[k] + 1.0 / 9.0 * k3[k] - 0.125 * g[c]);
-        const double sc = atol + rtol * fmax(fabs(y[k]), fabs(ynew[k]));
-        double q;                                            // the ratio in the transform precision
-        if constexpr (sizeof(T) == 4) q = (double)__fdiv_rn((float)fabs(E), (float)sc);
-        else q = fabs(E) / sc;
-        if (!(q == q) || isinf(q)) q = 1e300;
-        this->accmax = fmax(this->accmax, q);
-      } else if (!isfinite(g[c])) {
-        this->accmax = 1.0;
+        for (int w = 0; w < RU; ++w)
+          if (cls(m, w) == 1) this->P.hd[(i + (long long)j * q) * RU + w] = (T)sqrt(h2[j][w]);
       }
     }
   }
 };
+template <typename T, int E> using BStage = BStageT<T, E, false>;
+template <typename T, int E> using BStageKim = BStageT<T, E, true>;
 
+// j -> e (Eq. 13 / Ohm law): critical current jc, per cell or Kim-type jc / (1 + |h|/b0) when ib0 > 0
+// (|h| left by BStageKim), and the elliptic weight 1/gamma^2 of j_z
 template <typename T>
-struct BStoreJ : EpiBase<T> {              // readout of j = curl h (FP64)
-  BulkPtrs<T> P;
-  double* out;
-  __device__ void operator()(long long i, const T* in, T*) {
-    out[i] = in[0]; out[P.ncell + i] = in[1]; out[2 * P.ncell + i] = in[2];
-  }
-};
-
-template <typename T>
-struct BStoreE : EpiBase<T> {              // readout of e, the law of BPower (FP64)
-  BulkPtrs<T> P;
+struct BLaw : BEpi<T> {
+  static constexpr int RU = Lane<T>::RU, kBatch = 2;
+  static constexpr bool kJoint = true;
   T n, e0, jc, rho_out, ig2, ib0;
+  struct Ld { int m; Q<T> jc, h; };
+  __device__ __forceinline__ Ld load(long long i, long long) const {
+    Ld l;
+    l.m = this->msk(i);
+    if (this->P.jcmap) {
+      l.jc = ldg_q(this->P.jcmap + i * RU);
+    } else {
+#pragma unroll
+      for (int q = 0; q < RU; ++q) l.jc.v[q] = jc;
+    }
+    if (ib0 > (T)0) l.h = ld_q(this->P.hd + i * RU);
+    return l;
+  }
+  __device__ __forceinline__ void law(const Ld& l, const Q<T>* in, Q<T>* e) const {
+#pragma unroll
+    for (int q = 0; q < RU; ++q) {
+      const int m = cls(l.m, q);
+      T jcl = l.jc.v[q];
+      if (ib0 > (T)0 && m == 1) jcl = jcl / ((T)1 + l.h.v[q] * ib0);
+      const T a = m == 1 ? ig2 : (T)1;
+      const T x = in[0].v[q], y = in[1].v[q], z = in[2].v[q];
+      const T rho = resistivity<T>(x * x + y * y + z * z * a, jcl, m, n, e0, rho_out);
+      e[0].v[q] = rho * x; e[1].v[q] = rho * y; e[2].v[q] = rho * z * a;
+    }
+  }
+};
+template <typename T, int E>
+struct BPower : BLaw<T> {
+  using Ld = typename BLaw<T>::Ld;
+  __device__ __forceinline__ void apply(const Ld& l, int, int, long long, const Q<T>* in, Q<T>* out) { this->law(l, in, out); }
+};
+template <typename T, int E>
+struct BStoreE : BLaw<T> {                 // readout of e (FP64)
+  using Ld = typename BLaw<T>::Ld;
   double* out;
-  __device__ void operator()(long long i, const T* in, T*) {
-    const int m = __ldg(&P.mask[i]);
-    const T jcl = bulk_jc(P, i, m, jc, ib0);
-    const T a = m == 1 ? ig2 : (T)1;
-    const T rho = resistivity<T>(in[0] * in[0] + in[1] * in[1] + in[2] * in[2] * a, jcl, m, n, e0, rho_out);
-    out[i] = rho * in[0]; out[P.ncell + i] = rho * in[1]; out[2 * P.ncell + i] = rho * in[2] * a;
+  __device__ __forceinline__ void apply(const Ld& l, int, int, long long r, const Q<T>* in, Q<T>*) {
+    Q<T> e[3];
+    this->law(l, in, e);
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+#pragma unroll
+      for (int q = 0; q < Lane<T>::RU; ++q) out[c * this->P.ncell + r + (long long)q * this->P.nx] = e[c].v[q];
+    }
   }
 };
 
-template <typename T>
-struct BMoment : EpiBase<T> {              // m = 1/2 sum dV r x j over the conductor, component `comp`
-  BulkPtrs<T> P;
-  int comp;
-  __device__ void operator()(long long i, const T* in, T*) {
-    if (__ldg(&P.mask[i]) == 0) return;
-    const int x = (int)(i % P.nx), y = (int)((i / P.nx) % P.ny), z = (int)(i / ((long long)P.nx * P.ny));
-    const double rx = -P.Lx + (x + 0.5) * P.dx;
-    const double ry = -P.Ly + (y + 0.5) * P.dy;
-    const double rz = -P.Lz + (z + 0.5) * P.dz;
-    double v;
-    if (comp == 0) v = ry * in[2] - rz * in[1];
-    else if (comp == 1) v = rz * in[0] - rx * in[2];
-    else v = rx * in[1] - ry * in[0];
-    this->acc += v;
+template <typename T, int E>
+struct BInit : BEpi<T> {                   // h_dot^0: h_dot_in on the conductor, warm or h_e_dot outside
+  static constexpr int RU = Lane<T>::RU;
+  bool warm;
+  T hed[3];
+  struct Ld { int m; Q<T> w; };
+  __device__ __forceinline__ Ld load(int c, long long i, long long) const {
+    Ld l;
+    l.m = this->msk(i);
+    if (warm) l.w = ld_q(this->P.hd + (c * this->P.ncell + i * RU));
+    return l;
+  }
+  __device__ __forceinline__ void apply(const Ld& l, int c, int, long long i, long long, const Q<T>& in, Q<T>& out) {
+    const T he = c == 0 ? hed[0] : c == 1 ? hed[1] : hed[2];
+#pragma unroll
+    for (int q = 0; q < RU; ++q) out.v[q] = cls(l.m, q) != 0 ? in.v[q] : warm ? l.w.v[q] : he;   // -curl e (Eq. 14)
+    st_q(this->P.hd + (c * this->P.ncell + i * RU), out);
+  }
+};
+
+template <typename T, int E>
+struct BMaskCond : BEpi<T> {               // j_dot_in: keep on the conductor only
+  struct Ld { int m; };
+  __device__ __forceinline__ Ld load(int, long long i, long long) const { return Ld{this->msk(i)}; }
+  __device__ __forceinline__ void apply(const Ld& l, int, int, long long, long long, const Q<T>& in, Q<T>& out) {
+#pragma unroll
+    for (int q = 0; q < Lane<T>::RU; ++q) out.v[q] = cls(l.m, q) != 0 ? in.v[q] : (T)0;
+  }
+};
+
+template <typename T, int E>
+struct BUpdate : BEpi<T> {                 // Eq. 18 on free space, residual, forward
+  static constexpr int RU = Lane<T>::RU, kBatch = 2;
+  T hed[3];
+  T s[E][RU];                              // |h_dot^{i+1} - h_dot^i|^2 of the thread's cells, over the components
+  struct Ld { int m; Q<T> h; };
+  __device__ __forceinline__ Ld load(int c, long long i, long long) const {
+    return Ld{this->msk(i), ld_q(this->P.hd + (c * this->P.ncell + i * RU))};
+  }
+  __device__ __forceinline__ void apply(const Ld& l, int c, int j, long long i, long long, const Q<T>& in, Q<T>& out) {
+    const T he = c == 0 ? hed[0] : c == 1 ? hed[1] : hed[2];
+    out = l.h;
+    bool any = false;
+#pragma unroll
+    for (int q = 0; q < RU; ++q) {
+      T e = (T)0;
+      if (cls(l.m, q) == 0) {
+        const T n = he + in.v[q];
+        e = n - l.h.v[q];
+        out.v[q] = n;
+        any = true;
+      }
+      s[j][q] = c == 0 ? e * e : s[j][q] + e * e;
+    }
+    if (any) st_q(this->P.hd + (c * this->P.ncell + i * RU), out);
+  }
+  __device__ __forceinline__ void done(long long, int) {
+#pragma unroll
+    for (int j = 0; j < E; ++j) {
+#pragma unroll
+      for (int q = 0; q < RU; ++q) this->acc[0] += sqrt(s[j][q]);
+    }
+  }
+};
+
+template <typename T, int E, bool err>
+struct BFinalT : BEpi<T, 1, true> {        // h_dot out (FP64); optional BS23 error contribution
+  static constexpr int RU = Lane<T>::RU, NE = err ? RU : 1, kBatch = err ? 1 : 4;
+  double* kout;
+  double h, rtol, atol;
+  const double* k1; const double* k2; const double* k3; const double* y; const double* ynew;
+  struct Ld { Q<T> g; double a1[NE], a2[NE], a3[NE], y[NE], yn[NE]; };
+  __device__ __forceinline__ Ld load(int c, long long i, long long r) const {
+    Ld l;
+    l.g = ld_q(this->P.hd + (c * this->P.ncell + i * RU));
+    if constexpr (err) {
+#pragma unroll
+      for (int q = 0; q < RU; ++q) {
+        const long long o = c * this->P.ncell + r + (long long)q * this->P.nx;
+        l.a1[q] = ld_s(k1 + o); l.a2[q] = ld_s(k2 + o); l.a3[q] = ld_s(k3 + o);
+        l.y[q] = ld_s(y + o); l.yn[q] = ld_s(ynew + o);
+      }
+    }
+    return l;
+  }
+  __device__ __forceinline__ void apply(const Ld& l, int c, int, long long, long long r, const Q<T>&, Q<T>&) {
+#pragma unroll
+    for (int q = 0; q < RU; ++q) {
+      const double g = (double)l.g.v[q];
+      kout[c * this->P.ncell + r + (long long)q * this->P.nx] = g;
+      if constexpr (err) {
+        const double E_ = h * (-5.0 / 72.0 * l.a1[q] + 1.0 / 12.0 * l.a2[q] + 1.0 / 9.0 * l.a3[q] - 0.125 * g);
+        const double sc = atol + rtol * fmax(fabs(l.y[q]), fabs(l.yn[q]));
+        T e;                                                 // the ratio in the transform precision
+        if constexpr (sizeof(T) == 4) e = __fdiv_rn((float)fabs(E_), (float)sc);
+        else e = fabs(E_) / sc;
+        if (!(e == e)) e = (T)INFINITY;                      // non-finite -> rejected step
+        this->acc[0] = this->acc[0] > e ? this->acc[0] : e;
+      } else if (!isfinite(l.g.v[q])) {
+        this->acc[0] = (T)1;
+      }
+    }
+  }
+};
+template <typename T, int E> using BFinal = BFinalT<T, E, false>;
+template <typename T, int E> using BFinalErr = BFinalT<T, E, true>;
+
+template <typename T, int E>
+struct BStoreJ : BEpi<T> {                 // readout of j = curl h (FP64)
+  double* out;
+  using Ld = NoLd;
+  __device__ __forceinline__ Ld load(int, long long, long long) const { return Ld{}; }
+  __device__ __forceinline__ void apply(const Ld&, int c, int, long long, long long r, const Q<T>& in, Q<T>&) {
+#pragma unroll
+    for (int q = 0; q < Lane<T>::RU; ++q) out[c * this->P.ncell + r + (long long)q * this->P.nx] = in.v[q];
+  }
+};
+
+template <typename T, int E>
+struct BMoment : BEpi<T, 3> {              // m = 1/2 sum dV r x j over the conductor
+  static constexpr int RU = Lane<T>::RU, kBatch = 2;
+  static constexpr bool kJoint = true;
+  double acc[3];
+  double Lx, Ly, Lz, dx, dy, dz;
+  struct Ld { int m; };
+  __device__ __forceinline__ void reset() { acc[0] = acc[1] = acc[2] = 0.0; }
+  __device__ __forceinline__ Ld load(long long i, long long) const { return Ld{this->msk(i)}; }
+  __device__ __forceinline__ void apply(const Ld& l, int x, int unit, long long, const Q<T>* in, Q<T>*) {
+    if (l.m == 0) return;
+    const int row = unit * RU, z = row / this->P.ny, y0 = row - z * this->P.ny;
+    const double rx = -Lx + (x + 0.5) * dx, rz = -Lz + (z + 0.5) * dz;
+#pragma unroll
+    for (int q = 0; q < RU; ++q) {
+      if (cls(l.m, q) == 0) continue;
+      const double ry = -Ly + (y0 + q + 0.5) * dy;
+      const double jx = in[0].v[q], jy = in[1].v[q], jz = in[2].v[q];
+      acc[0] += ry * jz - rz * jy;
+      acc[1] += rz * jx - rx * jz;
+      acc[2] += rx * jy - ry * jx;
+    }
   }
 };
 
@@ -607,68 +690,80 @@ __device__ __noinline__ RhsOut bulk_rhs(Bulk<T>& B, double t, int seg, const Sta
                                         const double* e_k2, const double* e_k3, const double* e_y,
                                         const double* e_ynew) {
   const Desc& d = B.d;
+  Shared& sh = B.sh;
   RhsOut res{ST_OK, 0, 0.0, 0.0, 0};
-  const double hs = he_dot(d, t, seg);
-  const double hed[3] = {hs * d.he_dir[0], hs * d.he_dir[1], hs * d.he_dir[2]};
-  const double hed_norm = sqrt(hed[0] * hed[0] + hed[1] * hed[1] + hed[2] * hed[2]);
+  if (threadIdx.x == 0) {               // scalar FP64 work: one thread (see Control)
+    const double hs = he_dot(d, t, seg);
+    double n2 = 0.0;
+    for (int c = 0; c < 3; ++c) {
+      sh.hed3[c] = hs * d.he_dir[c];
+      sh.hed3f[c] = (float)sh.hed3[c];
+      n2 += sh.hed3[c] * sh.hed3[c];
+    }
+    sh.thresh = d.iter_tol * fmax(sqrt(n2), 1.0);
+    sh.r = 0.0;
+  }
+  auto hed = [&](T* e) {
+    for (int c = 0; c < 3; ++c) {
+      if constexpr (sizeof(T) == 4) e[c] = sh.hed3f[c];
+      else e[c] = sh.hed3[c];
+    }
+  };
 #define BSYNC(w) if (!B.sync(w)) { res.status = ST_BARRIER; return res; }
 #define BYZY(op, w) if (!B.yzy(op, w)) { res.status = ST_BARRIER; return res; }
-  { BStage<T> e; e.P = B.ptrs(); e.in = sin; e.kim = d.b0 > 0.0; B.xpass<0, 3>(e, -1); }
+  if (d.b0 > 0.0) B.template xpass<BStageKim, false, true>([&](auto& e) { e.in = sin; });
+  else B.template xpass<BStage, false, true>([&](auto& e) { e.in = sin; });
   BSYNC(101);
   BYZY(OP3_CURL, 102);                                                   // j = curl h
-  {
-    BPower<T> e; e.P = B.ptrs(); e.n = (T)d.n; e.e0 = (T)d.e0; e.jc = (T)d.jc; e.rho_out = (T)d.rho_out;
-    e.ig2 = (T)(1.0 / (d.gamma * d.gamma)); e.ib0 = d.b0 > 0.0 ? (T)(1.0 / d.b0) : (T)0;
-    B.xpass<3, 3>(e, -1);                                                // e = rho j
-  }
+  B.template xpass<BPower, true, true>([&](auto& e) { B.law(e); });      // e = rho j
   BSYNC(105);
   BYZY(OP3_CURLNEG, 106);                                                // -curl e
-  {
-    BInit<T> e; e.P = B.ptrs(); e.warm = B.sh.warm_valid != 0;
-    for (int c = 0; c < 3; ++c) e.hed[c] = (T)hed[c];
-    B.xpass<3, 3>(e, -1);                                                // h_dot^0
-  }
+  B.template xpass<BInit, true, true>([&](auto& e) { e.warm = sh.warm_valid != 0; hed(e.hed); });   // h_dot^0
   BSYNC(109);
   const bool have_out = d.nout > 0;
-  const double thresh = d.iter_tol * fmax(hed_norm, 1.0);
-  const bool forced = force_iters > 0;
-  const bool fixed = d.iter_tol <= 0.0;
-  const int itmax = forced ? force_iters : d.iter_max;
-  double r = 0.0;
+  const bool by_count = force_iters > 0 || d.iter_tol <= 0.0;
+  const int itmax = force_iters > 0 ? force_iters : d.iter_max;
   int i = 0;
   if (have_out) {
     for (; i < itmax; ++i) {
       BYZY(OP3_CURL, 110);                                               // j_dot = curl h_dot
-      { BMaskCond<T> e; e.P = B.ptrs(); B.xpass<3, 3>(e, -1); }                // j_dot_in
+      B.template xpass<BMaskCond, true, true>([&](auto&) {});            // j_dot_in
       BSYNC(113);
       BYZY(OP3_PHI, 114);                                                // Phi[j_dot_in]
-      {
-        BUpdate<T> e; e.P = B.ptrs();
-        for (int c = 0; c < 3; ++c) e.hed[c] = (T)hed[c];
-        B.xpass<3, 3>(e, 0);                                             // Eq. 18
-      }
+      B.template xpass<BUpdate, true, true>([&](auto& e) { hed(e.hed); }, 0);   // Eq. 18
       BSYNC(117);
-      r = B.total(0) / (double)d.nout;
-      if (!(forced || fixed) && r < thresh) { ++i; break; }
+      const double s = B.total(0);
+      if (threadIdx.x == 0) {
+        sh.r = s * sh.inv_nout;
+        sh.stop = !by_count && sh.r < sh.thresh;
+      }
+      __syncthreads();
+      if (sh.stop) { ++i; break; }
     }
     if (i > itmax) i = itmax;
   }
   res.iters = i;
-  res.r = r;
-  res.status = (!have_out || fixed || r < thresh) ? ST_OK : ST_NOCONV;
-  // a call that failed with a residual above 1e3 times the threshold (or not finite) diverged:
-  // the next call starts cold
-  B.sh.warm_valid = (res.status == ST_NOCONV && !(r < 1e3 * thresh)) ? 0 : 1;
+  if (threadIdx.x == 0) {
+    const double r = sh.r;
+    sh.ok = !have_out || d.iter_tol <= 0.0 || r < sh.thresh;
+    // a call that failed with a residual above 1e3 times the threshold (or not finite) diverged:
+    // the next call starts cold
+    sh.warm_valid = !sh.ok && !(r < 1e3 * sh.thresh) ? 0 : 1;
+  }
   {
-    BFinal<T> e; e.P = B.ptrs(); e.kout = kout; e.is_max = true;
-    e.err = want_err; e.h = h_err; e.rtol = d.rtol; e.atol = d.atol;
-    e.k1 = e_k1; e.k2 = e_k2; e.k3 = e_k3; e.y = e_y; e.ynew = e_ynew;
-    B.xpass<0, 0>(e, 3);
+    auto fill = [&](auto& e) {
+      e.kout = kout; e.h = h_err; e.rtol = d.rtol; e.atol = d.atol;
+      e.k1 = e_k1; e.k2 = e_k2; e.k3 = e_k3; e.y = e_y; e.ynew = e_ynew;
+    };
+    if (want_err) B.template xpass<BFinalErr, false, false>(fill, 3);
+    else B.template xpass<BFinal, false, false>(fill, 3);
   }
   BSYNC(120);
+  res.status = sh.ok ? ST_OK : ST_NOCONV;
+  res.r = sh.r;
   const double q = B.total(3, true);
-  if (want_err) res.err = q;
-  else res.nonfinite = q > 0.0;
+  if (want_err) res.err = isinf(q) ? 1e300 : q;
+  else res.nonfinite = __double_as_longlong(q) > 0;
 #undef BSYNC
 #undef BYZY
   return res;
@@ -688,7 +783,6 @@ struct BulkRhs {
 
 template <typename T>
 __global__ void __launch_bounds__(NT, 2) bulk_kernel(const Desc* __restrict__ dg, KernelArgs a) {
-  C2<T>* sm = dsm<T>();
   __shared__ Shared sh;
   // one copy of the pass object per CTA, in shared memory: its members are read as broadcasts
   // instead of per-thread local-memory copies
@@ -699,10 +793,19 @@ __global__ void __launch_bounds__(NT, 2) bulk_kernel(const Desc* __restrict__ dg
     sh.warm_valid = st->warm_valid;
     sh.bar_passed = 0;
     sh.A_prev = 0.0;
-    sh.tma_parity = 0;
-    mbar_init(&sh.tma_bar);
+    new (objraw) Bulk<T>(d, mf_dsmem, sh);
   }
-  if (threadIdx.x == 0) new (objraw) Bulk<T>(d, sm, sh);
+  {
+    // the twiddle tables, behind the exchange buffer (see film_tables)
+    uint4* to = (uint4*)mf_dsmem + bulk_slots(d);
+    auto copy = [&](const void* tab, int n) {
+      for (int k = threadIdx.x; k < n; k += NT) to[k] = ((const uint4*)tab)[k];
+      to += n;
+    };
+    copy(d.tw_x, core_table_len(d.lgx, d.ex));
+    copy(d.tw_y, core_table_len(d.lgy, d.ey));
+    copy(d.tw_z, core_table_len(d.lgz, d.ez));
+  }
   __syncthreads();
   Bulk<T>& B = *reinterpret_cast<Bulk<T>*>(objraw);
   const bool leader = blockIdx.x == 0 && threadIdx.x == 0;
@@ -716,23 +819,19 @@ __global__ void __launch_bounds__(NT, 2) bulk_kernel(const Desc* __restrict__ dg
     if (leader) { st->last_iters = r.iters; st->last_r = r.r; st->n_rhs += 1; st->n_iters += r.iters; }
   } else if (a.mode == MODE_J || a.mode == MODE_E || a.mode == MODE_MOMENT) {
     StageIn in{a.y_in, 0, {0, 0, 0}, {nullptr, nullptr, nullptr}, nullptr};
-    { BStage<T> e; e.P = B.ptrs(); e.in = in; e.kim = a.mode == MODE_E && d.b0 > 0.0; B.xpass<0, 3>(e, -1); }
+    if (a.mode == MODE_E && d.b0 > 0.0) B.template xpass<BStageKim, false, true>([&](auto& e) { e.in = in; });
+    else B.template xpass<BStage, false, true>([&](auto& e) { e.in = in; });
     bool ok = B.sync(201) && B.yzy(OP3_CURL, 202);
     if (ok) {
       if (a.mode == MODE_J) {
-        BStoreJ<T> e; e.P = B.ptrs(); e.out = a.out;
-        B.xpass<3, 0>(e, -1);
+        B.template xpass<BStoreJ, true, false>([&](auto& e) { e.out = a.out; });
       } else if (a.mode == MODE_E) {
-        BStoreE<T> e; e.P = B.ptrs(); e.out = a.out;
-        e.n = (T)d.n; e.e0 = (T)d.e0; e.jc = (T)d.jc; e.rho_out = (T)d.rho_out;
-        e.ig2 = (T)(1.0 / (d.gamma * d.gamma)); e.ib0 = d.b0 > 0.0 ? (T)(1.0 / d.b0) : (T)0;
-        B.xpass<3, 0>(e, -1);
+        B.template xpass<BStoreE, true, false>([&](auto& e) { B.law(e); e.out = a.out; });
       } else {
-        for (int c = 0; c < 3 && ok; ++c) {
-          BMoment<T> e; e.P = B.ptrs(); e.comp = c;
-          B.xpass<3, 0>(e, 4 + c);      // reads S1 only
-          ok = B.sync(205 + c);
-        }
+        B.template xpass<BMoment, true, false>([&](auto& e) {
+          e.Lx = d.Lx; e.Ly = d.Ly; e.Lz = d.Lz; e.dx = d.dx; e.dy = d.dy; e.dz = d.dz;
+        }, 4);
+        ok = B.sync(205);
         if (ok) {
           for (int c = 0; c < 3; ++c) {
             const double s = B.total(4 + c);
@@ -755,10 +854,10 @@ __global__ void __launch_bounds__(NT, 2) bulk_kernel(const Desc* __restrict__ dg
 int bulk_max_blocks(int precision, size_t smem) {
   int nb = 0;
   if (precision) {
-    cudaFuncSetAttribute(bulk_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaFuncSetAttribute(bulk_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)BULK_SMEM_MAX);
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, bulk_kernel<float>, NT, smem);
   } else {
-    cudaFuncSetAttribute(bulk_kernel<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaFuncSetAttribute(bulk_kernel<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)BULK_SMEM_MAX);
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, bulk_kernel<double>, NT, smem);
   }
   return nb;

@@ -10,16 +10,8 @@
 namespace mf {
 
 constexpr int NT = 256;           // threads per CTA of the persistent kernels
-constexpr int VPT = 16;           // complex values each thread holds per FFT stage
-constexpr int BATCH = NT * VPT;   // complex points one CTA transforms at once (4096)
-// shared-memory position of FFT element e: one padding slot every 16 complex values keeps the
-// strided butterfly writes of the early Stockham stages to at most 2-way bank conflicts
-__host__ __device__ __forceinline__ constexpr int sp(int e) { return e + (e >> 4); }
-constexpr int BATCH_PAD = BATCH + BATCH / 16;
-
-// The dynamic shared memory of the persistent kernels: two FFT buffers of BATCH_PAD complex
-// values each.  Passes address it by element offset from this base, so that every access is a
-// shared-memory access with 32-bit index arithmetic.
+// The dynamic shared memory of the persistent kernels: the transform core's exchange buffer and the
+// twiddle tables
 extern __shared__ __align__(16) unsigned char mf_dsmem[];
 
 // ------------------------------------------------------------------------------------------
@@ -27,37 +19,11 @@ extern __shared__ __align__(16) unsigned char mf_dsmem[];
 // ------------------------------------------------------------------------------------------
 // 8-byte (float) or 16-byte (double) alignment so that a complex value moves as one vector access
 template <typename T> struct alignas(2 * sizeof(T)) C2 { T x, y; };
-template <typename T> __device__ __forceinline__ C2<T> cadd(C2<T> a, C2<T> b) { return {a.x + b.x, a.y + b.y}; }
-template <typename T> __device__ __forceinline__ C2<T> csub(C2<T> a, C2<T> b) { return {a.x - b.x, a.y - b.y}; }
-template <typename T> __device__ __forceinline__ C2<T> cmul(C2<T> a, C2<T> b) {
-  return {a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x};
-}
-template <typename T> __device__ __forceinline__ C2<T> cconj(C2<T> a) { return {a.x, -a.y}; }
-template <typename T> __device__ __forceinline__ C2<T> cscale(C2<T> a, T s) { return {a.x * s, a.y * s}; }
-// a * (s i) for s = +-1
-template <typename T> __device__ __forceinline__ C2<T> cmul_si(C2<T> a, int s) {
-  return s > 0 ? C2<T>{-a.y, a.x} : C2<T>{a.y, -a.x};
-}
-
-template <typename T> __device__ __forceinline__ C2<T>* dsm() { return reinterpret_cast<C2<T>*>(mf_dsmem); }
-// element offset of a pointer into the dynamic shared memory
-template <typename T> __device__ __forceinline__ int dsm_off(const C2<T>* p) { return (int)(p - dsm<T>()); }
-
 // Loads with L1 placement hints.  Tables (twiddles, wavenumbers) are read over and over and
 // should stay in L1 (evict_last); field data streams through once per pass and should not
 // displace them (no_allocate).  ldg_* use the read-only path and are only for data that no
 // thread writes during the launch (plain asm: the compiler may move and batch them); lds_* are
 // coherent loads for data written by earlier phases (volatile, ordered with the barriers).
-__device__ __forceinline__ C2<float> ldg_c2(const C2<float>* p) {
-  float2 v;
-  asm("ld.global.nc.L1::evict_last.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(p));
-  return {v.x, v.y};
-}
-__device__ __forceinline__ C2<double> ldg_c2(const C2<double>* p) {
-  double2 v;
-  asm("ld.global.nc.L1::evict_last.v2.f64 {%0, %1}, [%2];" : "=d"(v.x), "=d"(v.y) : "l"(p));
-  return {v.x, v.y};
-}
 __device__ __forceinline__ float ldg_tab(const float* p) {
   float v;
   asm("ld.global.nc.L1::evict_last.f32 %0, [%1];" : "=f"(v) : "l"(p));
@@ -171,7 +137,7 @@ struct Desc {
   int rows_per_item;             // 2D row pass / 3D x pass rows per work item (even)
   int zs_per_item;               // 3D y pass z-lines per work item
   int grid;                      // CTAs of the persistent launch
-  int ex, ey;                    // elements per thread of the transform core along x, y
+  int ex, ey, ez;                // elements per thread of the transform core along x, y, z
   unsigned long long barrier_ns; // time limit of one grid-barrier wait (ns)
   const struct Desc* dev;        // device copy of this descriptor (what the kernels read)
 };
@@ -235,7 +201,7 @@ __device__ __forceinline__ bool grid_sync(GridBarrier* gb, unsigned int nblocks,
 }
 
 // ------------------------------------------------------------------------------------------
-// deterministic block reductions (fixed tree) of NT values
+// deterministic reductions
 // ------------------------------------------------------------------------------------------
 __device__ __forceinline__ double warp_sum(double v) {
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
@@ -249,61 +215,6 @@ __device__ __forceinline__ float warp_sum(float v) {
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;
 }
-// sum over the CTA of single-precision partials (warp level in FP32, across warps in FP64);
-// result valid in all threads
-__device__ __forceinline__ double block_sum(float v, double* red) {
-  v = warp_sum(v);
-  const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-  __syncthreads();
-  if (l == 0) red[w] = (double)v;
-  __syncthreads();
-  double s = 0.0;
-  if (threadIdx.x < 32) {
-    s = (l < NT / 32) ? red[l] : 0.0;
-    s = warp_sum(s);
-    if (l == 0) red[0] = s;
-  }
-  __syncthreads();
-  s = red[0];
-  __syncthreads();
-  return s;
-}
-// sum over the CTA; result valid in all threads.  `red` holds NT/32 doubles of shared memory.
-__device__ __forceinline__ double block_sum(double v, double* red) {
-  v = warp_sum(v);
-  const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-  __syncthreads();
-  if (l == 0) red[w] = v;
-  __syncthreads();
-  double s = 0.0;
-  if (threadIdx.x < 32) {
-    s = (l < NT / 32) ? red[l] : 0.0;
-    s = warp_sum(s);
-    if (l == 0) red[0] = s;
-  }
-  __syncthreads();
-  s = red[0];
-  __syncthreads();
-  return s;
-}
-__device__ __forceinline__ double block_max(double v, double* red) {
-  v = warp_max(v);
-  const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-  __syncthreads();
-  if (l == 0) red[w] = v;
-  __syncthreads();
-  double s = 0.0;
-  if (threadIdx.x < 32) {
-    s = (l < NT / 32) ? red[l] : 0.0;
-    s = warp_max(s);
-    if (l == 0) red[0] = s;
-  }
-  __syncthreads();
-  s = red[0];
-  __syncthreads();
-  return s;
-}
-
 // Sum (or max) of partials[slot * max_items + i] over i < n, in a fixed order, computed
 // identically by every CTA (loads through L2 only: the partials were written by other CTAs in this
 // launch).  Every thread loads, the warps reduce, thread 0 combines: one load latency and a short
@@ -387,6 +298,23 @@ __host__ __device__ inline bool film_one_table(const Desc& d) { return d.lgx == 
 constexpr size_t FILM_SMEM_MAX = 16 * ((size_t)slots_of(8) + 2 * core_table_len(11, 8));
 inline size_t film_smem_bytes(const Desc& d) {
   return 16 * ((size_t)film_slots(d) + core_table_len(d.lgx, d.ex) + (film_one_table(d) ? 0 : core_table_len(d.lgy, d.ey)));
+}
+// A bulk body's z pass runs 2^z_group_lg neighbouring lines per group (mf_bulk.cu), 4 where the CTA holds
+// so many; its shared memory: the widest pass's exchange buffer, then the three tables.
+__host__ __device__ constexpr int z_group_lg(int lgz, int ez) {
+  const int lines = (NT * ez) >> lgz;
+  return lines >= 4 ? 2 : lines >= 2 ? 1 : 0;
+}
+__host__ __device__ constexpr int z_slots(int lgz, int ez) {
+  return 3 * ((NT * ez) >> lgz) * ((1 << lgz) + ((1 << lgz) >> 3) + (8 >> z_group_lg(lgz, ez)));
+}
+__host__ __device__ inline int bulk_slots(const Desc& d) {
+  const int xy = slots_of(d.ex > d.ey ? d.ex : d.ey), z = z_slots(d.lgz, d.ez);
+  return xy > z ? xy : z;
+}
+constexpr size_t BULK_SMEM_MAX = 16 * ((size_t)slots_of(16) + 3 * 512);
+inline size_t bulk_smem_bytes(const Desc& d) {
+  return 16 * ((size_t)bulk_slots(d) + core_table_len(d.lgx, d.ex) + core_table_len(d.lgy, d.ey) + core_table_len(d.lgz, d.ez));
 }
 // Rows of the real fields that a film's row passes keep together (mf_film.cuh)
 constexpr int row_unit(int precision) { return precision ? 4 : 2; }

@@ -234,6 +234,7 @@ template <typename T, int E> struct Team {
   CV<V>* s;              // the line's part of the shared buffer
   const CV<V>* tw;       // twiddle table of this length and radix (shared memory)
   int i, lg, slot;       // thread of the line; log2 of its length; line of the CTA
+  static constexpr int fs = 0;
   __device__ __forceinline__ Team(CV<V>* buf, const CV<V>* table, int lgL) : tw(table), lg(lgL) {
     const int lgt = lg - LGE;
     slot = (int)threadIdx.x >> lgt;
@@ -249,12 +250,13 @@ template <typename T, int E> struct Team {
   }
 };
 
-// Transform of length 2^lg >= E, unnormalised.
-template <int DIR, typename T, int E>
-__device__ __forceinline__ void core_fft(CV<typename Lane<T>::V> (&v)[E], const Team<T, E>& t) {
-  using V = typename Lane<T>::V;
+// Transforms of length 2^lg >= E of NF fields together (they share the exchanges' barriers; field f's
+// buffer starts f t.fs elements behind the first one's), unnormalised.
+template <int DIR, int NF, class V, int E, class TM>
+__device__ __forceinline__ void core_fft_n(CV<V> (&v)[NF][E], const TM& t) {
   constexpr int e = lg_of(E), PAD = E == 16 ? 4 : 3;
-  dft_stage<DIR, E, e, true>(v, (const CV<V>*)nullptr);
+#pragma unroll
+  for (int f = 0; f < NF; ++f) dft_stage<DIR, E, e, true>(v[f], (const CV<V>*)nullptr);
   const int q = 1 << (t.lg - e), i = t.i;
   const CV<V>* tw = t.tw;
   int rem = t.lg - e;
@@ -265,27 +267,44 @@ __device__ __forceinline__ void core_fft(CV<typename Lane<T>::V> (&v)[E], const 
     if (lgp == e && E >= 8) {
       CV<V>* const w = t.s + (i << e) + ((i << e) >> PAD);
 #pragma unroll
-      for (int r = 0; r < E; ++r) w[r] = v[r];
+      for (int f = 0; f < NF; ++f) {
+#pragma unroll
+        for (int r = 0; r < E; ++r) w[f * t.fs + r] = v[f][r];
+      }
     } else if (lgp >= e + PAD) {
       const int pp = p >> e, kp = i & (pp - 1);
       CV<V>* const w = &t.at(((i - kp) << e) + kp);
       const int ws = pp + (pp >> PAD);
 #pragma unroll
-      for (int r = 0; r < E; ++r) w[r * ws] = v[r];
+      for (int f = 0; f < NF; ++f) {
+#pragma unroll
+        for (int r = 0; r < E; ++r) w[f * t.fs + r * ws] = v[f][r];
+      }
     } else {
       const int pp = p >> e, kp = i & (pp - 1), w = ((i - kp) << e) + kp;
 #pragma unroll
-      for (int r = 0; r < E; ++r) t.at(w + r * pp) = v[r];
+      for (int r = 0; r < E; ++r) {
+        CV<V>* const o = &t.at(w + r * pp);
+#pragma unroll
+        for (int f = 0; f < NF; ++f) o[f * t.fs] = v[f][r];
+      }
     }
     t.sync();
     if (q >= (1 << PAD)) {
       const CV<V>* const rd = &t.at(i);
       const int rds = q + (q >> PAD);
 #pragma unroll
-      for (int j = 0; j < E; ++j) v[j] = rd[j * rds];
+      for (int f = 0; f < NF; ++f) {
+#pragma unroll
+        for (int j = 0; j < E; ++j) v[f][j] = rd[f * t.fs + j * rds];
+      }
     } else {
 #pragma unroll
-      for (int j = 0; j < E; ++j) v[j] = t.at(i + j * q);
+      for (int j = 0; j < E; ++j) {
+        const CV<V>* const o = &t.at(i + j * q);
+#pragma unroll
+        for (int f = 0; f < NF; ++f) v[f][j] = o[f * t.fs];
+      }
     }
     if (rem >= e) {
       CV<V> w[e];
@@ -293,18 +312,26 @@ __device__ __forceinline__ void core_fft(CV<typename Lane<T>::V> (&v)[E], const 
 #pragma unroll
       for (int m = 0; m < e; ++m) w[m] = tw[(m << lgp) + k];
       tw += e << lgp;
-      dft_stage<DIR, E, e, false>(v, w);
+#pragma unroll
+      for (int f = 0; f < NF; ++f) dft_stage<DIR, E, e, false>(v[f], w);
     } else if (e > 3 && rem == 3) {
       const CV<V> w[3] = {tw[i], tw[q + i], tw[2 * q + i]};
-      dft_stage<DIR, E, (e > 3 ? 3 : 1), false>(v, w);
+#pragma unroll
+      for (int f = 0; f < NF; ++f) dft_stage<DIR, E, (e > 3 ? 3 : 1), false>(v[f], w);
     } else if (e > 2 && rem == 2) {
       const CV<V> w[2] = {tw[i], tw[q + i]};
-      dft_stage<DIR, E, (e > 2 ? 2 : 1), false>(v, w);
+#pragma unroll
+      for (int f = 0; f < NF; ++f) dft_stage<DIR, E, (e > 2 ? 2 : 1), false>(v[f], w);
     } else if (e > 1) {
       const CV<V> w[1] = {tw[i]};
-      dft_stage<DIR, E, 1, false>(v, w);
+#pragma unroll
+      for (int f = 0; f < NF; ++f) dft_stage<DIR, E, 1, false>(v[f], w);
     }
   }
+}
+template <int DIR, class V, int E, class TM>
+__device__ __forceinline__ void core_fft(CV<V> (&v)[E], const TM& t) {
+  core_fft_n<DIR, 1>(reinterpret_cast<CV<V>(&)[1][E]>(v), t);
 }
 
 }  // namespace mf

@@ -10,11 +10,10 @@ __global__ void __launch_bounds__(NT, FILM_CTAS) film_kernel(const Desc* __restr
   film_main<T>(*dg, a, (int)blockIdx.x, gridDim.x);
 }
 
-// film passes: the core's exchange buffer and twiddle tables; bulk passes: two FFT buffers and a third one for the next
-// item's gather
+// the core's exchange buffer and twiddle tables
 size_t kernel_smem_bytes(const Desc& d) {
   if (d.dim == 2) return film_smem_bytes(d);
-  return 3 * (size_t)BATCH_PAD * (d.precision ? sizeof(C2<float>) : sizeof(C2<double>));
+  return bulk_smem_bytes(d);
 }
 
 int film_max_blocks(int precision, size_t smem) {

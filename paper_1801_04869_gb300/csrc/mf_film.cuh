@@ -32,119 +32,11 @@
 // through shared memory and their latencies (979 -> 786 us), 512^2 and 1024^2 by both (350 -> 216 us,
 // 513 -> 304 us).
 #pragma once
-#include "mf_core.cuh"
-#include "mf_rhs_common.cuh"
+#include "mf_units.cuh"
 
 namespace mf {
 
 enum Op2 { OP_GRAD = 0, OP_CURLNEG = 1, OP_K1 = 2, OP_K2 = 3, OP_KH = 4, OP_ID = 5 };
-
-// ------------------------------------------------------------------------------------------
-// row units
-// ------------------------------------------------------------------------------------------
-// the RU rows of one element at one x: 16 bytes
-template <typename T> struct Q { T v[Lane<T>::RU]; };
-__device__ __forceinline__ Q<float> ld_q(const float* p) {
-  Q<float> r;
-  asm volatile("ld.global.L1::no_allocate.v4.f32 {%0, %1, %2, %3}, [%4];"
-               : "=f"(r.v[0]), "=f"(r.v[1]), "=f"(r.v[2]), "=f"(r.v[3]) : "l"(p) : "memory");
-  return r;
-}
-__device__ __forceinline__ Q<double> ld_q(const double* p) {
-  Q<double> r;
-  asm volatile("ld.global.L1::no_allocate.v2.f64 {%0, %1}, [%2];" : "=d"(r.v[0]), "=d"(r.v[1]) : "l"(p) : "memory");
-  return r;
-}
-// read-only for the whole launch (non-coherent path)
-__device__ __forceinline__ Q<float> ldg_q(const float* p) {
-  Q<float> r;
-  asm("ld.global.nc.L1::no_allocate.v4.f32 {%0, %1, %2, %3}, [%4];"
-      : "=f"(r.v[0]), "=f"(r.v[1]), "=f"(r.v[2]), "=f"(r.v[3]) : "l"(p));
-  return r;
-}
-__device__ __forceinline__ Q<double> ldg_q(const double* p) {
-  Q<double> r;
-  asm("ld.global.nc.L1::no_allocate.v2.f64 {%0, %1}, [%2];" : "=d"(r.v[0]), "=d"(r.v[1]) : "l"(p));
-  return r;
-}
-__device__ __forceinline__ void st_q(float* p, const Q<float>& q) { *(float4*)p = make_float4(q.v[0], q.v[1], q.v[2], q.v[3]); }
-__device__ __forceinline__ void st_q(double* p, const Q<double>& q) { *(double2*)p = make_double2(q.v[0], q.v[1]); }
-// element <-> rows: lines pack rows (0, 2) and (1, 3) in FP32, (0, 1) in FP64, as a + i b
-__device__ __forceinline__ Q<float> to_q(const CV<F2>& e) {
-  Q<float> q;
-  upk(e.x, q.v[0], q.v[1]);
-  upk(e.y, q.v[2], q.v[3]);
-  return q;
-}
-__device__ __forceinline__ Q<double> to_q(const CV<double>& e) { return Q<double>{{e.x, e.y}}; }
-__device__ __forceinline__ CV<F2> to_e(const Q<float>& q) { return {pk(q.v[0], q.v[1]), pk(q.v[2], q.v[3])}; }
-__device__ __forceinline__ CV<double> to_e(const Q<double>& q) { return {q.v[0], q.v[1]}; }
-// mask classes of a unit's rows, 2 bits each
-__device__ __forceinline__ int ld_mask(const uint8_t* p) {
-  unsigned m;
-  asm("ld.global.nc.L1::no_allocate.u8 %0, [%1];" : "=r"(m) : "l"(p));
-  return (int)m;
-}
-__device__ __forceinline__ int cls(int m, int r) { return (m >> (2 * r)) & 3; }
-
-// 32 bytes of one half-spectrum column: the complex values of a unit's rows at one x-wavenumber
-struct B32f { float a[8]; };
-struct B32d { double a[4]; };
-__device__ __forceinline__ B32f ld_b32(const C2<float>* p) {
-  B32f r;
-  asm volatile("ld.global.L1::no_allocate.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-               : "=f"(r.a[0]), "=f"(r.a[1]), "=f"(r.a[2]), "=f"(r.a[3]), "=f"(r.a[4]), "=f"(r.a[5]),
-                 "=f"(r.a[6]), "=f"(r.a[7]) : "l"(p) : "memory");
-  return r;
-}
-__device__ __forceinline__ B32d ld_b32(const C2<double>* p) {
-  B32d r;
-  asm volatile("ld.global.L1::no_allocate.v4.f64 {%0, %1, %2, %3}, [%4];"
-               : "=d"(r.a[0]), "=d"(r.a[1]), "=d"(r.a[2]), "=d"(r.a[3]) : "l"(p) : "memory");
-  return r;
-}
-// position k of the packed lines (a + i b per pair of rows) from the rows' half spectra A, B at k:
-// A + i B; at nx - k: conj(A) + i conj(B); at k = 0 and nx/2 the imaginary parts are dropped
-__device__ __forceinline__ CV<F2> pack_lo(const B32f& s) { return {pk(s.a[0] - s.a[5], s.a[2] - s.a[7]), pk(s.a[1] + s.a[4], s.a[3] + s.a[6])}; }
-__device__ __forceinline__ CV<F2> pack_hi(const B32f& s) { return {pk(s.a[0] + s.a[5], s.a[2] + s.a[7]), pk(s.a[4] - s.a[1], s.a[6] - s.a[3])}; }
-__device__ __forceinline__ CV<F2> pack_re(const B32f& s) { return {pk(s.a[0], s.a[2]), pk(s.a[4], s.a[6])}; }
-__device__ __forceinline__ CV<double> pack_lo(const B32d& s) { return {s.a[0] - s.a[3], s.a[1] + s.a[2]}; }
-__device__ __forceinline__ CV<double> pack_hi(const B32d& s) { return {s.a[0] + s.a[3], s.a[2] - s.a[1]}; }
-__device__ __forceinline__ CV<double> pack_re(const B32d& s) { return {s.a[0], s.a[2]}; }
-// twice the rows' half spectra at k from the packed lines' transforms at k and nx - k (the factor
-// 1/2 is in the column passes' scale)
-__device__ __forceinline__ void st_b32(C2<float>* p, const CV<F2>& zk, const CV<F2>& zm) {
-  float r[8];
-  upk(vadd(zk.x, zm.x), r[0], r[2]);
-  upk(vsub(zk.y, zm.y), r[1], r[3]);
-  upk(vadd(zk.y, zm.y), r[4], r[6]);
-  upk(vsub(zm.x, zk.x), r[5], r[7]);
-  asm volatile("st.global.v8.f32 [%8], {%0, %1, %2, %3, %4, %5, %6, %7};"
-               :: "f"(r[0]), "f"(r[1]), "f"(r[2]), "f"(r[3]), "f"(r[4]), "f"(r[5]), "f"(r[6]), "f"(r[7]), "l"(p) : "memory");
-}
-__device__ __forceinline__ void st_b32(C2<double>* p, const CV<double>& zk, const CV<double>& zm) {
-  asm volatile("st.global.v4.f64 [%4], {%0, %1, %2, %3};"
-               :: "d"(zk.x + zm.x), "d"(zk.y - zm.y), "d"(zk.y + zm.y), "d"(zm.x - zk.x), "l"(p) : "memory");
-}
-// one column element: the values of line kx (and, in FP32, of line kx + 1 at `stride`)
-__device__ __forceinline__ CV<F2> ld_col(const C2<float>* p, long long stride, bool two) {
-  const C2<float> a = lds_c2(p);
-  C2<float> b = {0.f, 0.f};
-  if (two) b = lds_c2(p + stride);
-  return {pk(a.x, b.x), pk(a.y, b.y)};
-}
-__device__ __forceinline__ CV<double> ld_col(const C2<double>* p, long long, bool) {
-  const C2<double> a = lds_c2(p);
-  return {a.x, a.y};
-}
-__device__ __forceinline__ void st_col(C2<float>* p, long long stride, bool two, const CV<F2>& e) {
-  C2<float> a, b;
-  upk(e.x, a.x, b.x);
-  upk(e.y, a.y, b.y);
-  p[0] = a;
-  if (two) p[stride] = b;
-}
-__device__ __forceinline__ void st_col(C2<double>* p, long long, bool, const CV<double>& e) { p[0] = C2<double>{e.x, e.y}; }
 
 // raw pointers and sizes the x-pass epilogues need, held by value (registers)
 template <typename T>
@@ -380,46 +272,6 @@ struct Film {
   }
 
   // ---- x pass over units of RU rows: inverse of NIN fields, epilogue, forward of NOUT ----
-  // The packed lines' upper half (positions nx - k) passes through the shared buffer: a thread
-  // loads the half spectrum at its k < nx/2 once, keeps Z[k] and hands Z[nx - k] over.
-  template <int E>
-  __device__ __forceinline__ void gather(CV<V> (&v)[E], const Team<T, E>& t, const C2<T>* src) {
-    const int nx = this->nx, q = t.step();
-    const long long ny = this->ny;
-    t.sync();
-#pragma unroll
-    for (int j = 0; j < E / 2; ++j) {
-      const int k = t.i + j * q;
-      const auto s = ld_b32(src + k * ny);
-      if (k == 0) {
-        v[j] = pack_re(s);
-      } else {
-        v[j] = pack_lo(s);
-        t.at(nx - k) = pack_hi(s);
-      }
-    }
-    if (t.i == 0) t.at(nx >> 1) = pack_re(ld_b32(src + (nx >> 1) * ny));
-    t.sync();
-#pragma unroll
-    for (int j = E / 2; j < E; ++j) v[j] = t.at(t.i + j * q);
-  }
-  template <int E>
-  __device__ __forceinline__ void scatter(CV<V> (&v)[E], const Team<T, E>& t, C2<T>* dst, bool mine) {
-    const int nx = this->nx, q = t.step();
-    const long long ny = this->ny;
-    t.sync();
-#pragma unroll
-    for (int j = E / 2; j < E; ++j) t.at(t.i + j * q) = v[j];
-    t.sync();
-#pragma unroll
-    for (int j = 0; j < E / 2; ++j) {
-      const int k = t.i + j * q;
-      const CV<V> zm = k == 0 ? v[j] : t.at(nx - k);
-      if (mine) st_b32(dst + k * ny, v[j], zm);
-    }
-    if (t.i == 0 && mine) st_b32(dst + (nx >> 1) * ny, v[E / 2], v[E / 2]);
-  }
-
   // Row pass over the units of RU rows with optional per-unit sums into partials slots `slot` (acc,
   // or the maximum of accmax) and `slot2` (acc2).  epi(i, r, in, out) is called for every element: i
   // is the index of the unit's 16-byte vector (and mask byte), r the row-major index of its first
@@ -429,7 +281,7 @@ struct Film {
   template <int E, int NIN, int NOUT, class Epi>
   __device__ __noinline__ void rows_e(const C2<T>* Sin, C2<T>* Sout, const Epi& epi_in, int slot, int slot2, T* tmp) {
     Epi epi = epi_in;                   // register copy of the epilogue
-    const int nx = this->nx;
+    const int nx = this->nx, ny = this->ny;
     const long long nspec = this->nspec;
     Team<T, E> t(sm, twx, lgx);
     const int q = t.step(), tt = t.threads();
@@ -452,14 +304,14 @@ struct Film {
       // inverse transform, each further one while the batch before is worked on
       constexpr int B = Epi::kBatch < E ? Epi::kBatch : E;
       typename Epi::Ld ld[2][B];
-      if constexpr (NIN > 0) gather<E>(v, t, Sin + y0);
+      if constexpr (NIN > 0) row_gather(v, t, Sin + y0, nx, ny);
       if constexpr (NIN == 2) {
         core_fft<+1>(v, t);
         if (mine) {
 #pragma unroll
           for (int j = 0; j < E; ++j) st_q(tmp + (iu + j * q) * RU, to_q(v[j]));
         }
-        gather<E>(v, t, Sin + nspec + y0);
+        row_gather(v, t, Sin + nspec + y0, nx, ny);
       }
 #pragma unroll
       for (int b = 0; b < B; ++b) ld[0][b] = epi.load(iu + b * q, ir + b * q);
@@ -491,13 +343,13 @@ struct Film {
       }
       if constexpr (NOUT > 0) {
         core_fft<-1>(v, t);
-        scatter<E>(v, t, Sout + y0, mine);
+        row_scatter(v, t, Sout + y0, nx, ny, mine);
       }
       if constexpr (NOUT == 2) {
 #pragma unroll
         for (int j = 0; j < E; ++j) v[j] = to_e(ld_q(tmp + (iu + j * q) * RU));
         core_fft<-1>(v, t);
-        scatter<E>(v, t, Sout + nspec + y0, mine);
+        row_scatter(v, t, Sout + nspec + y0, nx, ny, mine);
       }
       if (slot >= 0) unit_sums(epi, t, unit, mine, slot, slot2);
     }
@@ -634,14 +486,6 @@ struct Film {
 // in[f].v[0 .. RU) and sets the outputs out[f].v[0 .. RU).  kBatch elements are loaded together
 // (a store could alias a later load as far as the compiler knows, so a load placed behind a store
 // waits for the whole latency of the loads before it).
-struct NoLd {};
-
-// FP64 state fields are row-major (the caller's layout)
-__device__ __forceinline__ double ld_s(const double* p) {
-  double v;
-  asm volatile("ld.global.L1::no_allocate.f64 %0, [%1];" : "=d"(v) : "l"(p) : "memory");
-  return v;
-}
 
 // P1 / readouts: field from the FP64 stage input
 template <typename T>

@@ -432,18 +432,6 @@ __global__ void __launch_bounds__(1024) sums_kernel(long long n, const double* x
   if (threadIdx.x == 0) { out[0] = s1[0]; out[1] = s2[0]; }
 }
 
-// FP64 -> transform precision copy (a jc map set after creation)
-__global__ void to_float_kernel(long long n, const double* x, float* y) {
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-       i += (long long)gridDim.x * blockDim.x)
-    y[i] = (float)x[i];
-}
-
-cudaError_t adj_to_float(long long n, const double* x, float* y, cudaStream_t s) {
-  to_float_kernel<<<304, 256, 0, s>>>(n, x, y);
-  return cudaGetLastError();
-}
-
 cudaError_t adj_lincomb(long long n, double* out, int nt, const double* const* x, const double* c,
                         double b, cudaStream_t s) {
   const double* z = nullptr;
@@ -459,7 +447,7 @@ cudaError_t adj_sums(long long n, const double* x, double* out, cudaStream_t s) 
   return cudaGetLastError();
 }
 
-// Fields by row units (mf_film.cuh): element of (unit, x, row) for the row-major cell (y, x)
+// Fields by row units (mf_units.cuh): element of (unit, x, row) for the row-major cell (y, x)
 __device__ __forceinline__ long long unit_index(long long cell, int nx, int ru) {
   const long long y = cell / nx, x = cell - y * nx, u = y / ru;
   return (u * nx + x) * ru + (y - u * ru);
@@ -494,8 +482,8 @@ __global__ void to_units_kernel(int nx, long long n, const double* x, T* y) {
        i += (long long)gridDim.x * blockDim.x)
     y[unit_index(i, nx, Lane<T>::RU)] = (T)x[i];
 }
-cudaError_t film_to_units(int precision, int nx, int ny, const double* x, void* y, cudaStream_t s) {
-  const long long n = (long long)nx * ny;
+cudaError_t field_to_units(int precision, int nx, long long rows, const double* x, void* y, cudaStream_t s) {
+  const long long n = rows * nx;
   if (precision) to_units_kernel<float><<<608, 256, 0, s>>>(nx, n, x, (float*)y);
   else to_units_kernel<double><<<608, 256, 0, s>>>(nx, n, x, (double*)y);
   return cudaGetLastError();
@@ -520,8 +508,8 @@ __global__ void relayout_kernel(int nx, long long nvec, bool to_rows, const T* s
     }
   }
 }
-cudaError_t film_relayout(int precision, int nx, int ny, bool to_rows, const void* src, void* dst, cudaStream_t s) {
-  const long long nvec = (long long)nx * ny / row_unit(precision);
+cudaError_t field_relayout(int precision, int nx, long long rows, bool to_rows, const void* src, void* dst, cudaStream_t s) {
+  const long long nvec = rows * nx / row_unit(precision);
   if (precision) relayout_kernel<float><<<608, 256, 0, s>>>(nx, nvec, to_rows, (const float*)src, (float*)dst);
   else relayout_kernel<double><<<608, 256, 0, s>>>(nx, nvec, to_rows, (const double*)src, (double*)dst);
   return cudaGetLastError();

@@ -3,11 +3,28 @@
 #pragma once
 #include <new>
 
-#include "mf_passes.cuh"
+#include "mf_common.cuh"
 
 namespace mf {
 
 constexpr double PI_D = 3.14159265358979323846;
+
+__device__ __forceinline__ float powt(float a, float b) { return powf(a, b); }
+__device__ __forceinline__ double powt(double a, double b) { return pow(a, b); }
+
+// power law of Eq. 3 / Eq. 13:  rho = (e0/jc) (|j|/jc)^(n-1) in the superconductor (mask 1),
+// rho_out elsewhere.  Takes |j|^2.
+template <typename T>
+__device__ __forceinline__ T resistivity(T j2, T jc, int m, T n, T e0, T rho_out) {
+  if (m != 1) return rho_out;
+  const T x2 = j2 / (jc * jc);
+  // (|j|/jc)^(n-1) = (|j|^2/jc^2)^((n-1)/2); exactly 1 for n = 1 (including j = 0)
+  T pw;
+  if (n == (T)1) pw = (T)1;
+  else if (x2 <= (T)0) pw = (T)0;
+  else pw = powt(x2, (n - (T)1) * (T)0.5);
+  return e0 / jc * pw;
+}
 
 // stage input y + sum c_j k_j (FP64), optionally written to ynew
 struct StageIn {
@@ -31,6 +48,9 @@ struct Control {
 // per-CTA copy of the scalars every CTA agrees on
 struct Shared {
   double red[NT / 32], red2[NT / 32];
+  double redn[3][NT / 32];       // (3D) per-item sums
+  double hed3[3], thresh;        // (3D) h_e_dot; residual threshold of the stop test
+  float hed3f[3];
   double A, C, r, hed, N;
   float Af, Cf, rq;              // (2D) A, C and h_e_dot in the transform precision's FP32 form
   int stop, ok, diverged;        // decisions of the outside iteration
@@ -42,8 +62,6 @@ struct Shared {
   double inv_nout;               // 1 / free-space cells
   int attempt_first;             // (2D) the next right-hand side is the first of a step attempt
   unsigned long long bar_passed;  // grid barriers passed in this launch (thread 0)
-  unsigned long long tma_bar;     // (3D) mbarrier of the bulk copies into the staging buffer
-  unsigned tma_parity;            // (3D) phase parity the next wait on tma_bar expects
   Control ctl;
 };
 
@@ -89,10 +107,6 @@ struct EpiBase {
   Acc acc = 0, accmax = 0;
   Acc acc2 = 0;                 // a second sum (rows() with a second slot)
   bool is_max = false;
-  // kPair: the epilogue also has pair(ia, ib, ...) for the two rows of a cell pair, which issues
-  // every load of both before any store (a store may alias a later load as far as the compiler
-  // knows, so two separate calls would wait for the first call's loads before the second's)
-  static constexpr bool kPair = false;
 };
 
 struct RhsOut {

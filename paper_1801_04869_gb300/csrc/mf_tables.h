@@ -1,62 +1,15 @@
-// Host-side generation of the stage-ordered twiddle tables of the shared-memory FFT.
-//
-// For a transform of length L = 2^lgL with radices r_0 .. r_{m-1} (the plan rule of
-// fft_plan<T>: radix 16 while at least 4 factors of two remain, except when exactly 5 remain,
-// in single precision; radix 8 in double precision; then one radix 4 or 2), stage s has
-// p_s = r_0 ... r_{s-1} and needs w^(j k) = exp(-2 pi i j k / (p_s r_s)) for 1 <= j < r_s and
-// 0 <= k < p_s.  Entry (j - 1) p_s + k of the stage's block holds it, so the threads of a warp
-// (consecutive k) read consecutive entries.  Table A holds the blocks of the plan in order,
-// table B those of the reversed plan (used by the inverse half of a fused round trip); B
-// follows A.
+// Host-side tables and launch shapes: twiddles of the transform core, elements per thread, fields and
+// masks by row units.
 #pragma once
+#include <algorithm>
 #include <cmath>
 
 #include "mf_common.cuh"
 
 namespace mf {
 
-inline int plan_lgr(int lgL, bool single, int* lgr) {
-  int m = 0, rem = lgL;
-  while (rem > 0) {
-    int l;
-    if (single && VPT >= 16 && rem >= 4 && rem != 5) l = 4;
-    else if (rem >= 3) l = 3;
-    else l = rem;
-    lgr[m++] = l;
-    rem -= l;
-  }
-  return m;
-}
-
-// writes (re, im) pairs of tables A then B into out; returns the number of complex entries
-template <typename T>
-inline int stage_twiddles(int L, T* out) {
-  int lgL = 0;
-  while ((1 << lgL) < L) ++lgL;
-  int lgr[32];
-  const int m = plan_lgr(lgL, sizeof(T) == 4, lgr);
-  int n = 0;
-  for (int pass = 0; pass < 2; ++pass) {
-    int lgp = 0;
-    for (int s = 0; s < m; ++s) {
-      const int l = pass == 0 ? lgr[s] : lgr[m - 1 - s];
-      const int R = 1 << l, p = 1 << lgp;
-      for (int j = 1; j < R; ++j)
-        for (int k = 0; k < p; ++k) {
-          const double ang = -2.0 * M_PI * (double)j * (double)k / (double)(p * R);
-          out[2 * n] = (T)std::cos(ang);
-          out[2 * n + 1] = (T)std::sin(ang);
-          ++n;
-        }
-      lgp += l;
-    }
-  }
-  return n;
-}
-
-// Values of type T set aside per point of an axis for its twiddle tables: the bulk's tables A and B
-// hold fewer than 2 L complex entries; the core's hold fewer than L entries of 4 (single) or 2
-// (double) values
+// Values of type T set aside per point of an axis for its twiddle table, which holds fewer than L
+// entries of 4 (single) or 2 (double) values
 constexpr size_t TWIDDLE_VALUES = 4;
 
 // Table of the transform core (mf_core.cuh) for length L and E = 2^e elements per thread, stage after
@@ -110,6 +63,31 @@ inline int elems_per_thread(const Desc& d, int n) {
   const long long cells = (long long)d.nx * d.ny;
   if (d.precision == 0) return cells <= 65536 && n <= 2 * NT ? 2 : 8;
   return cells <= 1048576 && n <= 4 * NT ? 4 : 8;
+}
+
+// Elements per thread and items of a bulk body's passes.
+//   x: E = 8 (two exchanges per transform up to 512 points); E = 4 (FP32, to 64^3) or 2 (FP64, to 2^16
+//      cells) where a pass does not fill the chip and one thread's chain of instructions sets its time.
+//   y: E = 16 in FP32 (64 data registers, nothing else live: one exchange for lines of up to 256 points),
+//      8 in FP64; 4 for small bodies and lines shorter than E.
+//   z: three components are transformed together, so E = 4 (48 data registers); 2 for small FP64 bodies.
+// An x item is a block of row units whose residual is summed together: as many as fill a CTA, but at
+// least 304 items (two CTAs on each of 152 SMs), whatever the launch width, so that it changes nothing.
+inline void bulk_shape(Desc& d, int coresident) {
+  const bool f32 = d.precision != 0;
+  const bool small = d.ncell <= (f32 ? 262144 : 65536);
+  d.ex = small ? (f32 ? 4 : 2) : 8;
+  const int ey = small ? 4 : f32 ? 16 : 8;
+  d.ey = d.ny < ey ? 4 : ey;
+  d.ez = !f32 && small && d.nz <= 2 * NT ? 2 : 4;
+  const int ru = row_unit(d.precision);
+  const long long units = (long long)d.nz * d.ny / ru;
+  long long ub = NT / (d.nx / d.ex);
+  while (ub > 1 && (units / ub < 304 || units % ub)) ub /= 2;
+  d.rows_per_item = (int)ub * ru;
+  d.zs_per_item = 1;
+  const long long lines = 3LL * d.nz / (ru / 2) * (d.nx / 2 + 1);
+  d.grid = (int)std::min<long long>(coresident, std::max(units / ub, lines));
 }
 
 // mask classes of `units` row units from the row-major mask of their rows, 2 bits per row
