@@ -18,6 +18,8 @@
 //
 // The passes run on the transform core (mf_core.cuh); real fields and the mask lie by row units
 // (mf_units.cuh).
+#include <type_traits>
+
 #include "mf_units.cuh"
 
 namespace mf {
@@ -30,34 +32,7 @@ struct BulkPtrs {
   const uint8_t* mask;
   const T* jcmap;
   T* hd;
-  long long ncell;
-  int nx, ny;
-};
-
-// The threads of a group of G = 2^lgG neighbouring lines of the z pass: a line's element z lies nkx ny
-// values behind element z - 1, so the group's lines are interleaved on the lanes and a warp reads
-// G x 16 contiguous bytes per z.  Line u's buffer is 8/G elements longer than its padded length, which
-// spreads the lines of 8 neighbouring lanes over the banks.
-template <typename T, int E> struct GroupTeam {
-  using V = typename Lane<T>::V;
-  static constexpr int LGE = lg_of(E);
-  CV<V>* s;
-  const CV<V>* tw;
-  int i, lg, slot, u, lgt, fs;     // position; log2 length; group of the CTA; line of the group; log2 threads
-  __device__ __forceinline__ GroupTeam(CV<V>* buf, const CV<V>* table, int lgL, int lgG) : tw(table), lg(lgL) {
-    lgt = lg - LGE + lgG;
-    slot = (int)threadIdx.x >> lgt;
-    u = (int)threadIdx.x & ((1 << lgG) - 1);
-    i = ((int)threadIdx.x >> lgG) & ((1 << (lg - LGE)) - 1);
-    const int stride = spe<E>(1 << lg) + (8 >> lgG);
-    s = buf + ((slot << lgG) + u) * stride;
-    fs = ((NT >> lgt) << lgG) * stride;
-  }
-  __device__ __forceinline__ CV<V>& at(int e) const { return s[spe<E>(e)]; }
-  __device__ __forceinline__ void sync() const {
-    if (lgt <= 5) __syncwarp();
-    else asm volatile("bar.sync %0, %1;" :: "r"(1 + slot), "r"(1 << lgt) : "memory");
-  }
+  int ncell, nx, ny;
 };
 
 template <typename T>
@@ -65,10 +40,11 @@ struct Bulk {
   using V = typename Lane<T>::V;
   static constexpr int RU = Lane<T>::RU, NL = Lane<T>::NL;
   const Desc& d;
-  CV<V>* sm;         // the CTA's exchange buffer
+  CV<V>* sm;         // the CTA's shared memory: a pass's exchange buffers, then its staging buffer, in which
+                     // the next unit's spectra arrive while a unit is worked on
   Shared& sh;
   int nx, ny, nz, lgx, lgy, lgz, half, nkx;
-  long long nspec, ncell;
+  int nspec, ncell;  // indexes of the three components' values stay below 2^31 (512^3 cells)
   C2<T>* S;          // spectra of the three components, [c][z][kx][y]
   T* tmp;            // two real fields by row units (joint epilogues)
   T* hd;
@@ -78,7 +54,7 @@ struct Bulk {
   const T* ktab; const T* gtab;     // kx (nkx), ky (ny), kz (nz)
   T scale;           // 1/(2 cells): the x pass leaves twice the half spectra
   T ig2, ib0;        // 1/gamma^2; 1/b0 of the Kim law, 0: none
-  int ex, ey, ez, lgG, ub, lgu;     // elements per thread; lines per z group; row units per x item; log2 units per z
+  int ex, ey, ez, lgG, lgGx, ub, lgu;   // elements per thread; log2 lines per z, x group; row units per x item; log2 units per z
   int max_items;
   double* partials;
   GridBarrier* gb;
@@ -87,21 +63,23 @@ struct Bulk {
   __device__ Bulk(const Desc& dd, unsigned char* smem, Shared& shr) : d(dd), sm((CV<V>*)smem), sh(shr) {
     nx = d.nx; ny = d.ny; nz = d.nz; lgx = d.lgx; lgy = d.lgy; lgz = d.lgz;
     half = nx / 2; nkx = half + 1;
-    nspec = (long long)nkx * ny * nz;
-    ncell = (long long)nx * ny * nz;
+    nspec = nkx * ny * nz;
+    ncell = nx * ny * nz;
     S = (C2<T>*)d.Sa; tmp = (T*)d.Sb;
     hd = (T*)d.hd;
     mask = d.mask; jcmap = (const T*)d.jcmap;
     ex = d.ex; ey = d.ey; ez = d.ez;
     twx = sm + bulk_slots(d);
-    twy = twx + core_table_len(lgx, ex);
-    twz = twy + core_table_len(lgy, ey);
+    const CV<V>* const t = twx + core_table_len(lgx, ex);
+    twy = one_table(d) ? twx : t;
+    twz = one_table(d) ? t : t + core_table_len(lgy, ey);
     ktab = (const T*)d.ktab; gtab = (const T*)d.gtab;
     scale = (T)0.5 / (T)ncell;
     ig2 = (T)(1.0 / (d.gamma * d.gamma));
     ib0 = d.b0 > 0.0 ? (T)(1.0 / d.b0) : (T)0;
     lgG = z_group_lg(lgz, ez);
     ub = d.rows_per_item / RU;
+    lgGx = x_group_lg(d);
     lgu = lgy - (RU == 4 ? 2 : 1);
     max_items = d.max_items;
     partials = d.partials;
@@ -127,27 +105,45 @@ struct Bulk {
   __device__ __noinline__ void xpass_e(const Epi& epi_in, int slot) {
     Epi epi = epi_in;                   // register copy of the epilogue
     const int nx = this->nx, ub = this->ub;
-    const long long ny = this->ny, nspec = this->nspec, ncell = this->ncell;
-    Team<T, E> t(sm, twx, lgx);
+    const int ny = this->ny, nspec = this->nspec, ncell = this->ncell;
+    const int lgG = this->lgGx;
+    Team<T, E> t(sm, twx, lgx, lgG);
     const int q = t.step();
     const int nitems = (nz << lgu) / ub;
-    const int first = ((int)threadIdx.x & ~31) >> (lgx - lg_of(E));      // slot of the warp's first lane
+    const int first = (((int)threadIdx.x & ~31) >> t.lgt) << lgG;        // line of the warp's first lane
     const bool mine = t.slot < ub;
+    // the group's part of the staging buffer, and its values at nx/2
+    uint4* const stg0 = (uint4*)sm + x_slots(lgx, E);
+    uint4* const stg = stg0 + (((int)threadIdx.x >> t.lgt) << (lgx + lgG));
+    uint4* const top = stg0 + E * NT + (((int)threadIdx.x >> t.lgt) << (1 + lgG));
+    Q<T>* const park = (Q<T>*)(stg0 + x_stage(lgx, E)) + threadIdx.x;    // this thread's slots, NT apart
+    auto spectra = [&](int it, int slot) {
+      const int unit = it * ub + (mine ? slot : 0);
+      const int z = unit >> lgu, y0 = (unit - (z << lgu)) * RU;
+      return S + z * nkx * ny + y0;
+    };
+    const int slot0 = t.slot - t.u;                                      // the group's first unit
+    if (NIN && first < ub && (int)blockIdx.x < nitems) row_stage(t, lgG, stg, top, spectra((int)blockIdx.x, slot0), nx, ny);
     for (int it = (int)blockIdx.x; it < nitems; it += (int)gridDim.x) {
       epi.reset();
       if (first < ub) {
         const int unit = it * ub + (mine ? t.slot : 0);
-        const int z = unit >> lgu, y0 = (unit - (z << lgu)) * RU;
-        C2<T>* const Su = S + (long long)z * nkx * ny + y0;
-        const long long iu = (long long)unit * nx + t.i;                 // 16-byte vector of a component
-        const long long ir = (long long)unit * RU * nx + t.i;            // row-major cell of the first row
+        C2<T>* const Su = spectra(it, t.slot);
+        // component c's spectra from the staging buffer; the next component's (item's) are then issued
+        auto gather = [&](auto& v, int c) {
+          row_gather_staged(v, t, lgG, stg, top, nx);
+          const int nit = c < 2 ? it : it + (int)gridDim.x;
+          if (nit < nitems) row_stage(t, lgG, stg, top, spectra(nit, slot0) + (c < 2 ? c + 1 : 0) * nspec, nx, ny);
+        };
+        const int iu = unit * nx + t.i;                 // 16-byte vector of a component
+        const int ir = unit * RU * nx + t.i;            // row-major cell of the first row
         constexpr int B = Epi::kBatch < E ? Epi::kBatch : E;
         if constexpr (Epi::kJoint) {
           T* const tmp = this->tmp;
           CV<V> v[E];
 #pragma unroll 1
           for (int c = 0; c < 3; ++c) {
-            row_gather(v, t, Su + c * nspec, nx, ny);
+            gather(v, c);
             core_fft<+1>(v, t);
             if (c < 2 && mine) {
 #pragma unroll
@@ -161,7 +157,7 @@ struct Bulk {
               Q<T> in[B][3], out[3];
 #pragma unroll
               for (int b = 0; b < B; ++b) {
-                const long long i = iu + (j0 + b) * q;
+                const int i = iu + (j0 + b) * q;
                 ld[b] = epi.load(i, ir + (j0 + b) * q);
                 in[b][0] = ld_q(tmp + i * RU);
                 in[b][1] = ld_q(tmp + ncell + i * RU);
@@ -169,7 +165,7 @@ struct Bulk {
               }
 #pragma unroll
               for (int b = 0; b < B; ++b) {
-                const long long i = iu + (j0 + b) * q;
+                const int i = iu + (j0 + b) * q;
                 epi.apply(ld[b], t.i + (j0 + b) * q, unit, ir + (j0 + b) * q, in[b], out);
                 if constexpr (NOUT) {
                   st_q(tmp + i * RU, out[0]);
@@ -195,7 +191,7 @@ struct Bulk {
           for (int c = 0; c < 3; ++c) {
             CV<V> v[E];
             typename Epi::Ld ld[2][B];
-            if constexpr (NIN) row_gather(v, t, Su + c * nspec, nx, ny);
+            if constexpr (NIN) gather(v, c);
 #pragma unroll
             for (int b = 0; b < B; ++b) ld[0][b] = epi.load(c, iu + b * q, ir + b * q);
             if constexpr (NIN) core_fft<+1>(v, t);
@@ -211,7 +207,7 @@ struct Bulk {
                   const int j = j0 + b;
                   Q<T> in, out;
                   if constexpr (NIN) in = to_q(v[j]);
-                  epi.apply(ld[(j0 / B) & 1][b], c, j, iu + j * q, ir + j * q, in, out);
+                  epi.apply(ld[(j0 / B) & 1][b], c, park + j * NT, iu + j * q, ir + j * q, in, out);
                   if constexpr (NOUT) v[j] = to_e(out);
                 }
               }
@@ -221,7 +217,6 @@ struct Bulk {
               row_scatter(v, t, Su + c * nspec, nx, ny, mine);
             }
           }
-          if (mine) epi.done(iu, q);
         }
       }
       if (slot >= 0) {
@@ -270,23 +265,52 @@ struct Bulk {
   // ---- y pass: contiguous lines in place, z neighbours together in FP32; kx slowest ----
   template <int E, int DIR>
   __device__ __noinline__ void ypass_e() {
-    const long long ny = this->ny, nspec = this->nspec, nkx = this->nkx;
+    const int ny = this->ny, nspec = this->nspec, nkx = this->nkx;
     Team<T, E> t(sm, twy, lgy);
     const int q = t.step();
     const int nzp = nz / NL, units = 3 * nzp * (int)nkx;
     const int per = NT / t.threads(), want = (units + (int)gridDim.x - 1) / (int)gridDim.x;
     const int nuc = want < per ? want : per;
     const int first = ((int)threadIdx.x & ~31) >> (lgy - lg_of(E));
-    for (int u0 = (int)blockIdx.x * nuc; u0 < units; u0 += (int)gridDim.x * nuc) {
-      if (first >= nuc || u0 + first >= units) continue;
-      const bool mine = t.slot < nuc && u0 + t.slot < units;
-      const int u = mine ? u0 + t.slot : u0;
+    const int next = nkx * ny;         // the line of z + 1
+    auto line = [&](int u) {
       const int kx = u / (3 * nzp), r = u - kx * 3 * nzp, c = r / nzp, z = (r - c * nzp) * NL;
-      C2<T>* const p = S + c * nspec + (z * nkx + kx) * ny + t.i;
-      const long long next = nkx * ny;       // the line of z + 1
-      CV<V> v[E];
+      return S + c * nspec + (z * nkx + kx) * ny;
+    };
+    // a unit's NL lines lie one after the other in its part of the staging buffer, 16 bytes per copy
+    uint4* const stg = (uint4*)sm + slots_of(E) + ((t.slot * t.threads()) << lg_of(E));
+    auto issue = [&](const C2<T>* p) {
+      const int half_l = 1 << (lgy - (NL - 1));          // 16-byte pieces per line
 #pragma unroll
-      for (int j = 0; j < E; ++j) v[j] = ld_col(p + j * q, next, true);
+      for (int j = 0; j < E; ++j) {
+        const int k = t.i + j * q, l = NL == 2 ? k >> (lgy - 1) : 0;
+        cp16(stg + k, (const uint4*)(p + l * next) + (k & (half_l - 1)));
+      }
+      cp_commit();
+    };
+    if (first >= nuc) return;
+    int u0 = (int)blockIdx.x * nuc;
+    auto unit_of = [&](int u0) { return t.slot < nuc && u0 + t.slot < units ? u0 + t.slot : u0; };
+    if (u0 + first < units) issue(line(unit_of(u0)));
+    for (; u0 + first < units; u0 += (int)gridDim.x * nuc) {
+      const bool mine = t.slot < nuc && u0 + t.slot < units;
+      C2<T>* const p = line(unit_of(u0)) + t.i;
+      CV<V> v[E];
+      cp_wait();
+      t.sync();
+#pragma unroll
+      for (int j = 0; j < E; ++j) {
+        const C2<T>* const a = (const C2<T>*)stg + t.i + j * q;
+        if constexpr (NL == 2) {
+          const C2<T> x = a[0], y = a[1 << lgy];
+          v[j] = {pk(x.x, y.x), pk(x.y, y.y)};
+        } else {
+          v[j] = {a[0].x, a[0].y};
+        }
+      }
+      t.sync();                              // every thread has read: the next unit's lines may land
+      const int nu = u0 + (int)gridDim.x * nuc;
+      if (nu + first < units) issue(line(unit_of(nu)));
       core_fft<DIR>(v, t);
       if (mine) {
 #pragma unroll
@@ -295,18 +319,13 @@ struct Bulk {
     }
   }
   template <int DIR> __device__ __forceinline__ void ypass() {
-    constexpr int BIG = sizeof(T) == 4 ? 16 : 8;
     if (ey == 4) ypass_e<4, DIR>();
-    else ypass_e<BIG, DIR>();
+    else ypass_e<8, DIR>();
   }
 
   // ---- z pass: forward, 3x3 multiplier, inverse on groups of lines (kx, y0 ..) ----
-  static __device__ __forceinline__ CV<F2> ld_z(const C2<float>* p) {
-    float a, b, c, e;
-    asm volatile("ld.global.L1::no_allocate.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(a), "=f"(b), "=f"(c), "=f"(e) : "l"(p) : "memory");
-    return {pk(a, c), pk(b, e)};
-  }
-  static __device__ __forceinline__ CV<double> ld_z(const C2<double>* p) { return ld_col(p, 0, false); }
+  static __device__ __forceinline__ CV<F2> ld_z(const float4& f) { return {pk(f.x, f.z), pk(f.y, f.w)}; }
+  static __device__ __forceinline__ CV<double> ld_z(const double2& f) { return {f.x, f.y}; }
   static __device__ __forceinline__ void st_z(C2<float>* p, const CV<F2>& v) {
     float4 f;
     upk(v.x, f.x, f.z);
@@ -323,27 +342,48 @@ struct Bulk {
   template <int E>
   __device__ __noinline__ void zpass_e(int op) {
     const int ny = this->ny, half = this->half;
-    const long long nspec = this->nspec, zs = (long long)nkx * ny;
-    GroupTeam<T, E> t(sm, twz, lgz, lgG);
-    const int q = 1 << (lgz - lg_of(E));
+    const int nspec = this->nspec, zs = nkx * ny;
+    Team<T, E> t(sm, twz, lgz, lgG);
+    const int q = t.step();
     const int gl = NL << lgG, ngy = ny / gl;                  // y lines per group, groups per kx
     const int units = nkx * ngy;
-    const int per = NT >> t.lgt, want = (units + (int)gridDim.x - 1) / (int)gridDim.x;
+    const int per = NT >> t.lgt, slot = (int)threadIdx.x >> t.lgt, want = (units + (int)gridDim.x - 1) / (int)gridDim.x;
     const int nuc = want < per ? want : per;
     const int first = ((int)threadIdx.x & ~31) >> t.lgt;
-    for (int u0 = (int)blockIdx.x * nuc; u0 < units; u0 += (int)gridDim.x * nuc) {
-      if (first >= nuc || u0 + first >= units) continue;
-      const bool mine = t.slot < nuc && u0 + t.slot < units;
-      // from the last kx to the first: what the y pass before left in L2 last comes first
-      const int g = units - 1 - (mine ? u0 + t.slot : u0);
+    using Raw = typename std::conditional<sizeof(T) == 4, float4, double2>::type;
+    uint4* const stg = (uint4*)sm + z_slots(lgz, E) + threadIdx.x;       // this thread's elements, NT apart
+    // from the last kx to the first: what the y pass before left in L2 last comes first
+    auto group_of = [&](int u0) { return units - 1 - (slot < nuc && u0 + slot < units ? u0 + slot : u0); };
+    auto lines = [&](int g) {
       const int kx = g / ngy, y = (g - kx * ngy) * gl + t.u * NL;
-      C2<T>* const p = S + (long long)kx * ny + y + t.i * zs;
-      CV<V> v[3][E];
+      return S + kx * ny + y + t.i * zs;
+    };
+    auto issue = [&](const C2<T>* p) {
 #pragma unroll
       for (int c = 0; c < 3; ++c) {
 #pragma unroll
-        for (int j = 0; j < E; ++j) v[c][j] = ld_z(p + c * nspec + j * q * zs);
+        for (int j = 0; j < E; ++j) cp16(stg + (c * E + j) * NT, p + c * nspec + j * q * zs);
       }
+      cp_commit();
+    };
+    if (first >= nuc) return;
+    int u0 = (int)blockIdx.x * nuc;
+    if (u0 + first < units) issue(lines(group_of(u0)));
+    for (; u0 + first < units; u0 += (int)gridDim.x * nuc) {
+      const bool mine = slot < nuc && u0 + slot < units;
+      const int g = group_of(u0);
+      const int kx = g / ngy, y = (g - kx * ngy) * gl + t.u * NL;
+      C2<T>* const p = lines(g);
+      CV<V> v[3][E];
+      cp_wait();
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+#pragma unroll
+        for (int j = 0; j < E; ++j) v[c][j] = ld_z(*(const Raw*)(stg + (c * E + j) * NT));
+      }
+      t.sync();                              // the elements have been read: the next group's may land
+      const int nu = u0 + (int)gridDim.x * nuc;
+      if (nu + first < units) issue(lines(group_of(nu)));
       // wavenumbers of the line(s); odd multipliers are 0 at the Nyquist index of their axis
       const T kx1 = ldg_tab(&ktab[kx]), gx = ldg_tab(&gtab[kx]);
       const T kxo = kx == half ? (T)0 : kx1;
@@ -421,8 +461,9 @@ struct Bulk {
 // ------------------------------------------------------------------------------------------
 // Epilogues of the x pass.  load(c, i, r) reads what the RU rows of one element of component c need (i:
 // the component's 16-byte vector, r: the row-major cell of the first row, the others nx apart);
-// apply(ld, c, j, i, r, in, out) works on the thread's element j; done(i, q) follows the last component
-// (element j's vector is i + j q); reset() starts a unit.  Joint ones take the three components at once.
+// apply(ld, c, s, i, r, in, out) works on one element, which has 16 bytes of shared memory s of its own
+// for what passes from component to component; reset() starts an item.  Joint ones take the three
+// components at once.
 // ------------------------------------------------------------------------------------------
 template <typename T, int NS = 1, bool MAX = false>
 struct BEpi {
@@ -434,66 +475,73 @@ struct BEpi {
 #pragma unroll
     for (int k = 0; k < NS; ++k) acc[k] = 0;
   }
-  __device__ __forceinline__ void done(long long, int) {}
-  __device__ __forceinline__ int msk(long long i) const { return ld_mask(P.mask + i); }
+  __device__ __forceinline__ int msk(int i) const { return ld_mask(P.mask + i); }
 };
 
-// Stage state y + sum c_j k_j.  With a field-dependent critical current (KIM) the stage field's
-// magnitude |h| is kept, in the transform precision, in the first component of the h_dot iterate at
-// superconductor cells: those entries are rewritten by BInit before anything reads them as an iterate,
-// and the warm start lives on free space only.
-template <typename T, int E, bool KIM>
-struct BStageT : BEpi<T> {
+// Stage state y + sum c_j k_j.
+template <typename T, int E>
+struct BStage : BEpi<T> {
   static constexpr int RU = Lane<T>::RU, kBatch = 2;
   StageIn in;
-  double h2[KIM ? E : 1][RU];
   struct Ld { double v[RU]; };
-  __device__ __forceinline__ Ld load(int c, long long, long long r) const {
+  __device__ __forceinline__ double value(int o) const {
+    double v = ld_s(in.y + o);
+    for (int j = 0; j < in.nk; ++j) v += in.c[j] * ld_s(in.k[j] + o);
+    return v;
+  }
+  __device__ __forceinline__ Ld load(int c, int, int r) const {
     Ld l;
-    const long long o = c * this->P.ncell + r;
+    const int o = c * this->P.ncell + r;
 #pragma unroll
-    for (int q = 0; q < RU; ++q) l.v[q] = ld_s(in.y + o + (long long)q * this->P.nx);
+    for (int q = 0; q < RU; ++q) l.v[q] = ld_s(in.y + o + q * this->P.nx);
     for (int j = 0; j < in.nk; ++j) {
       double k[RU];
 #pragma unroll
-      for (int q = 0; q < RU; ++q) k[q] = ld_s(in.k[j] + o + (long long)q * this->P.nx);
+      for (int q = 0; q < RU; ++q) k[q] = ld_s(in.k[j] + o + q * this->P.nx);
 #pragma unroll
       for (int q = 0; q < RU; ++q) l.v[q] += in.c[j] * k[q];
     }
     return l;
   }
-  __device__ __forceinline__ void apply(const Ld& l, int c, int j, long long, long long r, const Q<T>&, Q<T>& out) {
+  __device__ __forceinline__ void apply(const Ld& l, int c, Q<T>*, int, int r, const Q<T>&, Q<T>& out) {
 #pragma unroll
     for (int q = 0; q < RU; ++q) {
-      if (in.ynew) in.ynew[c * this->P.ncell + r + (long long)q * this->P.nx] = l.v[q];
+      if (in.ynew) in.ynew[c * this->P.ncell + r + q * this->P.nx] = l.v[q];
       out.v[q] = (T)l.v[q];
-      if constexpr (KIM) h2[j][q] = l.v[q] * l.v[q] + (c == 0 ? 0.0 : h2[j][q]);
-    }
-  }
-  __device__ __forceinline__ void done(long long i, int q) {
-    if constexpr (KIM) {
-#pragma unroll
-      for (int j = 0; j < E; ++j) {
-        const int m = this->msk(i + (long long)j * q);
-#pragma unroll
-        for (int w = 0; w < RU; ++w)
-          if (cls(m, w) == 1) this->P.hd[(i + (long long)j * q) * RU + w] = (T)sqrt(h2[j][w]);
-      }
     }
   }
 };
-template <typename T, int E> using BStage = BStageT<T, E, false>;
-template <typename T, int E> using BStageKim = BStageT<T, E, true>;
+// The same with a field-dependent critical current: the stage field's magnitude |h| is kept, in the
+// transform precision, in the first component of the h_dot iterate at superconductor cells: those entries
+// are rewritten by BInit before anything reads them as an iterate, and the warm start lives on free space
+// only.  (The sum of squares in FP64, from all three components with the last one.)
+template <typename T, int E>
+struct BStageKim : BStage<T, E> {
+  static constexpr int RU = Lane<T>::RU, kBatch = 1;
+  using Ld = typename BStage<T, E>::Ld;
+  __device__ __forceinline__ void apply(const Ld& l, int c, Q<T>* s, int i, int r, const Q<T>& in, Q<T>& out) {
+    BStage<T, E>::apply(l, c, s, i, r, in, out);
+    if (c < 2) return;
+    const int m = this->msk(i);
+#pragma unroll
+    for (int q = 0; q < RU; ++q) {
+      if (cls(m, q) != 1) continue;
+      const int o = r + q * this->P.nx;
+      const double a = this->value(o), b = this->value(this->P.ncell + o);
+      this->P.hd[i * RU + q] = (T)sqrt(a * a + b * b + l.v[q] * l.v[q]);
+    }
+  }
+};
 
 // j -> e (Eq. 13 / Ohm law): critical current jc, per cell or Kim-type jc / (1 + |h|/b0) when ib0 > 0
 // (|h| left by BStageKim), and the elliptic weight 1/gamma^2 of j_z
 template <typename T>
 struct BLaw : BEpi<T> {
-  static constexpr int RU = Lane<T>::RU, kBatch = 2;
+  static constexpr int RU = Lane<T>::RU, kBatch = 1;
   static constexpr bool kJoint = true;
   T n, e0, jc, rho_out, ig2, ib0;
   struct Ld { int m; Q<T> jc, h; };
-  __device__ __forceinline__ Ld load(long long i, long long) const {
+  __device__ __forceinline__ Ld load(int i, int) const {
     Ld l;
     l.m = this->msk(i);
     if (this->P.jcmap) {
@@ -521,36 +569,36 @@ struct BLaw : BEpi<T> {
 template <typename T, int E>
 struct BPower : BLaw<T> {
   using Ld = typename BLaw<T>::Ld;
-  __device__ __forceinline__ void apply(const Ld& l, int, int, long long, const Q<T>* in, Q<T>* out) { this->law(l, in, out); }
+  __device__ __forceinline__ void apply(const Ld& l, int, int, int, const Q<T>* in, Q<T>* out) { this->law(l, in, out); }
 };
 template <typename T, int E>
 struct BStoreE : BLaw<T> {                 // readout of e (FP64)
   using Ld = typename BLaw<T>::Ld;
   double* out;
-  __device__ __forceinline__ void apply(const Ld& l, int, int, long long r, const Q<T>* in, Q<T>*) {
+  __device__ __forceinline__ void apply(const Ld& l, int, int, int r, const Q<T>* in, Q<T>*) {
     Q<T> e[3];
     this->law(l, in, e);
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
 #pragma unroll
-      for (int q = 0; q < Lane<T>::RU; ++q) out[c * this->P.ncell + r + (long long)q * this->P.nx] = e[c].v[q];
+      for (int q = 0; q < Lane<T>::RU; ++q) out[c * this->P.ncell + r + q * this->P.nx] = e[c].v[q];
     }
   }
 };
 
 template <typename T, int E>
 struct BInit : BEpi<T> {                   // h_dot^0: h_dot_in on the conductor, warm or h_e_dot outside
-  static constexpr int RU = Lane<T>::RU;
+  static constexpr int RU = Lane<T>::RU, kBatch = 2;
   bool warm;
   T hed[3];
   struct Ld { int m; Q<T> w; };
-  __device__ __forceinline__ Ld load(int c, long long i, long long) const {
+  __device__ __forceinline__ Ld load(int c, int i, int) const {
     Ld l;
     l.m = this->msk(i);
     if (warm) l.w = ld_q(this->P.hd + (c * this->P.ncell + i * RU));
     return l;
   }
-  __device__ __forceinline__ void apply(const Ld& l, int c, int, long long i, long long, const Q<T>& in, Q<T>& out) {
+  __device__ __forceinline__ void apply(const Ld& l, int c, Q<T>*, int i, int, const Q<T>& in, Q<T>& out) {
     const T he = c == 0 ? hed[0] : c == 1 ? hed[1] : hed[2];
 #pragma unroll
     for (int q = 0; q < RU; ++q) out.v[q] = cls(l.m, q) != 0 ? in.v[q] : warm ? l.w.v[q] : he;   // -curl e (Eq. 14)
@@ -561,8 +609,8 @@ struct BInit : BEpi<T> {                   // h_dot^0: h_dot_in on the conductor
 template <typename T, int E>
 struct BMaskCond : BEpi<T> {               // j_dot_in: keep on the conductor only
   struct Ld { int m; };
-  __device__ __forceinline__ Ld load(int, long long i, long long) const { return Ld{this->msk(i)}; }
-  __device__ __forceinline__ void apply(const Ld& l, int, int, long long, long long, const Q<T>& in, Q<T>& out) {
+  __device__ __forceinline__ Ld load(int, int i, int) const { return Ld{this->msk(i)}; }
+  __device__ __forceinline__ void apply(const Ld& l, int, Q<T>*, int, int, const Q<T>& in, Q<T>& out) {
 #pragma unroll
     for (int q = 0; q < Lane<T>::RU; ++q) out.v[q] = cls(l.m, q) != 0 ? in.v[q] : (T)0;
   }
@@ -572,13 +620,15 @@ template <typename T, int E>
 struct BUpdate : BEpi<T> {                 // Eq. 18 on free space, residual, forward
   static constexpr int RU = Lane<T>::RU, kBatch = 2;
   T hed[3];
-  T s[E][RU];                              // |h_dot^{i+1} - h_dot^i|^2 of the thread's cells, over the components
   struct Ld { int m; Q<T> h; };
-  __device__ __forceinline__ Ld load(int c, long long i, long long) const {
+  __device__ __forceinline__ Ld load(int c, int i, int) const {
     return Ld{this->msk(i), ld_q(this->P.hd + (c * this->P.ncell + i * RU))};
   }
-  __device__ __forceinline__ void apply(const Ld& l, int c, int j, long long i, long long, const Q<T>& in, Q<T>& out) {
+  // s: |h_dot^{i+1} - h_dot^i|^2 of the element's cells over the components so far
+  __device__ __forceinline__ void apply(const Ld& l, int c, Q<T>* s, int i, int, const Q<T>& in, Q<T>& out) {
     const T he = c == 0 ? hed[0] : c == 1 ? hed[1] : hed[2];
+    Q<T> e2;
+    if (c > 0) e2 = *s;
     out = l.h;
     bool any = false;
 #pragma unroll
@@ -590,16 +640,11 @@ struct BUpdate : BEpi<T> {                 // Eq. 18 on free space, residual, fo
         out.v[q] = n;
         any = true;
       }
-      s[j][q] = c == 0 ? e * e : s[j][q] + e * e;
+      e2.v[q] = c == 0 ? e * e : e2.v[q] + e * e;
+      if (c == 2) this->acc[0] += sqrt(e2.v[q]);
     }
     if (any) st_q(this->P.hd + (c * this->P.ncell + i * RU), out);
-  }
-  __device__ __forceinline__ void done(long long, int) {
-#pragma unroll
-    for (int j = 0; j < E; ++j) {
-#pragma unroll
-      for (int q = 0; q < RU; ++q) this->acc[0] += sqrt(s[j][q]);
-    }
+    if (c < 2) *s = e2;
   }
 };
 
@@ -610,24 +655,24 @@ struct BFinalT : BEpi<T, 1, true> {        // h_dot out (FP64); optional BS23 er
   double h, rtol, atol;
   const double* k1; const double* k2; const double* k3; const double* y; const double* ynew;
   struct Ld { Q<T> g; double a1[NE], a2[NE], a3[NE], y[NE], yn[NE]; };
-  __device__ __forceinline__ Ld load(int c, long long i, long long r) const {
+  __device__ __forceinline__ Ld load(int c, int i, int r) const {
     Ld l;
     l.g = ld_q(this->P.hd + (c * this->P.ncell + i * RU));
     if constexpr (err) {
 #pragma unroll
       for (int q = 0; q < RU; ++q) {
-        const long long o = c * this->P.ncell + r + (long long)q * this->P.nx;
+        const int o = c * this->P.ncell + r + q * this->P.nx;
         l.a1[q] = ld_s(k1 + o); l.a2[q] = ld_s(k2 + o); l.a3[q] = ld_s(k3 + o);
         l.y[q] = ld_s(y + o); l.yn[q] = ld_s(ynew + o);
       }
     }
     return l;
   }
-  __device__ __forceinline__ void apply(const Ld& l, int c, int, long long, long long r, const Q<T>&, Q<T>&) {
+  __device__ __forceinline__ void apply(const Ld& l, int c, Q<T>*, int, int r, const Q<T>&, Q<T>&) {
 #pragma unroll
     for (int q = 0; q < RU; ++q) {
       const double g = (double)l.g.v[q];
-      kout[c * this->P.ncell + r + (long long)q * this->P.nx] = g;
+      kout[c * this->P.ncell + r + q * this->P.nx] = g;
       if constexpr (err) {
         const double E_ = h * (-5.0 / 72.0 * l.a1[q] + 1.0 / 12.0 * l.a2[q] + 1.0 / 9.0 * l.a3[q] - 0.125 * g);
         const double sc = atol + rtol * fmax(fabs(l.y[q]), fabs(l.yn[q]));
@@ -649,10 +694,10 @@ template <typename T, int E>
 struct BStoreJ : BEpi<T> {                 // readout of j = curl h (FP64)
   double* out;
   using Ld = NoLd;
-  __device__ __forceinline__ Ld load(int, long long, long long) const { return Ld{}; }
-  __device__ __forceinline__ void apply(const Ld&, int c, int, long long, long long r, const Q<T>& in, Q<T>&) {
+  __device__ __forceinline__ Ld load(int, int, int) const { return Ld{}; }
+  __device__ __forceinline__ void apply(const Ld&, int c, Q<T>*, int, int r, const Q<T>& in, Q<T>&) {
 #pragma unroll
-    for (int q = 0; q < Lane<T>::RU; ++q) out[c * this->P.ncell + r + (long long)q * this->P.nx] = in.v[q];
+    for (int q = 0; q < Lane<T>::RU; ++q) out[c * this->P.ncell + r + q * this->P.nx] = in.v[q];
   }
 };
 
@@ -664,8 +709,8 @@ struct BMoment : BEpi<T, 3> {              // m = 1/2 sum dV r x j over the cond
   double Lx, Ly, Lz, dx, dy, dz;
   struct Ld { int m; };
   __device__ __forceinline__ void reset() { acc[0] = acc[1] = acc[2] = 0.0; }
-  __device__ __forceinline__ Ld load(long long i, long long) const { return Ld{this->msk(i)}; }
-  __device__ __forceinline__ void apply(const Ld& l, int x, int unit, long long, const Q<T>* in, Q<T>*) {
+  __device__ __forceinline__ Ld load(int i, int) const { return Ld{this->msk(i)}; }
+  __device__ __forceinline__ void apply(const Ld& l, int x, int unit, int, const Q<T>* in, Q<T>*) {
     if (l.m == 0) return;
     const int row = unit * RU, z = row / this->P.ny, y0 = row - z * this->P.ny;
     const double rx = -Lx + (x + 0.5) * dx, rz = -Lz + (z + 0.5) * dz;
@@ -803,7 +848,7 @@ __global__ void __launch_bounds__(NT, 2) bulk_kernel(const Desc* __restrict__ dg
       to += n;
     };
     copy(d.tw_x, core_table_len(d.lgx, d.ex));
-    copy(d.tw_y, core_table_len(d.lgy, d.ey));
+    if (!one_table(d)) copy(d.tw_y, core_table_len(d.lgy, d.ey));
     copy(d.tw_z, core_table_len(d.lgz, d.ez));
   }
   __syncthreads();

@@ -290,33 +290,53 @@ __host__ __device__ constexpr int core_table_len(int lg, int E) {
   for (int rem = lg - e; rem > 0; rem -= e, lgp += e) n += rem >= e ? e << lgp : rem << (lg - e);
   return n;
 }
+// Elements from one line's exchange buffer to the next when 2^lgG lines are interleaved on the lanes: the
+// padded length (one spare slot per 8, or per 16 with radix 16), and 8 / lines more where that is a
+// multiple of 4, so that the lines of 8 neighbouring lanes lie on distinct banks.
+__host__ __device__ constexpr int line_stride(int lg, int lgG, int E) {
+  return (1 << lg) + ((1 << lg) >> (E == 16 ? 4 : 3)) + (lgG > 0 && lg >= 5 ? 8 >> lgG : 0);
+}
+// Rows of the real fields that a film's row passes keep together (mf_film.cuh)
+__host__ __device__ constexpr int row_unit(int precision) { return precision ? 4 : 2; }
 // a film's shared memory: the exchange buffer's elements, then the tables (one if the axes agree)
 __host__ __device__ constexpr int slots_of(int E) { return NT * E + (NT * E >> (E == 16 ? 4 : 3)); }
 __host__ __device__ inline int film_slots(const Desc& d) { return slots_of(d.ex > d.ey ? d.ex : d.ey); }
-__host__ __device__ inline bool film_one_table(const Desc& d) { return d.lgx == d.lgy && d.ex == d.ey; }
+__host__ __device__ inline bool one_table(const Desc& d) { return d.lgx == d.lgy && d.ex == d.ey; }
 // the most that any film needs (what the kernels' attribute is set to, whatever is launched first)
 constexpr size_t FILM_SMEM_MAX = 16 * ((size_t)slots_of(8) + 2 * core_table_len(11, 8));
 inline size_t film_smem_bytes(const Desc& d) {
-  return 16 * ((size_t)film_slots(d) + core_table_len(d.lgx, d.ex) + (film_one_table(d) ? 0 : core_table_len(d.lgy, d.ey)));
+  return 16 * ((size_t)film_slots(d) + core_table_len(d.lgx, d.ex) + (one_table(d) ? 0 : core_table_len(d.lgy, d.ey)));
 }
-// A bulk body's z pass runs 2^z_group_lg neighbouring lines per group (mf_bulk.cu), 4 where the CTA holds
-// so many; its shared memory: the widest pass's exchange buffer, then the three tables.
+// A bulk body's passes (mf_bulk.cu).  The z pass runs 2^z_group_lg neighbouring lines per group, 4 where
+// the CTA holds so many; the x pass interleaves up to 4 of an item's row units (of one z): 128
+// contiguous bytes per kx.
 __host__ __device__ constexpr int z_group_lg(int lgz, int ez) {
   const int lines = (NT * ez) >> lgz;
   return lines >= 4 ? 2 : lines >= 2 ? 1 : 0;
 }
+__host__ __device__ inline int x_group_lg(const Desc& d) {
+  const int ru = row_unit(d.precision), ub = d.rows_per_item / ru, up = d.ny / ru;
+  const int m = ub < up ? ub : up;
+  return m >= 4 ? 2 : m >= 2 ? 1 : 0;
+}
+// Shared memory of the passes (16-byte elements): the exchange buffers, the staging buffer behind them
+// (x: E per thread and two per line; y: E per thread; z: 3 E per thread), in the x pass E per thread for
+// partial residuals; the tables follow the largest of the three.
+__host__ __device__ constexpr int x_slots(int lgx, int ex) { return ((NT * ex) >> lgx) * line_stride(lgx, 2, ex); }
+__host__ __device__ constexpr int x_stage(int lgx, int ex) { return NT * ex + 2 * ((NT * ex) >> lgx); }
 __host__ __device__ constexpr int z_slots(int lgz, int ez) {
-  return 3 * ((NT * ez) >> lgz) * ((1 << lgz) + ((1 << lgz) >> 3) + (8 >> z_group_lg(lgz, ez)));
+  return 3 * ((NT * ez) >> lgz) * line_stride(lgz, z_group_lg(lgz, ez), ez);
 }
 __host__ __device__ inline int bulk_slots(const Desc& d) {
-  const int xy = slots_of(d.ex > d.ey ? d.ex : d.ey), z = z_slots(d.lgz, d.ez);
-  return xy > z ? xy : z;
+  const int x = x_slots(d.lgx, d.ex) + x_stage(d.lgx, d.ex) + NT * d.ex;
+  const int y = slots_of(d.ey) + NT * d.ey, z = z_slots(d.lgz, d.ez) + 3 * NT * d.ez;
+  const int m = x > y ? x : y;
+  return m > z ? m : z;
 }
-constexpr size_t BULK_SMEM_MAX = 16 * ((size_t)slots_of(16) + 3 * 512);
+constexpr size_t BULK_SMEM_MAX = 128 << 10;
 inline size_t bulk_smem_bytes(const Desc& d) {
-  return 16 * ((size_t)bulk_slots(d) + core_table_len(d.lgx, d.ex) + core_table_len(d.lgy, d.ey) + core_table_len(d.lgz, d.ez));
+  return 16 * ((size_t)bulk_slots(d) + core_table_len(d.lgx, d.ex) +
+               (one_table(d) ? 0 : core_table_len(d.lgy, d.ey)) + core_table_len(d.lgz, d.ez));
 }
-// Rows of the real fields that a film's row passes keep together (mf_film.cuh)
-constexpr int row_unit(int precision) { return precision ? 4 : 2; }
 
 }  // namespace mf

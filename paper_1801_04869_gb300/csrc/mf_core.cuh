@@ -226,27 +226,32 @@ __device__ __forceinline__ void dft_stage(CV<V>* x, const CV<V>* w) {
 // ------------------------------------------------------------------------------------------
 __host__ __device__ constexpr int lg_of(int E) { return E == 2 ? 1 : E == 4 ? 2 : E == 8 ? 3 : 4; }
 
-// Lines of up to 32 threads lie inside a warp; longer ones (2, 4 or 8 warps) have a named
-// barrier each, so that the lines of a CTA do not wait for one another.
+// A group of G = 2^lgG lines (neighbours in memory) is interleaved on the lanes: thread i of line u is
+// thread (i << lgG) + u of the group, so that a warp moves G neighbouring values per position.  A group
+// of up to 32 threads lies inside a warp; longer ones (2, 4 or 8 warps) have a named barrier each, so
+// that the groups of a CTA do not wait for one another.
 template <typename T, int E> struct Team {
   using V = typename Lane<T>::V;
   static constexpr int LGE = lg_of(E);
   CV<V>* s;              // the line's part of the shared buffer
   const CV<V>* tw;       // twiddle table of this length and radix (shared memory)
-  int i, lg, slot;       // thread of the line; log2 of its length; line of the CTA
-  static constexpr int fs = 0;
-  __device__ __forceinline__ Team(CV<V>* buf, const CV<V>* table, int lgL) : tw(table), lg(lgL) {
-    const int lgt = lg - LGE;
-    slot = (int)threadIdx.x >> lgt;
-    i = (int)threadIdx.x & ((1 << lgt) - 1);
-    s = buf + slot * spe<E>(1 << lg);
+  int i, u, slot;        // thread of the line; line of the group; line of the CTA
+  int lg, lgt, fs;       // log2 of the length and of the group's threads; buffer elements per field
+  __device__ __forceinline__ Team(CV<V>* buf, const CV<V>* table, int lgL, int lgG = 0) : tw(table), lg(lgL) {
+    lgt = lg - LGE + lgG;
+    u = (int)threadIdx.x & ((1 << lgG) - 1);
+    i = ((int)threadIdx.x >> lgG) & ((1 << (lg - LGE)) - 1);
+    slot = (((int)threadIdx.x >> lgt) << lgG) + u;
+    const int stride = line_stride(lg, lgG, E);
+    s = buf + slot * stride;
+    fs = ((NT >> lgt) << lgG) * stride;
   }
   __device__ __forceinline__ int threads() const { return 1 << (lg - LGE); }
   __device__ __forceinline__ int step() const { return 1 << (lg - LGE); }    // position stride of a thread's elements
   __device__ __forceinline__ CV<V>& at(int e) const { return s[spe<E>(e)]; }
   __device__ __forceinline__ void sync() const {
-    if (lg - LGE <= 5) __syncwarp();
-    else asm volatile("bar.sync %0, %1;" :: "r"(1 + slot), "r"(1 << (lg - LGE)) : "memory");
+    if (lgt <= 5) __syncwarp();
+    else asm volatile("bar.sync %0, %1;" :: "r"(1 + ((int)threadIdx.x >> lgt)), "r"(1 << lgt) : "memory");
   }
 };
 

@@ -58,7 +58,7 @@ struct Film {
   CV<V>* sm;         // the CTA's exchange buffer
   Shared& sh;
   int nx, ny, lgx, lgy, half, nkx;
-  long long nspec, ncell;
+  int nspec, ncell;
   C2<T>* Sa;
   C2<T>* Sb;
   T* hd;
@@ -84,15 +84,15 @@ struct Film {
   __device__ Film(const Desc& dd, unsigned char* smem, Shared& shr, int vblock, unsigned nblk)
       : d(dd), sm((CV<V>*)smem), sh(shr) {
     nx = d.nx; ny = d.ny; lgx = d.lgx; lgy = d.lgy; half = nx / 2; nkx = half + 1;
-    nspec = (long long)nkx * ny;
-    ncell = (long long)nx * ny;
+    nspec = nkx * ny;
+    ncell = nx * ny;
     Sa = (C2<T>*)d.Sa; Sb = (C2<T>*)d.Sb;
     hd = (T*)d.hd; u = (T*)d.u; q1 = (const T*)d.q1; q2 = (const T*)d.q2;
     mask = d.mask; jcmap = (const T*)d.jcmap;
     ex = d.ex; ey = d.ey;
     const int slots = film_slots(d);
     twx = sm + slots;
-    twy = film_one_table(d) ? twx : twx + core_table_len(lgx, ex);
+    twy = one_table(d) ? twx : twx + core_table_len(lgx, ex);
     max_items = d.max_items;
     partials = d.partials;
     gb = d.gb;
@@ -162,7 +162,7 @@ struct Film {
   template <int E, int NIN, int NOUT>
   __device__ __noinline__ void cols_e(const C2<T>* Sin, C2<T>* Sout, int op) {
     const int ny = this->ny;
-    const long long nspec = this->nspec;
+    const int nspec = this->nspec;
     Team<T, E> t(sm, twy, lgy);
     const int units = (nkx + NL - 1) / NL;
     const int per = NT / t.threads();
@@ -176,8 +176,8 @@ struct Film {
       const bool mine = t.slot < nuc && u0 + t.slot < units;
       const int kx = mine ? (u0 + t.slot) * NL : 0;
       const bool two = NL == 2 && kx + 1 < nkx;
-      const C2<T>* const src = Sin + (long long)kx * ny + t.i;
-      C2<T>* const dst = Sout + (long long)kx * ny + t.i;
+      const C2<T>* const src = Sin + kx * ny + t.i;
+      C2<T>* const dst = Sout + kx * ny + t.i;
       const Coef c = coef_x(kx);
       CV<V> v[E];
 #pragma unroll
@@ -282,7 +282,7 @@ struct Film {
   __device__ __noinline__ void rows_e(const C2<T>* Sin, C2<T>* Sout, const Epi& epi_in, int slot, int slot2, T* tmp) {
     Epi epi = epi_in;                   // register copy of the epilogue
     const int nx = this->nx, ny = this->ny;
-    const long long nspec = this->nspec;
+    const int nspec = this->nspec;
     Team<T, E> t(sm, twx, lgx);
     const int q = t.step(), tt = t.threads();
     const int units = ny / RU;
@@ -294,8 +294,8 @@ struct Film {
       const bool mine = t.slot < nuc && u0 + t.slot < units;
       const int unit = mine ? u0 + t.slot : u0;
       const int y0 = unit * RU;
-      const long long iu = (long long)unit * nx + t.i;
-      const long long ir = (long long)y0 * nx + t.i;
+      const int iu = unit * nx + t.i;
+      const int ir = y0 * nx + t.i;
       epi.acc = 0;
       epi.accmax = 0;
       epi.acc2 = 0;
@@ -332,7 +332,7 @@ struct Film {
           for (int b = 0; b < B; ++b) {
             const int j = j0 + b;
             Q<T> in[NIN > 0 ? NIN : 1], out[NOUT > 0 ? NOUT : 1];
-            const long long i = iu + j * q;
+            const int i = iu + j * q;
             if constexpr (NIN == 2) { in[0] = in0[b]; in[1] = to_q(v[j]); }
             if constexpr (NIN == 1) in[0] = to_q(v[j]);
             epi.apply(ld[(j0 / B) & 1][b], i, ir + j * q, in, out);
@@ -495,23 +495,23 @@ struct EpiStage : EpiBase<T> {
   StageIn in;
   static constexpr int kBatch = 2;
   struct Ld { double v[RU]; };
-  __device__ __forceinline__ Ld load(long long, long long r) const {
+  __device__ __forceinline__ Ld load(int, int r) const {
     Ld l;
 #pragma unroll
-    for (int q = 0; q < RU; ++q) l.v[q] = ld_s(in.y + r + (long long)q * P.nx);
+    for (int q = 0; q < RU; ++q) l.v[q] = ld_s(in.y + r + q * P.nx);
     for (int j = 0; j < in.nk; ++j) {
       double k[RU];
 #pragma unroll
-      for (int q = 0; q < RU; ++q) k[q] = ld_s(in.k[j] + r + (long long)q * P.nx);
+      for (int q = 0; q < RU; ++q) k[q] = ld_s(in.k[j] + r + q * P.nx);
 #pragma unroll
       for (int q = 0; q < RU; ++q) l.v[q] += in.c[j] * k[q];
     }
     return l;
   }
-  __device__ __forceinline__ void apply(const Ld& l, long long, long long r, const Q<T>*, Q<T>* out) {
+  __device__ __forceinline__ void apply(const Ld& l, int, int r, const Q<T>*, Q<T>* out) {
     if (in.ynew) {
 #pragma unroll
-      for (int q = 0; q < RU; ++q) in.ynew[r + (long long)q * P.nx] = l.v[q];
+      for (int q = 0; q < RU; ++q) in.ynew[r + q * P.nx] = l.v[q];
     }
 #pragma unroll
     for (int q = 0; q < RU; ++q) out[0].v[q] = (T)l.v[q];
@@ -524,8 +524,8 @@ struct EpiOut : EpiBase<T> {
   FilmPtrs<T> P;
   static constexpr int kBatch = 4;
   struct Ld { int m; };
-  __device__ __forceinline__ Ld load(long long i, long long) const { return Ld{ld_mask(P.mask + i)}; }
-  __device__ __forceinline__ void apply(const Ld& l, long long, long long, const Q<T>*, Q<T>* out) {
+  __device__ __forceinline__ Ld load(int i, int) const { return Ld{ld_mask(P.mask + i)}; }
+  __device__ __forceinline__ void apply(const Ld& l, int, long long, const Q<T>*, Q<T>* out) {
 #pragma unroll
     for (int q = 0; q < Lane<T>::RU; ++q) out[0].v[q] = cls(l.m, q) == 0 ? (T)1 : (T)0;
   }
@@ -538,8 +538,8 @@ struct EpiStoreT : EpiBase<T> {
   T* dst;
   static constexpr int kBatch = 4;
   struct Ld { int m; };
-  __device__ __forceinline__ Ld load(long long i, long long) const { return Ld{ld_mask(P.mask + i)}; }
-  __device__ __forceinline__ void apply(const Ld& l, long long i, long long, const Q<T>* in, Q<T>*) {
+  __device__ __forceinline__ Ld load(int i, int) const { return Ld{ld_mask(P.mask + i)}; }
+  __device__ __forceinline__ void apply(const Ld& l, int i, int, const Q<T>* in, Q<T>*) {
     st_q(dst + i * Lane<T>::RU, in[0]);
 #pragma unroll
     for (int q = 0; q < Lane<T>::RU; ++q)
@@ -554,10 +554,10 @@ struct EpiStoreHz : EpiBase<T> {
   double he;
   static constexpr int kBatch = 4;
   using Ld = NoLd;
-  __device__ __forceinline__ Ld load(long long, long long) const { return Ld{}; }
-  __device__ __forceinline__ void apply(const Ld&, long long, long long r, const Q<T>* in, Q<T>*) {
+  __device__ __forceinline__ Ld load(int, int) const { return Ld{}; }
+  __device__ __forceinline__ void apply(const Ld&, int, int r, const Q<T>* in, Q<T>*) {
 #pragma unroll
-    for (int q = 0; q < Lane<T>::RU; ++q) dst[r + (long long)q * P.nx] = he + (double)in[0].v[q];
+    for (int q = 0; q < Lane<T>::RU; ++q) dst[r + q * P.nx] = he + (double)in[0].v[q];
   }
 };
 
@@ -570,7 +570,7 @@ struct EpiPower : EpiBase<T> {
   T n, e0, jc, rho_out, ig2;
   static constexpr int kBatch = 4;
   struct Ld { int m; Q<T> jc; };
-  __device__ __forceinline__ Ld load(long long i, long long) const {
+  __device__ __forceinline__ Ld load(int i, int) const {
     Ld l;
     l.m = ld_mask(P.mask + i);
     if (P.jcmap) {
@@ -581,7 +581,7 @@ struct EpiPower : EpiBase<T> {
     }
     return l;
   }
-  __device__ __forceinline__ void apply(const Ld& l, long long, long long, const Q<T>* in, Q<T>* out) {
+  __device__ __forceinline__ void apply(const Ld& l, int, long long, const Q<T>* in, Q<T>* out) {
 #pragma unroll
     for (int q = 0; q < Lane<T>::RU; ++q) {
       const T gx = in[0].v[q], gy = in[1].v[q];
@@ -604,14 +604,14 @@ struct EpiInit : EpiBase<T, T> {
   T A_prev, hed;
   static constexpr int kBatch = 4;
   struct Ld { int m; Q<T> w, q1; };
-  __device__ __forceinline__ Ld load(long long i, long long) const {
+  __device__ __forceinline__ Ld load(int i, int) const {
     Ld l;
     l.m = ld_mask(P.mask + i);
     if (warm) l.w = ld_q(wsrc + i * Lane<T>::RU);
     l.q1 = ldg_q(P.q1 + i * Lane<T>::RU);
     return l;
   }
-  __device__ __forceinline__ void apply(const Ld& l, long long i, long long, const Q<T>* in, Q<T>* out) {
+  __device__ __forceinline__ void apply(const Ld& l, int i, int, const Q<T>* in, Q<T>* out) {
 #pragma unroll
     for (int q = 0; q < Lane<T>::RU; ++q) {
       T h;
@@ -634,10 +634,10 @@ struct EpiU : EpiBase<T, T> {
   T A, C;
   static constexpr int kBatch = 4;
   struct Ld { int m; Q<T> q1; };
-  __device__ __forceinline__ Ld load(long long i, long long) const {
+  __device__ __forceinline__ Ld load(int i, int) const {
     return Ld{ld_mask(P.mask + i), ldg_q(P.q1 + i * Lane<T>::RU)};
   }
-  __device__ __forceinline__ void apply(const Ld& l, long long i, long long, const Q<T>* in, Q<T>* out) {
+  __device__ __forceinline__ void apply(const Ld& l, int i, int, const Q<T>* in, Q<T>* out) {
     Q<T> v;
 #pragma unroll
     for (int q = 0; q < Lane<T>::RU; ++q) {
@@ -658,10 +658,10 @@ struct EpiUpdate : EpiBase<T, T> {
   T A;
   static constexpr int kBatch = 4;
   struct Ld { int m; Q<T> h, q1; };
-  __device__ __forceinline__ Ld load(long long i, long long) const {
+  __device__ __forceinline__ Ld load(int i, int) const {
     return Ld{ld_mask(P.mask + i), ld_q(P.hd + i * Lane<T>::RU), ldg_q(P.q1 + i * Lane<T>::RU)};
   }
-  __device__ __forceinline__ void apply(const Ld& l, long long i, long long, const Q<T>* in, Q<T>* out) {
+  __device__ __forceinline__ void apply(const Ld& l, int i, int, const Q<T>* in, Q<T>* out) {
     Q<T> h = l.h;
 #pragma unroll
     for (int q = 0; q < Lane<T>::RU; ++q) {
@@ -684,26 +684,26 @@ struct EpiFinal : EpiBase<T, T> {
   const double* k1; const double* k2; const double* k3; const double* y; const double* ynew;
   static constexpr int RU = Lane<T>::RU, NE = err ? RU : 1, kBatch = err ? 1 : 4;
   struct Ld { int m; Q<T> u; double a1[NE], a2[NE], a3[NE], y[NE], yn[NE]; };
-  __device__ __forceinline__ Ld load(long long i, long long r) const {
+  __device__ __forceinline__ Ld load(int i, int r) const {
     Ld l;
     l.m = ld_mask(P.mask + i);
     l.u = ld_q(P.u + i * RU);                              // defined on the conductor's units only
     if constexpr (err) {
 #pragma unroll
       for (int q = 0; q < RU; ++q) {
-        const long long c = r + (long long)q * P.nx;
+        const int c = r + q * P.nx;
         l.a1[q] = ld_s(k1 + c); l.a2[q] = ld_s(k2 + c); l.a3[q] = ld_s(k3 + c);
         l.y[q] = ld_s(y + c); l.yn[q] = ld_s(ynew + c);
       }
     }
     return l;
   }
-  __device__ __forceinline__ void apply(const Ld& l, long long, long long r, const Q<T>*, Q<T>*) {
+  __device__ __forceinline__ void apply(const Ld& l, int, int r, const Q<T>*, Q<T>*) {
 #pragma unroll
     for (int q = 0; q < RU; ++q) {
       const bool in = cls(l.m, q) != 0;
       const double g = in ? (double)l.u.v[q] : 0.0;
-      kout[r + (long long)q * P.nx] = g;
+      kout[r + q * P.nx] = g;
       if constexpr (err) {
         const double E = h * (-5.0 / 72.0 * l.a1[q] + 1.0 / 12.0 * l.a2[q] + 1.0 / 9.0 * l.a3[q] - 0.125 * g);
         const double sc = atol + rtol * fmax(fabs(l.y[q]), fabs(l.yn[q]));
@@ -729,7 +729,7 @@ struct EpiStoreE : EpiBase<T> {
   FilmPtrs<T> P;
   T n, e0, jc, rho_out, ig2;
   double* dst;
-  long long ncell;
+  int ncell;
   static constexpr int kBatch = 4;
   using Ld = typename EpiPower<T>::Ld;
   __device__ __forceinline__ EpiPower<T> law() const {       // the law of P3
@@ -737,14 +737,14 @@ struct EpiStoreE : EpiBase<T> {
     p.P = P; p.n = n; p.e0 = e0; p.jc = jc; p.rho_out = rho_out; p.ig2 = ig2;
     return p;
   }
-  __device__ __forceinline__ Ld load(long long i, long long r) const { return law().load(i, r); }
-  __device__ __forceinline__ void apply(const Ld& l, long long i, long long r, const Q<T>* in, Q<T>*) {
+  __device__ __forceinline__ Ld load(int i, int r) const { return law().load(i, r); }
+  __device__ __forceinline__ void apply(const Ld& l, int i, int r, const Q<T>* in, Q<T>*) {
     Q<T> e[2];
     law().apply(l, i, r, in, e);
 #pragma unroll
     for (int q = 0; q < Lane<T>::RU; ++q) {
-      dst[r + (long long)q * P.nx] = (double)e[0].v[q];
-      dst[ncell + r + (long long)q * P.nx] = (double)e[1].v[q];
+      dst[r + q * P.nx] = (double)e[0].v[q];
+      dst[ncell + r + q * P.nx] = (double)e[1].v[q];
     }
   }
 };
@@ -756,13 +756,13 @@ struct EpiMoment : EpiBase<T> {
   const double* g;
   static constexpr int kBatch = 4;
   struct Ld { double v[Lane<T>::RU]; };
-  __device__ __forceinline__ Ld load(long long, long long r) const {
+  __device__ __forceinline__ Ld load(int, int r) const {
     Ld l;
 #pragma unroll
-    for (int q = 0; q < Lane<T>::RU; ++q) l.v[q] = ld_s(g + r + (long long)q * P.nx);
+    for (int q = 0; q < Lane<T>::RU; ++q) l.v[q] = ld_s(g + r + q * P.nx);
     return l;
   }
-  __device__ __forceinline__ void apply(const Ld& l, long long, long long, const Q<T>*, Q<T>*) {
+  __device__ __forceinline__ void apply(const Ld& l, int, long long, const Q<T>*, Q<T>*) {
 #pragma unroll
     for (int q = 0; q < Lane<T>::RU; ++q) this->acc += l.v[q];
   }
@@ -922,7 +922,7 @@ __device__ __forceinline__ void film_tables(const Desc& d) {
   uint4* const to = (uint4*)mf_dsmem + film_slots(d);
   const uint4* const x = (const uint4*)d.tw_x;
   const uint4* const y = (const uint4*)d.tw_y;
-  const int nx = core_table_len(d.lgx, d.ex), ny = film_one_table(d) ? 0 : core_table_len(d.lgy, d.ey);
+  const int nx = core_table_len(d.lgx, d.ex), ny = one_table(d) ? 0 : core_table_len(d.lgy, d.ey);
   for (int k = threadIdx.x; k < nx; k += NT) to[k] = x[k];
   for (int k = threadIdx.x; k < ny; k += NT) to[nx + k] = y[k];
 }

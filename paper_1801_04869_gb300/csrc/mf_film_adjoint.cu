@@ -52,7 +52,7 @@ struct AdjArgs {
 template <typename T>
 __device__ __forceinline__ void ld_rows(double (&v)[Lane<T>::RU], const double* p, int nx) {
 #pragma unroll
-  for (int q = 0; q < Lane<T>::RU; ++q) v[q] = ld_s(p + (long long)q * nx);
+  for (int q = 0; q < Lane<T>::RU; ++q) v[q] = ld_s(p + q * nx);
 }
 
 // full product, V1: gbar_{I-1} = conductor * v (with its sum) and g, forward of both
@@ -63,14 +63,14 @@ struct EpiPT0g : EpiBase<T, T> {
   const double* g;
   static constexpr int kBatch = 2;
   struct Ld { int m; double x[Lane<T>::RU], y[Lane<T>::RU]; };
-  __device__ __forceinline__ Ld load(long long i, long long r) const {
+  __device__ __forceinline__ Ld load(int i, int r) const {
     Ld l;
     l.m = ld_mask(P.mask + i);
     ld_rows<T>(l.x, v + r, P.nx);
     ld_rows<T>(l.y, g + r, P.nx);
     return l;
   }
-  __device__ __forceinline__ void apply(const Ld& l, long long, long long, const Q<T>*, Q<T>* out) {
+  __device__ __forceinline__ void apply(const Ld& l, int, long long, const Q<T>*, Q<T>* out) {
 #pragma unroll
     for (int q = 0; q < Lane<T>::RU; ++q) {
       const T gb = cls(l.m, q) != 0 ? (T)l.x[q] : (T)0;
@@ -89,8 +89,8 @@ struct EpiStoreJ : EpiBase<T, T> {
   T* jy;
   static constexpr int kBatch = 4;
   using Ld = NoLd;
-  __device__ __forceinline__ Ld load(long long, long long) const { return Ld{}; }
-  __device__ __forceinline__ void apply(const Ld&, long long i, long long, const Q<T>* in, Q<T>*) {
+  __device__ __forceinline__ Ld load(int, int) const { return Ld{}; }
+  __device__ __forceinline__ void apply(const Ld&, int i, int, const Q<T>* in, Q<T>*) {
     Q<T> b;
 #pragma unroll
     for (int q = 0; q < Lane<T>::RU; ++q) b.v[q] = -in[0].v[q];
@@ -107,14 +107,14 @@ struct EpiRbar : EpiBase<T, T> {
   double* wdst;         // cotangent of the warm start (free space) or null
   static constexpr int kBatch = 4;
   struct Ld { int m; Q<T> h; };
-  __device__ __forceinline__ Ld load(long long i, long long) const {
+  __device__ __forceinline__ Ld load(int i, int) const {
     return Ld{ld_mask(P.mask + i), ld_q(P.hd + i * Lane<T>::RU)};
   }
-  __device__ __forceinline__ void apply(const Ld& l, long long, long long r, const Q<T>*, Q<T>* out) {
+  __device__ __forceinline__ void apply(const Ld& l, int, int r, const Q<T>*, Q<T>* out) {
 #pragma unroll
     for (int q = 0; q < Lane<T>::RU; ++q) {
       out[0].v[q] = cls(l.m, q) != 0 ? -(l.h.v[q] - t_q) : (T)0;
-      if (wdst) wdst[r + (long long)q * P.nx] = cls(l.m, q) == 0 ? (double)(l.h.v[q] - t_q) : 0.0;
+      if (wdst) wdst[r + q * P.nx] = cls(l.m, q) == 0 ? (double)(l.h.v[q] - t_q) : 0.0;
     }
   }
 };
@@ -132,7 +132,7 @@ struct EpiPowVJP : EpiBase<T, T> {
   T n, e0, jc, rho_out, ig2;
   static constexpr int kBatch = 2;
   struct Ld { int m; Q<T> ax, ay, jc; };
-  __device__ __forceinline__ Ld load(long long i, long long) const {
+  __device__ __forceinline__ Ld load(int i, int) const {
     Ld l;
     l.m = ld_mask(P.mask + i);
     l.ax = ld_q(jx + i * Lane<T>::RU);
@@ -145,7 +145,7 @@ struct EpiPowVJP : EpiBase<T, T> {
     }
     return l;
   }
-  __device__ __forceinline__ void apply(const Ld& l, long long, long long r, const Q<T>* in, Q<T>* out) {
+  __device__ __forceinline__ void apply(const Ld& l, int, int r, const Q<T>* in, Q<T>* out) {
 #pragma unroll
     for (int q = 0; q < Lane<T>::RU; ++q) {
       const T ex = in[1].v[q], ey = -in[0].v[q];                 // transposed -curl
@@ -169,7 +169,7 @@ struct EpiPowVJP : EpiBase<T, T> {
       }
       out[0].v[q] = bx;
       out[1].v[q] = by;
-      jcbar[r + (long long)q * P.nx] = c;
+      jcbar[r + q * P.nx] = c;
     }
   }
 };
@@ -181,10 +181,10 @@ struct EpiGbar : EpiBase<T, T> {
   double* dst;
   static constexpr int kBatch = 4;
   using Ld = NoLd;
-  __device__ __forceinline__ Ld load(long long, long long) const { return Ld{}; }
-  __device__ __forceinline__ void apply(const Ld&, long long, long long r, const Q<T>* in, Q<T>*) {
+  __device__ __forceinline__ Ld load(int, int) const { return Ld{}; }
+  __device__ __forceinline__ void apply(const Ld&, int, int r, const Q<T>* in, Q<T>*) {
 #pragma unroll
-    for (int q = 0; q < Lane<T>::RU; ++q) dst[r + (long long)q * P.nx] = -(double)in[0].v[q];
+    for (int q = 0; q < Lane<T>::RU; ++q) dst[r + q * P.nx] = -(double)in[0].v[q];
   }
 };
 
@@ -195,13 +195,13 @@ struct EpiPT0 : EpiBase<T, T> {
   const double* v;
   static constexpr int kBatch = 4;
   struct Ld { int m; double x[Lane<T>::RU]; };
-  __device__ __forceinline__ Ld load(long long i, long long r) const {
+  __device__ __forceinline__ Ld load(int i, int r) const {
     Ld l;
     l.m = ld_mask(P.mask + i);
     ld_rows<T>(l.x, v + r, P.nx);
     return l;
   }
-  __device__ __forceinline__ void apply(const Ld& l, long long, long long, const Q<T>*, Q<T>* out) {
+  __device__ __forceinline__ void apply(const Ld& l, int, long long, const Q<T>*, Q<T>* out) {
 #pragma unroll
     for (int q = 0; q < Lane<T>::RU; ++q) {
       const T g = cls(l.m, q) != 0 ? (T)l.x[q] : (T)0;
@@ -220,7 +220,7 @@ struct EpiPTh : EpiBase<T, T> {
   T s_q1;               // S / n_out
   static constexpr int kBatch = 4;
   struct Ld { int m; Q<T> q1, z; };
-  __device__ __forceinline__ Ld load(long long i, long long r) const {
+  __device__ __forceinline__ Ld load(int i, int r) const {
     Ld l;
     l.m = ld_mask(P.mask + i);
     l.q1 = ldg_q(P.q1 + i * Lane<T>::RU);
@@ -236,7 +236,7 @@ struct EpiPTh : EpiBase<T, T> {
     }
     return l;
   }
-  __device__ __forceinline__ void apply(const Ld& l, long long i, long long, const Q<T>* in, Q<T>* out) {
+  __device__ __forceinline__ void apply(const Ld& l, int i, int, const Q<T>* in, Q<T>* out) {
     Q<T> h;
 #pragma unroll
     for (int q = 0; q < Lane<T>::RU; ++q) {
@@ -257,10 +257,10 @@ struct EpiPTg : EpiBase<T, T> {
   T t_q;                // tot / n_out
   static constexpr int kBatch = 4;
   struct Ld { int m; Q<T> q2, h; };
-  __device__ __forceinline__ Ld load(long long i, long long) const {
+  __device__ __forceinline__ Ld load(int i, int) const {
     return Ld{ld_mask(P.mask + i), ldg_q(P.q2 + i * Lane<T>::RU), ld_q(P.hd + i * Lane<T>::RU)};
   }
-  __device__ __forceinline__ void apply(const Ld& l, long long i, long long, const Q<T>* in, Q<T>* out) {
+  __device__ __forceinline__ void apply(const Ld& l, int i, int, const Q<T>* in, Q<T>* out) {
     Q<T> h = l.h;
 #pragma unroll
     for (int q = 0; q < Lane<T>::RU; ++q) {
@@ -282,15 +282,15 @@ struct EpiPTout : EpiBase<T, T> {
   T t_q;
   static constexpr int kBatch = 4;
   struct Ld { int m; Q<T> h; };
-  __device__ __forceinline__ Ld load(long long i, long long) const {
+  __device__ __forceinline__ Ld load(int i, int) const {
     return Ld{ld_mask(P.mask + i), ld_q(P.hd + i * Lane<T>::RU)};
   }
-  __device__ __forceinline__ void apply(const Ld& l, long long, long long r, const Q<T>*, Q<T>*) {
+  __device__ __forceinline__ void apply(const Ld& l, int, int r, const Q<T>*, Q<T>*) {
 #pragma unroll
     for (int q = 0; q < Lane<T>::RU; ++q) {
       const double x = (double)(l.h.v[q] - t_q);
-      dst[r + (long long)q * P.nx] = cls(l.m, q) != 0 ? x : 0.0;
-      if (wdst) wdst[r + (long long)q * P.nx] = cls(l.m, q) == 0 ? x : 0.0;
+      dst[r + q * P.nx] = cls(l.m, q) != 0 ? x : 0.0;
+      if (wdst) wdst[r + q * P.nx] = cls(l.m, q) == 0 ? x : 0.0;
     }
   }
 };

@@ -77,8 +77,7 @@ inline void bulk_shape(Desc& d, int coresident) {
   const bool f32 = d.precision != 0;
   const bool small = d.ncell <= (f32 ? 262144 : 65536);
   d.ex = small ? (f32 ? 4 : 2) : 8;
-  const int ey = small ? 4 : f32 ? 16 : 8;
-  d.ey = d.ny < ey ? 4 : ey;
+  d.ey = small ? 4 : 8;
   d.ez = !f32 && small && d.nz <= 2 * NT ? 2 : 4;
   const int ru = row_unit(d.precision);
   const long long units = (long long)d.nz * d.ny / ru;

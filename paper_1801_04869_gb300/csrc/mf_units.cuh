@@ -16,7 +16,7 @@ namespace mf {
 // row units
 // ------------------------------------------------------------------------------------------
 // the RU rows of one element at one x: 16 bytes
-template <typename T> struct Q { T v[Lane<T>::RU]; };
+template <typename T> struct alignas(16) Q { T v[Lane<T>::RU]; };
 __device__ __forceinline__ Q<float> ld_q(const float* p) {
   Q<float> r;
   asm volatile("ld.global.L1::no_allocate.v4.f32 {%0, %1, %2, %3}, [%4];"
@@ -100,24 +100,24 @@ __device__ __forceinline__ void st_b32(C2<double>* p, const CV<double>& zk, cons
                :: "d"(zk.x + zm.x), "d"(zk.y - zm.y), "d"(zk.y + zm.y), "d"(zm.x - zk.x), "l"(p) : "memory");
 }
 // one column element: the values of line kx (and, in FP32, of line kx + 1 at `stride`)
-__device__ __forceinline__ CV<F2> ld_col(const C2<float>* p, long long stride, bool two) {
+__device__ __forceinline__ CV<F2> ld_col(const C2<float>* p, int stride, bool two) {
   const C2<float> a = lds_c2(p);
   C2<float> b = {0.f, 0.f};
   if (two) b = lds_c2(p + stride);
   return {pk(a.x, b.x), pk(a.y, b.y)};
 }
-__device__ __forceinline__ CV<double> ld_col(const C2<double>* p, long long, bool) {
+__device__ __forceinline__ CV<double> ld_col(const C2<double>* p, int, bool) {
   const C2<double> a = lds_c2(p);
   return {a.x, a.y};
 }
-__device__ __forceinline__ void st_col(C2<float>* p, long long stride, bool two, const CV<F2>& e) {
+__device__ __forceinline__ void st_col(C2<float>* p, int stride, bool two, const CV<F2>& e) {
   C2<float> a, b;
   upk(e.x, a.x, b.x);
   upk(e.y, a.y, b.y);
   p[0] = a;
   if (two) p[stride] = b;
 }
-__device__ __forceinline__ void st_col(C2<double>* p, long long, bool, const CV<double>& e) { p[0] = C2<double>{e.x, e.y}; }
+__device__ __forceinline__ void st_col(C2<double>* p, int, bool, const CV<double>& e) { p[0] = C2<double>{e.x, e.y}; }
 
 // FP64 state fields are row-major (the caller's layout)
 __device__ __forceinline__ double ld_s(const double* p) {
@@ -128,16 +128,25 @@ __device__ __forceinline__ double ld_s(const double* p) {
 
 struct NoLd {};
 
+// Asynchronous copies global -> shared, 16 bytes each: issued without a register round trip, complete at
+// cp_wait (this thread's copies; a barrier of the threads that read them makes them visible).
+__device__ __forceinline__ void cp16(void* s, const void* g) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" :: "r"((unsigned)__cvta_generic_to_shared(s)), "l"(g) : "memory");
+}
+__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+__device__ __forceinline__ void cp_wait() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
+
 // The packed lines of a unit's rows from their half spectra at src + kx ny: a thread loads the half
 // spectrum at its k < nx/2 once, keeps Z[k] and hands Z[nx - k] over through the shared buffer.
-template <typename T, int E>
-__device__ __forceinline__ void row_gather(CV<typename Lane<T>::V> (&v)[E], const Team<T, E>& t, const C2<T>* src, int nx, long long ny) {
+// ld(j, k) gives the 32 bytes at the thread's j-th k (j = E/2: k = nx/2, asked for by thread 0).
+template <typename T, int E, class Ld>
+__device__ __forceinline__ void row_gather_from(CV<typename Lane<T>::V> (&v)[E], const Team<T, E>& t, int nx, Ld ld) {
   const int q = t.step();
   t.sync();
 #pragma unroll
   for (int j = 0; j < E / 2; ++j) {
     const int k = t.i + j * q;
-    const auto s = ld_b32(src + k * ny);
+    const auto s = ld(j, k);
     if (k == 0) {
       v[j] = pack_re(s);
     } else {
@@ -145,14 +154,50 @@ __device__ __forceinline__ void row_gather(CV<typename Lane<T>::V> (&v)[E], cons
       t.at(nx - k) = pack_hi(s);
     }
   }
-  if (t.i == 0) t.at(nx >> 1) = pack_re(ld_b32(src + (nx >> 1) * ny));
+  if (t.i == 0) t.at(nx >> 1) = pack_re(ld(E / 2, nx >> 1));
   t.sync();
 #pragma unroll
   for (int j = E / 2; j < E; ++j) v[j] = t.at(t.i + j * q);
 }
+template <typename T, int E>
+__device__ __forceinline__ void row_gather(CV<typename Lane<T>::V> (&v)[E], const Team<T, E>& t, const C2<T>* src, int nx, int ny) {
+  row_gather_from(v, t, nx, [&](int, int k) { return ld_b32(src + k * ny); });
+}
+// The same from a copy in shared memory that row_stage issued for the group's 2^lgG neighbouring units:
+// their 2^lgG x 32 contiguous bytes at each k < nx/2, one k after the other (stg), and at nx/2 (top).
+// src: the spectra of the group's first unit.
+template <typename T, int E>
+__device__ __forceinline__ void row_stage(const Team<T, E>& t, int lgG, uint4* stg, uint4* top, const C2<T>* src, int nx, int ny) {
+  const int g = (t.i << lgG) + t.u;                // thread of the group
+  const int lgc = 1 + lgG;                         // 16-byte pieces per k
+  const char* const base = (const char*)src;
+#pragma unroll
+  for (int m = 0; m < E; ++m) {
+    const int e = g + (m << t.lgt), k = e >> lgc;
+    cp16(stg + e, base + k * (ny * (int)sizeof(C2<T>)) + ((e & ((1 << lgc) - 1)) << 4));
+  }
+  for (int e = g; e < (1 << lgc); e += 1 << t.lgt)
+    cp16(top + e, base + (nx >> 1) * (ny * (int)sizeof(C2<T>)) + (e << 4));
+  cp_commit();
+}
+__device__ __forceinline__ B32f staged_b32(const uint4* a, const C2<float>*) {
+  const float4 x = *(const float4*)a, y = *(const float4*)(a + 1);
+  return B32f{{x.x, x.y, x.z, x.w, y.x, y.y, y.z, y.w}};
+}
+__device__ __forceinline__ B32d staged_b32(const uint4* a, const C2<double>*) {
+  const double2 x = *(const double2*)a, y = *(const double2*)(a + 1);
+  return B32d{{x.x, x.y, y.x, y.y}};
+}
+template <typename T, int E>
+__device__ __forceinline__ void row_gather_staged(CV<typename Lane<T>::V> (&v)[E], const Team<T, E>& t, int lgG, const uint4* stg, const uint4* top, int nx) {
+  cp_wait();                                       // (the gather's first barrier makes the copies visible)
+  row_gather_from(v, t, nx, [&](int j, int k) {
+    return staged_b32((j < E / 2 ? stg + (k << (1 + lgG)) : top) + 2 * t.u, (const C2<T>*)nullptr);
+  });
+}
 // The reverse: (twice) the half spectra of a unit's rows from the packed lines' transform.
 template <typename T, int E>
-__device__ __forceinline__ void row_scatter(CV<typename Lane<T>::V> (&v)[E], const Team<T, E>& t, C2<T>* dst, int nx, long long ny, bool mine) {
+__device__ __forceinline__ void row_scatter(CV<typename Lane<T>::V> (&v)[E], const Team<T, E>& t, C2<T>* dst, int nx, int ny, bool mine) {
   const int q = t.step();
   t.sync();
 #pragma unroll
