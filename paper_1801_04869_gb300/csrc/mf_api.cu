@@ -6,6 +6,7 @@
 #include <initializer_list>
 #include <cstdio>
 #include <cstring>
+#include <mutex>
 #include <string>
 #include <queue>
 #include <utility>
@@ -28,9 +29,12 @@ struct mf_problem {
   size_t ws_bytes;
   size_t used;
   double* scratch_m;            // device scalar(s) for moment readouts (in the workspace)
+  SolverState* mirror = nullptr;  // host copy of the solver state, written by the kernels; or null
+  bool mirror_ok = false;         // it is current (no launch or device write since)
   std::string err;
   bool have_knots;
   double batch_work = 0.0;      // field passes per step attempt in the last mf_advance_batch
+  ~mf_problem();
 };
 
 namespace mf {
@@ -182,20 +186,72 @@ mf_status cuda_fail(mf_problem* pb, cudaError_t e, const char* what) {
     if (r_ != MF_OK) return r_;      \
   } while (0)
 
+// Pinned, mapped blocks for the problems' host copies of the solver state: slabs of 256 blocks, at most
+// 64 of them, kept for the process; a problem takes a block at mf_create and gives it back at mf_destroy
+// (allocating and freeing pinned memory per problem would synchronise the device).  When none is left a
+// problem does without and copies the state from the device.
+struct StatePool {
+  static constexpr size_t BLOCK = 256, PER_SLAB = 256, MAX_SLABS = 64;
+  static_assert(sizeof(SolverState) <= BLOCK, "block size");
+  std::mutex m;
+  std::vector<void*> free;
+  size_t slabs = 0;
+  SolverState* take() {
+    std::lock_guard<std::mutex> lock(m);
+    if (free.empty() && slabs < MAX_SLABS) {
+      void* p = nullptr;
+      if (cudaHostAlloc(&p, BLOCK * PER_SLAB, cudaHostAllocPortable | cudaHostAllocMapped) == cudaSuccess) {
+        ++slabs;
+        for (size_t i = PER_SLAB; i-- > 0;) free.push_back((char*)p + i * BLOCK);
+      } else {
+        cudaGetLastError();
+      }
+    }
+    if (free.empty()) return nullptr;
+    void* b = free.back();
+    free.pop_back();
+    return (SolverState*)b;
+  }
+  void give(SolverState* b) {
+    if (!b) return;
+    std::lock_guard<std::mutex> lock(m);
+    free.push_back(b);
+  }
+};
+StatePool& state_pool() {
+  static StatePool* p = new StatePool();     // outlives every problem, also those destroyed at exit
+  return *p;
+}
+
+// The solver state as of the problem's last finished work.
 mf_status read_state(mf_problem* pb, SolverState* s) {
+  if (pb->mirror_ok) {
+    std::memcpy(s, pb->mirror, sizeof(SolverState));
+    return MF_OK;
+  }
   MF_CUDA(pb, cudaMemcpyAsync(s, pb->d.st, sizeof(SolverState), cudaMemcpyDeviceToHost, pb->stream));
   MF_CUDA(pb, cudaStreamSynchronize(pb->stream));
+  if (pb->mirror) {
+    std::memcpy(pb->mirror, s, sizeof(SolverState));
+    pb->mirror_ok = true;
+  }
   return MF_OK;
 }
 mf_status write_state(mf_problem* pb, const SolverState* s) {
+  pb->mirror_ok = false;
   MF_CUDA(pb, cudaMemcpyAsync(pb->d.st, s, sizeof(SolverState), cudaMemcpyHostToDevice, pb->stream));
   MF_CUDA(pb, cudaStreamSynchronize(pb->stream));
+  if (pb->mirror) {
+    std::memcpy(pb->mirror, s, sizeof(SolverState));
+    pb->mirror_ok = true;
+  }
   return MF_OK;
 }
 
 // enqueue one persistent launch on the problem's stream (no wait)
 mf_status launch_enqueue(mf_problem* pb, const KernelArgs& a) {
   MF_CUDA(pb, cudaSetDevice(pb->device));
+  pb->mirror_ok = false;
   MF_CUDA(pb, cudaMemsetAsync(pb->d.gb, 0, sizeof(GridBarrier), pb->stream));
   cudaError_t e = pb->d.dim == 2 ? film_launch(pb->d.precision, pb->d, a, pb->stream)
                                  : bulk_launch(pb->d.precision, pb->d, a, pb->stream);
@@ -205,6 +261,8 @@ mf_status launch_enqueue(mf_problem* pb, const KernelArgs& a) {
 // wait for the problem's stream and turn the kernel's sticky status into the return value
 mf_status launch_finish(mf_problem* pb) {
   SolverState s;
+  MF_CUDA(pb, cudaStreamSynchronize(pb->stream));
+  pb->mirror_ok = pb->mirror != nullptr;
   mf_status r = read_state(pb, &s);
   if (r != MF_OK) return r;
   if (s.status != ST_OK) {
@@ -223,6 +281,8 @@ mf_status launch(mf_problem* pb, const KernelArgs& a) {
 }
 
 }  // namespace
+
+mf_problem::~mf_problem() { state_pool().give(mirror); }
 
 extern "C" {
 
@@ -262,6 +322,7 @@ mf_status mf_create(const mf_params* p, void* d_workspace, size_t bytes, void* s
   pb->ws_bytes = bytes;
   pb->used = L.total;
   if (cudaGetDevice(&pb->device) != cudaSuccess) { delete pb; return MF_ERR_CUDA; }
+  pb->mirror = state_pool().take();
 
   const int nz = p->dim == 2 ? 1 : p->nz;
   Desc& d = pb->d;
@@ -295,6 +356,7 @@ mf_status mf_create(const mf_params* p, void* d_workspace, size_t bytes, void* s
   d.partials = (double*)(w + L.partials);
   d.max_items = L.max_items;
   d.st = (SolverState*)(w + L.st);
+  d.host_st = pb->mirror;
   d.gb = (GridBarrier*)(w + L.gb);
   d.log = (StepLog*)(w + L.log);
   d.log_cap = LOG_CAP;
@@ -565,6 +627,7 @@ static void advance_films_together(mf_problem* const* pbs, const std::vector<int
     for (int k : order) {
       if (launch[k] != j) continue;
       mf_problem* f = pbs[live[k]];
+      f->mirror_ok = false;
       if (e == cudaSuccess) e = cudaMemsetAsync(f->d.gb, 0, sizeof(GridBarrier), s);
       tab.job[tab.n++] = BatchJob{f->d.dev, t_targets[live[k]], max_attempts, b, ctas[k]};
       b += ctas[k];
@@ -934,6 +997,7 @@ mf_status mf_checkpoint_restore(mf_problem* pb, const void* src) {
     pb->err = "checkpoint does not match this problem (grid, dimension or precision)";
     return MF_ERR_ARG;
   }
+  pb->mirror_ok = false;
   const char* i = (const char*)src + sizeof(h);
   for (const auto& x : ckpt_regions(pb)) {
     if (void* rows = ckpt_rows(pb, x.first)) {
@@ -968,6 +1032,7 @@ static mf_status film_adjoint(mf_problem* pb, int iters, const double* d_v, doub
     return MF_ERR_ARG;
   }
   MF_CUDA(pb, cudaSetDevice(pb->device));
+  pb->mirror_ok = false;
   MF_CUDA(pb, cudaMemsetAsync(pb->d.gb, 0, sizeof(GridBarrier), pb->stream));
   cudaError_t e = film_adjoint_launch(pb->d.precision, pb->d, d_v, d_hin_bar, pb->scratch_m, iters,
                                       d_g, d_gbar, d_jcbar, d_wbar_out, d_wbar_in, pb->stream);
@@ -1285,6 +1350,6 @@ mf_status mf_get_log(mf_problem* pb, mf_step_log* out, long long cap, long long*
 
 const char* mf_last_error(const mf_problem* pb) { return pb ? pb->err.c_str() : "null handle"; }
 
-void mf_destroy(mf_problem* pb) { delete pb; }
+void mf_destroy(mf_problem* pb) { delete pb; }     // (its destructor gives the state block back)
 
 }  // extern "C"

@@ -893,6 +893,7 @@ __global__ void __launch_bounds__(NT, 2) bulk_kernel(const Desc* __restrict__ dg
   if (leader) {
     st->warm_valid = sh.warm_valid;
     st->status = status;
+    publish_state(d, st);
   }
 }
 

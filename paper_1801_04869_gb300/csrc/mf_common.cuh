@@ -131,6 +131,7 @@ struct Desc {
   double* partials;              // per-work-item partial reductions
   int max_items;
   SolverState* st;
+  SolverState* host_st;          // the host's copy of *st (pinned, mapped), written at the end of a launch; or null
   GridBarrier* gb;
   StepLog* log;
   long long log_cap;
@@ -141,6 +142,20 @@ struct Desc {
   unsigned long long barrier_ns; // time limit of one grid-barrier wait (ns)
   const struct Desc* dev;        // device copy of this descriptor (what the kernels read)
 };
+
+// The leader's last act in a launch: the solver state into the host's copy, which the host reads once
+// the stream has drained (a separate device-to-host copy costs it 5 to 10 us per call).
+__device__ __forceinline__ void publish_state(const Desc& d, const SolverState* st) {
+  if (!d.host_st) return;
+  static_assert(sizeof(SolverState) % 8 == 0, "copied by 8-byte words");
+  const volatile unsigned long long* s = (const volatile unsigned long long*)st;
+  volatile unsigned long long* h = (volatile unsigned long long*)d.host_st;
+  unsigned long long w[sizeof(SolverState) / 8];
+#pragma unroll
+  for (int k = 0; k < (int)(sizeof(SolverState) / 8); ++k) w[k] = s[k];
+#pragma unroll
+  for (int k = 0; k < (int)(sizeof(SolverState) / 8); ++k) h[k] = w[k];
+}
 
 // ------------------------------------------------------------------------------------------
 // bounded grid barrier for cooperative launches.  Every CTA is co-resident (cooperative

@@ -1014,6 +1014,7 @@ __device__ __forceinline__ void film_main(const Desc& d, const KernelArgs& a, in
     st->hd_sel = sh.hd_sel;
     st->A_com = sh.A_com;
     st->status = status;
+    publish_state(d, st);
   }
 }
 

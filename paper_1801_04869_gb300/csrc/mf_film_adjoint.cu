@@ -391,6 +391,7 @@ __global__ void __launch_bounds__(NT, FILM_CTAS) film_adjoint_kernel(const Desc*
     *a.sbar = sbar;
     st->warm_valid = 0; st->com_valid = 0; st->hd_sel = 0; st->A_prev = 0.0; st->A_com = 0.0;
     st->status = status;
+    publish_state(d, st);
   }
 }
 
