@@ -245,17 +245,17 @@ struct Bulk {
   // fill(epi) sets the epilogue's members
   template <template <class, int> class EPI, bool NIN, bool NOUT, class Fill>
   __device__ __forceinline__ void xpass(Fill fill, int slot = -1) {
-    constexpr int SMALL = sizeof(T) == 4 ? 4 : 2;
-    if (ex == SMALL) {
-      EPI<T, SMALL> e;
+    constexpr int FEW = sizeof(T) == 4 ? 4 : 2, MANY = 2 * FEW;
+    if (ex == FEW) {
+      EPI<T, FEW> e;
       e.P = ptrs();
       fill(e);
-      xpass_e<SMALL, NIN, NOUT>(e, slot);
+      xpass_e<FEW, NIN, NOUT>(e, slot);
     } else {
-      EPI<T, 8> e;
+      EPI<T, MANY> e;
       e.P = ptrs();
       fill(e);
-      xpass_e<8, NIN, NOUT>(e, slot);
+      xpass_e<MANY, NIN, NOUT>(e, slot);
     }
   }
   __device__ double total(int slot, bool is_max = false) {
@@ -319,7 +319,7 @@ struct Bulk {
     }
   }
   template <int DIR> __device__ __forceinline__ void ypass() {
-    if (ey == 4) ypass_e<4, DIR>();
+    if (sizeof(T) == 8 || ey == 4) ypass_e<4, DIR>();
     else ypass_e<8, DIR>();
   }
 

@@ -262,7 +262,7 @@ struct Film {
   template <int NIN, int NOUT>
   __device__ __forceinline__ void cols_n(const C2<T>* Sin, C2<T>* Sout, int op) {
     if (ey == 2) cols_e<2, NIN, NOUT>(Sin, Sout, op);
-    else if (sizeof(T) == 4 && ey == 4) cols_e<(sizeof(T) == 4 ? 4 : 2), NIN, NOUT>(Sin, Sout, op);
+    else if (ey == 4) cols_e<4, NIN, NOUT>(Sin, Sout, op);
     else cols_e<8, NIN, NOUT>(Sin, Sout, op);
   }
   __device__ __forceinline__ void cols(const C2<T>* Sin, int nin, C2<T>* Sout, int nout, int op) {
@@ -400,7 +400,7 @@ struct Film {
   template <int NIN, int NOUT, class Epi>
   __device__ __forceinline__ void rows(const C2<T>* Sin, C2<T>* Sout, const Epi& epi, int slot, int slot2 = -1, T* tmp = nullptr) {
     if (ex == 2) rows_e<2, NIN, NOUT>(Sin, Sout, epi, slot, slot2, tmp);
-    else if (sizeof(T) == 4 && ex == 4) rows_e<(sizeof(T) == 4 ? 4 : 2), NIN, NOUT>(Sin, Sout, epi, slot, slot2, tmp);
+    else if (ex == 4) rows_e<4, NIN, NOUT>(Sin, Sout, epi, slot, slot2, tmp);
     else rows_e<8, NIN, NOUT>(Sin, Sout, epi, slot, slot2, tmp);
   }
   // Sums over the units of slots a and (b >= 0) b, in a fixed order: the last warps first, which have

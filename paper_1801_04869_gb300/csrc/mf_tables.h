@@ -55,30 +55,37 @@ inline void film_shape(Desc& d, int coresident) {
 //   FP64: an FP64 instruction occupies an SM sub-partition for 64 cycles whatever the number of
 //     active lanes, so while E = 2 gives at most one warp per sub-partition (256^2 cells: 512 warps
 //     on 608) the pass takes a quarter of the instructions of E = 8.  One right-hand side with 4 / 5 /
-//     5 iterations at 64^2 / 128^2 / 256^2: 202 / 251 / 288 us against 389 / 514 / 550 us.
+//     5 iterations at 64^2 / 128^2 / 256^2: 202 / 251 / 288 us against 389 / 514 / 550 us.  E = 4 above:
+//     512 x 256 / 512^2 / 1024^2 427 / 540 / 2070 us against 441 / 570 us with E = 2 (lines of up to 512
+//     points) and, with E = 8, 625 us at 512^2 and 2082 us at 1024^2.
 //   FP32: E = 4 up to 2^20 cells (1024^2: 256 lines of 256 threads): 64^2 / 512^2 / 1024^2 with 5
 //     iterations 171 / 216 / 304 us against 230 / 240 / 339 us with E = 8; lines of 2048 points would
 //     need 512 threads.
 inline int elems_per_thread(const Desc& d, int n) {
   const long long cells = (long long)d.nx * d.ny;
-  if (d.precision == 0) return cells <= 65536 && n <= 2 * NT ? 2 : 8;
+  if (d.precision == 0) return cells <= 65536 && n <= 2 * NT ? 2 : n <= 4 * NT ? 4 : 8;
   return cells <= 1048576 && n <= 4 * NT ? 4 : 8;
 }
 
-// Elements per thread and items of a bulk body's passes.
-//   x: E = 8 (two exchanges per transform up to 512 points); E = 4 (FP32, to 64^3) or 2 (FP64, to 2^16
-//      cells) where a pass does not fill the chip and one thread's chain of instructions sets its time.
-//   y: E = 16 in FP32 (64 data registers, nothing else live: one exchange for lines of up to 256 points),
-//      8 in FP64; 4 for small bodies and lines shorter than E.
-//   z: three components are transformed together, so E = 4 (48 data registers); 2 for small FP64 bodies.
+// Elements per thread and items of a bulk body's passes (the kernel has E = 4 / 8 in FP32, 2 / 4 in FP64
+// along x, 4 and in FP32 8 along y, 4 and in FP64 2 along z).  Few elements where a pass does not fill
+// the chip and one thread's chain of instructions sets its time, more (fewer exchanges) where the passes
+// stream.  One right-hand side with 4 iterations, in us, with the smaller against the larger E:
+//   x FP32: 4 to 2^21 cells: 128 x 64 x 64 / 128^3 588 / 1098 against 718 / 1175; 256 x 128 x 128 / 256^3
+//     2140 / 8752 against 2004 / 7799.
+//   x FP64: 2 to 2^18 cells: 64^3 1363 against 1437 (1822 with 8: an item of 64^3 is 4 row units of 8
+//     threads then, one warp in a CTA, and three sub-partitions idle); 128 x 64 x 64 / 128 x 128 x 64 2358 /
+//     4738 against 2339 / 4580 (4725 with 8).
+//   y FP32: 4 to 2^18 cells: 64^3 460 against 467; 128 x 64 x 64 / 256^3 602 / 8534 against 588 / 7799.
+//   y FP64: 4: 64 x 64 x 32 / 128 x 128 x 64 / 128^3 823 / 4725 / 9345 against 863 / 4827 / 9712 with 8.
+//   z: three components are transformed together, so 4 (48 data registers); 2 for FP64 to 2^16 cells.
 // An x item is a block of row units whose residual is summed together: as many as fill a CTA, but at
 // least 304 items (two CTAs on each of 152 SMs), whatever the launch width, so that it changes nothing.
 inline void bulk_shape(Desc& d, int coresident) {
   const bool f32 = d.precision != 0;
-  const bool small = d.ncell <= (f32 ? 262144 : 65536);
-  d.ex = small ? (f32 ? 4 : 2) : 8;
-  d.ey = small ? 4 : 8;
-  d.ez = !f32 && small && d.nz <= 2 * NT ? 2 : 4;
+  d.ex = f32 ? (d.ncell <= 2097152 ? 4 : 8) : (d.ncell <= 262144 ? 2 : 4);
+  d.ey = f32 && d.ncell > 262144 ? 8 : 4;
+  d.ez = !f32 && d.ncell <= 65536 ? 2 : 4;
   const int ru = row_unit(d.precision);
   const long long units = (long long)d.nz * d.ny / ru;
   long long ub = NT / (d.nx / d.ex);
