@@ -173,3 +173,21 @@ def test_film_elliptic_law_rhs_vjp(precision, tol):
     assert rel_l2(gb.cpu().numpy(), gb_ref) < tol
     assert rel_l2(cb.cpu().numpy(), cb_ref) < tol
     assert abs(sb - sb_ref) <= tol * abs(sb_ref)
+
+
+@pytest.mark.parametrize("jc", [1.0, 1.7])
+@pytest.mark.parametrize("n", [1.0, 2.0, 3.0, 4.5, 30.0, 129.0, 130.0])
+@pytest.mark.parametrize("precision", [0, 1])
+def test_film_electric_field_readout_over_exponents(precision, n, jc):
+    """Whole exponents up to 129 take products in double, the others and single precision pow; the law's
+    relative error is (n - 1) times that of |j|, which the transforms leave near 1e-15 (2e-7): below
+    1e-9, and in single precision below 2e-6 (n + 1)."""
+    wl = film_workload(64, 64, L=(2.0, 2.0), shape="disk", radius=0.8, n=n, jc=jc, rho_out=5.0,
+                       precision=precision)
+    g = W.film_state(wl.mask, wl.Lx, wl.Ly, seed=31, amplitude=0.8)
+    o = oracle_of(wl)
+    p = native.from_workload(wl)
+    out = torch.zeros((2, wl.ny, wl.nx), dtype=torch.float64, device="cuda")
+    p.mf_readout(native.MF_READ_E, out=out, t=0.3, y=dev(g))
+    err = rel_l2(out.cpu().numpy(), np.stack(o.electric_field(*o.sheet_current(g))))
+    assert err < (TOL64 if precision == 0 else 2e-6 * (n + 1.0)), err
