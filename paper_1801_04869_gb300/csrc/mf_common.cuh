@@ -300,21 +300,21 @@ size_t kernel_smem_bytes(const Desc& d);
 
 // Entries (16 bytes each) of the core's twiddle table of length 2^lg for E elements per thread
 __host__ __device__ constexpr int core_table_len(int lg, int E) {
-  const int e = E == 2 ? 1 : E == 4 ? 2 : E == 8 ? 3 : 4;
+  const int e = E == 2 ? 1 : E == 4 ? 2 : 3;
   int n = 0, lgp = e;
   for (int rem = lg - e; rem > 0; rem -= e, lgp += e) n += rem >= e ? e << lgp : rem << (lg - e);
   return n;
 }
 // Elements from one line's exchange buffer to the next when 2^lgG lines are interleaved on the lanes: the
-// padded length (one spare slot per 8, or per 16 with radix 16), and 8 / lines more where that is a
+// padded length (one spare slot per 8), and 8 / lines more where that is a
 // multiple of 4, so that the lines of 8 neighbouring lanes lie on distinct banks.
-__host__ __device__ constexpr int line_stride(int lg, int lgG, int E) {
-  return (1 << lg) + ((1 << lg) >> (E == 16 ? 4 : 3)) + (lgG > 0 && lg >= 5 ? 8 >> lgG : 0);
+__host__ __device__ constexpr int line_stride(int lg, int lgG) {
+  return (1 << lg) + ((1 << lg) >> 3) + (lgG > 0 && lg >= 5 ? 8 >> lgG : 0);
 }
 // Rows of the real fields that a film's row passes keep together (mf_film.cuh)
 __host__ __device__ constexpr int row_unit(int precision) { return precision ? 4 : 2; }
 // a film's shared memory: the exchange buffer's elements, then the tables (one if the axes agree)
-__host__ __device__ constexpr int slots_of(int E) { return NT * E + (NT * E >> (E == 16 ? 4 : 3)); }
+__host__ __device__ constexpr int slots_of(int E) { return NT * E + NT * E / 8; }
 __host__ __device__ inline int film_slots(const Desc& d) { return slots_of(d.ex > d.ey ? d.ex : d.ey); }
 __host__ __device__ inline bool one_table(const Desc& d) { return d.lgx == d.lgy && d.ex == d.ey; }
 // the most that any film needs (what the kernels' attribute is set to, whatever is launched first)
@@ -337,10 +337,10 @@ __host__ __device__ inline int x_group_lg(const Desc& d) {
 // Shared memory of the passes (16-byte elements): the exchange buffers, the staging buffer behind them
 // (x: E per thread and two per line; y: E per thread; z: 3 E per thread), in the x pass E per thread for
 // partial residuals; the tables follow the largest of the three.
-__host__ __device__ constexpr int x_slots(int lgx, int ex) { return ((NT * ex) >> lgx) * line_stride(lgx, 2, ex); }
+__host__ __device__ constexpr int x_slots(int lgx, int ex) { return ((NT * ex) >> lgx) * line_stride(lgx, 2); }
 __host__ __device__ constexpr int x_stage(int lgx, int ex) { return NT * ex + 2 * ((NT * ex) >> lgx); }
 __host__ __device__ constexpr int z_slots(int lgz, int ez) {
-  return 3 * ((NT * ez) >> lgz) * line_stride(lgz, z_group_lg(lgz, ez), ez);
+  return 3 * ((NT * ez) >> lgz) * line_stride(lgz, z_group_lg(lgz, ez));
 }
 __host__ __device__ inline int bulk_slots(const Desc& d) {
   const int x = x_slots(d.lgx, d.ex) + x_stage(d.lgx, d.ex) + NT * d.ex;

@@ -68,10 +68,10 @@ template <class V> __device__ __forceinline__ CV<V> ezero();
 template <> __device__ __forceinline__ CV<F2> ezero<F2>() { return {F2{0ull}, F2{0ull}}; }
 template <> __device__ __forceinline__ CV<double> ezero<double>() { return {0.0, 0.0}; }
 
-// Shared-memory position of element e of a line: one spare slot per 8 (radix 16: per 16) keeps the
+// Shared-memory position of element e of a line: one spare slot per 8 keeps the
 // 16-byte accesses of 8 consecutive lanes (one wavefront) on distinct banks for every stage's
 // writes and reads.
-template <int E> __host__ __device__ __forceinline__ constexpr int spe(int e) { return e + (e >> (E == 16 ? 4 : 3)); }
+__host__ __device__ __forceinline__ constexpr int spe(int e) { return e + (e >> 3); }
 // ------------------------------------------------------------------------------------------
 // butterflies
 // ------------------------------------------------------------------------------------------
@@ -148,13 +148,6 @@ template <int DIR, class V> __device__ __forceinline__ void bf_oct3(CV<V>& a, CV
   }
 }
 
-// w (c + DIR i s)
-template <int DIR, class V> __device__ __forceinline__ Tw<V> tw_rot(const Tw<V>& w, double c, double s) {
-  const V vc = vconst(c, (V*)nullptr), vs = vconst(DIR * s, (V*)nullptr), ns = vconst(-DIR * s, (V*)nullptr);
-  const V y = vfma(w.y, vc, vmul(w.x, vs));
-  return {vfma(w.x, vc, vmul(w.y, ns)), y, vneg(y)};
-}
-
 __host__ __device__ constexpr int bitrev(int j, int r) {
   int o = 0;
   for (int k = 0; k < r; ++k) { o = (o << 1) | (j & 1); j >>= 1; }
@@ -169,7 +162,6 @@ __host__ __device__ constexpr int bitrev(int j, int r) {
 template <int DIR, int E, int r, bool FIRST, class V>
 __device__ __forceinline__ void dft_stage(CV<V>* x, const CV<V>* w) {
   constexpr int R = 1 << r, NS = E >> r;
-  constexpr double c1 = 0.92387953251128675613, s1 = 0.38268343236508977173;   // pi/8
   CV<V> y[E];                          // set s at y[s R ..], bit-reversed
 #pragma unroll
   for (int s = 0; s < NS; ++s) {
@@ -183,11 +175,6 @@ __device__ __forceinline__ void dft_stage(CV<V>* x, const CV<V>* w) {
     if constexpr (!FIRST) {
       t[0] = mk_tw<DIR>(w[r - l]);
       if constexpr (E == 8) t[1] = tw_oct<DIR>(t[0]);
-      if constexpr (E == 16) {
-        t[1] = tw_rot<DIR>(t[0], c1, s1);
-        t[2] = tw_oct<DIR>(t[0]);
-        t[3] = tw_rot<DIR>(t[0], s1, c1);
-      }
     }
 #pragma unroll
     for (int s = 0; s < NS; ++s) {
@@ -201,15 +188,11 @@ __device__ __forceinline__ void dft_stage(CV<V>* x, const CV<V>* w) {
         if (E == 2 || c < Q) {
           if (!FIRST) bf_tw(p, q, t[c % Q]);
           else if (c == 0) bf(p, q);
-          else if (2 * c == Q) bf_oct<DIR>(p, q);
-          else bf_tw(p, q, c == 1 ? Tw<V>{vconst(c1, (V*)nullptr), vconst(DIR * s1, (V*)nullptr), vconst(-DIR * s1, (V*)nullptr)}
-                                  : Tw<V>{vconst(s1, (V*)nullptr), vconst(DIR * c1, (V*)nullptr), vconst(-DIR * c1, (V*)nullptr)});
+          else bf_oct<DIR>(p, q);
         } else {
           if (!FIRST) bf_tw_i<DIR>(p, q, t[c % Q]);
           else if (c == Q) bf_i<DIR>(p, q);
-          else if (2 * c == 3 * Q) bf_oct3<DIR>(p, q);
-          else bf_tw_i<DIR>(p, q, c - Q == 1 ? Tw<V>{vconst(c1, (V*)nullptr), vconst(DIR * s1, (V*)nullptr), vconst(-DIR * s1, (V*)nullptr)}
-                                             : Tw<V>{vconst(s1, (V*)nullptr), vconst(DIR * c1, (V*)nullptr), vconst(-DIR * c1, (V*)nullptr)});
+          else bf_oct3<DIR>(p, q);
         }
       }
     }
@@ -224,7 +207,7 @@ __device__ __forceinline__ void dft_stage(CV<V>* x, const CV<V>* w) {
 // ------------------------------------------------------------------------------------------
 // the threads that share one line
 // ------------------------------------------------------------------------------------------
-__host__ __device__ constexpr int lg_of(int E) { return E == 2 ? 1 : E == 4 ? 2 : E == 8 ? 3 : 4; }
+__host__ __device__ constexpr int lg_of(int E) { return E == 2 ? 1 : E == 4 ? 2 : 3; }
 
 // A group of G = 2^lgG lines (neighbours in memory) is interleaved on the lanes: thread i of line u is
 // thread (i << lgG) + u of the group, so that a warp moves G neighbouring values per position.  A group
@@ -242,13 +225,13 @@ template <typename T, int E> struct Team {
     u = (int)threadIdx.x & ((1 << lgG) - 1);
     i = ((int)threadIdx.x >> lgG) & ((1 << (lg - LGE)) - 1);
     slot = (((int)threadIdx.x >> lgt) << lgG) + u;
-    const int stride = line_stride(lg, lgG, E);
+    const int stride = line_stride(lg, lgG);
     s = buf + slot * stride;
     fs = ((NT >> lgt) << lgG) * stride;
   }
   __device__ __forceinline__ int threads() const { return 1 << (lg - LGE); }
   __device__ __forceinline__ int step() const { return 1 << (lg - LGE); }    // position stride of a thread's elements
-  __device__ __forceinline__ CV<V>& at(int e) const { return s[spe<E>(e)]; }
+  __device__ __forceinline__ CV<V>& at(int e) const { return s[spe(e)]; }
   __device__ __forceinline__ void sync() const {
     if (lgt <= 5) __syncwarp();
     else asm volatile("bar.sync %0, %1;" :: "r"(1 + ((int)threadIdx.x >> lgt)), "r"(1 << lgt) : "memory");
@@ -259,7 +242,7 @@ template <typename T, int E> struct Team {
 // buffer starts f t.fs elements behind the first one's), unnormalised.
 template <int DIR, int NF, class V, int E, class TM>
 __device__ __forceinline__ void core_fft_n(CV<V> (&v)[NF][E], const TM& t) {
-  constexpr int e = lg_of(E), PAD = E == 16 ? 4 : 3;
+  constexpr int e = lg_of(E);
 #pragma unroll
   for (int f = 0; f < NF; ++f) dft_stage<DIR, E, e, true>(v[f], (const CV<V>*)nullptr);
   const int q = 1 << (t.lg - e), i = t.i;
@@ -270,16 +253,16 @@ __device__ __forceinline__ void core_fft_n(CV<V> (&v)[NF][E], const TM& t) {
     const int p = 1 << lgp;
     t.sync();
     if (lgp == e && E >= 8) {
-      CV<V>* const w = t.s + (i << e) + ((i << e) >> PAD);
+      CV<V>* const w = t.s + (i << e) + ((i << e) >> 3);
 #pragma unroll
       for (int f = 0; f < NF; ++f) {
 #pragma unroll
         for (int r = 0; r < E; ++r) w[f * t.fs + r] = v[f][r];
       }
-    } else if (lgp >= e + PAD) {
+    } else if (lgp >= e + 3) {
       const int pp = p >> e, kp = i & (pp - 1);
       CV<V>* const w = &t.at(((i - kp) << e) + kp);
-      const int ws = pp + (pp >> PAD);
+      const int ws = pp + (pp >> 3);
 #pragma unroll
       for (int f = 0; f < NF; ++f) {
 #pragma unroll
@@ -295,9 +278,9 @@ __device__ __forceinline__ void core_fft_n(CV<V> (&v)[NF][E], const TM& t) {
       }
     }
     t.sync();
-    if (q >= (1 << PAD)) {
+    if (q >= 8) {
       const CV<V>* const rd = &t.at(i);
-      const int rds = q + (q >> PAD);
+      const int rds = q + (q >> 3);
 #pragma unroll
       for (int f = 0; f < NF; ++f) {
 #pragma unroll
@@ -319,10 +302,6 @@ __device__ __forceinline__ void core_fft_n(CV<V> (&v)[NF][E], const TM& t) {
       tw += e << lgp;
 #pragma unroll
       for (int f = 0; f < NF; ++f) dft_stage<DIR, E, e, false>(v[f], w);
-    } else if (e > 3 && rem == 3) {
-      const CV<V> w[3] = {tw[i], tw[q + i], tw[2 * q + i]};
-#pragma unroll
-      for (int f = 0; f < NF; ++f) dft_stage<DIR, E, (e > 3 ? 3 : 1), false>(v[f], w);
     } else if (e > 2 && rem == 2) {
       const CV<V> w[2] = {tw[i], tw[q + i]};
 #pragma unroll
