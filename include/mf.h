@@ -310,8 +310,8 @@ mf_status mf_checkpoint_restore(mf_problem* pb, const void* src);
 
 /* Result of mf_autotune. */
 typedef struct {
-  int rows_per_item;          /* rows of the film row passes / bulk x pass per work item */
-  int zs_per_item;            /* bulk y pass z-lines per item (films: two-field row pass rows) */
+  int rows_per_item;          /* rows per work item of the x pass */
+  int zs_per_item;            /* 1 (bulk bodies); films: the rows of a row unit */
   int grid;                   /* CTAs of the persistent launch */
   int candidates;             /* configurations timed */
   double ms_per_rhs;          /* best time of one right-hand side with the forced iterations */
@@ -321,7 +321,7 @@ typedef struct {
 /* Time one right-hand side of the current state (force_iters outside iterations, reps timed
    launches after one warm-up) for every work-item shape and launch width the kernels accept
    for this grid, and keep the fastest; *out (may be NULL) receives it.  The candidates are the
-   power-of-two rows (and z-lines) per item that fit the shared-memory batch, times the launch
+   power-of-two rows per x item of a bulk body that fit a CTA (a film's are fixed), times the launch
    widths {size rule, all co-resident CTAs, half of them}.  Results change at rounding level
    with the item shape (the reductions are summed per item), not with the launch width.  The
    state, step size and counters are kept; the warm start of the outside iteration and the

@@ -18,6 +18,14 @@
 //
 // The passes run on the transform core (mf_core.cuh); real fields and the mask lie by row units
 // (mf_units.cuh).
+//
+// What bounds the passes, and what they measured (one right-hand side with 4 outside iterations; the
+// design before kept two spectra per component and transformed 16 values per thread through two shared
+// buffers): 256^3 FP32 by memory latency at 16 warps per SM, with 8 bytes per cell and component moved
+// each way per pass (13.3 -> 7.8 ms), so that every pass brings its next unit's spectra to shared memory
+// with asynchronous copies while it works on this one; 128^3 FP32 by the chain of loads, exchanges and
+// barriers per unit (1.66 -> 1.10 ms); FP64 from 64^3 by the FP64 unit (64^3 1.64 -> 1.36 ms, 128^3 12.1 ->
+// 9.2 ms); 32^3 by the latencies of 42 phases (FP32 390 -> 318 us, FP64 940 -> 578 us).
 #include <type_traits>
 
 #include "mf_units.cuh"
@@ -98,7 +106,9 @@ struct Bulk {
 
   __device__ BulkPtrs<T> ptrs() const { return BulkPtrs<T>{mask, jcmap, hd, ncell, nx, ny}; }
 
-  // ---- x pass: items of ub row units; per unit the components one after the other: inverse (NIN),
+  // ---- x pass: up to 4 row units side by side on the lanes, so that a warp's accesses to the spectra
+  // are 128 contiguous bytes per kx (32 with one unit); the spectra arrive by asynchronous copies (both
+  // together: 256^3 FP32 8.28 -> 7.77 ms, 128^3 1.43 -> 1.19 ms).  Items of ub row units; per unit the components one after the other: inverse (NIN),
   // epilogue, forward (NOUT).  An epilogue that needs the three components of a cell together (kJoint)
   // lets the first two wait in `tmp` (the same thread's elements) while the third is transformed. ----
   template <int E, bool NIN, bool NOUT, class Epi>
@@ -323,7 +333,10 @@ struct Bulk {
     else ypass_e<8, DIR>();
   }
 
-  // ---- z pass: forward, 3x3 multiplier, inverse on groups of lines (kx, y0 ..) ----
+  // ---- z pass: forward, 3x3 multiplier, inverse on groups of lines (kx, y0 ..), the three components of
+  // a line in one thread's registers, so that the multiplier needs no exchange and the transforms share
+  // their barriers; bound by the exchanges through shared memory and their barriers (256^3 FP32: some
+  // 27 k cycles per group of 4 lines, of which the exchanges' bytes account for 11 k) ----
   static __device__ __forceinline__ CV<F2> ld_z(const float4& f) { return {pk(f.x, f.z), pk(f.y, f.w)}; }
   static __device__ __forceinline__ CV<double> ld_z(const double2& f) { return {f.x, f.y}; }
   static __device__ __forceinline__ void st_z(C2<float>* p, const CV<F2>& v) {

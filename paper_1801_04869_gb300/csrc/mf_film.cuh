@@ -27,10 +27,13 @@
 // What bounds a pass, and what it measured (one right-hand side, 5 outside iterations = 24 passes with
 // their grid barriers; the design before transformed through two shared buffers at 16 values per
 // thread): small grids are bound by one thread's chain of instructions, the barrier and the load
-// latencies (128^2: FP32 250 -> 190 us, FP64 514 -> 251 us); FP64 grids from 512^2 by the FP64 unit,
-// 2 lanes per cycle and SM (1024^2 2.85 -> 2.10 ms, 2048^2 11.2 -> 8.6 ms); 2048^2 FP32 by exchanges
-// through shared memory and their latencies (979 -> 786 us), 512^2 and 1024^2 by both (350 -> 216 us,
-// 513 -> 304 us).
+// latencies (128^2: FP32 250 -> 166 us, FP64 514 -> 227 us); FP64 grids from 512^2 by the FP64 unit,
+// 2 lanes per cycle and SM, and the last round of units, 513 columns on 152 SMs (1024^2 2.85 -> 2.04 ms,
+// 2048^2 11.2 -> 8.5 ms); 2048^2 FP32 by the latency of exchanges and loads at 16 warps per SM (979 -> 760
+// us), 512^2 and 1024^2 by both (350 -> 195 us, 513 -> 290 us).  What did not pay at 2048^2: spectra
+// staged asynchronously as in the bulk passes (823 us: most CTAs have one unit or two), a second exchange
+// buffer in place of every other barrier (755 us, but 64^2 FP64 176 -> 182 us), k_y and its Gaussian in
+// shared memory (767 us).
 #pragma once
 #include "mf_units.cuh"
 
@@ -1019,8 +1022,10 @@ __device__ __forceinline__ void film_main(const Desc& d, const KernelArgs& a, in
 }
 
 // CTAs per SM of the film kernels: 2 leave 128 registers per thread.  4 (64 registers) spill in every
-// pass (2048^2 FP32, 5 iterations: 922 us against 852 us on otherwise the same source); 3 leave the 513
-// line pairs of a 2048^2 pass 456 places (1193 us).
+// pass, 3 spill too and leave the 513 line pairs of a 2048^2 pass 456 places.  One right-hand side with 5
+// iterations, 2 / 3 / 4 per SM: 2048^2 FP32 759 / 1120 / 935 us, 1024^2 FP32 289 / 312 / 333 us, 1024^2 FP64
+// 2080 / 2997 us.  A shared launch of 24 / 8 films of up to 128^2 cells with 3 per SM: FP32 5.1 / 2.7 ms
+// against 5.5 / 2.3 ms, FP64 24.4 / 10.6 ms against 23.9 / 8.7 ms.
 constexpr int FILM_CTAS = 2;
 
 }  // namespace mf
