@@ -300,9 +300,9 @@ size_t kernel_smem_bytes(const Desc& d);
 
 // Entries (16 bytes each) of the core's twiddle table of length 2^lg for E elements per thread
 __host__ __device__ constexpr int core_table_len(int lg, int E) {
-  const int e = E == 2 ? 1 : E == 4 ? 2 : 3;
+  const int e = E == 2 ? 1 : E == 4 ? 2 : 3, x = E == 8 ? 1 : 0;
   int n = 0, lgp = e;
-  for (int rem = lg - e; rem > 0; rem -= e, lgp += e) n += rem >= e ? e << lgp : rem << (lg - e);
+  for (int rem = lg - e; rem > 0; rem -= e, lgp += e) n += rem >= e ? (e + x) << lgp : (rem + x) << (lg - e);
   return n;
 }
 // Elements from one line's exchange buffer to the next when 2^lgG lines are interleaved on the lanes: the

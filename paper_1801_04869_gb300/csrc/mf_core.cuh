@@ -84,13 +84,6 @@ template <int DIR, class V> __device__ __forceinline__ Tw<V> mk_tw(const CV<V>& 
 }
 __device__ __forceinline__ double sqrt_half(double*) { return 0.70710678118654752440; }
 __device__ __forceinline__ F2 sqrt_half(F2*) { return pk(0.70710678118654752440f, 0.70710678118654752440f); }
-// w exp(DIR i pi/4)
-template <int DIR, class V> __device__ __forceinline__ Tw<V> tw_oct(const Tw<V>& w) {
-  const V h = sqrt_half((V*)nullptr);
-  const V a = vmul(w.x, h), b = vmul(w.y, h);
-  if (DIR > 0) { const V y = vadd(a, b); return {vsub(a, b), y, vneg(y)}; }
-  return {vadd(a, b), vsub(b, a), vsub(a, b)};
-}
 // (a, b) <- (a + w b, a - w b)
 __device__ __forceinline__ void bf_tw(CV<F2>& a, CV<F2>& b, const Tw<F2>& w) {
   const CV<F2> t = {vfma(w.x, b.x, vmul(w.ny, b.y)), vfma(w.x, b.y, vmul(w.y, b.x))};
@@ -174,7 +167,7 @@ __device__ __forceinline__ void dft_stage(CV<V>* x, const CV<V>* w) {
     Tw<V> t[E >= 8 ? E / 4 : 1];
     if constexpr (!FIRST) {
       t[0] = mk_tw<DIR>(w[r - l]);
-      if constexpr (E == 8) t[1] = tw_oct<DIR>(t[0]);
+      if constexpr (E == 8) t[1] = mk_tw<DIR>(w[r]);
     }
 #pragma unroll
     for (int s = 0; s < NS; ++s) {
@@ -242,7 +235,7 @@ template <typename T, int E> struct Team {
 // buffer starts f t.fs elements behind the first one's), unnormalised.
 template <int DIR, int NF, class V, int E, class TM>
 __device__ __forceinline__ void core_fft_n(CV<V> (&v)[NF][E], const TM& t) {
-  constexpr int e = lg_of(E);
+  constexpr int e = lg_of(E), X = E == 8 ? e + 1 : e;
 #pragma unroll
   for (int f = 0; f < NF; ++f) dft_stage<DIR, E, e, true>(v[f], (const CV<V>*)nullptr);
   const int q = 1 << (t.lg - e), i = t.i;
@@ -295,19 +288,19 @@ __device__ __forceinline__ void core_fft_n(CV<V> (&v)[NF][E], const TM& t) {
       }
     }
     if (rem >= e) {
-      CV<V> w[e];
+      CV<V> w[X];
       const int k = i & (p - 1);
 #pragma unroll
-      for (int m = 0; m < e; ++m) w[m] = tw[(m << lgp) + k];
-      tw += e << lgp;
+      for (int m = 0; m < X; ++m) w[m] = tw[(m << lgp) + k];
+      tw += X << lgp;
 #pragma unroll
       for (int f = 0; f < NF; ++f) dft_stage<DIR, E, e, false>(v[f], w);
     } else if (e > 2 && rem == 2) {
-      const CV<V> w[2] = {tw[i], tw[q + i]};
+      const CV<V> w[3] = {tw[i], tw[q + i], E == 8 ? tw[2 * q + i] : tw[i]};
 #pragma unroll
       for (int f = 0; f < NF; ++f) dft_stage<DIR, E, (e > 2 ? 2 : 1), false>(v[f], w);
     } else if (e > 1) {
-      const CV<V> w[1] = {tw[i]};
+      const CV<V> w[2] = {tw[i], E == 8 ? tw[q + i] : tw[i]};
 #pragma unroll
       for (int f = 0; f < NF; ++f) dft_stage<DIR, E, 1, false>(v[f], w);
     }
